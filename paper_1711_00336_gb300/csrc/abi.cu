@@ -53,7 +53,8 @@ template <typename FT>
 void launch_reaction_am(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename FT>
 void launch_reaction_drag(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
-void launch_dem_substep(const BoxDev *, const Tile *, int, int, int, int, int, int, int, int, cudaStream_t);
+void launch_dem_substep(const BoxDev *, const Tile *, int, int, int, int, int, int, int, cudaStream_t);
+void launch_dem_substep64(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
 void launch_build_nlist(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 long long scan_scratch_words(long long);
 void exclusive_scan(const int *, long long, int *, int *, cudaStream_t);
@@ -295,6 +296,7 @@ static void compute_phys(BoxHost *h) {
         p.kfac = (PI_H * PI_H + le * le) / (c.T_c * c.T_c);  // k_n / m_ij
         p.xfac = -2.0 * le / c.T_c;                          // xi_n / m_ij
         p.capfac = c.lub_cap / p.dt_dem;                     // lubrication cap / m_ij
+        p.fx = fx_box(h->d.g.n, h->dmin, h->dmax, c.h_c, c.h_min, p.mu);
     }
     // Verlet list: partners within (d_i+d_j)/2 + h_c + skin; linked cells of
     // +-R cells cover that range; particles may move skin/2 between sorts
@@ -599,23 +601,25 @@ static void enqueue_step(Batch *B) {
         tbegin(B);
         int ndl = 0;
         if (pl)
-            for (int sd = 0; sd < B->n_dem; ++sd)
+            for (int sd = 0; sd < B->n_dem; ++sd) {
+                const int key_out = sd == B->n_dem - 1;
+                if (B->prec == DPS_F64) {
+                    launch_dem_substep64(T, B->d_part, B->n_part, sd & 1, key_out, B->any_walls, u.part_tile, s);
+                    ndl += 2;  // pair kernel + gather kernel
+                    continue;
+                }
                 for (int c = 0; c < 4; ++c) {
                     const int nt = B->part_off[c + 1] - B->part_off[c];
                     if (nt <= 0) continue;
-                    // mixed forms: a block holds all lane groups of a particle tile,
-                    // at most 256 threads (two such blocks fit an SM); FP64 form:
-                    // the particle-kernel rule (its 200 registers a thread allow
-                    // one 256-thread block per SM)
-                    const int blk = B->prec != DPS_F64
-                                        ? (int)std::min<long long>(256, (std::max<long long>(u.part_block,
-                                                                                             (long long)u.part_tile << c) +
-                                                                         31) / 32 * 32)
-                                        : part_threads(u, 1 << c);
-                    launch_dem_substep(T, B->d_part + B->part_off[c], nt, sd & 1, sd == B->n_dem - 1,
-                                       B->prec != DPS_F64, 1 << c, B->any_walls, grid_of(nt), blk, s);
-                    ndl += 2;  // pair kernel + gather / integration kernel
+                    // a block holds all lane groups of a particle tile, at
+                    // most 256 threads (two such blocks fit an SM)
+                    const int blk = (int)std::min<long long>(
+                        256, (std::max<long long>(u.part_block, (long long)u.part_tile << c) + 31) / 32 * 32);
+                    launch_dem_substep(T, B->d_part + B->part_off[c], nt, sd & 1, key_out, 1 << c, B->any_walls,
+                                       grid_of(nt), blk, s);
+                    ndl += 2;  // pair kernel + integration kernel
                 }
+            }
         tend(B, PH_DEM, ndl);
         if (fork) cudaStreamWaitEvent(s, B->ev_join, 0);
         enqueue_sort_eps(B, B->n_dem & 1, 1, B->n_dem > 0);
@@ -699,15 +703,18 @@ static int ensure_lists(Batch *B) {
             if (pc >= (1LL << 31)) FAILB(B, DPS_ERR_ARG, "too many neighbour pairs for one box (%lld)", pc);
             void *hj = box_alloc(B, h, (size_t)pc * 4), *rr = box_alloc(B, h, (size_t)need * C * 4);
             void *pr = box_alloc(B, h, (size_t)pc * 48), *pg = box_alloc(B, h, (size_t)pc);
-            if (!hj || !rr || !pr || !pg) FAILB(B, DPS_ERR_OOM, "pair list allocation failed");
+            void *po = box_alloc(B, h, (size_t)pc);
+            if (!hj || !rr || !pr || !pg || !po) FAILB(B, DPS_ERR_OOM, "pair list allocation failed");
             box_release(B, h, h->d.hj);
             box_release(B, h, h->d.rrow);
             box_release(B, h, h->d.pres);
             box_release(B, h, h->d.pflag);
+            box_release(B, h, h->d.hl);
             h->d.hj = (int *)hj;
             h->d.rrow = (int *)rr;
             h->d.pres = (double *)pr;
             h->d.pflag = (unsigned char *)pg;
+            h->d.hl = (unsigned char *)po;
             h->d.pcap = pc;
         }
         h->d.maxn = need;
@@ -854,7 +861,8 @@ static size_t box_bytes(int prec, long long ncell, long long cap) {
     size_t b = 19 * N * pe + 27 * N * fe;
     b += 2 * (size_t)NPF * C * 8 + 2 * (size_t)NPI * C * 4 + 9 * C * 8 + 6 * C * 16 + C * 4 + 64 * C * 4 + 18 * C * 4;
     if (prec != DPS_F64) b += 6 * C * 8;  // mixed-form pair sums
-    if (prec == DPS_F64) b += 64 * C * 4 + 32 * C * (4 + 48 + 1);  // pair lists and results (64 partners)
+    if (prec == DPS_F64) b += 64 * C * 4 + 32 * C * (4 + 48 + 2);  // pair lists and results (64 partners)
+    if (prec == DPS_F64) b += C * (2 * sizeof(DemRec) + sizeof(DemPart));
     b += (3 * N + 1) * 4 + 3 * C * 4 + ((N + 8191) / 8192 + 1) * 4;
     b += 4096 + (size_t)reduce_partials_doubles() * 8;
     return b;
@@ -918,6 +926,9 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
     d.hj = d.rrow = nullptr;
     d.pres = nullptr;
     d.pflag = nullptr;
+    d.hl = nullptr;
+    for (int k = 0; k < 2; ++k) d.rec[k] = d.lowp ? nullptr : (DemRec *)A(cap * sizeof(DemRec));
+    d.part = d.lowp ? nullptr : (DemPart *)A(cap * sizeof(DemPart));
     d.pcap = 0;
     d.hoff = (int *)A(cap * 4);
     d.hn = (int *)A(cap * 4);

@@ -9,6 +9,19 @@
 
 namespace dps {
 
+// one particle as the FP64 pair kernel reads it (a gather of whole records:
+// two 32-byte sectors and one, where the separate planes would take nine)
+struct alignas(16) DemRec {
+    i64 x[3];      // position in units of 2^-Phys::fx.frac
+    double u[3];
+};
+struct alignas(16) DemPart {
+    i64 rad, inv_d;  // fx_radius, fx_inv_d
+    double im;       // 1/m
+    float imf;
+    int pad;
+};
+
 struct BoxDev {
     Geom g;
     Phys ph;
@@ -43,6 +56,11 @@ struct BoxDev {
     int *hj, *hoff, *hn, *rrow, *rn;
     double *pres;
     unsigned char *pflag;
+    unsigned char *hl;  // owner of a slot: its index within the chunk of 32 particles of its tile
+    // records of the pair kernel: the dynamic state of the current set / of
+    // the ping-pong planes, and the particle constants (set at every sort)
+    DemRec *rec[2];
+    DemPart *part;
     unsigned long long *ptop;
     long long pcap;    // slots
     int lowp;          // 1: low-precision form (FP32 coupling arithmetic)

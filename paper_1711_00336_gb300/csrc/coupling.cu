@@ -253,6 +253,21 @@ __global__ void k_bsort_gather(const BoxDev *__restrict__ boxes, const Tile *__r
             B.xf[0][k] = make_float4((float)xuw[i], (float)xuw[cap + i], (float)xuw[2 * cap + i], (float)dd);
             B.vf[0][k] = make_float4((float)xuw[3 * cap + i], (float)xuw[4 * cap + i], (float)xuw[5 * cap + i], (float)m);
             B.of[0][k] = make_float4((float)xuw[6 * cap + i], (float)xuw[7 * cap + i], (float)xuw[8 * cap + i], 0.f);
+            if (!B.lowp) {  // the records of the FP64 pair kernel
+                DemRec r;
+                DemPart q;
+                for (int a = 0; a < 3; ++a) {
+                    r.x[a] = fx_from(xuw[a * cap + i], B.ph.fx.frac);
+                    r.u[a] = xuw[(3 + a) * cap + i];
+                }
+                q.rad = fx_radius(dd);
+                q.inv_d = fx_inv_d(dd);
+                q.im = 1.0 / m;
+                q.imf = (float)q.im;
+                q.pad = 0;
+                B.rec[0][k] = r;
+                B.part[k] = q;
+            }
         }
     }
 }

@@ -9,8 +9,9 @@
 // the linked cells of the +-R cells around it, keeping every partner within
 // the interaction range plus the skin; the n_DEM substeps then loop over the
 // list only.  FP64 form: each pair of the list is evaluated once per substep
-// (k_dem_pairs64) and a gather kernel adds it to both partners in an order
-// fixed by the list (k_dem_gather64).  Mixed forms: a substep gives each
+// (k_dem_pairs64; lubrication pairs in 64-bit integer arithmetic of more than
+// FP64's precision, fx.cuh) and a gather kernel adds it to both partners in an
+// order fixed by the list (k_dem_gather64).  Mixed forms: a substep gives each
 // particle a group of LANES consecutive lanes of a warp: lane l takes the list
 // entries l, l + LANES, ... and the group's force and torque sums are combined
 // by warp shuffles (a fixed xor tree, so the result does not depend on the
@@ -315,73 +316,46 @@ __global__ void __launch_bounds__(256, DPS_NLIST_MINB) k_build_nlist(const BoxDe
     }
 }
 
-// the exact FP64 interaction with entry j (Sec. 3.1.1 / 3.1.3): a sphere
-// (j >= 0; separation from the FP64 positions) or a wall face
-// (j = -1 - (2 axis + side), side 1 the face at n[axis]; m_ij = m_i,
-// <d> = 2 d_i, partner at rest).  Both kinds run one contact / lubrication
-// body.  Out of line in the mixed forms, where it runs for the rare pairs
-// near contact only, so that its registers do not limit the occupancy of the
-// FP32 pair loop.
+// the FP64 interaction with sphere j (Sec. 3.1.1 / 3.1.3; separation from the
+// FP64 positions): F on particle i, and n x F_t in T (both partners take it
+// times their d/2)
 __device__ __forceinline__ void pair64_body(const PairPar<double> &pd, const double *__restrict__ xin,
                                             const double *__restrict__ pf, long long cap, const Geom &g, long long j,
                                             const double xi[3], const double ui[3], const double wi[3], double di,
-                                            double mi, double rng_extra, double lev, double F[3], double T[3],
-                                            unsigned &nlim) {
-    double n[3] = {0, 0, 0}, uj[3] = {0, 0, 0}, wjh[3] = {0, 0, 0};
-    double dist, sumr, dj = 0.0, mj = 1.0;
-    const bool wall = j < 0;
-    if (!wall) {
-        double dx[3];
+                                            double mi, double rng_extra, double F[3], double T[3], unsigned &nlim) {
+    double n[3], uj[3], wjh[3], dx[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) dx[a] = min_image(xin[a * cap + j] - xi[a], g.n[a], g.per[a]);
-        const double dist2 = dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2];
-        dj = pf[PD * cap + j];
-        sumr = 0.5 * (di + dj);
-        if (!(dist2 > 0.0)) return;
-        const double inv = rsqrt(dist2);  // 1/|dx| and |dx| from one reciprocal square root
-        dist = dist2 * inv;
-        if (!(dist < sumr + rng_extra)) return;
-        mj = pf[PM * cap + j];
+    for (int a = 0; a < 3; ++a) dx[a] = min_image(xin[a * cap + j] - xi[a], g.n[a], g.per[a]);
+    const double dist2 = dx[0] * dx[0] + dx[1] * dx[1] + dx[2] * dx[2];
+    const double dj = pf[PD * cap + j];
+    const double sumr = 0.5 * (di + dj);
+    if (!(dist2 > 0.0)) return;
+    const double inv = rsqrt(dist2);  // 1/|dx| and |dx| from one reciprocal square root
+    const double dist = dist2 * inv;
+    if (!(dist < sumr + rng_extra)) return;
+    const double mj = pf[PM * cap + j];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            n[a] = dx[a] * inv;
-            uj[a] = xin[(3 + a) * cap + j];
-        }
-    } else {
-        const int face = -1 - (int)j, ax = face >> 1, side = face & 1;
-        const double xa = ax == 0 ? xi[0] : (ax == 1 ? xi[1] : xi[2]);
-        const int L = ax == 0 ? g.n[0] : (ax == 1 ? g.n[1] : g.n[2]);
-        dist = side == 0 ? xa : L - xa;
-        sumr = 0.5 * di;
-        if (!(dist < sumr + rng_extra)) return;
-        const double sg = side == 0 ? -1.0 : 1.0;
-        n[0] = ax == 0 ? sg : 0.0;
-        n[1] = ax == 1 ? sg : 0.0;
-        n[2] = ax == 2 ? sg : 0.0;
+    for (int a = 0; a < 3; ++a) {
+        n[a] = dx[a] * inv;
+        uj[a] = xin[(3 + a) * cap + j];
     }
-    // m_ij = A / Bm and <d> = C / D: spheres m_i m_j / (m_i + m_j) and
-    // 2 d_i d_j / (d_i + d_j), walls m_i and 2 d_i; one division per pair
-    // (FP64 instructions bound this path on GB300)
-    const double A = wall ? mi : mi * mj, Bm = wall ? 1.0 : mi + mj;
-    const double C = wall ? 2.0 * di : 2.0 * di * dj, D = wall ? 1.0 : di + dj;
+    const double A = mi * mj, Bm = mi + mj;           // m_ij = A / Bm
+    const double C = 2.0 * di * dj, D = di + dj;      // <d> = C / D
     const double delta = sumr - dist;
     if (pd.contact && delta > 0.0) {
         // the partner's spin only matters in contact (the friction)
-        if (!wall) {
 #pragma unroll
-            for (int a = 0; a < 3; ++a) wjh[a] = 0.5 * dj * xin[(6 + a) * cap + j];
-        }
-        contact_force(pd, n, delta, ui, wi, di, uj, wjh, A / Bm, lev, F, T);
+        for (int a = 0; a < 3; ++a) wjh[a] = 0.5 * dj * xin[(6 + a) * cap + j];
+        contact_force(pd, n, delta, ui, wi, di, uj, wjh, A / Bm, 1.0, F, T);
     }
     const double h = dist - sumr;
     if (pd.lubrication && h >= 0.0 && h < pd.h_c) {
+        // one division for m_ij, <d>, r = <d>/hh and 1/r
         const double hh = fmax(h, pd.h_min);
         const double q = 1.0 / (Bm * D * hh * C);
-        const double dmean = wall ? C : C * C * Bm * hh * q;  // C / D
-        const double r = C * C * Bm * q;                      // <d> / hh
-        const double ir = Bm * D * D * hh * hh * q;           // hh / <d>
-        const double cap = (wall ? A : A * D * hh * C * q) * pd.capfac;  // m_ij capfac
-        lub_force(pd, n, dmean, r, ir, cap, ui, uj, F, nlim);
+        const double r = C * C * Bm * q;                // <d> / hh
+        const double ir = Bm * D * D * hh * hh * q;     // hh / <d>
+        lub_force(pd, n, C * C * Bm * hh * q, r, ir, A * D * hh * C * q * pd.capfac, ui, uj, F, nlim);
     }
 }
 // the mixed forms' pair within H_NEAR of contact.  The float copies of the
@@ -427,7 +401,7 @@ __device__ __noinline__ NearTerms near_pair32(const BoxDev &Bx, const double *__
 // one thread per particle: wall partners (WALLS; the FP64 form evaluates
 // them with the sphere pairs), then Eq. particle_motion (semi-implicit Euler)
 // and the outputs of the substep
-template <bool WALLS>
+template <bool WALLS, bool F64>
 __device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<double> &pd, long long i,
                                                int src_tmp, double F[3], double T[3], unsigned nlim, int key_out) {
     const double *xin = src_tmp ? Bx.xtmp : Bx.pf[Bx.cur];
@@ -496,6 +470,15 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<
     fout[i] = make_float4((float)xn3[0], (float)xn3[1], (float)xn3[2], pi.w);
     vout[i] = make_float4((float)un3[0], (float)un3[1], (float)un3[2], vi.w);
     oout[i] = make_float4((float)wn3[0], (float)wn3[1], (float)wn3[2], 0.f);
+    if (F64) {
+        DemRec r;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            r.x[a] = fx_from(xn3[a], ph.fx.frac);
+            r.u[a] = un3[a];
+        }
+        Bx.rec[1 - src_tmp][i] = r;
+    }
     if (key_out) {
         // last substep of the subcycle: the linked cell of the new position,
         // counted for the sort that follows (its counting pass)
@@ -624,7 +607,7 @@ __global__ void __launch_bounds__(128) k_dem_integrate(const BoxDev *__restrict_
                 F[a] = Bx.psum[a * cap + i];
                 T[a] = Bx.psum[(3 + a) * cap + i];
             }
-            finish_particle<WALLS>(Bx, pd, i, src_tmp, F, T, 0u, key_out);
+            finish_particle<WALLS, false>(Bx, pd, i, src_tmp, F, T, 0u, key_out);
         }
     }
 }
@@ -712,7 +695,10 @@ __global__ void __launch_bounds__(256) k_half_rows(const BoxDev *__restrict__ bo
             if (asc) {
                 const int lo = nn - nh;
                 for (int k = 0; k < lo; ++k) rr[k] = row[k];
-                for (int k = lo; k < nn; ++k) Bx.hj[h0 + k - lo] = row[k];
+                for (int k = lo; k < nn; ++k) {
+                    Bx.hj[h0 + k - lo] = row[k];
+                    Bx.hl[h0 + k - lo] = (unsigned char)((i - tl.begin) & 31);
+                }
                 continue;
             }
             for (int k = 0; k < nn; ++k) {
@@ -723,9 +709,10 @@ __global__ void __launch_bounds__(256) k_half_rows(const BoxDev *__restrict__ bo
                     const int o = row[m];
                     r += o < j && (up ? o > i : o < i);
                 }
-                if (up)
+                if (up) {
                     Bx.hj[h0 + r] = j;
-                else
+                    Bx.hl[h0 + r] = (unsigned char)((i - tl.begin) & 31);
+                } else
                     rr[r] = j;
             }
         }
@@ -765,108 +752,187 @@ __global__ void __launch_bounds__(256) k_reverse_slots(const BoxDev *__restrict_
     }
 }
 
-// The pairs of a substep.  Lane groups of LANES lanes screen the owned pairs
-// of a particle in FP32 (with a margin); a block-wide exclusive sum places the
-// entries that pass in a queue, evaluated one per thread by the exact FP64
-// contact / lubrication body (an FP64 instruction costs a warp the same
-// whatever number of its lanes are active), which writes the force on the
-// owner and n x F_t to the pair's slot.  Every owned slot gets its flag.
-constexpr int DQ_CAP = 512;
+// The pairs of a substep.  A warp takes chunks of 32 particles of a tile: their
+// owned pairs lie in consecutive slots (k_half_rows), which the lanes screen in
+// FP32 (with a margin) 32 at a time.  Pairs that pass go to a queue of the warp
+// and are evaluated 32 at a time, one per lane: separation, gap, logarithm and
+// reciprocal of a lubrication pair in 64-bit integers (fx_pair), its force in
+// 14 FP64 operations.  Pairs that overlap (or leave the range of that path) go to
+// a queue of the block, evaluated together by the exact FP64 contact /
+// lubrication body at the end of the tile, so that few warps pay for it (an FP64
+// instruction costs a warp the same whatever number of its lanes are active).
+// Every owned slot gets its flag; the result of a slot depends on its pair alone.
+// The FP64 body for every pair took ~120 FP64 warp instructions of ~19 cycles
+// per 32 pairs (70 % of the FP64 pipe).  DEM substep (this kernel and the
+// gather) before / after, FP64: 256^3, eps 0.2, d 1.5: 4.34 / 2.02 ms; 101 x 90
+// x 77, eps 0.36 with contacts: 1.13 / 0.48 ms.  At 128^3 this kernel takes
+// 140 us: 1100 instructions per 32 pairs, FP64 pipe 35 %.
+constexpr int PAIR_WARPS = 4;
+constexpr int EXACT_CAP = 512;  // queued pairs of a tile; past it a pair is evaluated at once
+
+struct PairQueue {
+    int slot[PAIR_WARPS][64], j[PAIR_WARPS][64], i[PAIR_WARPS][64];  // rings, one per warp
+    int eslot[EXACT_CAP], ej[EXACT_CAP], ei[EXACT_CAP], en;
+};
+
+// m_ij capfac and its reciprocal's FP64 Newton steps (x = 1/m_i + 1/m_j)
+__device__ __forceinline__ double fx_recip(double x, float xf) {
+    double y = (double)__fdividef(1.0f, xf);
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
 
 #ifndef DPS_PAIRS_MINB
-#define DPS_PAIRS_MINB 2  // 256-thread blocks per SM the register budget is sized for
+#define DPS_PAIRS_MINB 5  // 128-thread blocks per SM the register budget is sized for
 #endif
-template <int LANES>
-__global__ void __launch_bounds__(256, DPS_PAIRS_MINB) k_dem_pairs64(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles,
-                                                     int ntiles, int src_tmp) {
-    __shared__ int qS[DQ_CAP], qJ[DQ_CAP], qP[DQ_CAP];
-    __shared__ int ws[9];
-    const int lane = threadIdx.x % LANES, grp = threadIdx.x / LANES, ngrp = blockDim.x / LANES;
+__global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
+    k_dem_pairs64(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles, int ntiles, int src_tmp) {
+    __shared__ PairQueue Qs;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (threadIdx.x == 0) Qs.en = 0;
+    __syncthreads();
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &Bx = boxes[tl.box];
         const double *xin = src_tmp ? Bx.xtmp : Bx.pf[Bx.cur];
         const float4 *fin = Bx.xf[src_tmp];
+        const DemRec *rec = Bx.rec[src_tmp];
+        const DemPart *part = Bx.part;
         const double *pf = Bx.pf[Bx.cur];
         const long long cap = Bx.cap;
-        const Geom g = Bx.g;
+        const Geom &g = Bx.g;
         const Phys &ph = Bx.ph;
         const double rng_extra = ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0;
         const float rng_extra_f = (float)rng_extra;
         const float Lf[3] = {(float)g.n[0], (float)g.n[1], (float)g.n[2]};
         const PairPar<double> pd = pair_par<double>(ph);
+        const bool fx = ph.fx.ok != 0;
+        const float capf = (float)ph.capfac * 0.999f;
         unsigned nlim = 0;
-        for (long long base = tl.begin; base < tl.end; base += ngrp) {  // uniform trip count
-            const long long i = base + grp;
-            const bool act = i < tl.end;
-            float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
-            int nh = 0, h0 = 0;
-            if (act) {
-                pi = fin[i];
-                nh = Bx.hn[i];
-                h0 = Bx.hoff[i];
+
+        // the FP64 body of slot sl, the pair (i, j)
+        auto exact = [&](int sl, int i, int j) {
+            double xi[3], ui[3], wi[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                xi[a] = xin[a * cap + i];
+                ui[a] = xin[(3 + a) * cap + i];
+                wi[a] = xin[(6 + a) * cap + i];
             }
-            // the owned pairs of this lane (c = lane, lane + LANES, ...) that
-            // pass the FP32 screen, in order: fn(slot, j)
-            auto entries = [&](bool flag, auto &&fn) {
-                for (int c = lane; c < nh; c += LANES) {
-                    const int sl = h0 + c, j = Bx.hj[sl];
-                    const float4 pj = fin[j];
-                    const float fx = min_image_f(pj.x - pi.x, Lf[0], g.per[0]);
+            double Fq[3] = {0, 0, 0}, Cq[3] = {0, 0, 0};
+            pair64_body(pd, xin, pf, cap, g, j, xi, ui, wi, pf[PD * cap + i], pf[PM * cap + i], rng_extra, Fq, Cq,
+                        nlim);
+            // the force in the first plane; n x F_t, nonzero only for
+            // pairs in contact with friction, in the second, flagged 2
+            const long long sq = sl;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) Bx.pres[3 * sq + a] = Fq[a];
+            unsigned char fl = 1;
+            if (Cq[0] != 0.0 || Cq[1] != 0.0 || Cq[2] != 0.0) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) Bx.pres[3 * (Bx.pcap + sq) + a] = Cq[a];
+                fl = 2;
+            }
+            Bx.pflag[sq] = fl;
+        };
+        // entry k of the warp's queue
+        auto eval = [&](int k) {
+            const int sl = Qs.slot[wid][k & 63], i = Qs.i[wid][k & 63], j = Qs.j[wid][k & 63];
+            int kind = FX_EXACT;
+            if (fx) {
+                const DemRec ri = rec[i], rj = rec[j];
+                const DemPart pi = part[i], pj = part[j];
+                i64 dx[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    dx[a] = rj.x[a] - ri.x[a];
+                    if (g.per[a]) {
+                        const i64 L = (i64)g.n[a] << ph.fx.frac, h = L >> 1;
+                        dx[a] = dx[a] > h ? dx[a] - L : (dx[a] < -h ? dx[a] + L : dx[a]);
+                    }
+                }
+                FxPair o;
+                kind = fx_pair(dx, pi.rad + pj.rad, (u64)(pi.inv_d + pj.inv_d), ph.fx, o);
+                if (kind == FX_LUB && ph.lubrication) {
+                    double al = o.alpha, be = o.beta;
+                    if (ph.lub_limiter) {
+                        // a coefficient near its cap m_ij capfac: compare in FP64
+                        const float imf = pi.imf + pj.imf;
+                        if (!(fx_approx(be) * imf < capf && fx_approx(al) * imf < capf)) {
+                            const double lim = ph.capfac * fx_recip(pi.im + pj.im, imf);
+                            if (be > lim) { be = lim; ++nlim; }
+                            if (al > lim) { al = lim; ++nlim; }
+                        }
+                    }
+                    double du[3];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) du[a] = ri.u[a] - rj.u[a];
+                    const double un = du[0] * o.n[0] + du[1] * o.n[1] + du[2] * o.n[2];
+                    const double sn = (al - be) * un;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) Bx.pres[3 * (long long)sl + a] = sn * o.n[a] - al * du[a];
+                    Bx.pflag[sl] = 1;
+                } else if (kind != FX_EXACT) {
+                    Bx.pflag[sl] = 0;
+                }
+            }
+            if (kind == FX_EXACT) {
+                const int q = atomicAdd(&Qs.en, 1);
+                if (q < EXACT_CAP) {
+                    Qs.eslot[q] = sl;
+                    Qs.ei[q] = i;
+                    Qs.ej[q] = j;
+                } else {
+                    exact(sl, i, j);
+                }
+            }
+        };
+
+        int head = 0, qn = 0;  // the warp's ring: qn entries from head
+        for (long long c0 = tl.begin + 32 * wid; c0 < tl.end; c0 += 32 * nw) {
+            const long long p = c0 + lane;
+            const bool own = p < tl.end;
+            const int h0 = __shfl_sync(0xffffffffu, own ? Bx.hoff[p] : 0, 0);
+            const int total = __reduce_add_sync(0xffffffffu, own ? Bx.hn[p] : 0);
+            for (int t0 = 0; t0 < total; t0 += 32) {
+                const int sl = h0 + t0 + lane;
+                bool pass = false;
+                int i = 0, j = 0;
+                if (t0 + lane < total) {
+                    j = Bx.hj[sl];
+                    i = (int)c0 + Bx.hl[sl];
+                    const float4 pi = fin[i], pj = fin[j];
+                    const float fx_ = min_image_f(pj.x - pi.x, Lf[0], g.per[0]);
                     const float fy = min_image_f(pj.y - pi.y, Lf[1], g.per[1]);
                     const float fz = min_image_f(pj.z - pi.z, Lf[2], g.per[2]);
                     const float fr = 0.5f * (pi.w + pj.w) + rng_extra_f + SCREEN_MARGIN;
-                    const bool pass = fx * fx + fy * fy + fz * fz < fr * fr;
-                    if (flag) Bx.pflag[sl] = pass;
-                    if (pass) fn(sl, j);
+                    pass = fx_ * fx_ + fy * fy + fz * fz < fr * fr;
+                    if (!pass) Bx.pflag[sl] = 0;
                 }
-            };
-            int cnt = 0;
-            if (act) entries(true, [&](int, int) { ++cnt; });
-            int M;
-            const int off = block_excl_sum(cnt, ws, M);
-            for (int w0 = 0; w0 < M; w0 += DQ_CAP) {
-                const int mw = M - w0 < DQ_CAP ? M - w0 : DQ_CAP;
-                if (act && off < w0 + mw && off + cnt > w0) {
-                    int c = off;
-                    entries(false, [&](int sl, int j) {
-                        // (c < off + cnt: both passes screen alike; the bound only
-                        // keeps a lane inside its own slots)
-                        if (c >= w0 && c < w0 + mw && c < off + cnt) {
-                            qS[c - w0] = sl;
-                            qJ[c - w0] = j;
-                            qP[c - w0] = (int)(i - tl.begin);
-                        }
-                        ++c;
-                    });
+                const unsigned m = __ballot_sync(0xffffffffu, pass);
+                if (pass) {
+                    const int k = (head + qn + __popc(m & ((1u << lane) - 1))) & 63;
+                    Qs.slot[wid][k] = sl;
+                    Qs.i[wid][k] = i;
+                    Qs.j[wid][k] = j;
                 }
-                __syncthreads();
-                for (int q = threadIdx.x; q < mw; q += blockDim.x) {
-                    const long long ii = tl.begin + qP[q];
-                    double xi[3], ui[3], wi[3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        xi[a] = xin[a * cap + ii];
-                        ui[a] = xin[(3 + a) * cap + ii];
-                        wi[a] = xin[(6 + a) * cap + ii];
-                    }
-                    double Fq[3] = {0, 0, 0}, Cq[3] = {0, 0, 0};
-                    pair64_body(pd, xin, pf, cap, g, qJ[q], xi, ui, wi, pf[PD * cap + ii], pf[PM * cap + ii],
-                                rng_extra, 1.0, Fq, Cq, nlim);
-                    // the force in the first plane; n x F_t, nonzero only for
-                    // pairs in contact with friction, in the second, flagged 2
-                    const long long sq = qS[q];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) Bx.pres[3 * sq + a] = Fq[a];
-                    if (Cq[0] != 0.0 || Cq[1] != 0.0 || Cq[2] != 0.0) {
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) Bx.pres[3 * (Bx.pcap + sq) + a] = Cq[a];
-                        Bx.pflag[sq] = 2;
-                    }
+                qn += __popc(m);
+                __syncwarp();
+                if (qn >= 32) {
+                    eval(head + lane);
+                    head += 32;
+                    qn -= 32;
+                    __syncwarp();
                 }
-                __syncthreads();  // the next window overwrites the queue
             }
         }
+        if (lane < qn) eval(head + lane);
+        __syncthreads();
+        const int ne = min(Qs.en, EXACT_CAP);
+        for (int q = threadIdx.x; q < ne; q += blockDim.x) exact(Qs.eslot[q], Qs.ei[q], Qs.ej[q]);
+        __syncthreads();
+        if (threadIdx.x == 0) Qs.en = 0;
+        __syncthreads();
         // each capped coefficient acts on both partners (the count of the
         // per-particle evaluation of Sec. 3.1.3)
         if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], 2ull * nlim);
@@ -945,7 +1011,7 @@ __global__ void __launch_bounds__(128, WALLS ? 1 : DPS_GATHER_MINB) k_dem_gather
                     }
                 }
             }
-            finish_particle<WALLS>(Bx, pd, i, src_tmp, F, T, 0u, key_out);
+            finish_particle<WALLS, true>(Bx, pd, i, src_tmp, F, T, 0u, key_out);
         }
     }
 }
@@ -961,36 +1027,35 @@ void launch_build_nlist(const BoxDev *boxes, const Tile *tiles, int ntiles, int 
     }
 }
 
-// lanes: 1, 2, 4 or 8 lanes per particle (block a multiple of 32); the FP64
-// form launches its pair kernel and then its gather kernel; walls: some box
-// has a wall axis
+// mixed forms; lanes: 1, 2, 4 or 8 lanes per particle (block a multiple of
+// 32); walls: some box has a wall axis
 // key_out: the last substep of a subcycle also writes the particles' linked
 // cells and their counts for the sort that follows
-void launch_dem_substep(const BoxDev *boxes, const Tile *tiles, int ntiles, int src_tmp, int key_out, int mixed,
-                        int lanes, int walls, int grid, int block, cudaStream_t s) {
-#define DPS_DEM(K, L) K<L><<<grid, block, 0, s>>>(boxes, tiles, ntiles, src_tmp)
-    if (mixed) {
-        if (lanes >= 8) DPS_DEM(k_dem_pairsum_mixed, 8);
-        else if (lanes == 4) DPS_DEM(k_dem_pairsum_mixed, 4);
-        else if (lanes == 2) DPS_DEM(k_dem_pairsum_mixed, 2);
-        else DPS_DEM(k_dem_pairsum_mixed, 1);
-        if (walls)
-            k_dem_integrate<true><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
-        else
-            k_dem_integrate<false><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
-    } else {
-#define DPS_PAIRS(L) k_dem_pairs64<L><<<grid, block, 0, s>>>(boxes, tiles, ntiles, src_tmp)
-        if (lanes >= 8) DPS_PAIRS(8);
-        else if (lanes == 4) DPS_PAIRS(4);
-        else if (lanes == 2) DPS_PAIRS(2);
-        else DPS_PAIRS(1);
-#undef DPS_PAIRS
-        if (walls)
-            k_dem_gather64<true><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
-        else
-            k_dem_gather64<false><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
-    }
+void launch_dem_substep(const BoxDev *boxes, const Tile *tiles, int ntiles, int src_tmp, int key_out, int lanes,
+                        int walls, int grid, int block, cudaStream_t s) {
+#define DPS_DEM(L) k_dem_pairsum_mixed<L><<<grid, block, 0, s>>>(boxes, tiles, ntiles, src_tmp)
+    if (lanes >= 8) DPS_DEM(8);
+    else if (lanes == 4) DPS_DEM(4);
+    else if (lanes == 2) DPS_DEM(2);
+    else DPS_DEM(1);
 #undef DPS_DEM
+    if (walls)
+        k_dem_integrate<true><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
+    else
+        k_dem_integrate<false><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
+}
+
+// FP64 form: the pair kernel, then the gather kernel, over the particle tiles
+// of every box (one block per tile: blocks that finish make room for others)
+void launch_dem_substep64(const BoxDev *boxes, const Tile *tiles, int ntiles, int src_tmp, int key_out, int walls,
+                          int part_tile, cudaStream_t s) {
+    const int warps = part_tile < 32 * PAIR_WARPS ? (part_tile + 31) / 32 : PAIR_WARPS;
+    k_dem_pairs64<<<ntiles, 32 * warps, 0, s>>>(boxes, tiles, ntiles, src_tmp);
+    const int grid = ntiles < 152 * 8 ? ntiles : 152 * 8;
+    if (walls)
+        k_dem_gather64<true><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
+    else
+        k_dem_gather64<false><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
 }
 
 }  // namespace dps

@@ -21,6 +21,7 @@
 
 #include "dps.h"
 #include "tlog.cuh"
+#include "fx.cuh"
 
 namespace dps {
 
@@ -160,6 +161,7 @@ struct Phys {
     int drag, pressure, added_mass, lubrication, contact, lub_limiter;
     int lift;            // Table 1 shear lift (curl of u_f at the subcycle start)
     int eilers, smag;    // per-cell tau_e (Eqs. visc_eilers, tau_t, tau_e)
+    FxBox fx;            // constants of the integer pair path (fx.cuh)
 };
 
 // ---- precision-preserving math -----------------------------------------------

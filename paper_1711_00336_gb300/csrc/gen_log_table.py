@@ -9,6 +9,11 @@ unevaluated sum hi + lo with hi a multiple of 2^-42; ln 2 is split the same
 way, so that k ln2_hi + hi is exact for |k| < 2^11.  The values come from
 mpmath at 60 significant digits.
 
+The second table serves the integer logarithm of the pair kernel (fx.cuh): for
+m in [1, 2) and j the leading seven bits of its fraction, C_j = 2^16/(1 + (j +
+1/2)/128) rounded to an integer and -ln(C_j/2^16) in units of 2^-58, so that
+ln m = ln(1 + u) - ln(C_j/2^16) with u = m C_j/2^16 - 1, |u| < 2^-7.9.
+
     python gen_log_table.py    # rewrites log_table.cuh beside this file
 """
 import os
@@ -41,6 +46,14 @@ def main():
     for k, (F, inv, hi, lo) in enumerate(rows):
         sep = "," if k < 128 else ""
         out.append(f"    {{{F.hex()}, {inv.hex()}, {hi.hex()}, {lo.hex()}}}{sep} \\")
+    out.append("")
+    out.append("// Per j = 0..127: C_j = 2^16/(1 + (j + 1/2)/128) rounded, -ln(C_j/2^16) in units of 2^-58.")
+    out.append(f"#define DPS_FX_LN2_Q58 {int(mp.nint(mp.log(2) * mp.mpf(2) ** 58))}LL")
+    out.append("#define DPS_FX_LOG_ROWS \\")
+    for j in range(128):
+        C = int(mp.nint(mp.mpf(2) ** 16 / (1 + (mp.mpf(j) + mp.mpf("0.5")) / 128)))
+        T = int(mp.nint(-mp.log(mp.mpf(C) / 2 ** 16) * mp.mpf(2) ** 58))
+        out.append(f"    {{{C}LL, {T}LL}}{',' if j < 127 else ''} \\")
     out.append("")
     path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "log_table.cuh")
     with open(path, "w") as f:
