@@ -74,6 +74,7 @@ void launch_fluid_sums(const void *, const void *, const void *, const Geom &, c
                        cudaStream_t);
 void launch_particle_sums(const double *, const double *, long long, long long, double *, double *, cudaStream_t);
 void launch_particles_import(double *, int, long long, long long, const int *, const double *, cudaStream_t);
+void launch_rec_velocity(DemRec *, const double *, long long, long long, cudaStream_t);
 void launch_particles_export4(const BoxDev *, int, const double *, const int *, long long, long long, double *,
                               cudaStream_t);
 long long reduce_partials_doubles();
@@ -271,6 +272,10 @@ static void compute_phys(BoxHost *h) {
         h->d.R = 1;
         p.skin = 0.0;
         p.skin_half2 = 0.25;
+        p.skin_near2 = -1.0f;
+        p.shell = 0.0f;
+        p.shell_near2 = -1.0f;
+        p.far_ok = 0;
         return;
     }
     p.e_n = c.e_n;
@@ -304,6 +309,19 @@ static void compute_phys(BoxHost *h) {
     p.skin = c.skin;
     h->d.R = (int)std::floor(cutoff + c.skin + 1e-3) + 1;
     p.skin_half2 = 0.25 * c.skin * c.skin;
+    {
+        // both float positions are off by at most L 2^-24 per axis
+        const double L = std::max({h->d.g.n[0], h->d.g.n[1], h->d.g.n[2]});
+        const double near = 0.5 * c.skin - 4.0 * L * 0x1p-24;
+        p.skin_near2 = near > 0.0 ? (float)(0.999 * near * near) : -1.0f;
+        // inner shell of the list: a tenth of a cell holds the few per cent of
+        // extra pairs at ranges of 2-3 cells and lets a particle move 0.05
+        // cells between two sorts (|u| <= 0.1 at two subcycles a step)
+        const double shell = std::min(0.1, c.skin), half = 0.5 * shell - 4.0 * L * 0x1p-24;
+        p.shell = (float)shell;
+        p.shell_near2 = half > 0.0 ? (float)(0.999 * half * half) : -1.0f;
+        p.far_ok = L < 4096.0;
+    }
 }
 
 // ---- table and tiles ------------------------------------------------------------
@@ -415,11 +433,12 @@ static int push_layout(Batch *B) {
         B->any_lift |= h->d.ph.lift && h->d.np > 0;
         B->any_walls |= h->d.np > 0 && !(h->d.g.per[0] && h->d.g.per[1] && h->d.g.per[2]);
         std::vector<Tile> &ct = (h->d.ph.eilers || h->d.ph.smag) ? cellv : cell;
+        const int lc = dem_lanes_class(h), fl = force_lanes(h);
+        h->d.dem_lanes = 1 << lc;
         tab[k] = h->d;
         const long long N = h->d.g.ncell, np = h->d.np;
         for (long long c = 0; c < N; c += B->tune.cell_tile)
             ct.push_back(Tile{k, 0, c, std::min(N, c + B->tune.cell_tile)});
-        const int lc = dem_lanes_class(h), fl = force_lanes(h);
         B->cpl_lanes = std::max(B->cpl_lanes, fl);
         for (long long p = 0; p < np; p += B->tune.part_tile)
             partc[lc].push_back(Tile{k, fl, p, std::min(np, p + B->tune.part_tile)});
@@ -525,11 +544,12 @@ static void enqueue_sort_eps(Batch *B, int xsel, int mark_usub, bool have_keys) 
                             B->stream);
     }
     launch_bsort_flip(B->d_table, nb, mark_usub, B->stream);
-    const int pairs = B->prec == DPS_F64;  // the FP64 form evaluates each pair once
+    // pair rows (FP64: each pair is evaluated once), inner rows (FP16 storage)
+    const int rows = B->prec == DPS_F64 ? 1 : (B->prec == DPS_F16S ? 2 : 0);
     if (pl)
-        launch_build_nlist(T, B->d_part, B->n_part, grid_of(B->n_part), part_threads(u, B->cpl_lanes), pairs,
+        launch_build_nlist(T, B->d_part, B->n_part, grid_of(B->n_part), part_threads(u, B->cpl_lanes), rows,
                            B->stream);
-    tend(B, PH_SORT, cnt + 3 + 3 * pl + 1 + pl * (1 + 2 * pairs));
+    tend(B, PH_SORT, cnt + 3 + 3 * pl + 1 + pl * (1 + (rows == 1 ? 2 : rows == 2)));
     tbegin(B);
     if (B->fel == 8)
         launch_eps<double>(T, B->d_brick, B->n_brick, grid_of(B->n_brick), 256, B->stream);
@@ -702,20 +722,28 @@ static int ensure_lists(Batch *B) {
             const long long pc = pair_capacity(h, need);
             if (pc >= (1LL << 31)) FAILB(B, DPS_ERR_ARG, "too many neighbour pairs for one box (%lld)", pc);
             void *hj = box_alloc(B, h, (size_t)pc * 4), *rr = box_alloc(B, h, (size_t)need * C * 4);
-            void *pr = box_alloc(B, h, (size_t)pc * 48), *pg = box_alloc(B, h, (size_t)pc);
+            void *pr = box_alloc(B, h, (size_t)pc * sizeof(PairRes)), *pg = box_alloc(B, h, (size_t)pc * 24);
             void *po = box_alloc(B, h, (size_t)pc);
             if (!hj || !rr || !pr || !pg || !po) FAILB(B, DPS_ERR_OOM, "pair list allocation failed");
             box_release(B, h, h->d.hj);
             box_release(B, h, h->d.rrow);
             box_release(B, h, h->d.pres);
-            box_release(B, h, h->d.pflag);
+            box_release(B, h, h->d.ptan);
             box_release(B, h, h->d.hl);
             h->d.hj = (int *)hj;
             h->d.rrow = (int *)rr;
-            h->d.pres = (double *)pr;
-            h->d.pflag = (unsigned char *)pg;
+            h->d.pres = (PairRes *)pr;
+            h->d.ptan = (double *)pg;
             h->d.hl = (unsigned char *)po;
             h->d.pcap = pc;
+        }
+        if (!h->d.split) {
+            const int wide = (need + 7) / 8 * 8;  // rows of up to 8 lanes
+            void *q = box_alloc(B, h, (size_t)wide * C * 4);
+            if (!q) FAILB(B, DPS_ERR_OOM, "neighbour list allocation failed");
+            box_release(B, h, h->d.ilist);
+            h->d.ilist = (int *)q;
+            h->d.maxi = wide;
         }
         h->d.maxn = need;
         B->layout_dirty = true;
@@ -859,9 +887,10 @@ static size_t box_bytes(int prec, long long ncell, long long cap) {
     size_t pe = prec == DPS_F64 ? 8 : (prec == DPS_F32 ? 4 : 2), fe = prec == DPS_F64 ? 8 : 4;
     size_t N = (size_t)ncell, C = (size_t)(cap > 0 ? cap : 1);
     size_t b = 19 * N * pe + 27 * N * fe;
-    b += 2 * (size_t)NPF * C * 8 + 2 * (size_t)NPI * C * 4 + 9 * C * 8 + 6 * C * 16 + C * 4 + 64 * C * 4 + 18 * C * 4;
+    b += 2 * (size_t)NPF * C * 8 + 2 * (size_t)NPI * C * 4 + 9 * C * 8 + 7 * C * 16 + C * 4 + 64 * C * 4 + 22 * C * 4;
     if (prec != DPS_F64) b += 6 * C * 8;  // mixed-form pair sums
-    if (prec == DPS_F64) b += 64 * C * 4 + 32 * C * (4 + 48 + 2);  // pair lists and results (64 partners)
+    if (prec == DPS_F16S) b += 64 * C * 4 + C * 4;  // inner rows
+    if (prec == DPS_F64) b += 64 * C * 4 + 32 * C * (4 + sizeof(PairRes) + 24 + 1);  // pair lists and results (64 partners)
     if (prec == DPS_F64) b += C * (2 * sizeof(DemRec) + sizeof(DemPart));
     b += (3 * N + 1) * 4 + 3 * C * 4 + ((N + 8191) / 8192 + 1) * 4;
     b += 4096 + (size_t)reduce_partials_doubles() * 8;
@@ -916,8 +945,16 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
         d.vf[k] = (float4 *)A(cap * 16);
         d.of[k] = (float4 *)A(cap * 16);
     }
-    d.nlist_n = (int *)A(cap * 4);
     d.lowp = B->prec != DPS_F64;
+    d.xs = (float4 *)A(cap * 16);
+    d.nlist_n = (int *)A(cap * 4);
+    d.nlist_o = (int *)A(cap * 4);
+    d.split = B->prec != DPS_F16S;
+    d.ilist = nullptr;  // sized with nlist
+    d.ilist_n = d.split ? nullptr : (int *)A(cap * 4);
+    d.maxi = 0;
+    d.dem_lanes = 1;
+    d.moved = (int *)A(16);
     d.pwf = d.lowp ? (float *)A(9 * cap * 4) : nullptr;
     d.f32p = d.lowp ? (float *)A(6 * cap * 4) : nullptr;
     d.psum = d.lowp ? (double *)A(6 * cap * 8) : nullptr;
@@ -925,7 +962,7 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
     d.maxn = 0;
     d.hj = d.rrow = nullptr;
     d.pres = nullptr;
-    d.pflag = nullptr;
+    d.ptan = nullptr;
     d.hl = nullptr;
     for (int k = 0; k < 2; ++k) d.rec[k] = d.lowp ? nullptr : (DemRec *)A(cap * sizeof(DemRec));
     d.part = d.lowp ? nullptr : (DemPart *)A(cap * sizeof(DemPart));
@@ -933,6 +970,9 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
     d.hoff = (int *)A(cap * 4);
     d.hn = (int *)A(cap * 4);
     d.rn = (int *)A(cap * 4);
+    d.hoff2 = (int *)A(cap * 4);
+    d.hn2 = (int *)A(cap * 4);
+    d.rn2 = (int *)A(cap * 4);
     d.ptop = (unsigned long long *)A(16);
     d.cell_start = (int *)A((N + 1) * 4);
     d.count = (int *)A(N * 4);
@@ -966,7 +1006,8 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
     cudaMemsetAsync(d.rho, 0, N * B->fel, s);
     cudaMemsetAsync(d.ire, 0, N * B->fel, s);
     cudaMemsetAsync(d.nlist_n, 0, cap * 4, s);
-    for (int *z : {d.hoff, d.hn, d.rn}) cudaMemsetAsync(z, 0, cap * 4, s);
+    for (int *z : {d.hoff, d.hn, d.rn, d.hoff2, d.hn2, d.rn2, d.nlist_o}) cudaMemsetAsync(z, 0, cap * 4, s);
+    cudaMemsetAsync(d.moved, 0, 16, s);
     cudaMemsetAsync(d.ptop, 0, 16, s);
     for (int k = 0; k < 2; ++k) {
         cudaMemsetAsync(d.xf[k], 0, cap * 16, s);
@@ -1162,6 +1203,9 @@ static int box_write_particles(Batch *B, BoxHost *h, long long n, const double *
         CKB(B, cudaMemcpyAsync(buf, src[k], 8 * 3 * n, cudaMemcpyHostToDevice, B->stream));
         launch_particles_import(pf, 3 * k, h->d.cap, n, ids, buf, B->stream);
     }
+    // without new positions the box is not sorted again, which would renew
+    // the records of the FP64 pair kernel
+    if (u3 && !x3 && h->d.rec[0]) launch_rec_velocity(h->d.rec[0], pf, h->d.cap, n, B->stream);
     CKB(B, cudaFreeAsync(buf, B->stream));
     CKB(B, cudaStreamSynchronize(B->stream));
     if (x3) h->prepared = false;
@@ -1661,21 +1705,24 @@ int dps_read_neighbor_list(dps_handle h, int64_t *offsets, int32_t *partners, in
         for (long long i = 0; i <= np; ++i) offsets[i] = 0;
         return DPS_OK;
     }
-    std::vector<int> cnt((size_t)np), ids((size_t)np), rows((size_t)np * d.maxn);
+    std::vector<int> cnt((size_t)np), out((size_t)np), ids((size_t)np), rows((size_t)np * d.maxn);
     CKB(B, cudaMemcpy(cnt.data(), d.nlist_n, 4 * np, cudaMemcpyDeviceToHost));
+    CKB(B, cudaMemcpy(out.data(), d.nlist_o, 4 * np, cudaMemcpyDeviceToHost));
     CKB(B, cudaMemcpy(ids.data(), d.pi[d.cur] + IID * d.cap, 4 * np, cudaMemcpyDeviceToHost));
     CKB(B, cudaMemcpy(rows.data(), d.nlist, 4 * (size_t)np * d.maxn, cudaMemcpyDeviceToHost));
     // rows by insertion id, partners as insertion ids in ascending order
     std::vector<long long> len((size_t)np, 0);
-    for (long long s = 0; s < np; ++s) len[ids[s]] = cnt[s];
+    for (long long s = 0; s < np; ++s) len[ids[s]] = cnt[s] + out[s];
     offsets[0] = 0;
     for (long long i = 0; i < np; ++i) offsets[i + 1] = offsets[i] + len[i];
     if (!partners) return DPS_OK;
     if (cap < offsets[np]) FAILB(B, DPS_ERR_ARG, "capacity %lld < %lld list entries", (long long)cap, (long long)offsets[np]);
     for (long long s = 0; s < np; ++s) {
         int32_t *o = partners + offsets[ids[s]];
-        for (int k = 0; k < cnt[s]; ++k) o[k] = ids[rows[(size_t)s * d.maxn + k]];
-        std::sort(o, o + cnt[s]);
+        const int *row = rows.data() + (size_t)s * d.maxn;
+        for (int k = 0; k < cnt[s]; ++k) o[k] = ids[row[k] < 0 ? ~row[k] : row[k]];
+        for (int k = 0; k < out[s]; ++k) o[cnt[s] + k] = ids[row[d.maxn - 1 - k]];
+        std::sort(o, o + cnt[s] + out[s]);
     }
     return DPS_OK;
 }

@@ -22,6 +22,13 @@ struct alignas(16) DemPart {
     int pad;
 };
 
+// result of a pair and substep: the force on the owner of the slot, and 0: the
+// pair did not pass, 1: it did, 2: and its n x F_t is nonzero (BoxDev::ptan)
+struct alignas(32) PairRes {
+    double F[3];
+    i64 flag;
+};
+
 struct BoxDev {
     Geom g;
     Phys ph;
@@ -42,20 +49,25 @@ struct BoxDev {
     float4 *xf[2];     // float (x, y, z, d) of the current set / of the ping-pong planes
     float4 *vf[2];     // float (u, m) likewise
     float4 *of[2];     // float (omega, 0) likewise
-    int *nlist;        // Verlet list, row by row: nlist[i*maxn + k]
-    int *nlist_n;      // list length per particle
+    float4 *xs;        // float position at the last sort, and d
+    int *nlist;        // Verlet list, row by row (k_build_nlist)
+    int *nlist_n, *nlist_o;  // inner and outer partners per particle (one-row form: all, 0)
+    int split;         // 1: inner partners from the row's front, outer ones from its back; 0: one row
+    int *ilist;        // one-row form: the inner partners, ilist[i*maxi + k], dem_lanes columns, gaps -1
+    int *ilist_n;
+    int maxi, dem_lanes;
+    int *moved;        // [2], by source buffer of a substep: some particle has moved more than shell/2
     int maxn;          // list capacity per particle
     // FP64 form: the list as unordered pairs, each evaluated once per
     // substep (Newton's third law).  Particle i owns the pairs with its
     // partners j > i: hn[i] of them, in ascending j, at slots hoff[i] ...
     // (hj: the partner of a slot; slots are allocated per block from *ptop).
     // rn[i] / rrow[i*maxn + r]: the slots of the pairs (k, i), k < i, in
-    // ascending k.  pres[3 s ...]: force on the owner of slot s,
-    // pres[3 (pcap + s) ...]: its n x F_t; pflag[s]: 1 the pair passed the
-    // screen of this substep, 2 also n x F_t is nonzero (written).
+    // ascending k.
     int *hj, *hoff, *hn, *rrow, *rn;
-    double *pres;
-    unsigned char *pflag;
+    int *hoff2, *hn2, *rn2;  // the same of the outer partners (behind the inner ones in rrow)
+    PairRes *pres;
+    double *ptan;      // n x F_t of a slot [3] (written where flagged 2)
     unsigned char *hl;  // owner of a slot: its index within the chunk of 32 particles of its tile
     // records of the pair kernel: the dynamic state of the current set / of
     // the ping-pong planes, and the particle constants (set at every sort)

@@ -251,6 +251,7 @@ __global__ void k_bsort_gather(const BoxDev *__restrict__ boxes, const Tile *__r
             dsti[ICELL * cap + k] = B.key[i];
             dsti[IKEY * cap + k] = B.key[i];
             B.xf[0][k] = make_float4((float)xuw[i], (float)xuw[cap + i], (float)xuw[2 * cap + i], (float)dd);
+            B.xs[k] = B.xf[0][k];
             B.vf[0][k] = make_float4((float)xuw[3 * cap + i], (float)xuw[4 * cap + i], (float)xuw[5 * cap + i], (float)m);
             B.of[0][k] = make_float4((float)xuw[6 * cap + i], (float)xuw[7 * cap + i], (float)xuw[8 * cap + i], 0.f);
             if (!B.lowp) {  // the records of the FP64 pair kernel
@@ -280,6 +281,7 @@ __global__ void k_bsort_flip(BoxDev *boxes, int nboxes, int mark_usub) {
         boxes[b].cur ^= 1;
         if (mark_usub) boxes[b].have_usub = 1;
         *boxes[b].ptop = 0;  // pair slots of the list built next
+        boxes[b].moved[0] = boxes[b].moved[1] = 0;
     }
 }
 

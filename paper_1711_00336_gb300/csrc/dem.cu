@@ -161,7 +161,15 @@ __device__ __forceinline__ void partner(const PairPar<T> &ph, const T n[3], T ga
 }
 
 // list of particle i: partners j != i with |x_j - x_i| < (d_i+d_j)/2 + extra + skin
-// (screened in FP32 with a margin), stored row by row: nlist[i*maxn + k].
+// (screened in FP32 with a margin), stored row by row.  Partners within the
+// inner shell (range + Phys::shell) fill row i from the front, nlist[i*maxn + k],
+// k < nlist_n[i]; the rest fill it from the back, nlist[i*maxn + maxn-1-k],
+// k < nlist_o[i].  While no particle of the box has moved more than shell/2
+// since the sort, only inner pairs can interact and the substeps leave the
+// outer ones alone (BoxDev::moved): with the default skin of half a cell and
+// an interaction range of 3 cells the list has 20 partners a particle, the inner
+// shell 12.  The FP16-storage form (split = 0) keeps one row, outer partners
+// as ~j, and its inner rows apart (k_inner_rows).
 // LANES lanes share a particle (the tile's lanes of the particle-side
 // kernels): lane l scans the cell rows l, l + LANES, ...
 // of the (2R+1)^2 rows around it, counts its partners, takes its offset from
@@ -185,7 +193,8 @@ __global__ void __launch_bounds__(256, DPS_NLIST_MINB) k_build_nlist(const BoxDe
         const Geom g = Bx.g;
         const Phys &ph = Bx.ph;
         const float4 *xf = Bx.xf[0];
-        const float extra = (float)((ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0) + ph.skin) + SCREEN_MARGIN;
+        const float reach = (float)(ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0) + SCREEN_MARGIN;
+        const float extra = reach + (float)ph.skin, inner = reach + ph.shell;
         const float Lf[3] = {(float)g.n[0], (float)g.n[1], (float)g.n[2]};
         const int R = Bx.R, maxn = Bx.maxn;
         // the trip count is uniform over the block: every lane reaches the shuffles
@@ -263,55 +272,77 @@ __global__ void __launch_bounds__(256, DPS_NLIST_MINB) k_build_nlist(const BoxDe
                             const float dx = min_image_f(pj.x - pi.x, Lf[0], g.per[0]);
                             const float dy = min_image_f(pj.y - pi.y, Lf[1], g.per[1]);
                             const float dz = min_image_f(pj.z - pi.z, Lf[2], g.per[2]);
-                            const float rr = 0.5f * (pi.w + pj.w) + extra;
-                            if (dx * dx + dy * dy + dz * dz < rr * rr) fn(j);
+                            const float sr = 0.5f * (pi.w + pj.w), d2 = dx * dx + dy * dy + dz * dz;
+                            const float rr = sr + extra, ri = sr + inner;
+                            if (d2 < rr * rr) fn(j, d2 < ri * ri);
                         }
                 }
             };
             // one lane: a single pass writes the list.  Several lanes: pass 1
             // counts and keeps the first NL_CACHE partners of the lane in
-            // shared memory; pass 2 writes them (scanning again only past that)
-            int cnt = 0;
+            // shared memory (outer ones as ~j); pass 2 writes them (scanning
+            // again only past that)
             int *cache = nl_cache[threadIdx.x];
             int *lst = Bx.nlist + i * (long long)maxn;
-            if (LANES == 1) {
-                scan_rows([&](int j) {
-                    if (cnt < maxn) lst[cnt] = j;
-                    ++cnt;
-                });
-                if (act) {
-                    Bx.nlist_n[i] = min(cnt, maxn);
-                    if (cnt > maxn) atomicOr(Bx.status, ST_NLIST);
+            const bool split = Bx.split != 0;
+            int wi = 0, wo = 0;  // inner and outer partners written
+            auto put = [&](int j, bool in) {
+                // the callers keep wi + wo below maxn
+                lst[split && !in ? maxn - 1 - wo : (split ? wi : wi + wo)] = split || in ? j : ~j;
+                wi += in;
+                wo += !in;
+            };
+            auto counts = [&](int ci, int co) {
+                if (ci + co > maxn) {
+                    atomicOr(Bx.status, ST_NLIST);
+                    ci = co = 0;
                 }
+                Bx.nlist_n[i] = split ? ci : ci + co;
+                Bx.nlist_o[i] = split ? co : 0;
+            };
+            if (LANES == 1) {
+                scan_rows([&](int j, bool in) {
+                    if (wi + wo < maxn) put(j, in);
+                    else (in ? wi : wo)++;
+                });
+                if (act) counts(wi, wo);
                 continue;
             }
-            scan_rows([&](int j) {
-                if (cnt < NL_CACHE) cache[cnt] = j;
+            // counts: inner in the low, outer in the high half of a word (a
+            // box of several lanes has fewer than 2^15 particles)
+            int cnt = 0, cio = 0;
+            scan_rows([&](int j, bool in) {
+                if (cnt < NL_CACHE) cache[cnt] = in ? j : ~j;
                 ++cnt;
+                cio += in ? 1 : 0x10000;
             });
-            // exclusive sum of the counts over the lanes of the group
-            int off = cnt;
+            // exclusive sums of the counts over the lanes of the group
+            int off = cio;
             for (int o = 1; o < LANES; o <<= 1) {
                 const int v = __shfl_up_sync(0xffffffffu, off, o);
                 if (lane >= o) off += v;
             }
             const int total = __shfl_sync(0xffffffffu, off, (threadIdx.x & 31) - lane + LANES - 1);
-            off -= cnt;
+            off -= cio;
             if (!act) continue;
+            const int ti = total & 0xffff, to = total >> 16;
+            wi = off & 0xffff;
+            wo = off >> 16;
+            const bool fits = ti + to <= maxn;  // a row that does not stays empty: the run is flagged and stops
             if (cnt <= NL_CACHE) {
-                for (int c = 0; c < cnt; ++c)
-                    if (off + c < maxn) lst[off + c] = cache[c];
+                for (int c = 0; c < cnt; ++c) {
+                    const int e = cache[c];
+                    if (fits) put(e < 0 ? ~e : e, e >= 0);
+                }
             } else {
-                int w = off;
-                scan_rows([&](int j) {
-                    if (w < maxn && w < off + cnt) lst[w] = j;  // within the lane's counted slots
-                    ++w;
+                // (the second scan finds the partners of the first: the bound
+                // only keeps a lane inside its own counted slots)
+                const int ei = wi + (cio & 0xffff), eo = wo + (cio >> 16);
+                scan_rows([&](int j, bool in) {
+                    if (fits && (in ? wi < ei : wo < eo)) put(j, in);
                 });
             }
-            if (lane == 0) {
-                Bx.nlist_n[i] = min(total, maxn);
-                if (total > maxn) atomicOr(Bx.status, ST_NLIST);
-            }
+            if (lane == 0) counts(ti, to);
         }
     }
 }
@@ -398,21 +429,32 @@ __device__ __noinline__ NearTerms near_pair32(const BoxDev &Bx, const double *__
     return o;
 }
 
-// one thread per particle: wall partners (WALLS; the FP64 form evaluates
-// them with the sphere pairs), then Eq. particle_motion (semi-implicit Euler)
-// and the outputs of the substep
+// v rounded to single precision as the hardware conversion rounds it (nearest,
+// ties to even), in integer operations: the conversion instruction runs on the
+// FP64 pipe
+__device__ __forceinline__ float to_float(double v) {
+    const u64 b = fx_bits(v);
+    const u64 t = b + 0x0fffffffull + ((b >> 29) & 1);
+    if (((u32)(t >> 52) & 0x7ffu) - 897u < 254u)
+        return __uint_as_float((((u32)(t >> 29) - (896u << 23)) & 0x7fffffffu) | ((u32)(b >> 32) & 0x80000000u));
+    return (b << 1) == 0 ? __uint_as_float((u32)(b >> 32)) : (float)v;
+}
+
+// one thread per particle: wall partners (WALLS), then Eq. particle_motion
+// (semi-implicit Euler) and the outputs of the substep.  Comparisons and
+// conversions are integer or FP32 operations (an FP64 compare or conversion
+// costs as much as an FP64 multiply-add), and the spin is integrated only
+// under a torque: 10 FP64 instructions for a particle away from walls, where
+// ~55 were issued before.
 template <bool WALLS, bool F64>
-__device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<double> &pd, long long i,
-                                               int src_tmp, double F[3], double T[3], unsigned nlim, int key_out) {
+__device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, int src_tmp, double F[3], double T[3],
+                                               int key_out) {
     const double *xin = src_tmp ? Bx.xtmp : Bx.pf[Bx.cur];
     double *xout = src_tmp ? Bx.pf[Bx.cur] : Bx.xtmp;
-    const float4 *fin = Bx.xf[src_tmp], *vin = Bx.vf[src_tmp];
-    float4 *fout = Bx.xf[1 - src_tmp], *vout = Bx.vf[1 - src_tmp], *oout = Bx.of[1 - src_tmp];
     const double *pf = Bx.pf[Bx.cur];
     const long long cap = Bx.cap;
-    const Geom g = Bx.g;
+    const Geom &g = Bx.g;
     const Phys &ph = Bx.ph;
-    const double rng_extra = ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0;
     double xi[3], ui[3], wi[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -420,38 +462,54 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<
         ui[a] = xin[(3 + a) * cap + i];
         wi[a] = xin[(6 + a) * cap + i];
     }
-    const float4 pi = fin[i], vi = vin[i];
-    const double di = pf[PD * cap + i];
-    const double mi = pf[PM * cap + i];
-    // walls: the faces of every non-periodic axis (m_ij = m_i, <d> = 2 d_i)
-    const double zero[3] = {0, 0, 0};
+    const float4 xs = Bx.xs[i];  // position at the last sort, and d
+    // walls: the faces of every non-periodic axis (m_ij = m_i, <d> = 2 d_i),
+    // screened in FP32 (xs carries d) with the margin of the pair screen
+    if (WALLS && !(g.per[0] && g.per[1] && g.per[2])) {
+        const float reach = 0.5f * xs.w + (float)(ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0) + SCREEN_MARGIN;
+        const double zero[3] = {0, 0, 0};
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (!WALLS || g.per[a]) continue;
-#pragma unroll
-        for (int side = 0; side < 2; ++side) {
-            const double dist = side == 0 ? xi[a] : g.n[a] - xi[a];
-            const double range = 0.5 * di + rng_extra;
-            if (!(dist < range)) continue;
-            double n[3] = {0, 0, 0};
-            n[a] = side == 0 ? -1.0 : 1.0;
-            partner<double>(pd, n, dist - 0.5 * di, ui, wi, di, zero, zero, mi, 2.0 * di, F, T, nlim);
+        for (int a = 0; a < 3; ++a) {
+            if (g.per[a]) continue;
+            const float xf = to_float(xi[a]);
+            if (!(xf < reach) && !(((float)g.n[a] - xf) < reach) && ph.far_ok) continue;
+            const double rng_extra = ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0;
+            const PairPar<double> pd = pair_par<double>(ph);
+            const double di = pf[PD * cap + i];
+            const double mi = pf[PM * cap + i];
+            unsigned nlim = 0;
+#pragma unroll 1
+            for (int side = 0; side < 2; ++side) {
+                const double dist = side == 0 ? xi[a] : g.n[a] - xi[a];
+                const double range = 0.5 * di + rng_extra;
+                if (!(dist < range)) continue;
+                double n[3] = {0, 0, 0};
+                n[a] = side == 0 ? -1.0 : 1.0;
+                partner<double>(pd, n, dist - 0.5 * di, ui, wi, di, zero, zero, mi, 2.0 * di, F, T, nlim);
+            }
+            if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], (unsigned long long)nlim);
         }
     }
     // Eq. particle_motion, semi-implicit Euler with I = m d^2 / 10
-    const double dt_m = ph.dt_dem * pf[PIM * cap + i], dt_I = ph.dt_dem * pf[PII * cap + i];
-    double d2 = 0.0, xn3[3], un3[3], wn3[3];
+    const double dt_m = ph.dt_dem * pf[PIM * cap + i];
+    double xn3[3], un3[3], wn3[3] = {wi[0], wi[1], wi[2]};
+    if (T[0] != 0.0 || T[1] != 0.0 || T[2] != 0.0) {
+        const double dt_I = ph.dt_dem * pf[PII * cap + i];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) wn3[a] = wi[a] + dt_I * T[a];
+    }
+    float xf[3], d2f = 0.0f;
+    const float xsf[3] = {xs.x, xs.y, xs.z};
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const double Ft = pf[(PFH0 + a) * cap + i] + F[a];
         const double un = ui[a] + dt_m * Ft;
-        const double wn = wi[a] + dt_I * T[a];
         double xn = xi[a] + ph.dt_dem * un;
         if (g.per[a]) {
             const double L = g.n[a];
-            // a particle that left the box folds back in (two comparisons
-            // for the rest, which stay put)
-            if (!(xn >= 0.0 && xn < L)) {
+            // a particle that left the box folds back in; 0 <= xn < L compared
+            // as integers (the order of the bits is that of the values)
+            if (!(fx_bits(xn) < fx_bits(L))) {
                 if (xn >= L) xn -= L;
                 else if (xn < 0.0) xn += L;
                 if (xn >= L || xn < 0.0) xn -= L * floor(xn / L);
@@ -460,16 +518,14 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<
         }
         xn3[a] = xn;
         un3[a] = un;
-        wn3[a] = wn;
         xout[a * cap + i] = xn;
         xout[(3 + a) * cap + i] = un;
-        xout[(6 + a) * cap + i] = wn;
-        const double dd = min_image(xn - pf[(PXS0 + a) * cap + i], g.n[a], g.per[a]);
-        d2 += dd * dd;
+        xout[(6 + a) * cap + i] = wn3[a];
+        xf[a] = to_float(xn);
+        const float dd = min_image_f(xf[a] - xsf[a], (float)g.n[a], g.per[a]);
+        d2f += dd * dd;
     }
-    fout[i] = make_float4((float)xn3[0], (float)xn3[1], (float)xn3[2], pi.w);
-    vout[i] = make_float4((float)un3[0], (float)un3[1], (float)un3[2], vi.w);
-    oout[i] = make_float4((float)wn3[0], (float)wn3[1], (float)wn3[2], 0.f);
+    Bx.xf[1 - src_tmp][i] = make_float4(xf[0], xf[1], xf[2], xs.w);
     if (F64) {
         DemRec r;
 #pragma unroll
@@ -478,6 +534,10 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<
             r.u[a] = un3[a];
         }
         Bx.rec[1 - src_tmp][i] = r;
+    } else {
+        const float mf = Bx.vf[src_tmp][i].w;
+        Bx.vf[1 - src_tmp][i] = make_float4(to_float(un3[0]), to_float(un3[1]), to_float(un3[2]), mf);
+        Bx.of[1 - src_tmp][i] = make_float4(to_float(wn3[0]), to_float(wn3[1]), to_float(wn3[2]), 0.f);
     }
     if (key_out) {
         // last substep of the subcycle: the linked cell of the new position,
@@ -486,9 +546,19 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<
         Bx.key[i] = (int)c;
         atomicAdd(&Bx.count[c], 1);
     }
-    if (d2 > ph.skin_half2) atomicOr(Bx.status, ST_SKIN);
-    if (!(d2 < 1e30)) atomicOr(Bx.status, ST_NAN);
-    if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], (unsigned long long)nlim);
+    // moved beyond skin/2 since the sort, or not finite: decided in FP32
+    // where its rounding cannot matter, else in FP64
+    if (!(d2f < ph.shell_near2)) Bx.moved[1 - src_tmp] = 1;
+    if (!(d2f < ph.skin_near2)) {
+        double d2 = 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double dd = min_image(xn3[a] - pf[(PXS0 + a) * cap + i], g.n[a], g.per[a]);
+            d2 += dd * dd;
+        }
+        if (d2 > ph.skin_half2) atomicOr(Bx.status, ST_SKIN);
+        if (!(d2 < 1e30)) atomicOr(Bx.status, ST_NAN);
+    }
 }
 
 // ---- the substep of the mixed forms ----------------------------------------------------
@@ -504,7 +574,7 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, const PairPar<
 // pair loop waits on the partners' loads and needs every warp slot of the SM,
 // the FP64 update needs registers.
 #ifndef DPS_MIXED_MINB
-#define DPS_MIXED_MINB 8  // 256-thread blocks per SM the register budget of the pair loop is sized for
+#define DPS_MIXED_MINB 4  // 256-thread blocks per SM the register budget of the pair loop is sized for
 #endif
 template <int LANES>
 __global__ void __launch_bounds__(256, DPS_MIXED_MINB) k_dem_pairsum_mixed(const BoxDev *__restrict__ boxes,
@@ -522,6 +592,11 @@ __global__ void __launch_bounds__(256, DPS_MIXED_MINB) k_dem_pairsum_mixed(const
         const float Lf[3] = {(float)g.n[0], (float)g.n[1], (float)g.n[2]};
         const PairPar<float> pfl = pair_par<float>(ph);
         const long long cap = Bx.cap;
+        // outer partners only once a particle of the box has moved shell/2
+        const int outer = Bx.moved[src_tmp];
+        // cleared for this substep's update to set, by one thread of the box: a
+        // store from every block to the word all blocks read costs 20 us a launch
+        if (tl.begin == 0 && threadIdx.x == 0) Bx.moved[1 - src_tmp] = 0;
         // the trip count is uniform over the block, so every lane reaches the shuffles
         for (long long base = tl.begin; base < tl.end; base += ngrp) {
             const long long i = base + grp;
@@ -530,10 +605,19 @@ __global__ void __launch_bounds__(256, DPS_MIXED_MINB) k_dem_pairsum_mixed(const
             unsigned nlim = 0;
             if (act) {
                 const float4 pi = fin[i], vi = vin[i], oi = oin[i];
-                const int nn = Bx.nlist_n[i];
                 const int *row = Bx.nlist + i * (long long)Bx.maxn;
+                int ni = Bx.nlist_n[i], nn = ni + (outer ? Bx.nlist_o[i] : 0);
+                if (!Bx.split && !outer) {
+                    row = Bx.ilist + i * (long long)Bx.maxi;
+                    ni = nn = Bx.ilist_n[i];
+                }
+                const int back = Bx.maxn - 1 + ni;  // outer partner k - ni sits at maxn-1 - (k - ni)
                 for (int k = lane; k < nn; k += LANES) {
-                    const int j = row[k];
+                    int j = row[k < ni ? k : back - k];
+                    if (j < 0) {  // (one-row form) an outer partner, or a gap of the inner rows
+                        if (!outer) continue;
+                        j = ~j;
+                    }
                     const float4 pj = fin[j];
                     const float fx = min_image_f(pj.x - pi.x, Lf[0], g.per[0]);
                     const float fy = min_image_f(pj.y - pi.y, Lf[1], g.per[1]);
@@ -599,7 +683,6 @@ __global__ void __launch_bounds__(128) k_dem_integrate(const BoxDev *__restrict_
         const Tile tl = tiles[t];
         const BoxDev &Bx = boxes[tl.box];
         const long long cap = Bx.cap;
-        const PairPar<double> pd = pair_par<double>(Bx.ph);
         for (long long i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
             double F[3], T[3];
 #pragma unroll
@@ -607,7 +690,40 @@ __global__ void __launch_bounds__(128) k_dem_integrate(const BoxDev *__restrict_
                 F[a] = Bx.psum[a * cap + i];
                 T[a] = Bx.psum[(3 + a) * cap + i];
             }
-            finish_particle<WALLS, false>(Bx, pd, i, src_tmp, F, T, 0u, key_out);
+            finish_particle<WALLS, false>(Bx, i, src_tmp, F, T, key_out);
+        }
+    }
+}
+
+// The inner rows of the FP16-storage form: the inner partners of row i, each kept by
+// the lane (position in the full row modulo the box's lanes per particle) and
+// in the order that the full row gives it, so that a substep over the inner
+// rows adds in the same order as one over the full rows.  Lanes with fewer
+// inner partners end in gaps (-1).  (A change in the last bit of a force, far
+// inside the FP32 forms' tolerance, flips roundings of the FP16 populations:
+// 1e-3 of a force after a few steps.)
+__global__ void __launch_bounds__(128) k_inner_rows(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles,
+                                                    int ntiles) {
+    DPS_FOR_TILES(tiles, ntiles, t) {
+        const Tile tl = tiles[t];
+        const BoxDev &Bx = boxes[tl.box];
+        const int lanes = Bx.dem_lanes;
+        for (long long i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
+            const int n = Bx.nlist_n[i];
+            const int *row = Bx.nlist + i * (long long)Bx.maxn;
+            int *out = Bx.ilist + i * (long long)Bx.maxi;
+            int used[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rows = 0;
+            for (int k0 = 0; k0 < n; k0 += lanes)
+#pragma unroll
+                for (int l = 0; l < 8; ++l)
+                    if (l < lanes && k0 + l < n && row[k0 + l] >= 0) out[used[l]++ * lanes + l] = row[k0 + l];
+#pragma unroll
+            for (int l = 0; l < 8; ++l) rows = max(rows, used[l]);
+#pragma unroll
+            for (int l = 0; l < 8; ++l)
+                if (l < lanes)
+                    for (int m = used[l]; m < rows; ++m) out[m * lanes + l] = -1;
+            Bx.ilist_n[i] = rows * lanes;
         }
     }
 }
@@ -652,10 +768,12 @@ __device__ __forceinline__ int block_excl_sum(int v, int *ws, int &total) {
 // ascending partner, then the pairs owned by its lower partners by ascending
 // owner, then the walls), before the explicit update of Eq. particle_motion.
 
-// After the list build: the pairs particle i owns (partners j > i, ascending
-// j) get consecutive slots from a per-block allocation; its partners k < i
-// go to rrow (ascending k) until k_reverse_slots replaces them by the slots
-// of the pairs (k, i).  Ranks by counting keep the rows free of any sort.
+// After the list build: the pairs particle i owns (partners j > i) get
+// consecutive slots from a per-block allocation, inner ones first (hoff, hn),
+// outer ones (hoff2, hn2) behind the inner slots of the block, each by ascending
+// j; its partners k < i go to rrow (inner, then outer, ascending k) until
+// k_reverse_slots replaces them by the slots of the pairs (k, i).  Ranks by
+// counting keep the rows free of any sort.
 __global__ void __launch_bounds__(256) k_half_rows(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles,
                                                    int ntiles) {
     __shared__ int ws[9];
@@ -667,53 +785,70 @@ __global__ void __launch_bounds__(256) k_half_rows(const BoxDev *__restrict__ bo
         for (long long base = tl.begin; base < tl.end; base += blockDim.x) {  // uniform trip count
             const long long i = base + threadIdx.x;
             const bool act = i < tl.end;
-            int nn = 0, nh = 0;
-            const int *row = Bx.nlist;
+            // part 0: the inner partners (row from the front), part 1: the
+            // outer ones (from the back)
+            int nn[2] = {0, 0}, nh[2] = {0, 0}, off[2], total[2];
+            const int *row[2] = {Bx.nlist, Bx.nlist};
             if (act) {
-                nn = min(Bx.nlist_n[i], maxn);
-                row = Bx.nlist + i * (long long)maxn;
-                for (int k = 0; k < nn; ++k) nh += row[k] > i;
+                nn[0] = Bx.nlist_n[i];
+                nn[1] = Bx.nlist_o[i];
+                row[0] = Bx.nlist + i * (long long)maxn;
+                row[1] = row[0] + maxn - 1;
+                for (int k = 0; k < nn[0]; ++k) nh[0] += row[0][k] > i;
+                for (int k = 0; k < nn[1]; ++k) nh[1] += row[1][-k] > i;
             }
-            int total;
-            const int off = block_excl_sum(nh, ws, total);
-            if (threadIdx.x == 0) sbase = atomicAdd(Bx.ptop, (unsigned long long)total);
+            off[0] = block_excl_sum(nh[0], ws, total[0]);
+            off[1] = block_excl_sum(nh[1], ws, total[1]) + total[0];
+            if (threadIdx.x == 0) sbase = atomicAdd(Bx.ptop, (unsigned long long)(total[0] + total[1]));
             __syncthreads();
-            const long long h0 = (long long)sbase + off;
+            const long long sb = (long long)sbase;
             __syncthreads();  // sbase is written again in the next round
             if (!act) continue;
-            if (h0 + nh > Bx.pcap) {  // not reached: pcap bounds the pairs of any list
+            if (sb + total[0] + total[1] > Bx.pcap) {  // not reached: pcap bounds the pairs of any list
                 atomicOr(Bx.status, ST_NLIST);
-                Bx.hn[i] = Bx.rn[i] = 0;
+                Bx.hn[i] = Bx.rn[i] = Bx.hn2[i] = Bx.rn2[i] = 0;
                 continue;
             }
-            Bx.hoff[i] = (int)h0;
-            Bx.hn[i] = nh;
-            Bx.rn[i] = nn - nh;
+            Bx.hoff[i] = (int)(sb + off[0]);
+            Bx.hoff2[i] = (int)(sb + off[1]);
+            Bx.hn[i] = nh[0];
+            Bx.hn2[i] = nh[1];
+            Bx.rn[i] = nn[0] - nh[0];
+            Bx.rn2[i] = nn[1] - nh[1];
             int *rr = Bx.rrow + i * (long long)maxn;
-            bool asc = true;  // rows of one lane come out ascending
-            for (int k = 1; k < nn; ++k) asc = asc && row[k] > row[k - 1];
-            if (asc) {
-                const int lo = nn - nh;
-                for (int k = 0; k < lo; ++k) rr[k] = row[k];
-                for (int k = lo; k < nn; ++k) {
-                    Bx.hj[h0 + k - lo] = row[k];
-                    Bx.hl[h0 + k - lo] = (unsigned char)((i - tl.begin) & 31);
+            const unsigned char me = (unsigned char)((i - tl.begin) & 31);
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                const long long h0 = sb + off[w];
+                const int n = nn[w], st = w ? -1 : 1;
+                const int *r0 = row[w];
+                bool asc = true;  // rows of one lane come out ascending
+                for (int k = 1; k < n; ++k) asc = asc && r0[st * k] > r0[st * (k - 1)];
+                if (asc) {
+                    const int lo = n - nh[w];
+                    for (int k = 0; k < lo; ++k) rr[k] = r0[st * k];
+                    for (int k = lo; k < n; ++k) {
+                        Bx.hj[h0 + k - lo] = r0[st * k];
+                        Bx.hl[h0 + k - lo] = me;
+                    }
+                } else {
+                    for (int k = 0; k < n; ++k) {
+                        const int j = r0[st * k];
+                        const bool up = j > i;
+                        int r = 0;  // rank of j among the partners on its side of i
+                        for (int m = 0; m < n; ++m) {
+                            const int o = r0[st * m];
+                            r += o < j && (up ? o > i : o < i);
+                        }
+                        if (up) {
+                            Bx.hj[h0 + r] = j;
+                            Bx.hl[h0 + r] = me;
+                        } else {
+                            rr[r] = j;
+                        }
+                    }
                 }
-                continue;
-            }
-            for (int k = 0; k < nn; ++k) {
-                const int j = row[k];
-                const bool up = j > i;
-                int r = 0;  // rank of j among the partners on its side of i
-                for (int m = 0; m < nn; ++m) {
-                    const int o = row[m];
-                    r += o < j && (up ? o > i : o < i);
-                }
-                if (up) {
-                    Bx.hj[h0 + r] = j;
-                    Bx.hl[h0 + r] = (unsigned char)((i - tl.begin) & 31);
-                } else
-                    rr[r] = j;
+                rr += n - nh[w];
             }
         }
     }
@@ -727,11 +862,11 @@ __global__ void __launch_bounds__(256) k_reverse_slots(const BoxDev *__restrict_
         const Tile tl = tiles[t];
         const BoxDev &Bx = boxes[tl.box];
         for (long long i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
-            const int nr = Bx.rn[i];
+            const int ni = Bx.rn[i], nr = ni + Bx.rn2[i];
             int *rr = Bx.rrow + i * (long long)Bx.maxn;
             for (int r = 0; r < nr; ++r) {
                 const int k = rr[r];
-                const int hk = Bx.hn[k], ok = Bx.hoff[k];
+                const int hk = r < ni ? Bx.hn[k] : Bx.hn2[k], ok = r < ni ? Bx.hoff[k] : Bx.hoff2[k];
                 const int *h = Bx.hj + ok;
                 int lo = 0, hi = hk;
                 while (lo < hi) {
@@ -783,7 +918,7 @@ __device__ __forceinline__ double fx_recip(double x, float xf) {
 }
 
 #ifndef DPS_PAIRS_MINB
-#define DPS_PAIRS_MINB 5  // 128-thread blocks per SM the register budget is sized for
+#define DPS_PAIRS_MINB 7  // 128-thread blocks per SM the register budget is sized for
 #endif
 __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
     k_dem_pairs64(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles, int ntiles, int src_tmp) {
@@ -822,18 +957,16 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
             double Fq[3] = {0, 0, 0}, Cq[3] = {0, 0, 0};
             pair64_body(pd, xin, pf, cap, g, j, xi, ui, wi, pf[PD * cap + i], pf[PM * cap + i], rng_extra, Fq, Cq,
                         nlim);
-            // the force in the first plane; n x F_t, nonzero only for
-            // pairs in contact with friction, in the second, flagged 2
+            // n x F_t, nonzero only for pairs in contact with friction, in a
+            // plane of its own, flagged 2
             const long long sq = sl;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) Bx.pres[3 * sq + a] = Fq[a];
-            unsigned char fl = 1;
+            PairRes r = {{Fq[0], Fq[1], Fq[2]}, 1};
             if (Cq[0] != 0.0 || Cq[1] != 0.0 || Cq[2] != 0.0) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) Bx.pres[3 * (Bx.pcap + sq) + a] = Cq[a];
-                fl = 2;
+                for (int a = 0; a < 3; ++a) Bx.ptan[3 * sq + a] = Cq[a];
+                r.flag = 2;
             }
-            Bx.pflag[sq] = fl;
+            Bx.pres[sq] = r;
         };
         // entry k of the warp's queue
         auto eval = [&](int k) {
@@ -869,11 +1002,10 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
                     for (int a = 0; a < 3; ++a) du[a] = ri.u[a] - rj.u[a];
                     const double un = du[0] * o.n[0] + du[1] * o.n[1] + du[2] * o.n[2];
                     const double sn = (al - be) * un;
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) Bx.pres[3 * (long long)sl + a] = sn * o.n[a] - al * du[a];
-                    Bx.pflag[sl] = 1;
+                    const PairRes r = {{sn * o.n[0] - al * du[0], sn * o.n[1] - al * du[1], sn * o.n[2] - al * du[2]}, 1};
+                    Bx.pres[sl] = r;
                 } else if (kind != FX_EXACT) {
-                    Bx.pflag[sl] = 0;
+                    Bx.pres[sl].flag = 0;
                 }
             }
             if (kind == FX_EXACT) {
@@ -889,11 +1021,17 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
         };
 
         int head = 0, qn = 0;  // the warp's ring: qn entries from head
-        for (long long c0 = tl.begin + 32 * wid; c0 < tl.end; c0 += 32 * nw) {
+        // outer pairs only once a particle of the box has moved shell/2
+        const int parts = Bx.moved[src_tmp] ? 2 : 1;
+        // cleared for this substep's update to set, by one thread of the box: a
+        // store from every block to the word all blocks read costs 20 us a launch
+        if (tl.begin == 0 && threadIdx.x == 0) Bx.moved[1 - src_tmp] = 0;
+        for (long long c0 = tl.begin + 32 * wid; c0 < tl.end; c0 += 32 * nw)
+        for (int w = 0; w < parts; ++w) {
             const long long p = c0 + lane;
             const bool own = p < tl.end;
-            const int h0 = __shfl_sync(0xffffffffu, own ? Bx.hoff[p] : 0, 0);
-            const int total = __reduce_add_sync(0xffffffffu, own ? Bx.hn[p] : 0);
+            const int h0 = __shfl_sync(0xffffffffu, own ? (w ? Bx.hoff2[p] : Bx.hoff[p]) : 0, 0);
+            const int total = __reduce_add_sync(0xffffffffu, own ? (w ? Bx.hn2[p] : Bx.hn[p]) : 0);
             for (int t0 = 0; t0 < total; t0 += 32) {
                 const int sl = h0 + t0 + lane;
                 bool pass = false;
@@ -907,7 +1045,7 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
                     const float fz = min_image_f(pj.z - pi.z, Lf[2], g.per[2]);
                     const float fr = 0.5f * (pi.w + pj.w) + rng_extra_f + SCREEN_MARGIN;
                     pass = fx_ * fx_ + fy * fy + fz * fz < fr * fr;
-                    if (!pass) Bx.pflag[sl] = 0;
+                    if (!pass) Bx.pres[sl].flag = 0;
                 }
                 const unsigned m = __ballot_sync(0xffffffffu, pass);
                 if (pass) {
@@ -946,11 +1084,14 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
 // WALLS: some box of the batch has a wall axis (else the wall code is left
 // out: 128 registers instead of 168, more warps for a kernel that waits on
 // the scattered loads of the pair results)
+// A pair's force and flag share one 32-byte record, so an entry costs one
+// sector and one dependent load.  (A force plane and a flag array took three
+// sectors and two loads.)
 #ifndef DPS_GATHER_GC
 #define DPS_GATHER_GC 4  // entries whose loads are issued before any is added
 #endif
 #ifndef DPS_GATHER_MINB
-#define DPS_GATHER_MINB 4  // 128-thread blocks per SM the register budget is sized for
+#define DPS_GATHER_MINB 5  // 128-thread blocks per SM the register budget is sized for
 #endif
 template <bool WALLS>
 __global__ void __launch_bounds__(128, WALLS ? 1 : DPS_GATHER_MINB) k_dem_gather64(const BoxDev *__restrict__ boxes,
@@ -959,71 +1100,69 @@ __global__ void __launch_bounds__(128, WALLS ? 1 : DPS_GATHER_MINB) k_dem_gather
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &Bx = boxes[tl.box];
-        const double *pf = Bx.pf[Bx.cur];
-        const long long cap = Bx.cap;
-        const PairPar<double> pd = pair_par<double>(Bx.ph);
+        const PairRes *__restrict__ pres = Bx.pres;
+        const int parts = Bx.moved[src_tmp] ? 2 : 1;
         for (long long i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
-            const double lev = 0.5 * pf[PD * cap + i];
             double F[3] = {0, 0, 0}, T[3] = {0, 0, 0};
-            const int h0 = Bx.hoff[i], nh = Bx.hn[i];
-            const int nr = Bx.rn[i];
             const int *rr = Bx.rrow + i * (long long)Bx.maxn;
-            // the entries in chunks of GC: the slot indices, flags and results
-            // of a chunk are loaded before any is added (the loads, not the
-            // additions, bound this kernel), a screened-out pair adding zero;
-            // the additions keep the list order
+            // the entries in chunks of GC: the slot indices and records of a
+            // chunk are loaded before any is added; the additions keep the
+            // list order
             constexpr int GC = DPS_GATHER_GC;
+#pragma unroll 1
+            for (int w = 0; w < parts; ++w) {
+            const int h0 = w ? Bx.hoff2[i] : Bx.hoff[i], nh = w ? Bx.hn2[i] : Bx.hn[i];
+            const int nr = w ? Bx.rn2[i] : Bx.rn[i];
+            if (w) rr += Bx.rn[i];
             for (int c0 = 0; c0 < nh + nr; c0 += GC) {
-                long long sl[GC];
-                bool on[GC];
-                double sg[GC];
+                int sl[GC];
 #pragma unroll
                 for (int u = 0; u < GC; ++u) {
                     const int c = c0 + u;
-                    const int s = c < nh ? h0 + c : (c < nh + nr ? rr[c - nh] : -1);
-                    sl[u] = s < 0 ? 0 : s;
-                    on[u] = s >= 0;
-                    sg[u] = c < nh ? 1.0 : -1.0;  // the owner's force, or its opposite on the partner
+                    sl[u] = c < nh ? h0 + c : (c < nh + nr ? rr[c - nh] : -1);
                 }
-                int fl[GC];
+                PairRes r[GC];
 #pragma unroll
                 for (int u = 0; u < GC; ++u) {
-                    fl[u] = on[u] ? Bx.pflag[sl[u]] : 0;
-                    on[u] = fl[u] != 0;
+                    r[u].flag = 0;
+                    if (sl[u] >= 0) r[u] = pres[sl[u]];
                 }
-                // the force of every pair that passed; n x F_t only where the
-                // pair kernel flagged it (2): zero for all others
-                double v[GC][6];
-#pragma unroll
-                for (int u = 0; u < GC; ++u)
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        v[u][a] = on[u] ? Bx.pres[3 * sl[u] + a] : 0.0;
-                        v[u][3 + a] = fl[u] == 2 ? Bx.pres[3 * (Bx.pcap + sl[u]) + a] : 0.0;
-                    }
 #pragma unroll
                 for (int u = 0; u < GC; ++u) {
-                    if (!on[u]) continue;
+                    // the owner's force, its opposite on the partner, or zero:
+                    // selected, not branched on, since each side of a branch
+                    // would issue the three FP64 additions again
+                    const u64 sg = c0 + u < nh ? 0ull : 0x8000000000000000ull;
+                    const u64 on = r[u].flag != 0 ? ~0ull : 0ull;
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        F[a] += sg[u] * v[u][a];
-                        T[a] += lev * v[u][3 + a];
-                    }
+                    for (int a = 0; a < 3; ++a) F[a] += fx_double((fx_bits(r[u].F[a]) ^ sg) & on);
+                    if (r[u].flag == 2)
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) T[a] += Bx.ptan[3 * (long long)sl[u] + a];
                 }
             }
-            finish_particle<WALLS, true>(Bx, pd, i, src_tmp, F, T, 0u, key_out);
+            }
+            if (T[0] != 0.0 || T[1] != 0.0 || T[2] != 0.0) {  // (d_i/2) sum of n x F_t
+                const double lev = 0.5 * Bx.pf[Bx.cur][PD * Bx.cap + i];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) T[a] *= lev;
+            }
+            finish_particle<WALLS, true>(Bx, i, src_tmp, F, T, key_out);
         }
     }
 }
 
 // block: a multiple of 32 and of every tile's lanes (Tile::first).
-// pairs: also the pair rows of the FP64 form (two more launches)
-void launch_build_nlist(const BoxDev *boxes, const Tile *tiles, int ntiles, int grid, int block, int pairs,
+// rows: 1 also the pair rows of the FP64 form (two more launches), 2 the inner
+// rows of the FP16-storage form (one more)
+void launch_build_nlist(const BoxDev *boxes, const Tile *tiles, int ntiles, int grid, int block, int rows,
                         cudaStream_t s) {
     k_build_nlist<<<grid, block, 0, s>>>(boxes, tiles, ntiles);
-    if (pairs) {
+    if (rows == 1) {
         k_half_rows<<<grid, 128, 0, s>>>(boxes, tiles, ntiles);
         k_reverse_slots<<<grid, 128, 0, s>>>(boxes, tiles, ntiles);
+    } else if (rows == 2) {
+        k_inner_rows<<<grid, 128, 0, s>>>(boxes, tiles, ntiles);
     }
 }
 
@@ -1051,7 +1190,7 @@ void launch_dem_substep64(const BoxDev *boxes, const Tile *tiles, int ntiles, in
                           int part_tile, cudaStream_t s) {
     const int warps = part_tile < 32 * PAIR_WARPS ? (part_tile + 31) / 32 : PAIR_WARPS;
     k_dem_pairs64<<<ntiles, 32 * warps, 0, s>>>(boxes, tiles, ntiles, src_tmp);
-    const int grid = ntiles < 152 * 8 ? ntiles : 152 * 8;
+    const int grid = ntiles;
     if (walls)
         k_dem_gather64<true><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
     else

@@ -157,6 +157,10 @@ struct Phys {
     double kfac, xfac;   // k_n = m_ij kfac, xi_n = m_ij xfac (Eqs. damping_to_stiffness, collision_time)
     double capfac;       // lubrication cap = m_ij capfac
     double skin_half2;   // (skin / 2)^2: largest displacement between two sorts
+    float skin_near2;    // squared FP32 displacement below which skin/2 is not exceeded whatever the rounding
+    float shell;         // thickness of the list's inner shell beyond the interaction range
+    float shell_near2;   // squared FP32 displacement below which shell/2 is not exceeded whatever the rounding
+    int far_ok;          // the FP32 screen's margin covers the rounding of a wall distance (box below 2^12 cells)
     int n_int, n_dem;
     int drag, pressure, added_mass, lubrication, contact, lub_limiter;
     int lift;            // Table 1 shear lift (curl of u_f at the subcycle start)

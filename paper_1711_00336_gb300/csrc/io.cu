@@ -318,6 +318,14 @@ void launch_particles_import(double *base, int plane, long long cap, long long n
     if (np <= 0) return;
     k_particles_import<<<grid_for(np, 256), 256, 0, s>>>(base, plane, cap, np, ids, in);
 }
+// velocities of the pair records after an import that moved no particle
+__global__ void k_rec_velocity(DemRec *rec, const double *pf, long long cap, long long np) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < np; i += (long long)gridDim.x * blockDim.x)
+        for (int a = 0; a < 3; ++a) rec[i].u[a] = pf[(PU + a) * cap + i];
+}
+void launch_rec_velocity(DemRec *rec, const double *pf, long long cap, long long np, cudaStream_t s) {
+    if (np > 0) k_rec_velocity<<<grid_for(np, 256), 256, 0, s>>>(rec, pf, cap, np);
+}
 long long reduce_partials_doubles() { return (long long)RED_BLOCKS * FLUID_Q; }
 
 #define DPS_IO_INST_ST(ST, FT)                                                                                 \

@@ -81,3 +81,67 @@ def test_fp64_pairs_against_the_oracle(name):
     dx -= np.where(per, n, 0) * np.round(dx / np.array(n))
     assert np.abs(dx).max() <= TOL * np.abs(r["u"]).max()
     assert st["status"] == 0
+
+
+@pytest.mark.parametrize("fast", [0.0, 0.3])
+def test_written_velocities_and_moves_beyond_the_inner_shell(fast):
+    """Velocities written between sorts reach the pairs, and particles that
+    leave the list's inner shell within a subcycle (0.3 cells per step against
+    0.05) still meet every partner."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle as O
+    from paper_1711_00336_gb300 import dps
+    n, per = (14, 13, 12), (1, 0, 1)
+    p = lattice(np.array(n, float), np.array(per), seed=3, spacing=1.35, d=1.0, jitter=0.15)
+    u = p["u"].copy()
+    u[::17, 0] += fast
+    kw = dict(g=(0.0, 0.0, -1e-4), e_n=0.9, mu_c=0.25, T_c=2.0, h_c=0.5, h_min=1e-5, C_am=0.5, n_int=1, n_dem=20,
+              lub_limiter=1, lub_cap=0.25, eps_min=0.05)
+    dom = dps.Domain(n, per, 0.7, "f64", max_particles=len(p["x"]))
+    dom.add_particles(p["x"], p["d"], p["rho_p"], u=p["u"], w=p["w"])
+    dom.set_closure(fb_mode=0, fb=(0, 0, 0), skin=0.8, drag=0, pressure=0, added_mass=0, **kw)
+    dom.prepare()
+    dom.write_particles(u=u)
+    dom.step(1)
+    got = dom.read_particles()
+    dom.close()
+    P = O.make_params(n, per, 0.7, drag=0, pressure=0, added_mass=0, **kw)
+    ref = O.Domain(P, x=p["x"], u=u, w=p["w"], d=p["d"], rho_p=p["rho_p"])
+    ref.step(1)
+    r = ref.particles()
+    for k in ("u", "w"):
+        assert np.abs(got[k] - r[k]).max() <= TOL * np.abs(r[k]).max(), k
+
+
+@pytest.mark.parametrize("form", ["f64", "f16s"])
+@pytest.mark.parametrize("extra", [0, 3000])
+def test_outer_pairs_add_nothing_to_slow_particles(form, extra):
+    """A lone fast sphere makes every substep after the first visit the outer
+    pairs of the list; the other spheres, all slow, end with the same bits (the
+    FP32 form deals the entries to its lanes anew, so its sums round anew).
+    (extra: enough spheres that a particle is given fewer lanes.)"""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1711_00336_gb300 import dps
+    n, per = (14, 13, 40) if not extra else (26, 25, 40), (1, 1, 1)
+    p = lattice(np.array((n[0], n[1], 20 if not extra else 26), float), np.array(per), seed=4, spacing=1.25, d=1.0,
+                jitter=0.11)
+    assert len(p["x"]) > extra
+    kw = dict(g=(0.0, 0.0, -1e-4), fb_mode=0, fb=(0, 0, 0), e_n=0.9, mu_c=0.25, T_c=2.0, h_c=0.5, h_min=1e-5, C_am=0.5,
+              n_int=1, n_dem=8, lub_limiter=1, lub_cap=0.25, eps_min=0.05, skin=0.8, drag=0, pressure=0, added_mass=0)
+    out = []
+    for speed in (0.0, 0.35):
+        x = np.vstack([p["x"], [[n[0] / 2, n[1] / 2, 33.0]]])
+        u = np.vstack([p["u"], [[speed, 0.0, 0.0]]])
+        w = np.vstack([p["w"], [[0.0, 0.0, 0.0]]])
+        dom = dps.Domain(n, per, 0.7, form, max_particles=len(x))
+        dom.add_particles(x, np.append(p["d"], 1.0), np.append(p["rho_p"], 2.5), u=u, w=w)
+        dom.set_closure(**kw)
+        dom.step(1)
+        out.append(dom.read_particles())
+        dom.close()
+    for k in ("x", "u", "w"):
+        assert np.array_equal(out[0][k][:-1], out[1][k][:-1]), k
