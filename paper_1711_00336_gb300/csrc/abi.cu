@@ -44,15 +44,15 @@ void launch_bscan(const BoxDev *, int, const Tile *, int, cudaStream_t);
 int scan_tile_cells();
 void brick_tiles(int, const int *, std::vector<Tile> &);
 template <typename FT>
-void launch_eps(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+void launch_eps(const BoxDev *, const Tile *, int, cudaStream_t);
 template <typename FT>
 void launch_force_am(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename FT>
 void launch_force_drag(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 template <typename FT>
-void launch_reaction_am(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+void launch_reaction_am(const BoxDev *, const Tile *, int, cudaStream_t);
 template <typename FT>
-void launch_reaction_drag(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
+void launch_reaction_drag(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 void launch_dem_substep(const BoxDev *, const Tile *, int, int, int, int, int, int, int, cudaStream_t);
 void launch_dem_substep64(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
 void launch_build_nlist(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
@@ -552,16 +552,16 @@ static void enqueue_sort_eps(Batch *B, int xsel, int mark_usub, bool have_keys) 
     tend(B, PH_SORT, cnt + 3 + 3 * pl + 1 + pl * (1 + (rows == 1 ? 2 : rows == 2)));
     tbegin(B);
     if (B->fel == 8)
-        launch_eps<double>(T, B->d_brick, B->n_brick, grid_of(B->n_brick), 256, B->stream);
+        launch_eps<double>(T, B->d_brick, B->n_brick, B->stream);
     else
-        launch_eps<float>(T, B->d_brick, B->n_brick, grid_of(B->n_brick), 256, B->stream);
+        launch_eps<float>(T, B->d_brick, B->n_brick, B->stream);
     tend(B, PH_EPS, 1);
 }
 
 static void enqueue_step(Batch *B) {
     const BoxDev *T = B->d_table;
     const Tuning &u = B->tune;
-    const int gc = grid_of(B->n_cell), gp = grid_of(B->n_part), gb = grid_of(B->n_brick);
+    const int gc = grid_of(B->n_cell), gp = grid_of(B->n_part);
     const int pl = B->n_part > 0;
     const bool f64 = B->fel == 8;
     cudaStream_t s = B->stream;
@@ -591,8 +591,8 @@ static void enqueue_step(Batch *B) {
         }
         tend(B, PH_FAM, pl + nl);
         tbegin(B);
-        if (f64) launch_reaction_am<double>(T, B->d_brick, B->n_brick, gb, 256, s);
-        else launch_reaction_am<float>(T, B->d_brick, B->n_brick, gb, 256, s);
+        if (f64) launch_reaction_am<double>(T, B->d_brick, B->n_brick, s);
+        else launch_reaction_am<float>(T, B->d_brick, B->n_brick, s);
         tend(B, PH_RAM, 1);
         tbegin(B);
         if (pl) {
@@ -613,9 +613,9 @@ static void enqueue_step(Batch *B) {
         }
         tbegin(B, rs);
         if (f64)
-            launch_reaction_drag<double>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, gb, 256, rs);
+            launch_reaction_drag<double>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, rs);
         else
-            launch_reaction_drag<float>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, gb, 256, rs);
+            launch_reaction_drag<float>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, rs);
         tend(B, PH_RDRAG, 1, rs);
         if (fork) cudaEventRecord(B->ev_join, B->side);
         tbegin(B);

@@ -310,10 +310,10 @@ template <> __device__ __forceinline__ const float *weights_of<float>(const BoxD
 // ---- brick-tiled gathers ---------------------------------------------------------
 // A brick is a block of up to 8x8x8 cells of one box (Tile::begin and
 // Tile::end pack its origin and extent, 21 bits per axis).  The block first
-// stages the particle ranges of the brick's cells and their one-cell halo in
-// shared memory (one cell_start pair per halo cell instead of 27 per cell),
-// then every thread gathers over the 27 neighbours of its cells in a fixed
-// order: o_z, o_y, o_x ascending, then the sorted order inside a cell.
+// stages the particles of the brick's cells and their one-cell halo in
+// shared memory, then every thread gathers over the 27 neighbours of its cells
+// in a fixed order: o_z, o_y, o_x ascending, then the sorted order inside a
+// cell.
 constexpr int BRICK = 8;
 constexpr int HALO = BRICK + 2;
 constexpr int HALO3 = HALO * HALO * HALO;
@@ -327,32 +327,6 @@ __device__ __forceinline__ void brick_unpack(long long v, int &x, int &y, int &z
     z = (int)((v >> 42) & 0x1FFFFF);
 }
 
-struct BrickRanges {
-    int s[HALO3], e[HALO3];
-};
-
-// gather over the 27 halo neighbours of brick cell (lx,ly,lz) with weights w
-template <typename WT, typename Fn>
-__device__ __forceinline__ void gather27_staged(const BrickRanges &R, int lx, int ly, int lz, const WT *__restrict__ w,
-                                                long long cap, Fn &&fn) {
-#pragma unroll 1
-    for (int oz = -1; oz <= 1; ++oz) {
-        const WT *wz = w + (6 + 1 - oz) * cap;
-#pragma unroll 1
-        for (int oy = -1; oy <= 1; ++oy) {
-            const WT *wy = w + (3 + 1 - oy) * cap;
-            const int hrow = (lz + 1 + oz) * HALO * HALO + (ly + 1 + oy) * HALO + (lx + 1);
-#pragma unroll
-            for (int ox = -1; ox <= 1; ++ox) {
-                const int h = hrow + ox;
-                const int s = R.s[h], e = R.e[h];
-                const WT *wx = w + (1 - ox) * cap;
-                for (int p = s; p < e; ++p) fn(p, wx[p] * wy[p] * wz[p]);
-            }
-        }
-    }
-}
-
 // iterate the cells of the current brick tile: fn(cell index, lx, ly, lz)
 template <typename Fn>
 __device__ __forceinline__ void for_brick_cells(const Geom &g, int ox, int oy, int oz, int ex, int ey, int ez, Fn &&fn) {
@@ -363,32 +337,44 @@ __device__ __forceinline__ void for_brick_cells(const Geom &g, int ox, int oy, i
     }
 }
 
-// Compacted particle list of a brick and its halo: entry m is particle P[m]
-// of halo cell with x coordinate hx[m]; the entries of halo cell h are
-// [off[h], off[h+1]) in ascending h, then sorted order.  A warp gathers over
-// the rows (hz, hy) of the bounding box of its cells' supports only, so with
-// sparse particles it visits the few particles near it once, instead of each
-// lane testing all 27 neighbour cells (a warp pays for the busiest lane of
-// every neighbour cell).  The per-cell visit order is the one of
-// gather27_staged: ascending h is ascending (o_z, o_y, o_x) for a fixed cell.
+// The particles of a brick and its halo, staged in shared memory: entry m is a
+// particle of halo cell h for off[h] <= m < off[h+1] (ascending h, then sorted
+// order), with its nine kernel weights and the NV values that are spread.  The
+// three x neighbours of a cell are consecutive halo cells, so the 27
+// neighbours are nine runs of entries.  A thread first lists the entries of its
+// cell's support (integers only), then adds them in that order, so a warp pays
+// for the longest list among its 32 cells (~8 entries at 3 per cell) and not,
+// cell by cell of the support, for the busiest lane (~27 rounds of five
+// FP64 instructions); weights and values come from shared memory.  The three
+// gathers together, before / after: 17.9 / 7.6 ms a step (256^3, eps 0.2, two
+// subcycles, FP64), 3.1 / 2.1 ms (192^3, eps 0.38, FP32), 4.5 / 3.6 ms (256^3,
+// eps 0.05, FP16 storage); FP64 is bound by its five FP64 instructions an entry.
 constexpr int BRICK_THREADS = 256;  // block size of every brick kernel
-// entries; above it (about 0.13 particles per halo cell) the block takes the
-// per-cell walk of gather27_staged, faster once most probes find particles
-// (measured: the list wins at 0.02 particles per cell, the walk at 0.2)
-constexpr int BL_MAX = 128;
+constexpr int LIST_CAP = 24;        // entries a thread lists before it adds them
 constexpr int BL_PER_THREAD = (HALO3 + BRICK_THREADS - 1) / BRICK_THREADS;
+// staged entries: three (FP64) or four (FP32) blocks fit an SM's shared memory;
+// denser bricks take the walk over global memory
+template <typename FT> constexpr int stage_cap() { return sizeof(FT) == 8 ? 448 : 704; }
 
-struct BrickList {
-    BrickRanges R;
-    int off[HALO3 + 1];
-    int P[BL_MAX];
-    unsigned char hx[BL_MAX];
+template <typename FT, int NV>
+struct BrickStage {
+    static constexpr int CAP = stage_cap<FT>();
+    FT w[9][CAP], v[NV][CAP];
+    int off[HALO3 + 1], start[HALO3];
+    union {
+        int P[CAP];
+        unsigned short list[LIST_CAP][BRICK_THREADS];
+    };
     int wsum[BRICK_THREADS / 32];
-    int n;  // entries, or -1 when over BL_MAX
+    int n;  // entries, or -1 when over CAP
+    unsigned char hx[CAP];
 };
 
-// stage the ranges and the compacted list of brick (ox,oy,oz); ends with a barrier
-__device__ __forceinline__ void stage_list(const BoxDev &B, int ox, int oy, int oz, BrickList &L) {
+// stage brick (ox,oy,oz); value(p, k): the k-th value of particle p.  Ends with a barrier
+template <typename FT, int NV, typename Val>
+__device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int oz, int ex, int ey, int ez,
+                                            const FT *__restrict__ w, BrickStage<FT, NV> &S, Val &&value) {
+    constexpr int CAP = BrickStage<FT, NV>::CAP;
     const Geom &g = B.g;
     int s0[BL_PER_THREAD], cnt[BL_PER_THREAD], tot = 0;
 #pragma unroll
@@ -400,13 +386,13 @@ __device__ __forceinline__ void stage_list(const BoxDev &B, int ox, int oy, int 
             const int x = wrap_axis(ox + hx - 1, g.n[0], g.per[0]);
             const int y = wrap_axis(oy + hy - 1, g.n[1], g.per[1]);
             const int z = wrap_axis(oz + hz - 1, g.n[2], g.per[2]);
-            if (x >= 0 && y >= 0 && z >= 0) {
+            // (a clipped brick has a smaller halo)
+            if (hx <= ex + 1 && hy <= ey + 1 && hz <= ez + 1 && x >= 0 && y >= 0 && z >= 0) {
                 const long long n = cell_index(g, x, y, z);
                 a = B.cell_start[n];
                 e = B.cell_start[n + 1];
             }
-            L.R.s[h] = a;
-            L.R.e[h] = e;
+            S.start[h] = a;
         }
         s0[u] = a;
         cnt[u] = e - a;
@@ -420,88 +406,110 @@ __device__ __forceinline__ void stage_list(const BoxDev &B, int ox, int oy, int 
         const int v = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += v;
     }
-    if (lane == 31) L.wsum[wid] = incl;
+    if (lane == 31) S.wsum[wid] = incl;
     __syncthreads();
     int base = 0, total = 0;
 #pragma unroll
     for (int q = 0; q < BRICK_THREADS / 32; ++q) {
-        base += q < wid ? L.wsum[q] : 0;
-        total += L.wsum[q];
+        base += q < wid ? S.wsum[q] : 0;
+        total += S.wsum[q];
     }
     int run = base + incl - tot;
-    const bool fits = total <= BL_MAX;
+    const bool fits = total <= CAP;
 #pragma unroll
     for (int u = 0; u < BL_PER_THREAD; ++u) {
         const int h = BL_PER_THREAD * threadIdx.x + u;
         if (h < HALO3) {
-            L.off[h] = run;
+            S.off[h] = run;
             if (fits)
                 for (int m = 0; m < cnt[u]; ++m) {
-                    L.P[run + m] = s0[u] + m;
-                    L.hx[run + m] = (unsigned char)(h % HALO);
+                    S.P[run + m] = s0[u] + m;
+                    S.hx[run + m] = (unsigned char)(h % HALO);
                 }
         }
         run += cnt[u];
     }
     if (threadIdx.x == 0) {
-        L.off[HALO3] = total;
-        L.n = fits ? total : -1;
+        S.off[HALO3] = total;
+        S.n = fits ? total : -1;
     }
     __syncthreads();
+    if (fits)
+        for (int m = threadIdx.x; m < total; m += BRICK_THREADS) {
+            const int p = S.P[m];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) S.w[k][m] = w[k * B.cap + p];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) S.v[k][m] = value(p, k);
+        }
+    __syncthreads();  // P becomes the lists
 }
 
-// for every cell c of the brick: St st{}; acc(st, p, W_p(c)) over the
-// particles of its support in the order of gather27_staged; fin(st, c)
-template <typename St, typename WT, typename Acc, typename Fin>
-__device__ __forceinline__ void brick_gather(const Geom &g, const BrickList &L, int ox, int oy, int oz, int ex, int ey,
-                                             int ez, const WT *__restrict__ w, long long cap, Acc &&acc, Fin &&fin) {
-    if (L.n < 0) {
-        for_brick_cells(g, ox, oy, oz, ex, ey, ez, [&](long long c, int lx, int ly, int lz) {
-            St st{};
-            gather27_staged(L.R, lx, ly, lz, w, cap, [&](int p, WT W) { acc(st, p, W); });
-            fin(st, c);
-        });
-        return;
-    }
-    const int nb = ex * ey * ez;
-    for (int k0 = 0; k0 < nb; k0 += blockDim.x) {  // trip count uniform over the block
-        const int k = k0 + threadIdx.x;
-        const bool act = k < nb;
-        int lx = 0, ly = 0, lz = 0;
-        if (act) {
-            lx = k % ex;
-            ly = (k / ex) % ey;
-            lz = k / (ex * ey);
-        }
-        if (!__any_sync(0xffffffffu, act)) continue;
-        // halo bounding box of the warp's supports: [min l, max l + 2] per axis
-        const int BIG = 1 << 20;
-        const int bx0 = __reduce_min_sync(0xffffffffu, act ? lx : BIG);
-        const int by0 = __reduce_min_sync(0xffffffffu, act ? ly : BIG);
-        const int bz0 = __reduce_min_sync(0xffffffffu, act ? lz : BIG);
-        const int bx1 = __reduce_max_sync(0xffffffffu, act ? lx : -BIG) + 2;
-        const int by1 = __reduce_max_sync(0xffffffffu, act ? ly : -BIG) + 2;
-        const int bz1 = __reduce_max_sync(0xffffffffu, act ? lz : -BIG) + 2;
-        St st{};
-        for (int hz = bz0; hz <= bz1; ++hz) {
-            const int dz = hz - (lz + 1);
-            for (int hy = by0; hy <= by1; ++hy) {
-                const int dy = hy - (ly + 1);
-                const int hrow = (hz * HALO + hy) * HALO;
-                const int m0 = L.off[hrow + bx0], m1 = L.off[hrow + bx1 + 1];
-                if (!act || dz < -1 || dz > 1 || dy < -1 || dy > 1) continue;
-                const WT *wz = w + (6 + 1 - dz) * cap, *wy = w + (3 + 1 - dy) * cap;
-                for (int m = m0; m < m1; ++m) {
-                    const int dx = (int)L.hx[m] - (lx + 1);
-                    if (dx < -1 || dx > 1) continue;
-                    const int p = L.P[m];
-                    const WT *wx = w + (1 - dx) * cap;
-                    acc(st, p, wx[p] * wy[p] * wz[p]);
+// for every cell c of the brick: sums s[k] of W_p(c) v_k(p) over the particles
+// of its support, in the order o_z, o_y, o_x ascending, then sorted; fin(s, c)
+template <typename FT, int NV, typename Val, typename Fin>
+__device__ __forceinline__ void brick_gather(const BoxDev &B, BrickStage<FT, NV> &S, int ox, int oy, int oz, int ex,
+                                             int ey, int ez, const FT *__restrict__ w, Val &&value, Fin &&fin) {
+    const long long cap = B.cap;
+    for_brick_cells(B.g, ox, oy, oz, ex, ey, ez, [&](long long c, int lx, int ly, int lz) {
+        FT s[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) s[k] = FT(0);
+        if (S.n < 0) {  // over the staged size: the walk over global memory
+#pragma unroll 1
+            for (int r = 0; r < 9; ++r) {
+                const int dz = r / 3 - 1, dy = r % 3 - 1;
+                const FT *wz = w + (6 + 1 - dz) * cap, *wy = w + (3 + 1 - dy) * cap;
+                const int hrow = ((lz + 1 + dz) * HALO + ly + 1 + dy) * HALO + lx + 1;
+#pragma unroll
+                for (int dx = -1; dx <= 1; ++dx) {
+                    const int h = hrow + dx, p0 = S.start[h], p1 = p0 + S.off[h + 1] - S.off[h];
+                    const FT *wx = w + (1 - dx) * cap;
+                    for (int p = p0; p < p1; ++p) {
+                        const FT W = wx[p] * wy[p] * wz[p];
+#pragma unroll
+                        for (int k = 0; k < NV; ++k) s[k] += W * value(p, k);
+                    }
                 }
             }
+            fin(s, c);
+            return;
         }
-        if (act) fin(st, cell_index(g, ox + lx, oy + ly, oz + lz));
-    }
+        if (S.n > 0) {
+            // list LIST_CAP entries, add them, and so on (rounds in step over
+            // the warp: a lane that filled its list early and added alone
+            // would cost its whole round again)
+            unsigned short *list = &S.list[0][threadIdx.x];
+            const int h0 = (lz * HALO + ly) * HALO + lx;
+            int done = 0, total;
+            do {
+                total = 0;
+#pragma unroll
+                for (int r = 0; r < 9; ++r) {
+                    const int h = h0 + (r / 3 * HALO + r % 3) * HALO;
+                    const int m1 = S.off[h + 3];
+                    for (int m = S.off[h]; m < m1; ++m, ++total) {
+                        // weights of the particle's cell offset: index 1 - (dx, dy, dz)
+                        const int kx = lx + 2 - (int)S.hx[m], ky = 2 - r % 3, kz = 2 - r / 3;
+                        if ((unsigned)(total - done) < (unsigned)LIST_CAP)
+                            list[(total - done) * BRICK_THREADS] =
+                                (unsigned short)(m | (kx << 10) | (ky << 12) | (kz << 14));
+                    }
+                }
+                const int cnt = min(total - done, LIST_CAP);
+#pragma unroll 2
+                for (int q = 0; q < cnt; ++q) {
+                    const unsigned e = list[q * BRICK_THREADS];
+                    const int p = e & 1023, kx = (e >> 10) & 3, ky = (e >> 12) & 3, kz = e >> 14;
+                    const FT W = S.w[kx][p] * S.w[3 + ky][p] * S.w[6 + kz][p];
+#pragma unroll
+                    for (int k = 0; k < NV; ++k) s[k] += W * S.v[k][p];
+                }
+                done += LIST_CAP;
+            } while (done < total);
+        }
+        fin(s, c);
+    });
 }
 
 // ---- S2: eps_f ------------------------------------------------------------------
@@ -511,46 +519,38 @@ __device__ __forceinline__ void brick_gather(const Geom &g, const BrickList &L, 
 template <typename FT>
 __global__ void __launch_bounds__(BRICK_THREADS) k_eps_gather(const BoxDev *__restrict__ boxes,
                                                               const Tile *__restrict__ tiles, int ntiles) {
-    __shared__ BrickList L;
+    extern __shared__ __align__(16) unsigned char smem[];
+    BrickStage<FT, 1> &S = *(BrickStage<FT, 1> *)smem;
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
-        const Geom g = B.g;
         int ox, oy, oz, ex, ey, ez;
         brick_unpack(tl.begin, ox, oy, oz);
         brick_unpack(tl.end, ex, ey, ez);
-        __syncthreads();  // the previous brick is done with L
-        stage_list(B, ox, oy, oz, L);
+        __syncthreads();  // the previous brick is done with S
         const double *pf = B.pf[B.cur];
         const long long cap = B.cap;
         const FT *w = weights_of<FT>(B, pf);
         const float4 *xf = B.xf[0];
+        auto volume = [&](int p, int) -> FT {
+            if (sizeof(FT) == 8) return (FT)pf[PVOL * cap + p];  // stored at the sort
+            const FT d = (FT)xf[p].w;
+            return FT(PI_D / 6.0) * d * d * d;
+        };
+        stage_brick<FT, 1>(B, ox, oy, oz, ex, ey, ez, w, S, volume);
         FT *eps = (FT *)B.eps;
         const FT eps_min = (FT)B.ph.eps_min;
         unsigned nclamp = 0;
-        struct St {
-            FT ep;
-        };
-        brick_gather<St>(
-            g, L, ox, oy, oz, ex, ey, ez, w, cap,
-            [&](St &st, int p, FT W) {
-                if (sizeof(FT) == 8) {
-                    st.ep += W * (FT)pf[PVOL * cap + p];  // the volume stored at the sort
-                } else {
-                    const FT d = (FT)xf[p].w;
-                    st.ep += W * (FT(PI_D / 6.0) * d * d * d);
-                }
-            },
-            [&](St &st, long long c) {
-                FT e = FT(1) - st.ep;
-                if (e < eps_min) {
-                    if (e < FT(0)) atomicOr(B.status, ST_EPS_NEG);
-                    ++nclamp;
-                    e = eps_min;
-                }
-                eps[c] = e;
-                B.count[c] = 0;
-            });
+        brick_gather<FT, 1>(B, S, ox, oy, oz, ex, ey, ez, w, volume, [&](const FT *s, long long c) {
+            FT e = FT(1) - s[0];
+            if (e < eps_min) {
+                if (e < FT(0)) atomicOr(B.status, ST_EPS_NEG);
+                ++nclamp;
+                e = eps_min;
+            }
+            eps[c] = e;
+            B.count[c] = 0;
+        });
         if (nclamp) atomicAdd(&B.counters[CNT_EPS_CLAMP], (unsigned long long)nclamp);
     }
 }
@@ -804,35 +804,26 @@ template <> __device__ __forceinline__ const float *force_planes<float>(const Bo
 template <typename FT>
 __global__ void __launch_bounds__(BRICK_THREADS) k_reaction_am(const BoxDev *__restrict__ boxes,
                                                                const Tile *__restrict__ tiles, int ntiles) {
-    __shared__ BrickList L;
+    extern __shared__ __align__(16) unsigned char smem[];
+    BrickStage<FT, 3> &S = *(BrickStage<FT, 3> *)smem;
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
-        const Geom g = B.g;
         int ox, oy, oz, ex, ey, ez;
         brick_unpack(tl.begin, ox, oy, oz);
         brick_unpack(tl.end, ex, ey, ez);
         __syncthreads();
-        stage_list(B, ox, oy, oz, L);
-        const long long N = g.ncell, cap = B.cap;
+        const long long N = B.g.ncell, cap = B.cap;
         const double *pf = B.pf[B.cur];
         const FT *w = weights_of<FT>(B, pf), *Fa = force_planes<FT>(B, pf, 0);
+        auto force = [&](int p, int k) { return Fa[k * cap + p]; };
+        stage_brick<FT, 3>(B, ox, oy, oz, ex, ey, ez, w, S, force);
         FT *fam = (FT *)B.fam;
-        struct St {
-            FT s0, s1, s2;
-        };
-        brick_gather<St>(
-            g, L, ox, oy, oz, ex, ey, ez, w, cap,
-            [&](St &st, int p, FT W) {
-                st.s0 += W * Fa[p];
-                st.s1 += W * Fa[cap + p];
-                st.s2 += W * Fa[2 * cap + p];
-            },
-            [&](St &st, long long c) {
-                fam[c] = -st.s0;
-                fam[N + c] = -st.s1;
-                fam[2 * N + c] = -st.s2;
-            });
+        brick_gather<FT, 3>(B, S, ox, oy, oz, ex, ey, ez, w, force, [&](const FT *s, long long c) {
+            fam[c] = -s[0];
+            fam[N + c] = -s[1];
+            fam[2 * N + c] = -s[2];
+        });
     }
 }
 
@@ -842,43 +833,34 @@ template <typename FT>
 __global__ void __launch_bounds__(BRICK_THREADS) k_reaction_drag(const BoxDev *__restrict__ boxes,
                                                                  const Tile *__restrict__ tiles, int ntiles, int first,
                                                                  int last) {
-    __shared__ BrickList L;
+    extern __shared__ __align__(16) unsigned char smem[];
+    BrickStage<FT, 3> &S = *(BrickStage<FT, 3> *)smem;
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
-        const Geom g = B.g;
         int ox, oy, oz, ex, ey, ez;
         brick_unpack(tl.begin, ox, oy, oz);
         brick_unpack(tl.end, ex, ey, ez);
         __syncthreads();
-        stage_list(B, ox, oy, oz, L);
-        const long long N = g.ncell, cap = B.cap;
+        const long long N = B.g.ncell, cap = B.cap;
         const double *pf = B.pf[B.cur];
         const FT *w = weights_of<FT>(B, pf), *Fd = force_planes<FT>(B, pf, 1);
+        auto force = [&](int p, int k) { return Fd[k * cap + p]; };
+        stage_brick<FT, 3>(B, ox, oy, oz, ex, ey, ez, w, S, force);
         const FT *fam = (const FT *)B.fam;
         FT *acc = (FT *)B.acc, *fpf = (FT *)B.fpf;
         const FT inv_nint = (FT)B.ph.dt_sub;
-        struct St {
-            FT s[3];
-        };
-        brick_gather<St>(
-            g, L, ox, oy, oz, ex, ey, ez, w, cap,
-            [&](St &st, int p, FT W) {
-                st.s[0] += W * Fd[p];
-                st.s[1] += W * Fd[cap + p];
-                st.s[2] += W * Fd[2 * cap + p];
-            },
-            [&](St &st, long long c) {
+        brick_gather<FT, 3>(B, S, ox, oy, oz, ex, ey, ez, w, force, [&](const FT *s, long long c) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const FT k = fam[a * N + c] - st.s[a];
-                    const FT v = first ? k : acc[a * N + c] + k;
-                    if (last)
-                        fpf[a * N + c] = v * inv_nint;
-                    else
-                        acc[a * N + c] = v;
-                }
-            });
+            for (int a = 0; a < 3; ++a) {
+                const FT k = fam[a * N + c] - s[a];
+                const FT v = first ? k : acc[a * N + c] + k;
+                if (last)
+                    fpf[a * N + c] = v * inv_nint;
+                else
+                    acc[a * N + c] = v;
+            }
+        });
     }
 }
 
@@ -936,9 +918,15 @@ void launch_bsort_flip(BoxDev *b, int nb, int mark_usub, cudaStream_t s) {
 }
 void launch_end_step(BoxDev *b, int nb, cudaStream_t s) { k_end_step<<<(nb + 127) / 128, 128, 0, s>>>(b, nb); }
 
+// brick kernels: one block per brick and opt-in shared memory for the stage
+template <typename K, typename... Args>
+static void launch_brick(K kernel, size_t smem, int nt, cudaStream_t s, Args... args) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kernel<<<nt, BRICK_THREADS, smem, s>>>(args...);
+}
 template <typename FT>
-void launch_eps(const BoxDev *b, const Tile *t, int nt, int grid, int block, cudaStream_t s) {
-    k_eps_gather<FT><<<grid, BRICK_THREADS, 0, s>>>(b, t, nt);
+void launch_eps(const BoxDev *b, const Tile *t, int nt, cudaStream_t s) {
+    launch_brick(k_eps_gather<FT>, sizeof(BrickStage<FT, 1>), nt, s, b, t, nt);
 }
 template <typename FT>
 void launch_force_am(const BoxDev *b, const Tile *t, int nt, int grid, int block, cudaStream_t s) {
@@ -949,21 +937,20 @@ void launch_force_drag(const BoxDev *b, const Tile *t, int nt, int first, int gr
     k_force_drag<FT><<<grid, block, 0, s>>>(b, t, nt, first);
 }
 template <typename FT>
-void launch_reaction_am(const BoxDev *b, const Tile *t, int nt, int grid, int block, cudaStream_t s) {
-    k_reaction_am<FT><<<grid, BRICK_THREADS, 0, s>>>(b, t, nt);
+void launch_reaction_am(const BoxDev *b, const Tile *t, int nt, cudaStream_t s) {
+    launch_brick(k_reaction_am<FT>, sizeof(BrickStage<FT, 3>), nt, s, b, t, nt);
 }
 template <typename FT>
-void launch_reaction_drag(const BoxDev *b, const Tile *t, int nt, int first, int last, int grid, int block,
-                          cudaStream_t s) {
-    k_reaction_drag<FT><<<grid, BRICK_THREADS, 0, s>>>(b, t, nt, first, last);
+void launch_reaction_drag(const BoxDev *b, const Tile *t, int nt, int first, int last, cudaStream_t s) {
+    launch_brick(k_reaction_drag<FT>, sizeof(BrickStage<FT, 3>), nt, s, b, t, nt, first, last);
 }
 
 #define DPS_CPL_INST(FT)                                                                                  \
-    template void launch_eps<FT>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);              \
+    template void launch_eps<FT>(const BoxDev *, const Tile *, int, cudaStream_t);                        \
     template void launch_force_am<FT>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);         \
     template void launch_force_drag<FT>(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);  \
-    template void launch_reaction_am<FT>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);      \
-    template void launch_reaction_drag<FT>(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
+    template void launch_reaction_am<FT>(const BoxDev *, const Tile *, int, cudaStream_t);                \
+    template void launch_reaction_drag<FT>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 DPS_CPL_INST(double)
 DPS_CPL_INST(float)
 
