@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "box.cuh"
+#include "lbm_fx.cuh"
 
 namespace dps {
 // launchers (lbm.cu, coupling.cu, dem.cu, scan.cu, io.cu)
@@ -22,8 +23,8 @@ template <typename ST, typename FT, typename CT>
 void launch_collide_stream(const BoxDev *, const Tile *, int, int, int, bool, bool, int, int, cudaStream_t);
 template <typename ST, typename FT, typename CT>
 void launch_moments(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
-template <typename FT, typename CT>
-void launch_fields(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+void launch_fields64(const BoxDev *, const Tile *, int, cudaStream_t);
+void launch_fields32(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename FT, typename CT>
 void launch_curl(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename ST>
@@ -262,6 +263,7 @@ static void compute_phys(BoxHost *h) {
             p.fb[a] = c.fb[a];
     }
     for (int a = 0; a < 3; ++a) p.fb_f[a] = (float)p.fb[a];
+    p.ff = fx_fluid(p.omega, p.kf, p.fb);
     p.lift = h->have_closure ? c.lift : 0;
     p.eilers = h->have_closure ? c.eilers : 0;
     p.smag = h->have_closure ? c.smagorinsky : 0;
@@ -582,9 +584,9 @@ static void enqueue_step(Batch *B) {
               (launch_moments<float, float, float>(T, B->d_cell, B->n_cell, par, gc, u.cell_block, s)),
               (launch_moments<__half, float, float>(T, B->d_cell, B->n_cell, par, gc, u.cell_block, s)));
     if (f64)
-        launch_fields<double, double>(T, B->d_cell, B->n_cell, gc, u.cell_block, s);
+        launch_fields64(T, B->d_brick, B->n_brick, s);
     else
-        launch_fields<float, float>(T, B->d_cell, B->n_cell, gc, u.cell_block, s);
+        launch_fields32(T, B->d_cell, B->n_cell, gc, u.cell_block, s);
     tend(B, PH_MOM, 2);
     const int nl = pl && B->any_lift;
     for (int k = 0; k < B->n_int; ++k) {

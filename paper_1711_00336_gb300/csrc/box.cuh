@@ -96,4 +96,14 @@ struct Tile {
 // iterate the tiles of a launch: one block per tile, blocks stride over tiles
 #define DPS_FOR_TILES(tiles, ntiles, t) for (int t = blockIdx.x; t < (ntiles); t += gridDim.x)
 
+// a brick tile packs its origin (Tile::begin) and extent (Tile::end), 21 bits an axis
+__host__ __device__ inline long long brick_pack(int x, int y, int z) {
+    return (long long)x | ((long long)y << 21) | ((long long)z << 42);
+}
+__device__ __forceinline__ void brick_unpack(long long v, int &x, int &y, int &z) {
+    x = (int)(v & 0x1FFFFF);
+    y = (int)((v >> 21) & 0x1FFFFF);
+    z = (int)((v >> 42) & 0x1FFFFF);
+}
+
 }  // namespace dps

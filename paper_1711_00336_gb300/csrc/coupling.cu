@@ -318,15 +318,6 @@ constexpr int BRICK = 8;
 constexpr int HALO = BRICK + 2;
 constexpr int HALO3 = HALO * HALO * HALO;
 
-__host__ __device__ inline long long brick_pack(int x, int y, int z) {
-    return (long long)x | ((long long)y << 21) | ((long long)z << 42);
-}
-__device__ __forceinline__ void brick_unpack(long long v, int &x, int &y, int &z) {
-    x = (int)(v & 0x1FFFFF);
-    y = (int)((v >> 21) & 0x1FFFFF);
-    z = (int)((v >> 42) & 0x1FFFFF);
-}
-
 // iterate the cells of the current brick tile: fn(cell index, lx, ly, lz)
 template <typename Fn>
 __device__ __forceinline__ void for_brick_cells(const Geom &g, int ox, int oy, int oz, int ex, int ey, int ez, Fn &&fn) {

@@ -144,6 +144,14 @@ __device__ __forceinline__ long long particle_cell(const Geom &g, double x, doub
     return cell_index(g, ix, iy, iz);
 }
 
+// constants of the fixed-point relaxation (lbm_fx.cuh), units of 2^-63 / 2^-64
+struct FxFluid {
+    i64 om1;               // 1 - omega, 2^-63
+    u64 om12, om36, kf12;  // omega/12, omega/36, (1 - omega/2)/12, 2^-64
+    i64 fb[3];             // body force, 2^-64
+    int ok;
+};
+
 // closure constants, derived once on the host
 struct Phys {
     double tau, omega, kf, rho_f, mu;   // kf = 1 - 1/(2 tau) (Eq. Forcing)
@@ -165,6 +173,7 @@ struct Phys {
     int drag, pressure, added_mass, lubrication, contact, lub_limiter;
     int lift;            // Table 1 shear lift (curl of u_f at the subcycle start)
     int eilers, smag;    // per-cell tau_e (Eqs. visc_eilers, tau_t, tau_e)
+    FxFluid ff;          // constants of the fixed-point relaxation
     FxBox fx;            // constants of the integer pair path (fx.cuh)
 };
 

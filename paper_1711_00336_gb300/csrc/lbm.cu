@@ -6,13 +6,19 @@
 //    direction q goes to plane opp(q)); odd parity reads the upstream values
 //    and writes the downstream cells.  Halfway bounce-back at wall faces is
 //    folded into the odd-parity index map.  HBM traffic per cell: 19 loads and
-//    19 stores of the PDF type plus eps_f and f_pf (4 loads of the field type);
-//    in the FP64 coupled step also rho and j from K2a (4 more).
+//    19 stores of the PDF type plus eps_f and f_pf (4 loads of the field type).
+//    FP64: 207 FP64 warp instructions of ~19 cycles per 32 cells bound this
+//    pass; it runs in 64-bit fixed point (lbm_fx.cuh), ~1500 integer
+//    instructions of which two to four issue per cycle.  128^3, walls at z:
+//    815 -> 311 us; 256^3, coupled step: 4.88 -> 2.64 ms (floor at the
+//    measured copy rate: 0.10 and 0.83 ms).  Boxes with a per-cell tau_e keep
+//    the FP64 relaxation, with rho and j from K2a.
 // K2a moments: rho, j of f(x,t), u_D = (j + f_ext/2)/(rho eps_f) and
 //    1/(rho eps_f); one PDF read.
 // K2b fields: stencil over rho and u_D giving grad(eps_f p) and Du_f/Dt.
 #include "box.cuh"
 #include "lbm_dev.cuh"
+#include "lbm_fx.cuh"
 
 namespace dps {
 
@@ -64,9 +70,9 @@ template <typename ST, typename FT, typename CT, int PAR, bool VISC, bool MOMIN>
 __device__ __forceinline__ void relax_store_cell(ST *__restrict__ pdf, CT f[Q], const NbDelta &D, bool in,
                                                  const Geom &g, CT e, CT fpx, CT fpy, CT fpz, long long N, long long c,
                                                  CT fbx, CT fby, CT fbz, CT omega_box, CT kf_box, CT tau, int vmode,
-                                                 int *status, const CT *mom);
+                                                 int *status, const CT *mom, const FxFluid *ff = nullptr);
 
-// the moments of cell c from K2a (MOMIN), else nothing
+// the moments of cell c from K2a (MOMIN: FP64 with a per-cell tau_e), else nothing
 template <typename FT, typename CT, bool MOMIN>
 __device__ __forceinline__ void load_moments(const FT *__restrict__ rho, const FT *__restrict__ j, long long N,
                                              long long c, CT mom[4]) {
@@ -83,7 +89,7 @@ __device__ __forceinline__ void collide_stream_cell(ST *__restrict__ pdf, const 
                                                     const FT *__restrict__ fpf, const FT *__restrict__ rho_m,
                                                     const FT *__restrict__ j_m, const Geom &g, long long c, CT fbx,
                                                     CT fby, CT fbz, CT omega_box, CT kf_box, CT tau, int vmode,
-                                                    int *status) {
+                                                    int *status, const FxFluid *ff = nullptr) {
     const long long N = g.ncell;
     NbDelta D;
     bool in = false;
@@ -104,7 +110,7 @@ __device__ __forceinline__ void collide_stream_cell(ST *__restrict__ pdf, const 
     load_moments<FT, CT, MOMIN>(rho_m, j_m, N, c, mom);
     relax_store_cell<ST, FT, CT, PAR, VISC, MOMIN>(pdf, f, D, in, g, (CT)eps[c], (CT)fpf[c], (CT)fpf[N + c],
                                                    (CT)fpf[2 * N + c], N, c, fbx, fby, fbz, omega_box, kf_box, tau,
-                                                   vmode, status, mom);
+                                                   vmode, status, mom, ff);
 }
 
 // two cells per thread (c and c + stride): the loads of both are issued before
@@ -289,7 +295,7 @@ __device__ __forceinline__ double r_sub(double a, double b) { return __dsub_rn(a
 // O = K3 cu + K4 cF, with K0..K4 fixed per weight class.
 // `flag`: report a non-finite or non-positive density.
 // MOMIN: the moments s, j of these populations were computed by K2a in this
-// step with the same sums (the FP64 form): they are passed in, not re-summed.
+// step (the FP64 form with a per-cell tau_e): they are passed in, not re-summed.
 template <typename ST, typename CT, bool VISC, bool MOMIN = false>
 __device__ __forceinline__ void relax_cell(CT f[Q], CT e, CT fpx, CT fpy, CT fpz, CT fbx, CT fby, CT fbz,
                                            CT omega_box, CT kf_box, CT tau, int vmode, bool flag, int *status,
@@ -359,9 +365,17 @@ template <typename ST, typename FT, typename CT, int PAR, bool VISC, bool MOMIN>
 __device__ __forceinline__ void relax_store_cell(ST *__restrict__ pdf, CT f[Q], const NbDelta &D, bool in,
                                                  const Geom &g, CT e, CT fpx, CT fpy, CT fpz, long long N, long long c,
                                                  CT fbx, CT fby, CT fbz, CT omega_box, CT kf_box, CT tau, int vmode,
-                                                 int *status, const CT *mom) {
-    relax_cell<ST, CT, VISC, MOMIN>(f, e, fpx, fpy, fpz, fbx, fby, fbz, omega_box, kf_box, tau, vmode, true, status,
-                                    mom);
+                                                 int *status, const CT *mom, const FxFluid *ff) {
+    bool done = false;
+    if constexpr (sizeof(ST) == 8 && !VISC) {
+        u64 b[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) b[q] = fx_bits(f[q]);
+        done = fx_relax(b, e, fpx, fpy, fpz, *ff, f);
+    }
+    if (!done)
+        relax_cell<ST, CT, VISC, MOMIN>(f, e, fpx, fpy, fpz, fbx, fby, fbz, omega_box, kf_box, tau, vmode, true, status,
+                                        mom);
     Store<ST>::store(pdf + (unsigned)c, f[0]);
 #pragma unroll
     for (int k = 1; k <= 9; ++k) {
@@ -376,8 +390,11 @@ template <typename CT> __device__ __forceinline__ CT pick(double d, float f);
 template <> __device__ __forceinline__ double pick<double>(double d, float) { return d; }
 template <> __device__ __forceinline__ float pick<float>(double, float f) { return f; }
 
+#ifndef DPS_K1_MINB
+#define DPS_K1_MINB 3  // FP64: 128-thread blocks per SM the register budget is sized for
+#endif
 // K1: every cell tile of every box, AA parity PAR (common to the batch).
-// MOMIN: rho and j come from K2a of the same step (FP64 coupled step)
+// MOMIN: rho and j come from K2a of the same step (FP64 coupled step, VISC)
 template <typename ST, typename FT, typename CT, int PAR, int MINB, bool VISC, int CPT, bool MOMIN = false>
 __global__ void __launch_bounds__(128, MINB) k_collide_stream(const BoxDev *__restrict__ boxes,
                                                            const Tile *__restrict__ tiles, int ntiles) {
@@ -402,7 +419,7 @@ __global__ void __launch_bounds__(128, MINB) k_collide_stream(const BoxDev *__re
         } else if (CPT == 1 || CPT == 3) {
             for (long long c = tl.begin + threadIdx.x; c < tl.end; c += blockDim.x)
                 collide_stream_cell<ST, FT, CT, PAR, VISC, MOMIN>(pdf, eps, fpf, rho_m, j_m, g, c, fbx, fby, fbz,
-                                                                  omega, kf, tau, vmode, st);
+                                                                  omega, kf, tau, vmode, st, &B.ph.ff);
         } else {
             for (long long c = tl.begin + threadIdx.x; c < tl.end; c += 2 * blockDim.x) {
                 const long long c2 = c + blockDim.x;
@@ -425,24 +442,48 @@ __device__ __forceinline__ void moments_cell(const ST *__restrict__ pdf, const F
     NbDelta D = neighbour_deltas(g, ix, iy, iz);
     CT f[Q];
     load_pdfs<ST, CT, PAR>(pdf, N, c, D, f);
-    CT rho, jx, jy, jz;
-    moments(f, rho, jx, jy, jz);
-    if (Store<ST>::shifted) rho += CT(1);  // deviations: sum of the shifts w_q is 1
     const CT e = (CT)eps[c];
+    CT rho, jx, jy, jz, s = 0;
+    bool exact = false;
+    if constexpr (sizeof(ST) == 8) {
+        // the sums are exact in units of 2^-62 (FP64: 57 FP64 instructions a
+        // cell, here 9); 1/(rho eps) by Newton's iteration on integers
+        u64 b[Q];
+        i64 fi[Q], r, j[3];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) b[q] = fx_bits(f[q]);
+        if (fx_populations(b, fi, r, j) && r > (1ll << 61) && e > 0.125 && e <= 1.0) {
+            int lz;
+            const u64 R = fx_recip(r, fx_from_pos(e, 62), lz);
+            s = fx_to_double(R, 64 - lz);
+            rho = fx_to_double((u64)r, 62);
+            jx = fx_signed_to_double(j[0], 62);
+            jy = fx_signed_to_double(j[1], 62);
+            jz = fx_signed_to_double(j[2], 62);
+            exact = true;
+        }
+    }
+    if (!exact) {
+        moments(f, rho, jx, jy, jz);
+        if (Store<ST>::shifted) rho += CT(1);  // deviations: sum of the shifts w_q is 1
+        s = CT(1) / (rho * e);
+    }
     const CT Fx = (CT)fpf[c] + e * fbx, Fy = (CT)fpf[N + c] + e * fby, Fz = (CT)fpf[2 * N + c] + e * fbz;
     rho_o[c] = (FT)rho;
     j_o[c] = (FT)jx;
     j_o[N + c] = (FT)jy;
     j_o[2 * N + c] = (FT)jz;
-    const CT s = CT(1) / (rho * e);
     ire[c] = (FT)s;  // the first subcycle's drag interpolation reuses it
     uD[c] = (FT)((jx + CT(0.5) * Fx) * s);
     uD[N + c] = (FT)((jy + CT(0.5) * Fy) * s);
     uD[2 * N + c] = (FT)((jz + CT(0.5) * Fz) * s);
 }
 
+#ifndef DPS_MOM_MINB
+#define DPS_MOM_MINB 3  // FP64: 128-thread blocks per SM the register budget is sized for
+#endif
 template <typename ST, typename FT, typename CT, int PAR>
-__global__ void __launch_bounds__(128, sizeof(CT) == 8 ? 2 : 4) k_moments(const BoxDev *__restrict__ boxes,
+__global__ void __launch_bounds__(128, sizeof(CT) == 8 ? DPS_MOM_MINB : 4) k_moments(const BoxDev *__restrict__ boxes,
                                                     const Tile *__restrict__ tiles, int ntiles) {
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
@@ -513,6 +554,151 @@ __global__ void __launch_bounds__(256) k_fields(const BoxDev *__restrict__ boxes
                 const CT up = have_prev ? (CT)uprev[b * N + c] : u[b];
                 DuDt[b * N + c] = (FT)((u[b] - up) + conv);
                 uprev[b * N + c] = (FT)u[b];
+            }
+        }
+    }
+}
+
+// K2b of the FP64 form over bricks of 8^3 cells: rho and u_D of the brick and its
+// halo are staged in shared memory as integers of 58 bits relative to the
+// largest of the block (rho apart from u_D), so that the 18-neighbour sums are
+// exact integer additions and the convective products 64-bit ones; 12 FP64
+// instructions a cell are left of 135, which bound this kernel.  A block with a
+// non-finite value takes FP64 throughout.  K2a and K2b together at 256^3: 6.34
+// -> 2.35 ms; at 64^3: 115 -> 51 us.
+constexpr int FB = 8, FH = FB + 2, FH3 = FH * FH * FH;
+
+__device__ __forceinline__ void fields_cell64(const double *__restrict__ rho, const double *__restrict__ uD,
+                                              const Geom &g, int ix, int iy, int iz, double gp[3], double cv[3]) {
+    const long long N = g.ncell, c = cell_index(g, ix, iy, iz);
+    const int ii[3] = {ix, iy, iz};
+    double gu[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+    gp[0] = gp[1] = gp[2] = 0.0;
+#pragma unroll 1
+    for (int q = 1; q < Q; ++q) {
+        const int cc[3] = {CX(q), CY(q), CZ(q)};
+        int t[3];
+        for (int a = 0; a < 3; ++a) {
+            t[a] = ii[a] + cc[a];
+            if (t[a] < 0) t[a] = g.per[a] ? g.n[a] - 1 : 0;
+            if (t[a] >= g.n[a]) t[a] = g.per[a] ? 0 : g.n[a] - 1;
+        }
+        const long long n = cell_index(g, t[0], t[1], t[2]);
+        const double r = rho[n], u0 = uD[n], u1 = uD[N + n], u2 = uD[2 * N + n];
+        for (int a = 0; a < 3; ++a) {
+            const double wc = WQ(q) * cc[a];
+            gp[a] += wc * r;
+            gu[a][0] += wc * u0;
+            gu[a][1] += wc * u1;
+            gu[a][2] += wc * u2;
+        }
+    }
+    const double u[3] = {uD[c], uD[N + c], uD[2 * N + c]};
+    for (int b = 0; b < 3; ++b) cv[b] = 3.0 * (u[0] * gu[0][b] + u[1] * gu[1][b] + u[2] * gu[2][b]);
+}
+
+// 36 sum_q w_q c_q phi(x + c_q) at entry p of the staged field
+__device__ __forceinline__ void stencil36(const i64 *__restrict__ s, int p, i64 G[3]) {
+    constexpr int Y = FH, Z = FH * FH;
+    const i64 xpyp = s[p + 1 + Y], xpym = s[p + 1 - Y], xmyp = s[p - 1 + Y], xmym = s[p - 1 - Y];
+    const i64 xpzp = s[p + 1 + Z], xpzm = s[p + 1 - Z], xmzp = s[p - 1 + Z], xmzm = s[p - 1 - Z];
+    const i64 ypzp = s[p + Y + Z], ypzm = s[p + Y - Z], ymzp = s[p - Y + Z], ymzm = s[p - Y - Z];
+    G[0] = 2 * (s[p + 1] - s[p - 1]) + (xpyp - xmym) + (xpym - xmyp) + (xpzp - xmzm) + (xpzm - xmzp);
+    G[1] = 2 * (s[p + Y] - s[p - Y]) + (xpyp - xmym) - (xpym - xmyp) + (ypzp - ymzm) + (ypzm - ymzp);
+    G[2] = 2 * (s[p + Z] - s[p - Z]) + (xpzp - xmzm) - (xpzm - xmzp) + (ypzp - ymzm) - (ypzm - ymzp);
+}
+
+__global__ void __launch_bounds__(256) k_fields64(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles,
+                                                  int ntiles) {
+    __shared__ i64 S[4][FH3];
+    __shared__ u32 top[2];
+    DPS_FOR_TILES(tiles, ntiles, t) {
+        const Tile tl = tiles[t];
+        const BoxDev &B = boxes[tl.box];
+        const Geom g = B.g;
+        const long long N = g.ncell;
+        int ox, oy, oz, ex, ey, ez;
+        brick_unpack(tl.begin, ox, oy, oz);
+        brick_unpack(tl.end, ex, ey, ez);
+        const double *rho = (const double *)B.rho, *uD = (const double *)B.uD;
+        if (threadIdx.x < 2) top[threadIdx.x] = 0;
+        __syncthreads();  // (also: the previous brick is done with S)
+        // stage the raw bits and the largest exponents (neighbours beyond a
+        // wall are mirrored into the box: coordinate clamped)
+        u32 mr = 0, mu = 0;
+        for (int h = threadIdx.x; h < FH3; h += 256) {
+            const int hx = h % FH, hy = (h / FH) % FH, hz = h / (FH * FH);
+            u64 v[4] = {0, 0, 0, 0};
+            if (hx <= ex + 1 && hy <= ey + 1 && hz <= ez + 1) {
+                int p[3] = {ox + hx - 1, oy + hy - 1, oz + hz - 1};
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    if (p[a] < 0) p[a] = g.per[a] ? g.n[a] - 1 : 0;
+                    else if (p[a] >= g.n[a]) p[a] = g.per[a] ? 0 : g.n[a] - 1;
+                }
+                const long long n = cell_index(g, p[0], p[1], p[2]);
+                v[0] = fx_bits(rho[n]);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    v[1 + k] = fx_bits(uD[k * N + n]);
+                    mu = max(mu, fx_abs_hi(v[1 + k]));
+                }
+                mr = max(mr, fx_abs_hi(v[0]));
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) S[k][h] = (i64)v[k];
+        }
+        mr = __reduce_max_sync(0xffffffffu, mr);
+        mu = __reduce_max_sync(0xffffffffu, mu);
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&top[0], mr);
+            atomicMax(&top[1], mu);
+        }
+        __syncthreads();
+        // |v| < 2^(e + 1): units of 2^(e - 57) leave four bits for the sums
+        const int er = (int)(top[0] >> 20) - 1023, eu = max((int)(top[1] >> 20) - 1023, -400);
+        const bool fixed = er < 1024 && er > -400 && eu < 400;
+        const int fr = 57 - er, fu = 57 - eu;
+        if (fixed) {
+            for (int h = threadIdx.x; h < FH3; h += 256) {
+                S[0][h] = fx_from(fx_double((u64)S[0][h]), fr);
+#pragma unroll
+                for (int k = 1; k < 4; ++k) S[k][h] = fx_from(fx_double((u64)S[k][h]), fu);
+            }
+        }
+        __syncthreads();
+        double *uprev = (double *)B.uprev, *gradP = (double *)B.gradP, *DuDt = (double *)B.DuDt;
+        const int have_prev = B.have_uprev;
+        const int nb = ex * ey * ez;
+        for (int k = threadIdx.x; k < nb; k += 256) {
+            const int lx = k % ex, ly = (k / ex) % ey, lz = k / (ex * ey);
+            const long long c = cell_index(g, ox + lx, oy + ly, oz + lz);
+            double gp[3], cv[3], u[3];
+#pragma unroll
+            for (int b = 0; b < 3; ++b) u[b] = uD[b * N + c];
+            if (fixed) {
+                const int p = ((lz + 1) * FH + ly + 1) * FH + lx + 1;
+                i64 G[3];
+                stencil36(S[0], p, G);
+#pragma unroll
+                for (int b = 0; b < 3; ++b) gp[b] = fx_signed_to_double(G[b], fr) * (1.0 / 36.0);
+                const i64 v[3] = {S[1][p] * 16, S[2][p] * 16, S[3][p] * 16};
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    stencil36(S[1 + b], p, G);
+                    // (u . grad) u_b = 3/36 sum_a u_a G_a: three products of the high halves
+                    const i64 C = fx_mulhi_s(v[0], G[0]) + fx_mulhi_s(v[1], G[1]) + fx_mulhi_s(v[2], G[2]) + 1;
+                    cv[b] = fx_signed_to_double(C, 2 * fu + 4 - 64) * (1.0 / 12.0);
+                }
+            } else {
+                fields_cell64(rho, uD, g, ox + lx, oy + ly, oz + lz, gp, cv);
+            }
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                gradP[b * N + c] = gp[b];
+                const double up = have_prev ? uprev[b * N + c] : u[b];
+                DuDt[b * N + c] = (u[b] - up) + cv[b];
+                uprev[b * N + c] = u[b];
             }
         }
     }
@@ -634,14 +820,13 @@ void launch_collide_stream(const BoxDev *boxes, const Tile *tiles, int ntiles, i
 #define DPS_K1V(MB, V, CPT) DPS_K1VM(MB, V, CPT, false)
 #define DPS_K1(MB, CPT) DPS_K1V(MB, false, CPT)
     if constexpr (sizeof(CT) == 8) {
-        // the FP64 coupled step takes rho and j from K2a (same sums, one
-        // fifth fewer FP64 instructions)
+        // per-cell tau_e: FP64 relaxation, rho and j of the coupled step
+        // from K2a.  Else the fixed-point relaxation, which sums them itself
         if (visc) {
             if (mom_in) DPS_K1VM(2, true, 1, true);
             else DPS_K1V(2, true, 1);
         } else {
-            if (mom_in) DPS_K1VM(2, false, 1, true);
-            else DPS_K1(2, 1);
+            DPS_K1(DPS_K1_MINB, 1);
         }
     } else if (visc)
         DPS_K1V(3, true, 1);
@@ -676,9 +861,11 @@ void launch_moments(const BoxDev *boxes, const Tile *tiles, int ntiles, int pari
         k_moments<ST, FT, CT, 0><<<grid, block, 0, s>>>(boxes, tiles, ntiles);
 }
 
-template <typename FT, typename CT>
-void launch_fields(const BoxDev *boxes, const Tile *tiles, int ntiles, int grid, int block, cudaStream_t s) {
-    k_fields<FT, CT><<<grid, block, 0, s>>>(boxes, tiles, ntiles);
+void launch_fields64(const BoxDev *boxes, const Tile *bricks, int nbricks, cudaStream_t s) {
+    k_fields64<<<nbricks, 256, 0, s>>>(boxes, bricks, nbricks);
+}
+void launch_fields32(const BoxDev *boxes, const Tile *tiles, int ntiles, int grid, int block, cudaStream_t s) {
+    k_fields<float, float><<<grid, block, 0, s>>>(boxes, tiles, ntiles);
 }
 
 template <typename FT, typename CT>
@@ -708,8 +895,6 @@ void launch_pdf_import(void *pdf, long long N, const double *in, cudaStream_t s)
 DPS_LBM_INST(double, double, double)
 DPS_LBM_INST(float, float, float)
 DPS_LBM_INST(__half, float, float)
-template void launch_fields<double, double>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
-template void launch_fields<float, float>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template void launch_curl<double, double>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template void launch_curl<float, float>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template void launch_pdf_export<double>(const void *, const Geom &, int, double *, cudaStream_t);

@@ -1,0 +1,187 @@
+// lbm_fx.cuh -- the BGK relaxation of the FP64 form (Eqs. LBM_Equation, LBM_EQ,
+// Forcing) in 64-bit fixed point.
+//
+// The populations of a fluid near rest are below 1/2 and their rounding errors
+// absolute (2^-58 for the diagonals), so units of 2^-62 ... 2^-64 hold every
+// quantity of the update more precisely than FP64 does: sums are exact, and a
+// product (the high half of a 64 x 64-bit multiplication) costs a third of an
+// FP64 multiply on GB300, a sum a tenth.  With A = omega rho u / 12, G = kf F /
+// 12, H = A + G and V = u / eps the update of Sec. 3.2.2, divided by 36, is
+//   E' = omega rho / 36 - (Dx + Dy + Dz)/3,  D_a = 3/2 (H_a + G_a) V_a,
+//   X_ab = 3 (H_a V_b + G_b V_a),
+//   f0  <- (1 - omega) f0 + 12 E',
+//   f+-a <- (1 - omega) f + 2 (E' + D_a) +- 2 H_a,
+//   f+-a+-b <- (1 - omega) f + E' + D_a + D_b +- X_ab +- H_a +- H_b,
+// which needs no multiplication per direction beyond (1 - omega) f.  Cells
+// outside the ranges below (a third of them per axis or more from rest) take
+// the FP64 path, as do non-finite ones.  Products round down; the constants
+// added below balance the mean of that, so that neither mass nor momentum
+// drifts.
+#pragma once
+#include "dps_internal.cuh"
+
+namespace dps {
+
+// v in (-1, 1) in units of 2^-62, bits below dropped (none above 2^-10)
+__host__ __device__ __forceinline__ i64 fx_q62(u64 b) {
+    const int s = 1024 - (int)((b >> 52) & 0x7ff);
+    const u64 top = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 11;
+    const u64 m = s < 64 ? top >> s : 0ull;
+    return (i64)b < 0 ? -(i64)m : (i64)m;
+}
+__host__ __device__ __forceinline__ double fx_signed_to_double(i64 v, int frac) {
+    const double d = fx_to_double((u64)(v < 0 ? -v : v), frac);
+    return v < 0 ? -d : d;
+}
+__host__ __device__ __forceinline__ u32 fx_abs_hi(u64 b) { return (u32)(b >> 32) & 0x7fffffffu; }
+
+// populations in units of 2^-62 and their exact moments; false when |f_0| >=
+// 1/2, |f| >= 1/8 along an axis or |f| >= 1/16 along a diagonal (their sum could
+// pass 2), or a value is not finite
+__host__ __device__ __forceinline__ bool fx_populations(const u64 b[Q], i64 f[Q], i64 &rho, i64 j[3]) {
+    u32 axis = 0, diag = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int q = 1; q < Q; ++q) {
+        const u32 h = fx_abs_hi(b[q]);
+        if (CX(q) * CX(q) + CY(q) * CY(q) + CZ(q) * CZ(q) == 1) axis = axis > h ? axis : h;
+        else diag = diag > h ? diag : h;
+    }
+    if (!(fx_abs_hi(b[0]) < 0x3fe00000u && axis < 0x3fc00000u && diag < 0x3fb00000u)) return false;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int q = 0; q < Q; ++q) f[q] = fx_q62(b[q]);
+    rho = f[0];
+    j[0] = j[1] = j[2] = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int k = 1; k <= 9; ++k) {
+        rho += f[k] + f[k + 9];
+        const i64 d = f[k] - f[k + 9];
+        if (CX(k) != 0) j[0] += CX(k) > 0 ? d : -d;
+        if (CY(k) != 0) j[1] += CY(k) > 0 ? d : -d;
+        if (CZ(k) != 0) j[2] += CZ(k) > 0 ? d : -d;
+    }
+    return true;
+}
+
+// box constants of the relaxation
+__host__ __device__ inline FxFluid fx_fluid(double omega, double kf, const double fb[3]) {
+    FxFluid x;
+    std::memset(&x, 0, sizeof x);
+    x.ok = omega > 0.0 && omega < 2.0 && kf > 0.0 && kf < 1.0 && fabs(fb[0]) < 0.125 && fabs(fb[1]) < 0.125 &&
+           fabs(fb[2]) < 0.125;
+    if (!x.ok) return x;
+    x.om1 = fx_from(1.0 - omega, 62) * 2;
+    const u64 o = (u64)fx_from_pos(omega, 60), k = (u64)fx_from_pos(kf, 60);
+    // omega/12, omega/36, kf/12 in units of 2^-64: 16/12 = 4/3 and 16/36 = 4/9 of the 2^-60 value
+    x.om12 = o / 3 * 4 + (o % 3) * 4 / 3;
+    x.om36 = o / 9 * 4 + (o % 9) * 4 / 9;
+    x.kf12 = k / 3 * 4 + (k % 3) * 4 / 3;
+    for (int a = 0; a < 3; ++a) x.fb[a] = fx_from(fb[a], 63) * 2;  // 2^-64
+    return x;
+}
+
+// 1/(rho eps) = R 2^(lz-64), R in (2^62, 2^63] (Newton from a single-precision
+// seed); rho eps in (1/16, 2), both in units of 2^-62
+__host__ __device__ __forceinline__ u64 fx_recip(i64 rho, i64 e62, int &lz) {
+    u64 P = fx_mulhi((u64)rho << 1, (u64)e62 << 1);  // 2^-62
+    lz = fx_clz(P);
+    P <<= lz;
+    u32 Y = (u32)(fx_rcp_seed((float)(u32)(P >> 32) * 0x1p-32f) * 0x1p30f);
+    Y = Y > 0x7fffffffu ? 0x7fffffffu : Y;
+    const i64 e1 = (i64)((1ull << 63) - fx_mulhi(P, (u64)Y << 33));  // y (1 + e1 + e1^2)
+    const i64 f1 = (i64)(int)(e1 >> 12);
+    const i64 c1 = e1 + ((f1 * f1) >> 39);
+    return ((u64)Y << 32) + (u64)(((c1 >> 32) * (i64)Y) * 2) + (((u64)(u32)c1 * Y) >> 31);
+}
+
+// One cell: b the bits of the populations, e = eps_f, fp = f_pf; f receives the
+// post-collision populations.  False: outside the range, nothing is written.
+__host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, double fp0, double fp1, double fp2,
+                                                  const FxFluid &x, double out[Q]) {
+    i64 f[Q], rho, j[3];
+    const u64 eb = fx_bits(e), p0 = fx_bits(fp0), p1 = fx_bits(fp1), p2 = fx_bits(fp2);
+    // 1/8 < eps <= 1, |f_pf| < 1/8
+    if (!(eb > 0x3fc0000000000000ull && eb <= 0x3ff0000000000000ull && fx_abs_hi(p0) < 0x3fc00000u &&
+          fx_abs_hi(p1) < 0x3fc00000u && fx_abs_hi(p2) < 0x3fc00000u && x.ok))
+        return false;
+    if (!fx_populations(b, f, rho, j)) return false;
+    const i64 e62 = fx_from_pos(e, 62);
+    i64 F[3] = {fx_q62(p0), fx_q62(p1), fx_q62(p2)}, J[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < 3; ++a) {
+        F[a] += fx_mulhi_s(e62, x.fb[a]);  // f_ext = f_pf + eps_f f_b (|.| < 1/4)
+        J[a] = j[a] + (F[a] >> 1);
+    }
+    // 1/2 < rho < 2, |j + F/2| < 1/8 per component
+    const i64 lim = 1ll << 59;
+    if (!(rho > (1ll << 61) && J[0] < lim && J[0] > -lim && J[1] < lim && J[1] > -lim && J[2] < lim && J[2] > -lim))
+        return false;
+    int lz;
+    const u64 R = fx_recip(rho, e62, lz);
+    const i64 ir = (i64)(fx_mulhi((u64)e62, R) << lz);  // 1/rho, 2^-62, < 2
+    const u64 m = fx_mulhi((u64)rho << 1, R);
+    const i64 ie = (i64)(lz >= 3 ? m << (lz - 3) : m >> (3 - lz));  // 1/eps, 2^-60, < 8
+    const u64 c12 = fx_mulhi(x.om12, (u64)rho << 1) << 1;           // omega rho / 12, 2^-64
+    i64 H[3], G[3], V[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < 3; ++a) {
+        const i64 u = fx_mulhi_s(J[a] * 4, ir);  // 2^-62, |u| < 1/4
+        G[a] = fx_mulhi_s(F[a] * 4, (i64)x.kf12);  // 2^-64
+        H[a] = fx_mulhi_s(u * 4, (i64)c12) + G[a] + 1;
+        V[a] = fx_mulhi_s(u * 4, ie);  // 2^-60
+    }
+    i64 D[3], S = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < 3; ++a) {
+        const i64 p = fx_mulhi_s(H[a] + G[a], V[a]);  // 2^-60
+        D[a] = p + (p >> 1);
+        S += D[a];
+    }
+    // E' in units of 2^-63
+    const i64 E = (i64)fx_mulhi(x.om36, (u64)rho << 1) - fx_mulhi_s(S * 4, 6148914691236517205ll) * 2;
+    const i64 xy = fx_mulhi_s(H[0], V[1]) + fx_mulhi_s(G[1], V[0]);
+    const i64 xz = fx_mulhi_s(H[0], V[2]) + fx_mulhi_s(G[2], V[0]);
+    const i64 yz = fx_mulhi_s(H[1], V[2]) + fx_mulhi_s(G[2], V[1]);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int a = 0; a < 3; ++a) {
+        D[a] *= 8;  // 2^-63
+        H[a] = (H[a] + 1) >> 1;
+    }
+    const i64 Xxy = xy * 24, Xxz = xz * 24, Xyz = yz * 24;
+    // (-4: the mean of the rounded-down products over the 19 populations)
+    out[0] = fx_signed_to_double(fx_mulhi_s(x.om1, f[0] * 2) + 6 * E - 4, 62);
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int k = 1; k <= 9; ++k) {
+        i64 ev = E, od = 0;
+        if (CX(k) != 0) { ev += D[0]; od += CX(k) > 0 ? H[0] : -H[0]; }
+        if (CY(k) != 0) { ev += D[1]; od += CY(k) > 0 ? H[1] : -H[1]; }
+        if (CZ(k) != 0) { ev += D[2]; od += CZ(k) > 0 ? H[2] : -H[2]; }
+        if (CX(k) * CY(k) != 0) ev += CX(k) * CY(k) > 0 ? Xxy : -Xxy;
+        if (CX(k) * CZ(k) != 0) ev += CX(k) * CZ(k) > 0 ? Xxz : -Xxz;
+        if (CY(k) * CZ(k) != 0) ev += CY(k) * CZ(k) > 0 ? Xyz : -Xyz;
+        if (CX(k) * CX(k) + CY(k) * CY(k) + CZ(k) * CZ(k) == 1) {
+            ev *= 2;
+            od *= 2;
+        }
+        out[k] = fx_signed_to_double(fx_mulhi_s(x.om1, f[k] * 4) + ev + od, 63);
+        out[k + 9] = fx_signed_to_double(fx_mulhi_s(x.om1, f[k + 9] * 4) + ev - od, 63);
+    }
+    return true;
+}
+
+}  // namespace dps
