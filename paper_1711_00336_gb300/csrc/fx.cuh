@@ -112,6 +112,10 @@ __host__ __device__ __forceinline__ double fx_to_double(u64 v, int frac) {
     return v ? fx_double(b) : 0.0;
 }
 
+// the sign of s on v >= 0, as bits (a negation would be an FP64 instruction)
+__host__ __device__ __forceinline__ double fx_with_sign(double v, i64 s) {
+    return fx_double(fx_bits(v) | ((u64)s & 0x8000000000000000ull));
+}
 // the particle constants of the pair path: the radius in units of 2^-56 and
 // 1/d in units of 2^-58 (1/4 <= d < 8: both exact to below an FP64 rounding)
 __host__ __device__ __forceinline__ i64 fx_radius(double d) { return fx_from_pos(0.5 * d, 56); }
@@ -275,8 +279,7 @@ __host__ __device__ __forceinline__ int fx_pair(const i64 dx[3], i64 S, u64 I, c
 #pragma unroll
 #endif
     for (int k = 0; k < 3; ++k) {
-        const double t = fx_to_double(fx_mulhi(X[k], R), 61);
-        o.n[k] = dx[k] < 0 ? -t : t;
+        o.n[k] = fx_with_sign(fx_to_double(fx_mulhi(X[k], R), 61), dx[k]);
     }
     return FX_LUB;
 }

@@ -10,7 +10,7 @@
 //    FP64: 207 FP64 warp instructions of ~19 cycles per 32 cells bound this
 //    pass; it runs in 64-bit fixed point (lbm_fx.cuh), ~1500 integer
 //    instructions of which two to four issue per cycle.  128^3, walls at z:
-//    815 -> 311 us; 256^3, coupled step: 4.88 -> 2.64 ms (floor at the
+//    815 -> 228 us; 256^3, coupled step: 4.88 -> 1.93 ms (floor at the
 //    measured copy rate: 0.10 and 0.83 ms).  Boxes with a per-cell tau_e keep
 //    the FP64 relaxation, with rho and j from K2a.
 // K2a moments: rho, j of f(x,t), u_D = (j + f_ext/2)/(rho eps_f) and
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(256) k_fields(const BoxDev *__restrict__ boxes
 // exact integer additions and the convective products 64-bit ones; 12 FP64
 // instructions a cell are left of 135, which bound this kernel.  A block with a
 // non-finite value takes FP64 throughout.  K2a and K2b together at 256^3: 6.34
-// -> 2.35 ms; at 64^3: 115 -> 51 us.
+// -> 2.12 ms; at 64^3: 115 -> 46 us.
 constexpr int FB = 8, FH = FB + 2, FH3 = FH * FH * FH;
 
 __device__ __forceinline__ void fields_cell64(const double *__restrict__ rho, const double *__restrict__ uD,

@@ -9,12 +9,12 @@
 // 12, H = A + G and V = u / eps the update of Sec. 3.2.2, divided by 36, is
 //   E' = omega rho / 36 - (Dx + Dy + Dz)/3,  D_a = 3/2 (H_a + G_a) V_a,
 //   X_ab = 3 (H_a V_b + G_b V_a),
-//   f0  <- (1 - omega) f0 + 12 E',
-//   f+-a <- (1 - omega) f + 2 (E' + D_a) +- 2 H_a,
-//   f+-a+-b <- (1 - omega) f + E' + D_a + D_b +- X_ab +- H_a +- H_b,
-// which needs no multiplication per direction beyond (1 - omega) f.  Cells
-// outside the ranges below (a third of them per axis or more from rest) take
-// the FP64 path, as do non-finite ones.  Products round down; the constants
+//   f0  <- f0 - omega f0 + 12 E',
+//   f+-a <- f - omega f + 2 (E' + D_a) +- 2 H_a,
+//   f+-a+-b <- f - omega f + E' + D_a + D_b +- X_ab +- H_a +- H_b,
+// which needs no multiplication per direction beyond omega f.  Cells
+// outside the ranges below (populations about twice those at rest, or below
+// 2^-10) take the FP64 path, as do non-finite ones.  Products round down; the constants
 // added below balance the mean of that, so that neither mass nor momentum
 // drifts.
 #pragma once
@@ -22,33 +22,48 @@
 
 namespace dps {
 
-// v in (-1, 1) in units of 2^-62, bits below dropped (none above 2^-10)
+// v in [2^-10, 1) in units of 2^-62, exactly: its 53 bits moved up by 0 to 9
 __host__ __device__ __forceinline__ i64 fx_q62(u64 b) {
-    const int s = 1024 - (int)((b >> 52) & 0x7ff);
-    const u64 top = ((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << 11;
-    const u64 m = s < 64 ? top >> s : 0ull;
-    return (i64)b < 0 ? -(i64)m : (i64)m;
+    return (i64)(((b & 0x000fffffffffffffull) | 0x0010000000000000ull) << (((u32)(b >> 52) + 11) & 31));
 }
 __host__ __device__ __forceinline__ double fx_signed_to_double(i64 v, int frac) {
-    const double d = fx_to_double((u64)(v < 0 ? -v : v), frac);
-    return v < 0 ? -d : d;
+    return fx_with_sign(fx_to_double((u64)(v < 0 ? -v : v), frac), v);
+}
+// v >= 2^32, units of 2^-frac, rounded to double
+__host__ __device__ __forceinline__ double fx_positive_to_double(u64 v, int frac) {
+#ifdef __CUDA_ARCH__
+    const u32 hi = (u32)(v >> 32), lo = (u32)v;
+    const int lz = __clz((int)hi);
+    const u32 h = __funnelshift_l(lo, hi, lz), l = lo << lz;
+    const u64 r = (((u64)h << 32 | l) >> 11) + ((l >> 10) & 1);
+    return fx_double(r + ((u64)((u32)(1022 + 63 - frac - lz) << 20) << 32));
+#else
+    return fx_to_double(v, frac);
+#endif
+}
+// a b 2^-64 for a, b >= 0, rounded down, the product of the low halves left
+// out: at most 3 units low, 1.25 in the mean
+__host__ __device__ __forceinline__ u64 fx_mulhi_short(u64 a, u64 b) {
+    const u32 ah = (u32)(a >> 32), al = (u32)a, bh = (u32)(b >> 32), bl = (u32)b;
+    return (u64)ah * bh + (((u64)ah * bl) >> 32) + (((u64)al * bh) >> 32);
 }
 __host__ __device__ __forceinline__ u32 fx_abs_hi(u64 b) { return (u32)(b >> 32) & 0x7fffffffu; }
 
-// populations in units of 2^-62 and their exact moments; false when |f_0| >=
-// 1/2, |f| >= 1/8 along an axis or |f| >= 1/16 along a diagonal (their sum could
-// pass 2), or a value is not finite
+// populations in units of 2^-62 and their exact moments; false when one is
+// below 2^-10, or not below 1/2 (f_0), 1/8 (along an axis), 1/16 (along a
+// diagonal: their sum stays below 2), or not finite
 __host__ __device__ __forceinline__ bool fx_populations(const u64 b[Q], i64 f[Q], i64 &rho, i64 j[3]) {
-    u32 axis = 0, diag = 0;
+    int axis = 0, diag = 0, low = (int)(b[0] >> 32);  // high words: ordered like the values
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
     for (int q = 1; q < Q; ++q) {
-        const u32 h = fx_abs_hi(b[q]);
+        const int h = (int)(b[q] >> 32);
         if (CX(q) * CX(q) + CY(q) * CY(q) + CZ(q) * CZ(q) == 1) axis = axis > h ? axis : h;
         else diag = diag > h ? diag : h;
+        low = low < h ? low : h;
     }
-    if (!(fx_abs_hi(b[0]) < 0x3fe00000u && axis < 0x3fc00000u && diag < 0x3fb00000u)) return false;
+    if (!(low >= 0x3f500000 && (int)(b[0] >> 32) < 0x3fe00000 && axis < 0x3fc00000 && diag < 0x3fb00000)) return false;
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
@@ -75,7 +90,7 @@ __host__ __device__ inline FxFluid fx_fluid(double omega, double kf, const doubl
     x.ok = omega > 0.0 && omega < 2.0 && kf > 0.0 && kf < 1.0 && fabs(fb[0]) < 0.125 && fabs(fb[1]) < 0.125 &&
            fabs(fb[2]) < 0.125;
     if (!x.ok) return x;
-    x.om1 = fx_from(1.0 - omega, 62) * 2;
+    x.om = (u64)fx_from_pos(omega, 60) * 8;
     const u64 o = (u64)fx_from_pos(omega, 60), k = (u64)fx_from_pos(kf, 60);
     // omega/12, omega/36, kf/12 in units of 2^-64: 16/12 = 4/3 and 16/36 = 4/9 of the 2^-60 value
     x.om12 = o / 3 * 4 + (o % 3) * 4 / 3;
@@ -111,7 +126,7 @@ __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, doub
         return false;
     if (!fx_populations(b, f, rho, j)) return false;
     const i64 e62 = fx_from_pos(e, 62);
-    i64 F[3] = {fx_q62(p0), fx_q62(p1), fx_q62(p2)}, J[3];
+    i64 F[3] = {fx_from(fp0, 62), fx_from(fp1, 62), fx_from(fp2, 62)}, J[3];
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
@@ -161,8 +176,11 @@ __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, doub
         H[a] = (H[a] + 1) >> 1;
     }
     const i64 Xxy = xy * 24, Xxz = xz * 24, Xyz = yz * 24;
-    // (-4: the mean of the rounded-down products over the 19 populations)
-    out[0] = fx_signed_to_double(fx_mulhi_s(x.om1, f[0] * 2) + 6 * E - 4, 62);
+    // f - omega f + ...; the constant in f_0 balances the mean of the
+    // rounded-down products over the 19 populations
+    i64 v[Q];
+    v[0] = (f[0] - (i64)fx_mulhi(x.om, (u64)f[0] << 1) + 6 * E) * 2 - 42;
+    int low = (int)(v[0] >> 32);
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
@@ -178,8 +196,22 @@ __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, doub
             ev *= 2;
             od *= 2;
         }
-        out[k] = fx_signed_to_double(fx_mulhi_s(x.om1, f[k] * 4) + ev + od, 63);
-        out[k + 9] = fx_signed_to_double(fx_mulhi_s(x.om1, f[k + 9] * 4) + ev - od, 63);
+        v[k] = f[k] * 2 - (i64)fx_mulhi_short(x.om, (u64)f[k] << 2) + ev + od;
+        v[k + 9] = f[k + 9] * 2 - (i64)fx_mulhi_short(x.om, (u64)f[k + 9] << 2) + ev - od;
+        const int a = (int)(v[k] >> 32), c = (int)(v[k + 9] >> 32);
+        low = low < a ? low : a;
+        low = low < c ? low : c;
+    }
+    if (low > 0) {
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int q = 0; q < Q; ++q) out[q] = fx_positive_to_double((u64)v[q], 63);
+    } else {  // a population at or below zero
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int q = 0; q < Q; ++q) out[q] = fx_signed_to_double(v[q], 63);
     }
     return true;
 }
