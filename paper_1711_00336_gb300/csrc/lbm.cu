@@ -203,9 +203,10 @@ __device__ __forceinline__ void relax_cell(CT f[Q], CT e, CT fpx, CT fpy, CT fpz
                                            CT omega_box, CT kf_box, CT tau, int vmode, bool flag, int *status,
                                            const CT *mom);
 
-// two cells c, c+1 of one x row (c even, nx even: the plane offsets, the
-// pair and every y / z neighbour offset are even), both without a wall
-// neighbour: a population whose memory offset keeps the pair aligned (even
+// two consecutive cells c, c+1 (c and ncell even).  Even parity: own-cell
+// accesses only, any pair.  Odd parity: two cells of one x row (nx even: the
+// plane offsets, the pair and every y / z neighbour offset are even), both
+// without a wall neighbour.  A population whose memory offset keeps the pair aligned (even
 // parity: every one; odd parity: those with c_x = 0) moves as one
 // two-element vector, half the load and store instructions of the scalar
 // path; the x-moving populations of the odd parity stay scalar.  A pair next
@@ -217,10 +218,14 @@ __device__ __forceinline__ void collide_stream_vec2(ST *__restrict__ pdf, const 
                                                     CT fby, CT fbz, CT omega_box, CT kf_box, CT tau, int vmode,
                                                     int *status) {
     const long long N = g.ncell;
-    int ix, iy, iz;
-    cell_coords(g, c, ix, iy, iz);
-    const NbDelta D = neighbour_deltas(g, ix, iy, iz), D1 = neighbour_deltas(g, ix + 1, iy, iz);
-    if (!no_wall_neighbour(D) || !no_wall_neighbour(D1)) {
+    NbDelta D, D1;
+    if (PAR) {
+        int ix, iy, iz;
+        cell_coords(g, c, ix, iy, iz);
+        D = neighbour_deltas(g, ix, iy, iz);
+        D1 = neighbour_deltas(g, ix + 1, iy, iz);
+    }
+    if (PAR && (!no_wall_neighbour(D) || !no_wall_neighbour(D1))) {
         collide_stream_cell<ST, FT, CT, PAR, VISC, false>(pdf, eps, fpf, nullptr, nullptr, g, c, fbx, fby, fbz,
                                                           omega_box, kf_box, tau, vmode, status);
         collide_stream_cell<ST, FT, CT, PAR, VISC, false>(pdf, eps, fpf, nullptr, nullptr, g, c + 1, fbx, fby, fbz,
@@ -411,12 +416,15 @@ __global__ void __launch_bounds__(128, MINB) k_collide_stream(const BoxDev *__re
         const CT tau = (CT)B.ph.tau;
         const int vmode = VISC ? (B.ph.eilers ? 1 : 0) | (B.ph.smag ? 2 : 0) : 0;
         int *st = B.status;
-        if (CPT == 3 && sizeof(ST) < 8 && !MOMIN && !(g.n[0] & 1) && !(tl.begin & 1)) {
-            // vector pairs (c even; nx even, so the tile ends are even too)
+        if (CPT == 3 && sizeof(ST) < 8 && !MOMIN && !(g.ncell & 1) && !((tl.begin | tl.end) & 1) &&
+            (!PAR || !(g.n[0] & 1))) {
+            // vector pairs; the odd parity at odd nx moves scalars, two cells a
+            // thread in FP16 (161 x 150 x 139: 131 -> 107 us a step), one in
+            // FP32 (two: 148 us against 135)
             for (long long c = tl.begin + 2 * threadIdx.x; c < tl.end; c += 2 * blockDim.x)
                 collide_stream_vec2<ST, FT, CT, PAR, VISC>(pdf, eps, fpf, g, c, fbx, fby, fbz, omega, kf, tau, vmode,
                                                            st);
-        } else if (CPT == 1 || CPT == 3) {
+        } else if (CPT == 1 || (CPT == 3 && sizeof(ST) == 4)) {
             for (long long c = tl.begin + threadIdx.x; c < tl.end; c += blockDim.x)
                 collide_stream_cell<ST, FT, CT, PAR, VISC, MOMIN>(pdf, eps, fpf, rho_m, j_m, g, c, fbx, fby, fbz,
                                                                   omega, kf, tau, vmode, st, &B.ph.ff);
