@@ -41,7 +41,7 @@ void launch_sort_rank(const int *, const int *, long long, const int *, const in
 void launch_bsort_count(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 void launch_bsort_scatter(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 void launch_bsort_rank(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
-void launch_bsort_gather(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
+void launch_bsort_gather(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
 void launch_bsort_flip(BoxDev *, int, int, cudaStream_t);
 void launch_end_step(BoxDev *, int, cudaStream_t);
 void launch_bscan(const BoxDev *, int, const Tile *, int, cudaStream_t);
@@ -381,6 +381,7 @@ static void compute_phys(BoxHost *h) {
         p.skin = 0.0;
         p.skin_half2 = 0.25;
         p.skin_near2 = -1.0f;
+        p.dmax = 0.0f;
         p.shell = 0.0f;
         p.shell_near2 = -1.0f;
         p.far_ok = 0;
@@ -426,6 +427,7 @@ static void compute_phys(BoxHost *h) {
         // extra pairs at ranges of 2-3 cells and lets a particle move 0.05
         // cells between two sorts (|u| <= 0.1 at two subcycles a step)
         const double shell = std::min(0.1, c.skin), half = 0.5 * shell - 4.0 * L * 0x1p-24;
+        p.dmax = (float)(h->dmax * (1.0 + 1e-6));
         p.shell = (float)shell;
         p.shell_near2 = half > 0.0 ? (float)(0.999 * half * half) : -1.0f;
         p.far_ok = L < 4096.0;
@@ -656,8 +658,8 @@ static void enqueue_sort_eps(Batch *B, int xsel, int mark_usub, bool have_keys) 
     if (pl) {
         launch_bsort_scatter(T, B->d_part, B->n_part, grid_of(B->n_part), u.part_block, B->stream);
         launch_bsort_rank(T, B->d_part, B->n_part, grid_of(B->n_part), u.part_block, B->stream);
-        launch_bsort_gather(T, B->d_part, B->n_part, xsel, grid_of(B->n_part), part_threads(u, B->cpl_lanes),
-                            B->stream);
+        launch_bsort_gather(T, B->d_part, B->n_part, xsel, !mark_usub, grid_of(B->n_part),
+                            part_threads(u, B->cpl_lanes), B->stream);
     }
     launch_bsort_flip(B->d_table, nb, mark_usub, B->stream);
     // pair rows (FP64: each pair is evaluated once), inner rows (FP16 storage)
@@ -1012,7 +1014,7 @@ static size_t box_bytes(int prec, long long ncell, long long cap) {
     if (prec != DPS_F64) b += 6 * C * 8;  // mixed-form pair sums
     if (prec == DPS_F16S) b += 64 * C * 4 + C * 4;  // inner rows
     if (prec == DPS_F64) b += 64 * C * 4 + 32 * C * (4 + sizeof(PairRes) + 24 + 1);  // pair lists and results (64 partners)
-    if (prec == DPS_F64) b += C * (2 * sizeof(DemRec) + sizeof(DemPart));
+    if (prec == DPS_F64) b += 2 * C * (sizeof(DemRec) + sizeof(DemPart));
     b += (3 * N + 1) * 4 + 3 * C * 4 + ((N + 8191) / 8192 + 1) * 4;
     b += 4096 + (size_t)reduce_partials_doubles() * 8;
     return b;
@@ -1086,7 +1088,7 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
     d.ptan = nullptr;
     d.hl = nullptr;
     for (int k = 0; k < 2; ++k) d.rec[k] = d.lowp ? nullptr : (DemRec *)A(cap * sizeof(DemRec));
-    d.part = d.lowp ? nullptr : (DemPart *)A(cap * sizeof(DemPart));
+    for (int k = 0; k < 2; ++k) d.part[k] = d.lowp ? nullptr : (DemPart *)A(cap * sizeof(DemPart));
     d.pcap = 0;
     d.hoff = (int *)A(cap * 4);
     d.hn = (int *)A(cap * 4);

@@ -72,7 +72,7 @@ struct BoxDev {
     // records of the pair kernel: the dynamic state of the current set / of
     // the ping-pong planes, and the particle constants (set at every sort)
     DemRec *rec[2];
-    DemPart *part;
+    DemPart *part[2];  // by particle set
     unsigned long long *ptop;
     long long pcap;    // slots
     int lowp;          // 1: low-precision form (FP32 coupling arithmetic)

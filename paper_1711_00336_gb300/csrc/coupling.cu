@@ -31,27 +31,37 @@ __device__ __forceinline__ double roma_phi(double r) {
 }
 
 // weights of cells i-1, i, i+1 around the containing cell i; across a wall the
-// missing cell gets weight 0 and the rest is renormalised to sum 1.
+// missing cell gets weight 0 and the rest is renormalised to sum 1.  With s the
+// offset from the centre of cell i (|s| <= 1/2) the inner branch of phi at s and
+// the outer one at 1 -+ s share q = sqrt(1 - 3 s^2): one square root an axis
+// instead of three, of the ~25 FP64 instructions each costs with its branch.
 __device__ __forceinline__ void axis_weights(double x, int L, int periodic, double w[3]) {
-    int i = containing_cell(x, L);
-    double sum = 0.0;
-#pragma unroll
-    for (int o = -1; o <= 1; ++o) {
-        int c = i + o;
-        bool ok = periodic || (c >= 0 && c < L);
-        w[o + 1] = ok ? roma_phi((c + 0.5) - x) : 0.0;
-        sum += w[o + 1];
-    }
-    if (!periodic) {
-        if (sum > 0.0) {
-            double inv = 1.0 / sum;
-            w[0] *= inv;
-            w[1] *= inv;
-            w[2] *= inv;
-        } else {
-            w[0] = w[2] = 0.0;
-            w[1] = 1.0;
+    const int i = containing_cell(x, L);
+    const double s = x - (i + 0.5);
+    if (!(fabs(s) <= 0.5)) {  // beyond a wall: clamped into the edge cell
+        double sum = 0.0;
+#pragma unroll 1
+        for (int o = -1; o <= 1; ++o) {
+            const int c = i + o;
+            w[o + 1] = periodic || (c >= 0 && c < L) ? roma_phi((c + 0.5) - x) : 0.0;
+            sum += w[o + 1];
         }
+        if (periodic) return;
+        const bool none = !(sum > 0.0);
+        for (int o = 0; o < 3; ++o) w[o] = none ? (o == 1 ? 1.0 : 0.0) : w[o] / sum;
+        return;
+    }
+    const double q = sqrt(1.0 - 3.0 * s * s);
+    w[0] = (2.0 - 3.0 * s - q) * (1.0 / 6.0);
+    w[1] = (1.0 + q) * (1.0 / 3.0);
+    w[2] = (2.0 + 3.0 * s - q) * (1.0 / 6.0);
+    if (!periodic && (i == 0 || i == L - 1)) {
+        if (i == 0) w[0] = 0.0;
+        if (i == L - 1) w[2] = 0.0;
+        const double inv = 1.0 / (w[0] + w[1] + w[2]);
+        w[0] *= inv;
+        w[1] *= inv;
+        w[2] *= inv;
     }
 }
 
@@ -196,9 +206,12 @@ __global__ void k_bsort_rank(const BoxDev *__restrict__ boxes, const Tile *__res
 }
 
 // reorder every particle field into the other set in the sorted order;
-// record the sort position and the kernel weights (Eq. filter_def) per axis
+// record the sort position and the kernel weights (Eq. filter_def) per axis.
+// fresh: the initialisation sort, which also derives the constants of a
+// particle (mass, inverse factors, volume, the pair records' radius and 1/d);
+// later sorts move them along.  XXBS
 __global__ void k_bsort_gather(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles, int ntiles,
-                               int xsel) {
+                               int xsel, int fresh) {
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
@@ -219,7 +232,7 @@ __global__ void k_bsort_gather(const BoxDev *__restrict__ boxes, const Tile *__r
             // all plane copies issued back to back (predicated per lane)
 #pragma unroll
             for (int f = 0; f < PXS0; ++f)
-                if ((f & lm) == lane) dstf[f * cap + k] = f < 9 ? xuw[f * cap + i] : srcf[f * cap + i];
+                if ((f & lm) == lane && !(fresh && f >= PM && f <= PVOL)) dstf[f * cap + k] = f < 9 ? xuw[f * cap + i] : srcf[f * cap + i];
             for (int a = lane; a < 3; a += lanes) {
                 const double xa = xuw[a * cap + i];
                 const int La = a == 0 ? g.n[0] : (a == 1 ? g.n[1] : g.n[2]);
@@ -240,34 +253,53 @@ __global__ void k_bsort_gather(const BoxDev *__restrict__ boxes, const Tile *__r
                 }
             }
             if ((3 & lm) != lane) continue;
-            // mass and the inverse factors of Eq. particle_motion (I = m d^2 / 10)
             const double dd = srcf[PD * cap + i];
-            const double m = srcf[PRHO * cap + i] * PI_D / 6.0 * dd * dd * dd;
-            dstf[PM * cap + k] = m;
-            dstf[PIM * cap + k] = 1.0 / m;
-            dstf[PII * cap + k] = 10.0 / (m * dd * dd);
-            dstf[PVOL * cap + k] = double(PI_D / 6.0) * dd * dd * dd;
+            const float df = to_float(dd);
+            double m = 0.0;
+            if (fresh) {
+                // mass and the inverse factors of Eq. particle_motion (I = m d^2 / 10)
+                m = srcf[PRHO * cap + i] * PI_D / 6.0 * dd * dd * dd;
+                dstf[PM * cap + k] = m;
+                dstf[PIM * cap + k] = 1.0 / m;
+                dstf[PII * cap + k] = 10.0 / (m * dd * dd);
+                dstf[PVOL * cap + k] = double(PI_D / 6.0) * dd * dd * dd;
+            }
             dsti[IID * cap + k] = srci[IID * cap + i];
             dsti[ICELL * cap + k] = B.key[i];
             dsti[IKEY * cap + k] = B.key[i];
-            B.xf[0][k] = make_float4((float)xuw[i], (float)xuw[cap + i], (float)xuw[2 * cap + i], (float)dd);
-            B.xs[k] = B.xf[0][k];
-            B.vf[0][k] = make_float4((float)xuw[3 * cap + i], (float)xuw[4 * cap + i], (float)xuw[5 * cap + i], (float)m);
-            B.of[0][k] = make_float4((float)xuw[6 * cap + i], (float)xuw[7 * cap + i], (float)xuw[8 * cap + i], 0.f);
-            if (!B.lowp) {  // the records of the FP64 pair kernel
+            double x[3], u[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                x[a] = xuw[a * cap + i];
+                u[a] = xuw[(3 + a) * cap + i];
+            }
+            const float4 xf = make_float4(to_float(x[0]), to_float(x[1]), to_float(x[2]), df);
+            B.xf[0][k] = xf;
+            B.xs[k] = xf;
+            if (B.lowp) {
+                if (!fresh) m = srcf[PM * cap + i];
+                B.vf[0][k] = make_float4(to_float(u[0]), to_float(u[1]), to_float(u[2]), to_float(m));
+                B.of[0][k] = make_float4(to_float(xuw[6 * cap + i]), to_float(xuw[7 * cap + i]),
+                                         to_float(xuw[8 * cap + i]), 0.f);
+            } else {  // the records of the FP64 pair kernel
                 DemRec r;
-                DemPart q;
+#pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    r.x[a] = fx_from(xuw[a * cap + i], B.ph.fx.frac);
-                    r.u[a] = xuw[(3 + a) * cap + i];
+                    r.x[a] = fx_from(x[a], B.ph.fx.frac);
+                    r.u[a] = u[a];
                 }
-                q.rad = fx_radius(dd);
-                q.inv_d = fx_inv_d(dd);
-                q.im = 1.0 / m;
-                q.imf = (float)q.im;
-                q.pad = 0;
                 B.rec[0][k] = r;
-                B.part[k] = q;
+                DemPart q;
+                if (fresh) {
+                    q.rad = fx_radius(dd);
+                    q.inv_d = fx_inv_d(dd);
+                    q.im = 1.0 / m;
+                    q.imf = (float)q.im;
+                    q.pad = 0;
+                } else {
+                    q = B.part[B.cur][i];
+                }
+                B.part[1 - B.cur][k] = q;
             }
         }
     }
@@ -901,8 +933,9 @@ void launch_bsort_scatter(const BoxDev *b, const Tile *t, int nt, int grid, int 
 void launch_bsort_rank(const BoxDev *b, const Tile *t, int nt, int grid, int block, cudaStream_t s) {
     k_bsort_rank<<<grid, block, 0, s>>>(b, t, nt);
 }
-void launch_bsort_gather(const BoxDev *b, const Tile *t, int nt, int xsel, int grid, int block, cudaStream_t s) {
-    k_bsort_gather<<<grid, block, 0, s>>>(b, t, nt, xsel);
+void launch_bsort_gather(const BoxDev *b, const Tile *t, int nt, int xsel, int fresh, int grid, int block,
+                         cudaStream_t s) {
+    k_bsort_gather<<<grid, block, 0, s>>>(b, t, nt, xsel, fresh);
 }
 void launch_bsort_flip(BoxDev *b, int nb, int mark_usub, cudaStream_t s) {
     k_bsort_flip<<<(nb + 127) / 128, 128, 0, s>>>(b, nb, mark_usub);

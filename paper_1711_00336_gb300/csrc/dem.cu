@@ -222,24 +222,24 @@ __global__ void __launch_bounds__(256, DPS_NLIST_MINB) k_build_nlist(const BoxDe
                 }
             }
             const int ny = hi[1] - lo[1] + 1, nz = hi[2] - lo[2] + 1, nrows = act ? ny * nz : 0;
-            // the x segments of a cell row (two where the row wraps
-            // periodically), and the rows, are visited in ascending cell index
-            // of the wrapped cells, so that one lane's partners come out in
-            // ascending sorted index (the cells are the sort's keys)
-            int xs0[2] = {lo[0], 0}, xs1[2] = {hi[0], -1};
-            if (lo[0] < 0) {
-                xs0[0] = 0;
-                xs1[0] = hi[0];
-                xs0[1] = lo[0] + g.n[0];
-                xs1[1] = g.n[0] - 1;
-            } else if (hi[0] > g.n[0] - 1) {
-                xs0[0] = 0;
-                xs1[0] = hi[0] - g.n[0];
-                xs0[1] = lo[0];
-                xs1[1] = g.n[0] - 1;
-            }
+            // the rows, and the x segments of a row (two where it wraps
+            // periodically), are visited in ascending cell index of the
+            // wrapped cells, so that one lane's partners come out in ascending
+            // sorted index (the cells are the sort's keys).  Rows, and row
+            // ends, beyond the reach of the particle are left out: of the 9 x 9
+            // x 9 cells at a reach of 3.5 cells about half remain (256^3, eps 0.2,
+            // FP64: XXNL).  rm: the largest distance that can be listed, with a
+            // margin for the rounding of float positions (boxes below 2^12)
+            const float rm = 0.5f * (pi.w + ph.dmax) + extra + SCREEN_MARGIN;
+            const bool trim = ph.far_ok != 0, trimx = trim && !(g.per[0] && 2 * R + 1 >= g.n[0]);
             const int roty = lo[1] < 0 ? -lo[1] : (hi[1] > g.n[1] - 1 ? g.n[1] - lo[1] : 0);
             const int rotz = lo[2] < 0 ? -lo[2] : (hi[2] > g.n[2] - 1 ? g.n[2] - lo[2] : 0);
+            // distance from coordinate x to the cells [c, c+1) of an axis
+            auto away = [&](float x, int c, int ax) {
+                float d = fabsf(((float)c + 0.5f) - x);
+                if (g.per[ax]) d = fminf(d, fabsf(Lf[ax] - d));
+                return fmaxf(d - 0.5f, 0.0f);
+            };
             // partners of particle i in this lane's rows r = lane, lane +
             // LANES, ..., in row order, then the sorted order inside a row; the
             // particle ranges of RB rows are loaded together before any is
@@ -256,13 +256,30 @@ __global__ void __launch_bounds__(256, DPS_NLIST_MINB) k_build_nlist(const BoxDe
                         const int yy = lo[1] + (r % ny + roty) % ny, zz = lo[2] + (r / ny + rotz) % nz;
                         const int z = zz < 0 ? zz + g.n[2] : (zz >= g.n[2] ? zz - g.n[2] : zz);
                         const int y = yy < 0 ? yy + g.n[1] : (yy >= g.n[1] ? yy - g.n[1] : yy);
-                        const long long row = cell_index(g, 0, y, z);
-#pragma unroll
-                        for (int sg = 0; sg < 2; ++sg)
-                            if (xs1[sg] >= xs0[sg]) {
-                                s[2 * u + sg] = Bx.cell_start[row + xs0[sg]];
-                                e[2 * u + sg] = Bx.cell_start[row + xs1[sg] + 1];
+                        int a = lo[0], b = hi[0];
+                        if (trim) {
+                            const float dy = away(pi.y, yy, 1), dz = away(pi.z, zz, 2);
+                            const float h2 = rm * rm - dy * dy - dz * dz;
+                            if (!(h2 > 0.0f)) continue;
+                            if (trimx) {
+                                const float h = sqrtf(h2) + SCREEN_MARGIN;
+                                a = max(a, (int)floorf(pi.x - h));
+                                b = min(b, (int)floorf(pi.x + h));
+                                // a position outside the box or not finite
+                                // (the run is flagged): no cells
+                                if (a > b || b < 0 || a > g.n[0] - 1) continue;
                             }
+                        }
+                        const long long row = cell_index(g, 0, y, z);
+                        // [a, b] on the axis, or [0, b'] and [a', n-1] where it wraps
+                        const int n0 = g.n[0], a1 = a < 0 ? a + n0 : a, b0 = b > n0 - 1 ? b - n0 : b;
+                        const bool wraps = a < 0 || b > n0 - 1;
+                        s[2 * u] = Bx.cell_start[row + (wraps ? 0 : a)];
+                        e[2 * u] = Bx.cell_start[row + b0 + 1];
+                        if (wraps) {
+                            s[2 * u + 1] = Bx.cell_start[row + a1];
+                            e[2 * u + 1] = Bx.cell_start[row + n0];
+                        }
                     }
 #pragma unroll
                     for (int v = 0; v < 2 * RB; ++v)
@@ -427,17 +444,6 @@ __device__ __noinline__ NearTerms near_pair32(const BoxDev &Bx, const double *__
     const float dmean = 2.0f * pi.w * pj.w / (pi.w + pj.w);
     partner<float>(pfl, n, gap, uif, wif, pi.w, uj, wjh, m_ij, dmean, o.F, o.T, o.nlim);
     return o;
-}
-
-// v rounded to single precision as the hardware conversion rounds it (nearest,
-// ties to even), in integer operations: the conversion instruction runs on the
-// FP64 pipe
-__device__ __forceinline__ float to_float(double v) {
-    const u64 b = fx_bits(v);
-    const u64 t = b + 0x0fffffffull + ((b >> 29) & 1);
-    if (((u32)(t >> 52) & 0x7ffu) - 897u < 254u)
-        return __uint_as_float((((u32)(t >> 29) - (896u << 23)) & 0x7fffffffu) | ((u32)(b >> 32) & 0x80000000u));
-    return (b << 1) == 0 ? __uint_as_float((u32)(b >> 32)) : (float)v;
 }
 
 // one thread per particle: wall partners (WALLS), then Eq. particle_motion
@@ -932,7 +938,7 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
         const double *xin = src_tmp ? Bx.xtmp : Bx.pf[Bx.cur];
         const float4 *fin = Bx.xf[src_tmp];
         const DemRec *rec = Bx.rec[src_tmp];
-        const DemPart *part = Bx.part;
+        const DemPart *part = Bx.part[Bx.cur];
         const double *pf = Bx.pf[Bx.cur];
         const long long cap = Bx.cap;
         const Geom &g = Bx.g;

@@ -166,6 +166,7 @@ struct Phys {
     double capfac;       // lubrication cap = m_ij capfac
     double skin_half2;   // (skin / 2)^2: largest displacement between two sorts
     float skin_near2;    // squared FP32 displacement below which skin/2 is not exceeded whatever the rounding
+    float dmax;          // largest diameter, rounded up
     float shell;         // thickness of the list's inner shell beyond the interaction range
     float shell_near2;   // squared FP32 displacement below which shell/2 is not exceeded whatever the rounding
     int far_ok;          // the FP32 screen's margin covers the rounding of a wall distance (box below 2^12 cells)
@@ -189,6 +190,17 @@ __device__ __forceinline__ float m_min(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ double m_min(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ float m_max(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double m_max(double a, double b) { return fmax(a, b); }
+
+// v rounded to single precision as the hardware conversion rounds it (nearest,
+// ties to even), in integer operations: the conversion instruction runs on the
+// FP64 pipe
+__device__ __forceinline__ float to_float(double v) {
+    const u64 b = fx_bits(v);
+    const u64 t = b + 0x0fffffffull + ((b >> 29) & 1);
+    if (((u32)(t >> 52) & 0x7ffu) - 897u < 254u)
+        return __uint_as_float((((u32)(t >> 29) - (896u << 23)) & 0x7fffffffu) | ((u32)(b >> 32) & 0x80000000u));
+    return (b << 1) == 0 ? __uint_as_float((u32)(b >> 32)) : (float)v;
+}
 
 // ---- PDF storage traits ---------------------------------------------------
 // FP64 stores f_q itself; the low-precision forms store the deviation
