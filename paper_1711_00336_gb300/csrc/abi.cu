@@ -54,7 +54,7 @@ void launch_force_am(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename FT>
 void launch_force_drag(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 template <typename FT>
-void launch_reaction_am(const BoxDev *, const Tile *, int, cudaStream_t);
+void launch_reaction_am(const BoxDev *, const Tile *, int, int, cudaStream_t);
 template <typename FT>
 void launch_reaction_drag(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 void launch_dem_substep(const BoxDev *, const Tile *, int, int, int, int, int, int, int, cudaStream_t);
@@ -553,6 +553,9 @@ static int push_layout(Batch *B) {
         std::vector<Tile> &ct = (h->d.ph.eilers || h->d.ph.smag) ? cellv : cell;
         const int lc = dem_lanes_class(h), fl = force_lanes(h);
         h->d.dem_lanes = 1 << lc;
+        // a cell evaluation costs the drag pass as much as it costs the
+        // gather, plus the plane's traffic: worth it from 2 supports a cell
+        h->d.ufield = B->prec == DPS_F64 && 27 * h->d.np >= 2 * h->d.g.ncell;
         tab[k] = h->d;
         const long long N = h->d.g.ncell, np = h->d.np;
         for (long long c = 0; c < N; c += B->tune.cell_tile)
@@ -709,8 +712,8 @@ static void enqueue_step(Batch *B) {
         }
         tend(B, PH_FAM, pl + nl);
         tbegin(B);
-        if (f64) launch_reaction_am<double>(T, B->d_brick, B->n_brick, s);
-        else launch_reaction_am<float>(T, B->d_brick, B->n_brick, s);
+        if (f64) launch_reaction_am<double>(T, B->d_brick, B->n_brick, k == 0, s);
+        else launch_reaction_am<float>(T, B->d_brick, B->n_brick, k == 0, s);
         tend(B, PH_RAM, 1);
         tbegin(B);
         if (pl) {

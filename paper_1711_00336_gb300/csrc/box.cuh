@@ -75,6 +75,7 @@ struct BoxDev {
     DemPart *part[2];  // by particle set
     unsigned long long *ptop;
     long long pcap;    // slots
+    int ufield;        // 1: the added-mass reaction writes u_f of the subcycle to the u_D planes (FP64 form)
     int lowp;          // 1: low-precision form (FP32 coupling arithmetic)
     float *pwf;        // FP32 kernel weights [9][cap] (low-precision forms)
     float *f32p;       // FP32 copies of F_am (3 planes) and F_d (3 planes) [6][cap]
