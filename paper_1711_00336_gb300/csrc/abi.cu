@@ -477,19 +477,25 @@ static int ensure_buf(Batch *B, Tile **p, size_t *cap, size_t need) {
 }
 
 // lanes per particle in the DEM substep of a box (class 0..3 = 1, 2, 4, 8
-// lanes): about one neighbour-list entry per lane or more, from the expected
-// list length (number density times the list sphere).  A property of the box
-// alone, so a box gets the same arithmetic alone and in any batch.
+// lanes).  A property of the box alone, so a box gets the same arithmetic
+// alone and in any batch.  A lane group pays seven sums over its lanes, so two
+// lanes (one for short rows) are best once they fill the chip: DEM of 40
+// substeps, FP32, 1.5 million spheres with 22 partners: 22.8 / 22.3 / 23.7 / 26.2
+// ms with 1 / 2 / 4 / 8 lanes, 190 thousand 3.80 / 3.71 / 3.92 / 4.29, 63
+// thousand 1.59 / 1.32 / 1.34 / -, 19 thousand 0.97 with 4, 0.77 with 8.
+// The FP16-storage form keeps the lanes (and with them the summation order) of
+// the full list's length.
 static int dem_lanes_class(const BoxHost *h) {
     if (!h->have_closure || h->d.np == 0) return 0;
     const dps_closure &c = h->cl;
-    const double rl = h->dmax + (c.lubrication ? std::fmax(c.h_c, 0.0) : 0.0) + c.skin;
-    const double est = (double)h->d.np / (double)h->d.g.ncell * 4.18879 * rl * rl * rl;
-    int cls = est >= 24.0 ? 3 : est >= 8.0 ? 2 : est >= 3.0 ? 1 : 0;
-    // few particles: a warp costs the longest list among its particles and
+    const double reach = h->dmax + (c.lubrication ? std::fmax(c.h_c, 0.0) : 0.0);
+    const double rl = reach + (h->d.split ? std::min(0.1, c.skin) : c.skin);
+    const double est = (double)h->d.np / (double)h->d.g.ncell * 4.18879 * rl * rl * rl;  // expected row length
+    int cls = h->d.split ? (est >= 8.0 ? 1 : 0) : est >= 24.0 ? 3 : est >= 8.0 ? 2 : est >= 3.0 ? 1 : 0;
+    // few particles: a warp costs the longest row among its particles and
     // there are few warps per SM, so spread every particle over more lanes
-    // (about one warp per SM scheduler at np x lanes / 32)
-    for (long long lanes = 1LL << cls; cls < 3 && h->d.np * lanes < 19456; lanes <<= 1) ++cls;
+    const long long fill = h->d.split ? 126000 : 19456;
+    for (long long lanes = 1LL << cls; cls < 3 && h->d.np * lanes < fill; lanes <<= 1) ++cls;
     return cls;
 }
 
@@ -749,17 +755,22 @@ static void enqueue_step(Batch *B) {
                     ndl += 2;  // pair kernel + gather kernel
                     continue;
                 }
-                for (int c = 0; c < 4; ++c) {
-                    const int nt = B->part_off[c + 1] - B->part_off[c];
-                    if (nt <= 0) continue;
-                    // a block holds all lane groups of a particle tile, at
-                    // most 256 threads (two such blocks fit an SM)
-                    const int blk = (int)std::min<long long>(
-                        256, (std::max<long long>(u.part_block, (long long)u.part_tile << c) + 31) / 32 * 32);
-                    launch_dem_substep(T, B->d_part + B->part_off[c], nt, sd & 1, key_out, 1 << c, B->any_walls,
-                                       grid_of(nt), blk, s);
-                    ndl += 2;  // pair kernel + integration kernel
-                }
+                // lanes per particle: those of the one class present, or 0:
+                // each tile its box's
+                int lanes = 0, classes = 0;
+                for (int c = 0; c < 4; ++c)
+                    if (B->part_off[c + 1] > B->part_off[c]) {
+                        lanes = 1 << c;
+                        ++classes;
+                    }
+                if (classes > 1) lanes = 0;
+                // a block holds all lane groups of a particle tile, at most
+                // 256 threads (four such blocks fit an SM)
+                const int blk = (int)std::min<long long>(
+                    256, (std::max<long long>(u.part_block, (long long)u.part_tile * (lanes ? lanes : 8)) + 31) / 32 * 32);
+                launch_dem_substep(T, B->d_part, B->n_part, sd & 1, key_out, lanes, B->any_walls, grid_of(B->n_part),
+                                   blk, s);
+                ndl += 2;  // pair kernel + integration kernel
             }
         tend(B, PH_DEM, ndl);
         if (fork) cudaStreamWaitEvent(s, B->ev_join, 0);
