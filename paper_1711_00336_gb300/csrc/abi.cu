@@ -28,8 +28,8 @@ template <typename ST, typename FT, typename CT>
 void launch_moments(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 void launch_fields64(const BoxDev *, const Tile *, int, cudaStream_t);
 void launch_fields32(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
-template <typename FT, typename CT>
-void launch_curl(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+void launch_curl64(const BoxDev *, const Tile *, int, cudaStream_t);
+void launch_curl32(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename ST>
 void launch_pdf_export(const void *, const Geom &, int, double *, cudaStream_t);
 template <typename ST>
@@ -709,8 +709,8 @@ static void enqueue_step(Batch *B) {
     for (int k = 0; k < B->n_int; ++k) {
         tbegin(B);
         if (nl) {
-            if (f64) launch_curl<double, double>(T, B->d_cell, B->n_cell, gc, u.cell_block, s);
-            else launch_curl<float, float>(T, B->d_cell, B->n_cell, gc, u.cell_block, s);
+            if (f64) launch_curl64(T, B->d_brick, B->n_brick, s);
+            else launch_curl32(T, B->d_cell, B->n_cell, gc, u.cell_block, s);
         }
         if (pl) {
             if (f64) launch_force_am<double>(T, B->d_part, B->n_part, gp, part_threads(u, B->cpl_lanes), s);

@@ -684,7 +684,18 @@ __global__ void k_force_am(const BoxDev *__restrict__ boxes, const Tile *__restr
             Support<FT> S;
             if (act) {
                 S = support_of<FT>(B, pf, p);
-                if (lift)
+                if (lift && sizeof(FT) == 8) {
+                    // u_f of the subcycle start written by the curl pass
+                    const FT *uf = (const FT *)B.fam;
+                    for_support_lanes(g, S, lane, lanes, [&](long long c, FT W) {
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            v[a] += W * DuDt[a * N + c];
+                            v[3 + a] += W * uf[a * N + c];
+                            v[6 + a] += W * curl[a * N + c];
+                        }
+                    });
+                } else if (lift)
                     for_support_lanes(g, S, lane, lanes, [&](long long c, FT W) {
                         v[0] += W * DuDt[c];
                         v[1] += W * DuDt[N + c];
