@@ -118,6 +118,37 @@ __device__ __forceinline__ void contact_force(const PairPar<T> &ph, const T n[3]
     }
 }
 
+// the FP64 form of it: |F_n| = |k_n delta + xi u_n| since n is a unit vector,
+// and the friction is xi u_t unless mu_c |F_n| caps it, so the square root and
+// the divisions of the general form shrink to one reciprocal square root on
+// the sliding branch (an FP64 square root or division costs ~8.5 multiply-adds)
+__device__ __forceinline__ void contact_force(const PairPar<double> &ph, const double n[3], double delta,
+                                              const double ui[3], const double wi[3], double di, const double uj[3],
+                                              const double wjh[3], double m_ij, double lev, double F[3], double Tq[3]) {
+    double ws[3], wx[3], ur[3], ut[3], Ft[3], nF[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) ws[a] = 0.5 * di * wi[a] + wjh[a];
+    cross3(ws, n, wx);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) ur[a] = ui[a] - uj[a] + wx[a];
+    const double urn = ur[0] * n[0] + ur[1] * n[1] + ur[2] * n[2];
+    const double xi = m_ij * ph.xfac, fn = m_ij * ph.kfac * delta + xi * urn;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) ut[a] = ur[a] - urn * n[a];
+    const double ut2 = ut[0] * ut[0] + ut[1] * ut[1] + ut[2] * ut[2];
+    const double lim = ph.mu_c * fabs(fn);
+    double mag = xi;
+    if (!(xi * xi * ut2 <= lim * lim)) mag = lim * rsqrt(ut2);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) Ft[a] = -mag * ut[a];
+    cross3(n, Ft, nF);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        F[a] += Ft[a] - fn * n[a];
+        Tq[a] += lev * nF[a];
+    }
+}
+
 // lubrication correction (Sec. 3.1.3) at the floored gap hh, given <d>,
 // r = <d>/hh, ir = 1/r and the limiter cap m_ij capfac
 template <typename T>
@@ -151,7 +182,7 @@ __device__ __forceinline__ void partner(const PairPar<T> &ph, const T n[3], T ga
                                         T di, const T uj[3], const T wjh[3], T m_ij, T dmean, T F[3], T Tq[3],
                                         unsigned &nlim) {
     const T delta = -gap;
-    if (ph.contact && delta > T(0)) contact_force(ph, n, delta, ui, wi, di, uj, wjh, m_ij, T(0.5) * di, F, Tq);
+    if (ph.contact && delta > T(0)) contact_force<T>(ph, n, delta, ui, wi, di, uj, wjh, m_ij, T(0.5) * di, F, Tq);
     const T h = gap;
     if (ph.lubrication && h >= T(0) && h < ph.h_c) {
         const T hh = m_max(h, ph.h_min);
@@ -459,6 +490,23 @@ __device__ __noinline__ NearTerms near_pair32(const BoxDev &Bx, const double *__
     return o;
 }
 
+// contact or lubrication with face `side` of axis a, in FP64 (out of line: few
+// particles of few warps need it)
+__device__ __noinline__ void wall_exact(const BoxDev &Bx, long long i, int a, int side, double xa, const double ui[3],
+                                        const double wi[3], double F[3], double T[3]) {
+    const Phys &ph = Bx.ph;
+    const double *pf = Bx.pf[Bx.cur];
+    const double di = pf[PD * Bx.cap + i], mi = pf[PM * Bx.cap + i];
+    const double dist = side == 0 ? xa : Bx.g.n[a] - xa;
+    if (!(dist < 0.5 * di + (ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0))) return;
+    const PairPar<double> pd = pair_par<double>(ph);
+    const double zero[3] = {0, 0, 0}, s = side == 0 ? -1.0 : 1.0;
+    const double n[3] = {a == 0 ? s : 0.0, a == 1 ? s : 0.0, a == 2 ? s : 0.0};
+    unsigned nlim = 0;
+    partner<double>(pd, n, dist - 0.5 * di, ui, wi, di, zero, zero, mi, 2.0 * di, F, T, nlim);
+    if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], (unsigned long long)nlim);
+}
+
 // one thread per particle: wall partners (WALLS), then Eq. particle_motion
 // (semi-implicit Euler) and the outputs of the substep.  Comparisons and
 // conversions are integer or FP32 operations (an FP64 compare or conversion
@@ -483,30 +531,47 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
     }
     const float4 xs = Bx.xs[i];  // position at the last sort, and d
     // walls: the faces of every non-periodic axis (m_ij = m_i, <d> = 2 d_i),
-    // screened in FP32 (xs carries d) with the margin of the pair screen
+    // screened in FP32 (xs carries d) with the margin of the pair screen.  The
+    // FP64 form takes the lubrication from the integer path of the pairs and
+    // leaves contact to the FP64 body out of line: inlined, six faces' worth of
+    // FP64 cost 211 registers a thread (closures with walls, 75 x 61 x 90: DEM
+    // substep 67 -> 55 us with three blocks per SM, 64 with one)
     if (WALLS && !(g.per[0] && g.per[1] && g.per[2])) {
         const float reach = 0.5f * xs.w + (float)(ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0) + SCREEN_MARGIN;
-        const double zero[3] = {0, 0, 0};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (g.per[a]) continue;
-            const float xf = to_float(xi[a]);
-            if (!(xf < reach) && !(((float)g.n[a] - xf) < reach) && ph.far_ok) continue;
-            const double rng_extra = ph.lubrication ? fmax(ph.h_c, 0.0) : 0.0;
-            const PairPar<double> pd = pair_par<double>(ph);
-            const double di = pf[PD * cap + i];
-            const double mi = pf[PM * cap + i];
-            unsigned nlim = 0;
+        const float fx3[3] = {to_float(xi[0]), to_float(xi[1]), to_float(xi[2])};
 #pragma unroll 1
-            for (int side = 0; side < 2; ++side) {
-                const double dist = side == 0 ? xi[a] : g.n[a] - xi[a];
-                const double range = 0.5 * di + rng_extra;
-                if (!(dist < range)) continue;
-                double n[3] = {0, 0, 0};
-                n[a] = side == 0 ? -1.0 : 1.0;
-                partner<double>(pd, n, dist - 0.5 * di, ui, wi, di, zero, zero, mi, 2.0 * di, F, T, nlim);
+        for (int f = 0; f < 6; ++f) {
+            const int a = f >> 1, side = f & 1;
+            const float xf = a == 0 ? fx3[0] : (a == 1 ? fx3[1] : fx3[2]);
+            const int n_a = a == 0 ? g.n[0] : (a == 1 ? g.n[1] : g.n[2]);
+            const int per = a == 0 ? g.per[0] : (a == 1 ? g.per[1] : g.per[2]);
+            const float away = side ? (float)n_a - xf : xf;
+            if (per || (!(away < reach) && ph.far_ok)) continue;
+            const double xa = a == 0 ? xi[0] : (a == 1 ? xi[1] : xi[2]);
+            int kind = FX_EXACT;
+            if (F64 && ph.fx.ok && ph.lubrication && away > 0.f && away < 16.f) {
+                // lubrication as for a pair, with the wall a partner of no
+                // radius: 1/<d> = 1/(2 d_i)
+                const DemPart q = Bx.part[Bx.cur][i];
+                const i64 x = fx_from(xa, ph.fx.frac);
+                const i64 dx[3] = {0, 0, side ? ((i64)n_a << ph.fx.frac) - x : x};
+                FxPair o;
+                kind = dx[2] > 0 ? fx_pair(dx, q.rad, (u64)q.inv_d, ph.fx, o) : FX_EXACT;
+                if (kind == FX_LUB) {
+                    double al = o.alpha, be = o.beta;
+                    const float capf = (float)ph.capfac * 0.999f;
+                    if (ph.lub_limiter && !(fx_approx(be) * q.imf < capf && fx_approx(al) * q.imf < capf)) {
+                        const double lim = pf[PM * cap + i] * ph.capfac;
+                        const unsigned nlim = (be > lim) + (al > lim);
+                        be = be > lim ? lim : be;
+                        al = al > lim ? lim : al;
+                        if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], (unsigned long long)nlim);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) F[k] -= (k == a ? be : al) * ui[k];
+                }
             }
-            if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], (unsigned long long)nlim);
+            if (kind == FX_EXACT) wall_exact(Bx, i, a, side, xa, ui, wi, F, T);
         }
     }
     // Eq. particle_motion, semi-implicit Euler with I = m d^2 / 10
@@ -1132,7 +1197,7 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
 #define DPS_GATHER_MINB 5  // 128-thread blocks per SM the register budget is sized for
 #endif
 template <bool WALLS>
-__global__ void __launch_bounds__(128, WALLS ? 1 : DPS_GATHER_MINB) k_dem_gather64(const BoxDev *__restrict__ boxes,
+__global__ void __launch_bounds__(128, WALLS ? 3 : DPS_GATHER_MINB) k_dem_gather64(const BoxDev *__restrict__ boxes,
                                                         const Tile *__restrict__ tiles, int ntiles, int src_tmp,
                                                         int key_out) {
     // slots of a particle's pairs in contact with friction: listed while the

@@ -83,6 +83,40 @@ def test_fp64_pairs_against_the_oracle(name):
     assert st["status"] == 0
 
 
+@pytest.mark.parametrize("per", [(0, 1, 1), (1, 0, 0), (0, 0, 0)])
+@pytest.mark.parametrize("gap", [-0.1, -1e-6, 1e-7, 9e-6, 1e-4, 0.03, 0.499, 0.501])
+def test_fp64_walls_against_the_oracle(per, gap):
+    """One sphere at each face (gaps from overlap over the floor, the limiter
+    and the cut-off to beyond it), each far from the others."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import oracle as O
+    from paper_1711_00336_gb300 import dps
+    n = (14, 15, 13)
+    rng = np.random.default_rng(7)
+    d = rng.uniform(0.9, 1.6, 6)
+    x = np.tile(np.array(n) / 2.0, (6, 1))
+    for f in range(6):
+        near = gap + 0.5 * d[f]
+        x[f, f // 2] = n[f // 2] - near if f % 2 else near
+    u, w = 0.01 * rng.standard_normal((6, 3)), 0.01 * rng.standard_normal((6, 3))
+    kw = dict(g=(0.0, 0.0, -1e-4), e_n=0.9, mu_c=0.25, T_c=20.0, h_c=0.5, h_min=1e-5, C_am=0.5, n_int=1, n_dem=10,
+              lub_limiter=1, lub_cap=0.25, eps_min=0.05)
+    dom = dps.Domain(n, per, 0.7, "f64", max_particles=6)
+    dom.add_particles(x, d, 2.5, u=u, w=w)
+    dom.set_closure(fb_mode=0, fb=(0, 0, 0), skin=0.6, drag=0, pressure=0, added_mass=0, **kw)
+    dom.step(1)
+    got = dom.read_particles()
+    dom.close()
+    P = O.make_params(n, per, 0.7, drag=0, pressure=0, added_mass=0, **kw)
+    ref = O.Domain(P, x=x, u=u, w=w, d=d, rho_p=np.full(6, 2.5))
+    ref.step(1)
+    r = ref.particles()
+    for k in ("u", "w"):
+        assert np.abs(got[k] - r[k]).max() <= TOL * np.abs(r[k]).max(), k
+
+
 @pytest.mark.parametrize("fast", [0.0, 0.3])
 def test_written_velocities_and_moves_beyond_the_inner_shell(fast):
     """Velocities written between sorts reach the pairs, and particles that
