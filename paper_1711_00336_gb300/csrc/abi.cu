@@ -48,15 +48,16 @@ void launch_bscan(const BoxDev *, int, const Tile *, int, cudaStream_t);
 int scan_tile_cells();
 void brick_tiles(int, const int *, std::vector<Tile> &);
 template <typename FT>
-void launch_eps(const BoxDev *, const Tile *, int, cudaStream_t);
+void launch_eps(const BoxDev *, const Tile *, int, int, cudaStream_t);
 template <typename FT>
 void launch_force_am(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename FT>
 void launch_force_drag(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 template <typename FT>
-void launch_reaction_am(const BoxDev *, const Tile *, int, int, cudaStream_t);
+void launch_reaction_am(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename FT>
-void launch_reaction_drag(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+void launch_reaction_drag(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
+int sparse_stage_mean();
 void launch_dem_substep(const BoxDev *, const Tile *, int, int, int, int, int, int, int, cudaStream_t);
 void launch_dem_substep64(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
 void launch_build_nlist(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
@@ -153,6 +154,7 @@ struct Batch {
     bool any_lift = false;        // some box applies the lift force (curl launch per subcycle)
     bool any_walls = true;        // some box with particles has a wall axis (DEM wall code)
     int part_off[5] = {0, 0, 0, 0, 0};  // particle tiles grouped by DEM lanes class (1, 2, 4, 8)
+    int sparse = 1;  // every box is dilute: brick gathers with the small stage
     int cpl_lanes = 1;            // most lanes per particle of the force kernels over the batch
     int n_cell_plain = 0;         // cell tiles of boxes with a constant tau (listed first);
                                   // the rest relax with a per-cell tau_e (K1 variant)
@@ -551,6 +553,7 @@ static int push_layout(Batch *B) {
     B->any_lift = false;
     B->any_walls = false;
     B->cpl_lanes = 1;
+    B->sparse = 1;
     for (int k = 0; k < nb; ++k) {
         BoxHost *h = B->boxes[k];
         compute_phys(h);
@@ -564,6 +567,7 @@ static int push_layout(Batch *B) {
         h->d.ufield = B->prec == DPS_F64 && 27 * h->d.np >= 2 * h->d.g.ncell;
         tab[k] = h->d;
         const long long N = h->d.g.ncell, np = h->d.np;
+        B->sparse &= 1000 * np <= sparse_stage_mean() * N;
         for (long long c = 0; c < N; c += B->tune.cell_tile)
             ct.push_back(Tile{k, 0, c, std::min(N, c + B->tune.cell_tile)});
         B->cpl_lanes = std::max(B->cpl_lanes, fl);
@@ -679,9 +683,9 @@ static void enqueue_sort_eps(Batch *B, int xsel, int mark_usub, bool have_keys) 
     tend(B, PH_SORT, cnt + 3 + 3 * pl + 1 + pl * (1 + (rows == 1 ? 2 : rows == 2)));
     tbegin(B);
     if (B->fel == 8)
-        launch_eps<double>(T, B->d_brick, B->n_brick, B->stream);
+        launch_eps<double>(T, B->d_brick, B->n_brick, B->sparse, B->stream);
     else
-        launch_eps<float>(T, B->d_brick, B->n_brick, B->stream);
+        launch_eps<float>(T, B->d_brick, B->n_brick, B->sparse, B->stream);
     tend(B, PH_EPS, 1);
 }
 
@@ -718,8 +722,8 @@ static void enqueue_step(Batch *B) {
         }
         tend(B, PH_FAM, pl + nl);
         tbegin(B);
-        if (f64) launch_reaction_am<double>(T, B->d_brick, B->n_brick, k == 0, s);
-        else launch_reaction_am<float>(T, B->d_brick, B->n_brick, k == 0, s);
+        if (f64) launch_reaction_am<double>(T, B->d_brick, B->n_brick, k == 0, B->sparse, s);
+        else launch_reaction_am<float>(T, B->d_brick, B->n_brick, k == 0, B->sparse, s);
         tend(B, PH_RAM, 1);
         tbegin(B);
         if (pl) {
@@ -740,9 +744,9 @@ static void enqueue_step(Batch *B) {
         }
         tbegin(B, rs);
         if (f64)
-            launch_reaction_drag<double>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, rs);
+            launch_reaction_drag<double>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, B->sparse, rs);
         else
-            launch_reaction_drag<float>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, rs);
+            launch_reaction_drag<float>(T, B->d_brick, B->n_brick, k == 0, k == B->n_int - 1, B->sparse, rs);
         tend(B, PH_RDRAG, 1, rs);
         if (fork) cudaEventRecord(B->ev_join, B->side);
         tbegin(B);

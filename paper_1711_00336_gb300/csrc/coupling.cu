@@ -371,20 +371,37 @@ __device__ __forceinline__ void for_brick_cells(const Geom &g, int ox, int oy, i
 // cell by cell of the support, for the busiest lane (~27 rounds of five
 // FP64 instructions); weights and values come from shared memory.  The three
 // gathers together, before / after: 17.9 / 7.6 ms a step (256^3, eps 0.2, two
-// subcycles, FP64), 3.1 / 2.1 ms (192^3, eps 0.38, FP32), 4.5 / 3.6 ms (256^3,
+// subcycles, FP64), 3.1 / 1.9 ms (192^3, eps 0.38, FP32), 4.5 / 3.7 ms (256^3,
 // eps 0.05, FP16 storage); FP64 is bound by its five FP64 instructions an entry.
+//
+// A dilute brick is a chain of waits instead (cell ranges, particles, cells),
+// so what counts is how many blocks an SM holds.  Boxes with at most 5/8 of
+// SPARSE_CAP particles in a brick and its halo on average take the SPARSE
+// instances: a stage of SPARSE_CAP entries and lists of SPARSE_LIST, 8 (FP32)
+// or 6 (FP64) blocks per SM; a brick over that (particles that settled) is
+// staged in slabs of two layers (0.5 particles per cell), and walks global
+// memory past that.  Dilute cases: 3.7 -> 2.8 ms (FP16 storage), 7.6 -> 6.5 ms
+// (FP64 256^3); SPARSE_CAP 128 sends that FP64 box to the dense stage and 256
+// costs the dilute one 5%.
 constexpr int BRICK_THREADS = 256;  // block size of every brick kernel
-constexpr int LIST_CAP = 24;        // entries a thread lists before it adds them
+constexpr int SPARSE_CAP = 192, SPARSE_LIST = 12;
+// blocks per SM the registers of a brick kernel are sized for
+template <typename FT, bool SPARSE> constexpr int brick_minb() {
+    return SPARSE ? (sizeof(FT) == 8 ? 6 : 8) : (sizeof(FT) == 8 ? 3 : 4);
+}
 constexpr int BL_PER_THREAD = (HALO3 + BRICK_THREADS - 1) / BRICK_THREADS;
 // staged entries: three (FP64) or four (FP32) blocks fit an SM's shared memory;
 // denser bricks take the walk over global memory
-template <typename FT> constexpr int stage_cap() { return sizeof(FT) == 8 ? 448 : 704; }
+template <typename FT, bool SPARSE> constexpr int stage_cap() {
+    return SPARSE ? SPARSE_CAP : (sizeof(FT) == 8 ? 448 : 704);
+}
 
-template <typename FT, int NV>
+template <typename FT, int NV, bool SPARSE>
 struct BrickStage {
-    static constexpr int CAP = stage_cap<FT>();
+    static constexpr int CAP = stage_cap<FT, SPARSE>();
+    static constexpr int LIST_CAP = SPARSE ? SPARSE_LIST : 24;  // entries a thread lists before it adds them
     FT w[9][CAP], v[NV][CAP];
-    int off[HALO3 + 1], start[HALO3];
+    unsigned short off[HALO3 + 2];
     union {
         int P[CAP];
         unsigned short list[LIST_CAP][BRICK_THREADS];
@@ -395,10 +412,10 @@ struct BrickStage {
 };
 
 // stage brick (ox,oy,oz); value(p, k): the k-th value of particle p.  Ends with a barrier
-template <typename FT, int NV, typename Val>
+template <typename FT, int NV, bool SPARSE, typename Val>
 __device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int oz, int ex, int ey, int ez,
-                                            const FT *__restrict__ w, BrickStage<FT, NV> &S, Val &&value) {
-    constexpr int CAP = BrickStage<FT, NV>::CAP;
+                                            const FT *__restrict__ w, BrickStage<FT, NV, SPARSE> &S, Val &&value) {
+    constexpr int CAP = BrickStage<FT, NV, SPARSE>::CAP;
     const Geom &g = B.g;
     int s0[BL_PER_THREAD], cnt[BL_PER_THREAD], tot = 0;
 #pragma unroll
@@ -416,7 +433,6 @@ __device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int
                 a = B.cell_start[n];
                 e = B.cell_start[n + 1];
             }
-            S.start[h] = a;
         }
         s0[u] = a;
         cnt[u] = e - a;
@@ -443,9 +459,9 @@ __device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int
 #pragma unroll
     for (int u = 0; u < BL_PER_THREAD; ++u) {
         const int h = BL_PER_THREAD * threadIdx.x + u;
-        if (h < HALO3) {
-            S.off[h] = run;
-            if (fits)
+        if (h < HALO3 && fits) {
+            S.off[h] = (unsigned short)run;
+            if (cnt[u])
                 for (int m = 0; m < cnt[u]; ++m) {
                     S.P[run + m] = s0[u] + m;
                     S.hx[run + m] = (unsigned char)(h % HALO);
@@ -454,7 +470,7 @@ __device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int
         run += cnt[u];
     }
     if (threadIdx.x == 0) {
-        S.off[HALO3] = total;
+        S.off[HALO3] = (unsigned short)total;
         S.n = fits ? total : -1;
     }
     __syncthreads();
@@ -471,25 +487,31 @@ __device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int
 
 // for every cell c of the brick: sums s[k] of W_p(c) v_k(p) over the particles
 // of its support, in the order o_z, o_y, o_x ascending, then sorted; fin(s, c)
-template <typename FT, int NV, typename Val, typename Fin>
-__device__ __forceinline__ void brick_gather(const BoxDev &B, BrickStage<FT, NV> &S, int ox, int oy, int oz, int ex,
+template <typename FT, int NV, bool SPARSE, typename Val, typename Fin>
+__device__ __forceinline__ void brick_cells(const BoxDev &B, BrickStage<FT, NV, SPARSE> &S, int ox, int oy, int oz, int ex,
                                              int ey, int ez, const FT *__restrict__ w, Val &&value, Fin &&fin) {
-    const long long cap = B.cap;
+    constexpr int LIST_CAP = BrickStage<FT, NV, SPARSE>::LIST_CAP;
     for_brick_cells(B.g, ox, oy, oz, ex, ey, ez, [&](long long c, int lx, int ly, int lz) {
         FT s[NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k) s[k] = FT(0);
         if (S.n < 0) {  // over the staged size: the walk over global memory
+            const Geom &g = B.g;
 #pragma unroll 1
             for (int r = 0; r < 9; ++r) {
                 const int dz = r / 3 - 1, dy = r % 3 - 1;
-                const FT *wz = w + (6 + 1 - dz) * cap, *wy = w + (3 + 1 - dy) * cap;
-                const int hrow = ((lz + 1 + dz) * HALO + ly + 1 + dy) * HALO + lx + 1;
-#pragma unroll
+                const FT *wz = w + (6 + 1 - dz) * B.cap, *wy = w + (3 + 1 - dy) * B.cap;
+                const int y = wrap_axis(oy + ly + dy, g.n[1], g.per[1]), z = wrap_axis(oz + lz + dz, g.n[2], g.per[2]);
+                if (y < 0 || z < 0) continue;
+#pragma unroll 1
                 for (int dx = -1; dx <= 1; ++dx) {
-                    const int h = hrow + dx, p0 = S.start[h], p1 = p0 + S.off[h + 1] - S.off[h];
-                    const FT *wx = w + (1 - dx) * cap;
-                    for (int p = p0; p < p1; ++p) {
+                    const int x = wrap_axis(ox + lx + dx, g.n[0], g.per[0]);
+                    if (x < 0) continue;
+                    const long long h = cell_index(g, x, y, z);
+                    const int p1 = B.cell_start[h + 1];
+                    const FT *wx = w + (1 - dx) * B.cap;
+#pragma unroll 1
+                    for (int p = B.cell_start[h]; p < p1; ++p) {
                         const FT W = wx[p] * wy[p] * wz[p];
 #pragma unroll
                         for (int k = 0; k < NV; ++k) s[k] += W * value(p, k);
@@ -536,22 +558,41 @@ __device__ __forceinline__ void brick_gather(const BoxDev &B, BrickStage<FT, NV>
     });
 }
 
+// stage and gather one brick; a sparse stage takes a brick over its size in
+// slabs of two layers
+template <bool SPARSE, typename FT, int NV, typename Val, typename Fin>
+__device__ __forceinline__ void brick_gather(const BoxDev &B, unsigned char *smem, const Tile &tl,
+                                             const FT *__restrict__ w, Val &&value, Fin &&fin) {
+    BrickStage<FT, NV, SPARSE> &S = *(BrickStage<FT, NV, SPARSE> *)smem;
+    int ox, oy, oz, ex, ey, ez;
+    brick_unpack(tl.begin, ox, oy, oz);
+    brick_unpack(tl.end, ex, ey, ez);
+    int z = 0, dz = ez;
+#pragma unroll 1
+    while (z < ez) {
+        __syncthreads();  // the previous stage is done with
+        stage_brick(B, ox, oy, oz + z, ex, ey, dz, w, S, value);
+        if (SPARSE && S.n < 0 && dz > 2) {
+            dz = 2;
+            continue;
+        }
+        brick_cells(B, S, ox, oy, oz + z, ex, ey, dz, w, value, fin);
+        z += dz;
+        dz = min(dz, ez - z);
+    }
+}
+
 // ---- S2: eps_f ------------------------------------------------------------------
 // FT is the compute type of the form: FP64 for the plain method, FP32 (with
 // FP32 kernel weights) for the low-precision forms.  Also clears the sort
 // counts for the next sort (every cell is visited once).
-template <typename FT>
-__global__ void __launch_bounds__(BRICK_THREADS) k_eps_gather(const BoxDev *__restrict__ boxes,
+template <typename FT, bool SPARSE>
+__global__ void __launch_bounds__(BRICK_THREADS, brick_minb<FT, SPARSE>()) k_eps_gather(const BoxDev *__restrict__ boxes,
                                                               const Tile *__restrict__ tiles, int ntiles) {
     extern __shared__ __align__(16) unsigned char smem[];
-    BrickStage<FT, 1> &S = *(BrickStage<FT, 1> *)smem;
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
-        int ox, oy, oz, ex, ey, ez;
-        brick_unpack(tl.begin, ox, oy, oz);
-        brick_unpack(tl.end, ex, ey, ez);
-        __syncthreads();  // the previous brick is done with S
         const double *pf = B.pf[B.cur];
         const long long cap = B.cap;
         const FT *w = weights_of<FT>(B, pf);
@@ -561,11 +602,10 @@ __global__ void __launch_bounds__(BRICK_THREADS) k_eps_gather(const BoxDev *__re
             const FT d = (FT)xf[p].w;
             return FT(PI_D / 6.0) * d * d * d;
         };
-        stage_brick<FT, 1>(B, ox, oy, oz, ex, ey, ez, w, S, volume);
         FT *eps = (FT *)B.eps;
         const FT eps_min = (FT)B.ph.eps_min;
         unsigned nclamp = 0;
-        brick_gather<FT, 1>(B, S, ox, oy, oz, ex, ey, ez, w, volume, [&](const FT *s, long long c) {
+        brick_gather<SPARSE, FT, 1>(B, smem, tl, w, volume, [&](const FT *s, long long c) {
             FT e = FT(1) - s[0];
             if (e < eps_min) {
                 if (e < FT(0)) atomicOr(B.status, ST_EPS_NEG);
@@ -887,25 +927,19 @@ template <> __device__ __forceinline__ const float *force_planes<float>(const Bo
 }
 
 // K6a: f_pf,am(c) = -sum_p W F_am
-template <typename FT>
-__global__ void __launch_bounds__(BRICK_THREADS) k_reaction_am(const BoxDev *__restrict__ boxes,
+template <typename FT, bool SPARSE>
+__global__ void __launch_bounds__(BRICK_THREADS, brick_minb<FT, SPARSE>()) k_reaction_am(const BoxDev *__restrict__ boxes,
                                                                const Tile *__restrict__ tiles, int ntiles, int first) {
     extern __shared__ __align__(16) unsigned char smem[];
-    BrickStage<FT, 3> &S = *(BrickStage<FT, 3> *)smem;
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
-        int ox, oy, oz, ex, ey, ez;
-        brick_unpack(tl.begin, ox, oy, oz);
-        brick_unpack(tl.end, ex, ey, ez);
-        __syncthreads();
         const long long N = B.g.ncell, cap = B.cap;
         const double *pf = B.pf[B.cur];
         const FT *w = weights_of<FT>(B, pf), *Fa = force_planes<FT>(B, pf, 0);
         auto force = [&](int p, int k) { return Fa[k * cap + p]; };
-        stage_brick<FT, 3>(B, ox, oy, oz, ex, ey, ez, w, S, force);
         FT *fam = (FT *)B.fam;
-        brick_gather<FT, 3>(B, S, ox, oy, oz, ex, ey, ez, w, force, [&](const FT *s, long long c) {
+        brick_gather<SPARSE, FT, 3>(B, smem, tl, w, force, [&](const FT *s, long long c) {
             fam[c] = -s[0];
             fam[N + c] = -s[1];
             fam[2 * N + c] = -s[2];
@@ -937,28 +971,22 @@ __global__ void __launch_bounds__(BRICK_THREADS) k_reaction_am(const BoxDev *__r
 
 // K6b: acc = (first ? 0 : acc) + f_pf,am - sum_p W F_d; after the last subcycle
 // the applied f_pf is the subcycle average.
-template <typename FT>
-__global__ void __launch_bounds__(BRICK_THREADS) k_reaction_drag(const BoxDev *__restrict__ boxes,
+template <typename FT, bool SPARSE>
+__global__ void __launch_bounds__(BRICK_THREADS, brick_minb<FT, SPARSE>()) k_reaction_drag(const BoxDev *__restrict__ boxes,
                                                                  const Tile *__restrict__ tiles, int ntiles, int first,
                                                                  int last) {
     extern __shared__ __align__(16) unsigned char smem[];
-    BrickStage<FT, 3> &S = *(BrickStage<FT, 3> *)smem;
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
-        int ox, oy, oz, ex, ey, ez;
-        brick_unpack(tl.begin, ox, oy, oz);
-        brick_unpack(tl.end, ex, ey, ez);
-        __syncthreads();
         const long long N = B.g.ncell, cap = B.cap;
         const double *pf = B.pf[B.cur];
         const FT *w = weights_of<FT>(B, pf), *Fd = force_planes<FT>(B, pf, 1);
         auto force = [&](int p, int k) { return Fd[k * cap + p]; };
-        stage_brick<FT, 3>(B, ox, oy, oz, ex, ey, ez, w, S, force);
         const FT *fam = (const FT *)B.fam;
         FT *acc = (FT *)B.acc, *fpf = (FT *)B.fpf;
         const FT inv_nint = (FT)B.ph.dt_sub;
-        brick_gather<FT, 3>(B, S, ox, oy, oz, ex, ey, ez, w, force, [&](const FT *s, long long c) {
+        brick_gather<SPARSE, FT, 3>(B, smem, tl, w, force, [&](const FT *s, long long c) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const FT k = fam[a * N + c] - s[a];
@@ -1034,8 +1062,9 @@ static void launch_brick(K kernel, size_t smem, int nt, cudaStream_t s, Args... 
     kernel<<<nt, BRICK_THREADS, smem, s>>>(args...);
 }
 template <typename FT>
-void launch_eps(const BoxDev *b, const Tile *t, int nt, cudaStream_t s) {
-    launch_brick(k_eps_gather<FT>, sizeof(BrickStage<FT, 1>), nt, s, b, t, nt);
+void launch_eps(const BoxDev *b, const Tile *t, int nt, int sparse, cudaStream_t s) {
+    if (sparse) launch_brick(k_eps_gather<FT, true>, sizeof(BrickStage<FT, 1, true>), nt, s, b, t, nt);
+    else launch_brick(k_eps_gather<FT, false>, sizeof(BrickStage<FT, 1, false>), nt, s, b, t, nt);
 }
 template <typename FT>
 void launch_force_am(const BoxDev *b, const Tile *t, int nt, int grid, int block, cudaStream_t s) {
@@ -1046,20 +1075,24 @@ void launch_force_drag(const BoxDev *b, const Tile *t, int nt, int first, int gr
     k_force_drag<FT><<<grid, block, 0, s>>>(b, t, nt, first);
 }
 template <typename FT>
-void launch_reaction_am(const BoxDev *b, const Tile *t, int nt, int first, cudaStream_t s) {
-    launch_brick(k_reaction_am<FT>, sizeof(BrickStage<FT, 3>), nt, s, b, t, nt, first);
+void launch_reaction_am(const BoxDev *b, const Tile *t, int nt, int first, int sparse, cudaStream_t s) {
+    if (sparse) launch_brick(k_reaction_am<FT, true>, sizeof(BrickStage<FT, 3, true>), nt, s, b, t, nt, first);
+    else launch_brick(k_reaction_am<FT, false>, sizeof(BrickStage<FT, 3, false>), nt, s, b, t, nt, first);
 }
 template <typename FT>
-void launch_reaction_drag(const BoxDev *b, const Tile *t, int nt, int first, int last, cudaStream_t s) {
-    launch_brick(k_reaction_drag<FT>, sizeof(BrickStage<FT, 3>), nt, s, b, t, nt, first, last);
+void launch_reaction_drag(const BoxDev *b, const Tile *t, int nt, int first, int last, int sparse, cudaStream_t s) {
+    if (sparse) launch_brick(k_reaction_drag<FT, true>, sizeof(BrickStage<FT, 3, true>), nt, s, b, t, nt, first, last);
+    else launch_brick(k_reaction_drag<FT, false>, sizeof(BrickStage<FT, 3, false>), nt, s, b, t, nt, first, last);
 }
+// particles in a brick and its halo up to which the sparse stage is taken on average
+int sparse_stage_mean() { return SPARSE_CAP * 5 / 8; }
 
 #define DPS_CPL_INST(FT)                                                                                  \
-    template void launch_eps<FT>(const BoxDev *, const Tile *, int, cudaStream_t);                        \
+    template void launch_eps<FT>(const BoxDev *, const Tile *, int, int, cudaStream_t);                   \
     template void launch_force_am<FT>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);         \
     template void launch_force_drag<FT>(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);  \
-    template void launch_reaction_am<FT>(const BoxDev *, const Tile *, int, int, cudaStream_t);           \
-    template void launch_reaction_drag<FT>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+    template void launch_reaction_am<FT>(const BoxDev *, const Tile *, int, int, int, cudaStream_t);      \
+    template void launch_reaction_drag<FT>(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 DPS_CPL_INST(double)
 DPS_CPL_INST(float)
 

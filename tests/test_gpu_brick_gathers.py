@@ -23,6 +23,11 @@ CASES = {
     "fp32_stage_edge": ((16, 16, 16), (1, 1, 1), 2884, (0.5, 0.55)),  # ~704
     "over_the_stage": ((16, 8, 24), (1, 1, 1), 6000, (0.3, 0.35)),
     "half_empty": ((32, 16, 16), (1, 1, 1), 900, (0.7, 0.8)),
+    # dilute boxes (on average under 120 per brick and halo) with a dense
+    # corner: bricks over the small stage, in slabs and over the slabs' size
+    "dilute": ((24, 21, 18), (1, 1, 0), 700, (0.7, 1.1)),
+    "dilute_slabs": ((48, 47, 46), (1, 1, 1), 1500, (0.5, 0.6)),
+    "dilute_walk": ((48, 47, 46), (1, 1, 1), 3500, (0.4, 0.45)),
 }
 
 
@@ -39,6 +44,8 @@ def test_gathers_against_the_oracle(name, form, teps, tforce):
     L = np.array(n, float)
     if name == "half_empty":
         L[0] /= 2
+    if name.startswith("dilute_"):
+        L[:] = 16.0
     lo = np.where(per, 0.0, 0.6)
     x = lo + rng.random((count, 3)) * (L - 2 * lo)
     dia = rng.uniform(*d, count)
