@@ -378,6 +378,7 @@ static void compute_phys(BoxHost *h) {
     p.rho_f = h->rho_f;
     p.mu = h->rho_f * (h->tau - 0.5) / 3.0;  // Eq. visc_tau
     const double cells = (double)h->d.g.ncell;
+    for (int a = 0; a < 3; ++a) p.Lbits[a] = fx_bits((double)h->d.g.n[a]);
     for (int a = 0; a < 3; ++a) {
         p.g[a] = h->have_closure ? c.g[a] : 0.0;
         if (!h->have_closure)

@@ -507,6 +507,42 @@ __device__ __noinline__ void wall_exact(const BoxDev &Bx, long long i, int a, in
     if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], (unsigned long long)nlim);
 }
 
+// the rare branches of the update: a position off a periodic axis, the exact
+// displacement, the linked cell after the last substep
+__device__ __forceinline__ double fold_axis(double xn, int n) {
+    const double L = n;
+    if (xn >= L) xn -= L;
+    else if (xn < 0.0) xn += L;
+    if (xn >= L || xn < 0.0) xn -= L * floor(xn / L);
+    if (xn >= L) xn -= L;
+    return xn;
+}
+__device__ __forceinline__ void check_skin(const BoxDev &Bx, long long i, double x, double y, double z) {
+    const double *xs = Bx.pf[Bx.cur] + PXS0 * Bx.cap + i;
+    const double xn3[3] = {x, y, z};
+    double d2 = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double dd = min_image(xn3[a] - xs[a * Bx.cap], Bx.g.n[a], Bx.g.per[a]);
+        d2 += dd * dd;
+    }
+    if (d2 > Bx.ph.skin_half2) atomicOr(Bx.status, ST_SKIN);
+    if (!(d2 < 1e30)) atomicOr(Bx.status, ST_NAN);
+}
+__device__ __forceinline__ int new_cell(const BoxDev &Bx, double x, double y, double z) {
+    return (int)particle_cell(Bx.g, x, y, z, Bx.status);
+}
+// out of line in boxes without walls, where occupancy counts (a box with walls
+// calls the wall contact already): with FP64 comparisons and conversions gone
+// and 5 -> 7 blocks per SM the DEM of 101x90x77 at eps 0.36 took 6.5 -> 6.2 ms a
+// step, and the update of the mixed forms with 3 -> 4 blocks 11.7 -> 11.0 ms
+// (192^3, eps 0.38, FP32) and 9.7 -> 8.8 ms (32^3)
+__device__ __noinline__ double fold_axis_call(double xn, int n) { return fold_axis(xn, n); }
+__device__ __noinline__ void check_skin_call(const BoxDev &Bx, long long i, double x, double y, double z) {
+    check_skin(Bx, i, x, y, z);
+}
+__device__ __noinline__ int new_cell_call(const BoxDev &Bx, double x, double y, double z) { return new_cell(Bx, x, y, z); }
+
 // one thread per particle: wall partners (WALLS), then Eq. particle_motion
 // (semi-implicit Euler) and the outputs of the substep.  Comparisons and
 // conversions are integer or FP32 operations (an FP64 compare or conversion
@@ -577,7 +613,7 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
     // Eq. particle_motion, semi-implicit Euler with I = m d^2 / 10
     const double dt_m = ph.dt_dem * pf[PIM * cap + i];
     double xn3[3], un3[3], wn3[3] = {wi[0], wi[1], wi[2]};
-    if (T[0] != 0.0 || T[1] != 0.0 || T[2] != 0.0) {
+    if ((fx_bits(T[0]) | fx_bits(T[1]) | fx_bits(T[2])) << 1) {  // (either zero shifts out its sign)
         const double dt_I = ph.dt_dem * pf[PII * cap + i];
 #pragma unroll
         for (int a = 0; a < 3; ++a) wn3[a] = wi[a] + dt_I * T[a];
@@ -590,15 +626,9 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
         const double un = ui[a] + dt_m * Ft;
         double xn = xi[a] + ph.dt_dem * un;
         if (g.per[a]) {
-            const double L = g.n[a];
             // a particle that left the box folds back in; 0 <= xn < L compared
             // as integers (the order of the bits is that of the values)
-            if (!(fx_bits(xn) < fx_bits(L))) {
-                if (xn >= L) xn -= L;
-                else if (xn < 0.0) xn += L;
-                if (xn >= L || xn < 0.0) xn -= L * floor(xn / L);
-                if (xn >= L) xn -= L;
-            }
+            if (!(fx_bits(xn) < ph.Lbits[a])) xn = WALLS ? fold_axis(xn, g.n[a]) : fold_axis_call(xn, g.n[a]);
         }
         xn3[a] = xn;
         un3[a] = un;
@@ -626,22 +656,16 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
     if (key_out) {
         // last substep of the subcycle: the linked cell of the new position,
         // counted for the sort that follows (its counting pass)
-        const long long c = particle_cell(g, xn3[0], xn3[1], xn3[2], Bx.status);
-        Bx.key[i] = (int)c;
+        const int c = WALLS ? new_cell(Bx, xn3[0], xn3[1], xn3[2]) : new_cell_call(Bx, xn3[0], xn3[1], xn3[2]);
+        Bx.key[i] = c;
         atomicAdd(&Bx.count[c], 1);
     }
     // moved beyond skin/2 since the sort, or not finite: decided in FP32
     // where its rounding cannot matter, else in FP64
     if (!(d2f < ph.shell_near2)) Bx.moved[1 - src_tmp] = 1;
     if (!(d2f < ph.skin_near2)) {
-        double d2 = 0.0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const double dd = min_image(xn3[a] - pf[(PXS0 + a) * cap + i], g.n[a], g.per[a]);
-            d2 += dd * dd;
-        }
-        if (d2 > ph.skin_half2) atomicOr(Bx.status, ST_SKIN);
-        if (!(d2 < 1e30)) atomicOr(Bx.status, ST_NAN);
+        if (WALLS) check_skin(Bx, i, xn3[0], xn3[1], xn3[2]);
+        else check_skin_call(Bx, i, xn3[0], xn3[1], xn3[2]);
     }
 }
 
@@ -657,6 +681,9 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
 // per particle.  Two kernels so that each has its own register budget: the
 // pair loop waits on the partners' loads and needs every warp slot of the SM,
 // the FP64 update needs registers.
+#ifndef DPS_INTEG_MINB
+#define DPS_INTEG_MINB 4  // 128-thread blocks per SM the register budget of the update is sized for
+#endif
 #ifndef DPS_MIXED_MINB
 #define DPS_MIXED_MINB 4  // 256-thread blocks per SM the register budget of the pair loop is sized for
 #endif
@@ -779,7 +806,7 @@ __global__ void __launch_bounds__(256, DPS_MIXED_MINB) k_dem_pairsum_mixed(const
 
 // walls and Eq. particle_motion of the mixed forms, one thread per particle
 template <bool WALLS>
-__global__ void __launch_bounds__(128) k_dem_integrate(const BoxDev *__restrict__ boxes,
+__global__ void __launch_bounds__(128, DPS_INTEG_MINB) k_dem_integrate(const BoxDev *__restrict__ boxes,
                                                                      const Tile *__restrict__ tiles, int ntiles,
                                                                      int src_tmp, int key_out) {
     DPS_FOR_TILES(tiles, ntiles, t) {
@@ -1194,7 +1221,7 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
 #define DPS_GATHER_GC 4  // entries whose loads are issued before any is added
 #endif
 #ifndef DPS_GATHER_MINB
-#define DPS_GATHER_MINB 5  // 128-thread blocks per SM the register budget is sized for
+#define DPS_GATHER_MINB 7  // 128-thread blocks per SM the register budget is sized for
 #endif
 template <bool WALLS>
 __global__ void __launch_bounds__(128, WALLS ? 3 : DPS_GATHER_MINB) k_dem_gather64(const BoxDev *__restrict__ boxes,
@@ -1238,13 +1265,13 @@ __global__ void __launch_bounds__(128, WALLS ? 3 : DPS_GATHER_MINB) k_dem_gather
                 }
 #pragma unroll
                 for (int u = 0; u < GC; ++u) {
-                    // the owner's force, its opposite on the partner, or zero:
-                    // selected, not branched on, since each side of a branch
+                    // the owner's force or its opposite on the partner: the sign
+                    // is selected, not branched on, since each side of a branch
                     // would issue the three FP64 additions again
                     const u64 sg = c0 + u < nh ? 0ull : 0x8000000000000000ull;
-                    const u64 on = r[u].flag != 0 ? ~0ull : 0ull;
+                    if (r[u].flag)
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) F[a] += fx_double((fx_bits(r[u].F[a]) ^ sg) & on);
+                        for (int a = 0; a < 3; ++a) F[a] += fx_double(fx_bits(r[u].F[a]) ^ sg);
                     if (r[u].flag == 2) {  // rare: its n x F_t is added below
                         if (nc < TAN_CAP)
                             tan_slot[nc][threadIdx.x] = sl[u];

@@ -164,6 +164,7 @@ struct Phys {
     double skin;         // Verlet skin (dx)
     double kfac, xfac;   // k_n = m_ij kfac, xi_n = m_ij xfac (Eqs. damping_to_stiffness, collision_time)
     double capfac;       // lubrication cap = m_ij capfac
+    u64 Lbits[3];        // the box lengths as bits of a double
     double skin_half2;   // (skin / 2)^2: largest displacement between two sorts
     float skin_near2;    // squared FP32 displacement below which skin/2 is not exceeded whatever the rounding
     float dmax;          // largest diameter, rounded up
