@@ -46,7 +46,7 @@ void launch_bsort_rank(const BoxDev *, const Tile *, int, int, int, cudaStream_t
 void launch_bsort_gather(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
 void launch_bsort_flip(BoxDev *, int, int, cudaStream_t);
 void launch_end_step(BoxDev *, int, cudaStream_t);
-void launch_bscan(const BoxDev *, int, const Tile *, int, cudaStream_t);
+int launch_bscan(const BoxDev *, int, const Tile *, int, int, cudaStream_t);
 int scan_tile_cells();
 void brick_tiles(int, const int *, std::vector<Tile> &);
 template <typename FT>
@@ -156,6 +156,7 @@ struct Batch {
     bool any_lift = false;        // some box applies the lift force (curl launch per subcycle)
     bool any_walls = true;        // some box with particles has a wall axis (DEM wall code)
     int part_off[5] = {0, 0, 0, 0, 0};  // particle tiles grouped by DEM lanes class (1, 2, 4, 8)
+    int most_scan = 0;            // scan tiles of the largest box
     int sparse = 1;  // every box is dilute: brick gathers with the small stage
     int cpl_lanes = 1;            // most lanes per particle of the force kernels over the batch
     int n_cell_plain = 0;         // cell tiles of boxes with a constant tau (listed first);
@@ -587,6 +588,7 @@ static int push_layout(Batch *B) {
     B->any_walls = false;
     B->cpl_lanes = 1;
     B->sparse = 1;
+    B->most_scan = 0;
     for (int k = 0; k < nb; ++k) {
         BoxHost *h = B->boxes[k];
         compute_phys(h);
@@ -608,6 +610,7 @@ static int push_layout(Batch *B) {
             partc[lc].push_back(Tile{k, fl, p, std::min(np, p + B->tune.part_tile)});
         int idx = 0;
         for (long long c = 0; c < N; c += ST) scan.push_back(Tile{k, idx++, c, std::min(N, c + ST)});
+        B->most_scan = std::max(B->most_scan, idx);
         brick_tiles(k, h->d.g.n, brick);
     }
     B->n_cell_plain = (int)cell.size();
@@ -700,7 +703,7 @@ static void enqueue_sort_eps(Batch *B, int xsel, int mark_usub, bool have_keys) 
     const int cnt = pl && !have_keys;
     tbegin(B);
     if (cnt) launch_bsort_count(T, B->d_part, B->n_part, xsel, grid_of(B->n_part), u.part_block, B->stream);
-    launch_bscan(T, nb, B->d_scan, B->n_scan, B->stream);
+    const int nscan = launch_bscan(T, nb, B->d_scan, B->n_scan, B->most_scan, B->stream);
     if (pl) {
         launch_bsort_scatter(T, B->d_part, B->n_part, grid_of(B->n_part), u.part_block, B->stream);
         launch_bsort_rank(T, B->d_part, B->n_part, grid_of(B->n_part), u.part_block, B->stream);
@@ -713,7 +716,7 @@ static void enqueue_sort_eps(Batch *B, int xsel, int mark_usub, bool have_keys) 
     if (pl)
         launch_build_nlist(T, B->d_part, B->n_part, grid_of(B->n_part), part_threads(u, B->cpl_lanes), rows,
                            B->stream);
-    tend(B, PH_SORT, cnt + 3 + 3 * pl + 1 + pl * (1 + (rows == 1 ? 2 : rows == 2)));
+    tend(B, PH_SORT, cnt + nscan + 3 * pl + 1 + pl * (1 + (rows == 1 ? 2 : rows == 2)));
     tbegin(B);
     if (B->fel == 8)
         launch_eps<double>(T, B->d_brick, B->n_brick, B->sparse, B->stream);
@@ -1066,7 +1069,7 @@ static size_t box_bytes(int prec, long long ncell, long long cap) {
     if (prec == DPS_F16S) b += 64 * C * 4 + C * 4;  // inner rows
     if (prec == DPS_F64) b += 64 * C * 4 + 32 * C * (4 + sizeof(PairRes) + 24 + 1);  // pair lists and results (64 partners)
     if (prec == DPS_F64) b += 2 * C * (sizeof(DemRec) + sizeof(DemPart));
-    b += (3 * N + 1) * 4 + 3 * C * 4 + ((N + 8191) / 8192 + 1) * 4;
+    b += (2 * N + 1) * 4 + 3 * C * 4 + (N / scan_tile_cells() + 2) * 4;
     b += 4096 + (size_t)reduce_partials_doubles() * 8;
     return b;
 }
@@ -1150,11 +1153,10 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
     d.ptop = (unsigned long long *)A(16);
     d.cell_start = (int *)A((N + 1) * 4);
     d.count = (int *)A(N * 4);
-    d.fill = (int *)A(N * 4);
     d.key = (int *)A(cap * 4);
     d.tmp = (int *)A(cap * 4);
     d.perm = (int *)A(cap * 4);
-    d.scan_part = (int *)A(((N + 8191) / 8192 + 1) * 4);
+    d.scan_part = (int *)A((N / scan_tile_cells() + 2) * 4);
     d.status = (int *)A(64);
     d.counters = (unsigned long long *)A(8 * CNT_N);
     h->d_red = (double *)A((size_t)reduce_partials_doubles() * 8);
@@ -1192,7 +1194,6 @@ static int box_create(Batch *B, const int n[3], const int per[3], double tau, do
     }
     cudaMemsetAsync(d.cell_start, 0, (N + 1) * 4, s);
     cudaMemsetAsync(d.count, 0, N * 4, s);
-    cudaMemsetAsync(d.fill, 0, N * 4, s);
     cudaMemsetAsync(d.status, 0, 64, s);
     cudaMemsetAsync(d.counters, 0, 8 * CNT_N, s);
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {

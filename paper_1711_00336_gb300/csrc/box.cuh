@@ -81,7 +81,7 @@ struct BoxDev {
     float *f32p;       // FP32 copies of F_am (3 planes) and F_d (3 planes) [6][cap]
     double *psum;      // mixed-form DEM: pair sums of a substep, force and torque [6][cap]
     // linked cells
-    int *cell_start, *count, *fill, *key, *tmp, *perm;
+    int *cell_start, *count, *key, *tmp, *perm;
     int *scan_part;    // per scan tile partial sums of this box
     // status
     int *status;

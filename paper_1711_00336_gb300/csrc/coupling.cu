@@ -180,13 +180,14 @@ __global__ void k_bsort_count(const BoxDev *__restrict__ boxes, const Tile *__re
     }
 }
 
+// counts the cells back down: they are zero again for the next sort
 __global__ void k_bsort_scatter(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles, int ntiles) {
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
         for (long long i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
             int k = B.key[i];
-            B.tmp[B.cell_start[k] + atomicAdd(&B.fill[k], 1)] = (int)i;
+            B.tmp[B.cell_start[k] + atomicSub(&B.count[k], 1) - 1] = (int)i;
         }
     }
 }
@@ -584,8 +585,7 @@ __device__ __forceinline__ void brick_gather(const BoxDev &B, unsigned char *sme
 
 // ---- S2: eps_f ------------------------------------------------------------------
 // FT is the compute type of the form: FP64 for the plain method, FP32 (with
-// FP32 kernel weights) for the low-precision forms.  Also clears the sort
-// counts for the next sort (every cell is visited once).
+// FP32 kernel weights) for the low-precision forms.
 template <typename FT, bool SPARSE>
 __global__ void __launch_bounds__(BRICK_THREADS, brick_minb<FT, SPARSE>()) k_eps_gather(const BoxDev *__restrict__ boxes,
                                                               const Tile *__restrict__ tiles, int ntiles) {
@@ -613,7 +613,6 @@ __global__ void __launch_bounds__(BRICK_THREADS, brick_minb<FT, SPARSE>()) k_eps
                 e = eps_min;
             }
             eps[c] = e;
-            B.count[c] = 0;
         });
         if (nclamp) atomicAdd(&B.counters[CNT_EPS_CLAMP], (unsigned long long)nclamp);
     }
