@@ -29,7 +29,7 @@ void launch_collide_stream(const BoxDev *, const Tile *, int, int, int, bool, bo
 template <typename ST, typename FT, typename CT>
 void launch_moments(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 void launch_fields64(const BoxDev *, const Tile *, int, cudaStream_t);
-void launch_fields32(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+void launch_fields32(const BoxDev *, const Tile *, int, cudaStream_t);
 void launch_curl64(const BoxDev *, const Tile *, int, cudaStream_t);
 void launch_curl32(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
 template <typename ST>
@@ -743,7 +743,7 @@ static void enqueue_step(Batch *B) {
     if (f64)
         launch_fields64(T, B->d_brick, B->n_brick, s);
     else
-        launch_fields32(T, B->d_cell, B->n_cell, gc, u.cell_block, s);
+        launch_fields32(T, B->d_brick, B->n_brick, s);
     tend(B, PH_MOM, 2);
     const int nl = pl && B->any_lift;
     for (int k = 0; k < B->n_int; ++k) {

@@ -510,58 +510,80 @@ __global__ void __launch_bounds__(128, sizeof(CT) == 8 ? DPS_MOM_MINB : 4) k_mom
 // K2b: grad P with P = eps_f p = c_s^2 rho, and Du_f/Dt = (u_D - u_prev) +
 // (u_D . grad) u_D, with the lattice gradient of Sec. 3.2.3.  Neighbours
 // beyond a wall are mirrored into the box (coordinate clamped).
-template <typename FT, typename CT>
-__global__ void __launch_bounds__(256) k_fields(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles,
-                                                int ntiles) {
+#ifndef DPS_FIELDS32_MINB
+#define DPS_FIELDS32_MINB 8  // 256-thread blocks per SM the register budget is sized for
+#endif
+constexpr int FB = 8, FH = FB + 2, FH3 = FH * FH * FH;
+
+// coordinate of the cell at i on axis a, wrapped or mirrored
+__device__ __forceinline__ int near_cell(const Geom &g, int a, int i) {
+    if (i < 0) return g.per[a] ? g.n[a] - 1 : 0;
+    if (i >= g.n[a]) return g.per[a] ? 0 : g.n[a] - 1;
+    return i;
+}
+
+// The FP32 forms over bricks of 8^3 cells: rho and u_D of the brick and its
+// halo are staged in shared memory as one float4 a cell, so a neighbour is one
+// 16-byte load off a constant offset and not four words of global memory with
+// a 64-bit address: K2a and K2b together 1.53 -> 1.07 ms (256^3, FP16 storage),
+// 0.66 -> 0.44 ms (192^3, FP32).  Each sum keeps the order of q.
+__global__ void __launch_bounds__(256, DPS_FIELDS32_MINB) k_fields32(const BoxDev *__restrict__ boxes,
+                                                                      const Tile *__restrict__ tiles, int ntiles) {
+    __shared__ float4 S[FH3];
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &B = boxes[tl.box];
         const Geom g = B.g;
         const long long N = g.ncell;
-        const FT *rho = (const FT *)B.rho, *uD = (const FT *)B.uD;
-        FT *uprev = (FT *)B.uprev, *gradP = (FT *)B.gradP, *DuDt = (FT *)B.DuDt;
+        int ox, oy, oz, ex, ey, ez;
+        brick_unpack(tl.begin, ox, oy, oz);
+        brick_unpack(tl.end, ex, ey, ez);
+        const float *rho = (const float *)B.rho, *uD = (const float *)B.uD;
+        float *uprev = (float *)B.uprev, *gradP = (float *)B.gradP, *DuDt = (float *)B.DuDt;
         const int have_prev = B.have_uprev;
-        for (long long c = tl.begin + threadIdx.x; c < tl.end; c += blockDim.x) {
-            int ix, iy, iz;
-            cell_coords(g, c, ix, iy, iz);
-            long long stride[3] = {1, g.n[0], (long long)g.n[0] * g.n[1]};
-            const int ii[3] = {ix, iy, iz};
-            long long dd[3][3];
+        __syncthreads();  // the previous brick is done with S
+        for (int h = threadIdx.x; h < FH3; h += 256) {
+            const int hx = h % FH, hy = (h / FH) % FH, hz = h / (FH * FH);
+            if (hx > ex + 1 || hy > ey + 1 || hz > ez + 1) continue;
+            const long long n = cell_index(g, near_cell(g, 0, ox + hx - 1), near_cell(g, 1, oy + hy - 1),
+                                           near_cell(g, 2, oz + hz - 1));
+            S[h] = make_float4(rho[n], uD[n], uD[N + n], uD[2 * N + n]);
+        }
+        __syncthreads();
+        const int nb = ex * ey * ez;
+        for (int k = threadIdx.x; k < nb; k += 256) {
+            const int lx = k % ex, ly = (k / ex) % ey, lz = k / (ex * ey);
+            const long long c = cell_index(g, ox + lx, oy + ly, oz + lz);
+            const int p = ((lz + 1) * FH + ly + 1) * FH + lx + 1;
+            const float4 s = S[p];
+            const float u[3] = {s.y, s.z, s.w};
+            float up[3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                int L = g.n[a];
-                dd[a][1] = 0;
-                dd[a][0] = ii[a] > 0 ? -stride[a] : (g.per[a] ? (long long)(L - 1) * stride[a] : 0);
-                dd[a][2] = ii[a] < L - 1 ? stride[a] : (g.per[a] ? -(long long)(L - 1) * stride[a] : 0);
-            }
-            CT gp[3] = {0, 0, 0};
-            CT gu[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};  // gu[a][b] = sum w c_a u_b
+            for (int b = 0; b < 3; ++b) up[b] = have_prev ? uprev[b * N + c] : u[b];
+            float gp[3] = {0, 0, 0};
+            float gu[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};  // gu[a][b] = sum w c_a u_b
 #pragma unroll
             for (int q = 1; q < Q; ++q) {
-                const long long n = c + dd[0][CX(q) + 1] + dd[1][CY(q) + 1] + dd[2][CZ(q) + 1];
-                const CT w = (CT)WQ(q);
-                const CT r = (CT)rho[n];
-                const CT u0 = (CT)uD[n], u1 = (CT)uD[N + n], u2 = (CT)uD[2 * N + n];
+                const float4 v = S[p + (CZ(q) * FH + CY(q)) * FH + CX(q)];
+                const float w = (float)WQ(q);
                 const int cc[3] = {CX(q), CY(q), CZ(q)};
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     if (cc[a] == 0) continue;
-                    const CT wc = w * (CT)cc[a];
-                    gp[a] += wc * r;
-                    gu[a][0] += wc * u0;
-                    gu[a][1] += wc * u1;
-                    gu[a][2] += wc * u2;
+                    const float wc = w * (float)cc[a];
+                    gp[a] += wc * v.x;
+                    gu[a][0] += wc * v.y;
+                    gu[a][1] += wc * v.z;
+                    gu[a][2] += wc * v.w;
                 }
             }
             // c_s^-2 sum w c phi; for P = c_s^2 rho the c_s^2 cancels
-            const CT u[3] = {(CT)uD[c], (CT)uD[N + c], (CT)uD[2 * N + c]};
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
-                gradP[b * N + c] = (FT)gp[b];
-                const CT conv = CT(3) * (u[0] * gu[0][b] + u[1] * gu[1][b] + u[2] * gu[2][b]);
-                const CT up = have_prev ? (CT)uprev[b * N + c] : u[b];
-                DuDt[b * N + c] = (FT)((u[b] - up) + conv);
-                uprev[b * N + c] = (FT)u[b];
+                gradP[b * N + c] = gp[b];
+                const float conv = 3.0f * (u[0] * gu[0][b] + u[1] * gu[1][b] + u[2] * gu[2][b]);
+                DuDt[b * N + c] = (u[b] - up[b]) + conv;
+                uprev[b * N + c] = u[b];
             }
         }
     }
@@ -574,7 +596,6 @@ __global__ void __launch_bounds__(256) k_fields(const BoxDev *__restrict__ boxes
 // instructions a cell are left of 135, which bound this kernel.  A block with a
 // non-finite value takes FP64 throughout.  K2a and K2b together at 256^3: 6.34
 // -> 2.12 ms; at 64^3: 115 -> 46 us.
-constexpr int FB = 8, FH = FB + 2, FH3 = FH * FH * FH;
 
 __device__ __forceinline__ void fields_cell64(const double *__restrict__ rho, const double *__restrict__ uD,
                                               const Geom &g, int ix, int iy, int iz, double gp[3], double cv[3]) {
@@ -638,13 +659,8 @@ __global__ void __launch_bounds__(256) k_fields64(const BoxDev *__restrict__ box
             const int hx = h % FH, hy = (h / FH) % FH, hz = h / (FH * FH);
             u64 v[4] = {0, 0, 0, 0};
             if (hx <= ex + 1 && hy <= ey + 1 && hz <= ez + 1) {
-                int p[3] = {ox + hx - 1, oy + hy - 1, oz + hz - 1};
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    if (p[a] < 0) p[a] = g.per[a] ? g.n[a] - 1 : 0;
-                    else if (p[a] >= g.n[a]) p[a] = g.per[a] ? 0 : g.n[a] - 1;
-                }
-                const long long n = cell_index(g, p[0], p[1], p[2]);
+                const long long n = cell_index(g, near_cell(g, 0, ox + hx - 1), near_cell(g, 1, oy + hy - 1),
+                                               near_cell(g, 2, oz + hz - 1));
                 v[0] = fx_bits(rho[n]);
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
@@ -971,8 +987,8 @@ void launch_moments(const BoxDev *boxes, const Tile *tiles, int ntiles, int pari
 void launch_fields64(const BoxDev *boxes, const Tile *bricks, int nbricks, cudaStream_t s) {
     k_fields64<<<nbricks, 256, 0, s>>>(boxes, bricks, nbricks);
 }
-void launch_fields32(const BoxDev *boxes, const Tile *tiles, int ntiles, int grid, int block, cudaStream_t s) {
-    k_fields<float, float><<<grid, block, 0, s>>>(boxes, tiles, ntiles);
+void launch_fields32(const BoxDev *boxes, const Tile *bricks, int nbricks, cudaStream_t s) {
+    k_fields32<<<nbricks, 256, 0, s>>>(boxes, bricks, nbricks);
 }
 
 void launch_curl64(const BoxDev *boxes, const Tile *bricks, int nbricks, cudaStream_t s) {
