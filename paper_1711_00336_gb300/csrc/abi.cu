@@ -61,6 +61,8 @@ template <typename FT>
 void launch_reaction_drag(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 int sparse_stage_mean();
 void launch_dem_substep(const BoxDev *, const Tile *, int, int, int, int, int, int, int, cudaStream_t);
+void launch_dem_solo64(const BoxDev *, const Tile *, int, int, int, cudaStream_t);
+void launch_dem_mixed8(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
 void launch_dem_substep64(const BoxDev *, const Tile *, int, int, int, int, int, cudaStream_t);
 void launch_build_nlist(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 long long scan_scratch_words(long long);
@@ -156,6 +158,7 @@ struct Batch {
     bool any_lift = false;        // some box applies the lift force (curl launch per subcycle)
     bool any_walls = true;        // some box with particles has a wall axis (DEM wall code)
     int part_off[5] = {0, 0, 0, 0, 0};  // particle tiles grouped by DEM lanes class (1, 2, 4, 8)
+    int solo = 0;                 // the particles of every box are one tile
     int most_scan = 0;            // scan tiles of the largest box
     int sparse = 1;  // every box is dilute: brick gathers with the small stage
     int cpl_lanes = 1;            // most lanes per particle of the force kernels over the batch
@@ -588,6 +591,7 @@ static int push_layout(Batch *B) {
     B->any_walls = false;
     B->cpl_lanes = 1;
     B->sparse = 1;
+    B->solo = 1;
     B->most_scan = 0;
     for (int k = 0; k < nb; ++k) {
         BoxHost *h = B->boxes[k];
@@ -602,6 +606,7 @@ static int push_layout(Batch *B) {
         h->d.ufield = B->prec == DPS_F64 && 27 * h->d.np >= 2 * h->d.g.ncell;
         tab[k] = h->d;
         const long long N = h->d.g.ncell, np = h->d.np;
+        B->solo &= np <= std::min(128, B->tune.part_tile);
         B->sparse &= 1000 * np <= sparse_stage_mean() * N;
         for (long long c = 0; c < N; c += B->tune.cell_tile)
             ct.push_back(Tile{k, 0, c, std::min(N, c + B->tune.cell_tile)});
@@ -641,6 +646,7 @@ static int push_layout(Batch *B) {
     B->n_brick = (int)brick.size();
     B->dev_order = B->boxes;
     B->layout_dirty = false;
+    B->launches_step = 0;
     invalidate_graph(B);
     return DPS_OK;
 }
@@ -787,7 +793,10 @@ static void enqueue_step(Batch *B) {
         if (fork) cudaEventRecord(B->ev_join, B->side);
         tbegin(B);
         int ndl = 0;
-        if (pl)
+        if (pl && f64 && B->solo && B->n_part <= 4 * 152) {
+            launch_dem_solo64(T, B->d_part, B->n_part, B->n_dem, B->any_walls, s);
+            ndl = 1;
+        } else if (pl)
             for (int sd = 0; sd < B->n_dem; ++sd) {
                 const int key_out = sd == B->n_dem - 1;
                 if (B->prec == DPS_F64) {
@@ -804,6 +813,13 @@ static void enqueue_step(Batch *B) {
                         ++classes;
                     }
                 if (classes > 1) lanes = 0;
+                if (lanes == 8 && u.part_tile <= 32) {
+                    const int n = B->solo ? B->n_dem : 1;
+                    launch_dem_mixed8(T, B->d_part, B->n_part, sd, n, B->n_dem, B->any_walls, s);
+                    sd += n - 1;
+                    ++ndl;
+                    continue;
+                }
                 // a block holds all lane groups of a particle tile, at most
                 // 256 threads (four such blocks fit an SM)
                 const int blk = (int)std::min<long long>(
@@ -1936,13 +1952,14 @@ static void b_get_timing(Batch *B, double *ms, int64_t *nl, int reset) {
     }
 }
 static long long b_launches_per_step(Batch *B) {
+    if (B->launches_step > 0) return B->launches_step;  // counted as the step was recorded
     long long np = 0;
     for (BoxHost *h : B->boxes) np += h->d.np;
     const int pl = np > 0;
     const int n_int = B->boxes.empty() ? 1 : B->boxes[0]->cl.n_int;
     const int n_dem = B->boxes.empty() ? 1 : B->boxes[0]->cl.n_dem;
     const int f64 = B->prec == DPS_F64;
-    return 2 + 2 + (long long)n_int * (2 * pl + 2 + pl * n_dem * 2 + 3 + (5 + 2 * f64) * pl + 1 + 1);
+    return 2 + 2 + (long long)n_int * (2 * pl + 2 + pl * n_dem * 2 + 2 + (5 + 2 * f64) * pl + 1 + 1);
 }
 
 int dps_set_timing(dps_handle h, int enable) { return h ? b_set_timing(&h->B, enable) : DPS_ERR_ARG; }

@@ -56,7 +56,8 @@ struct BoxDev {
     int *ilist;        // one-row form: the inner partners, ilist[i*maxi + k], dem_lanes columns, gaps -1
     int *ilist_n;
     int maxi, dem_lanes;
-    int *moved;        // [2], by source buffer of a substep: some particle has moved more than shell/2
+    int *moved;        // [3], by source buffer of a substep (k_dem_mixed8: by substep mod 3): some particle has
+                       // moved more than shell/2
     int maxn;          // list capacity per particle
     // FP64 form: the list as unordered pairs, each evaluated once per
     // substep (Newton's third law).  Particle i owns the pairs with its

@@ -315,7 +315,7 @@ __global__ void k_bsort_flip(BoxDev *boxes, int nboxes, int mark_usub) {
         boxes[b].cur ^= 1;
         if (mark_usub) boxes[b].have_usub = 1;
         *boxes[b].ptop = 0;  // pair slots of the list built next
-        boxes[b].moved[0] = boxes[b].moved[1] = 0;
+        boxes[b].moved[0] = boxes[b].moved[1] = boxes[b].moved[2] = 0;
     }
 }
 

@@ -551,7 +551,7 @@ __device__ __noinline__ int new_cell_call(const BoxDev &Bx, double x, double y, 
 // ~55 were issued before.
 template <bool WALLS, bool F64>
 __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, int src_tmp, double F[3], double T[3],
-                                               int key_out) {
+                                               int key_out, int *moved_out) {
     const double *xin = src_tmp ? Bx.xtmp : Bx.pf[Bx.cur];
     double *xout = src_tmp ? Bx.pf[Bx.cur] : Bx.xtmp;
     const double *pf = Bx.pf[Bx.cur];
@@ -662,7 +662,7 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
     }
     // moved beyond skin/2 since the sort, or not finite: decided in FP32
     // where its rounding cannot matter, else in FP64
-    if (!(d2f < ph.shell_near2)) Bx.moved[1 - src_tmp] = 1;
+    if (!(d2f < ph.shell_near2)) *moved_out = 1;
     if (!(d2f < ph.skin_near2)) {
         if (WALLS) check_skin(Bx, i, xn3[0], xn3[1], xn3[2]);
         else check_skin_call(Bx, i, xn3[0], xn3[1], xn3[2]);
@@ -687,8 +687,8 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
 #ifndef DPS_MIXED_MINB
 #define DPS_MIXED_MINB 4  // 256-thread blocks per SM the register budget of the pair loop is sized for
 #endif
-template <int LANES>
-__device__ __forceinline__ void pairsum_tile(const BoxDev &Bx, const Tile &tl, int src_tmp) {
+template <int LANES, typename Sink>
+__device__ __forceinline__ void pairsum_tile(const BoxDev &Bx, const Tile &tl, int src_tmp, int outer, Sink &&sink) {
     const int lane = threadIdx.x % LANES, grp = threadIdx.x / LANES, ngrp = blockDim.x / LANES;
     {
         const double *xin = src_tmp ? Bx.xtmp : Bx.pf[Bx.cur];
@@ -699,11 +699,6 @@ __device__ __forceinline__ void pairsum_tile(const BoxDev &Bx, const Tile &tl, i
         const float Lf[3] = {(float)g.n[0], (float)g.n[1], (float)g.n[2]};
         const PairPar<float> pfl = pair_par<float>(ph);
         const long long cap = Bx.cap;
-        // outer partners only once a particle of the box has moved shell/2
-        const int outer = Bx.moved[src_tmp];
-        // cleared for this substep's update to set, by one thread of the box: a
-        // store from every block to the word all blocks read costs 20 us a launch
-        if (tl.begin == 0 && threadIdx.x == 0) Bx.moved[1 - src_tmp] = 0;
         // the trip count is uniform over the block, so every lane reaches the shuffles
         for (long long base = tl.begin; base < tl.end; base += ngrp) {
             const long long i = base + grp;
@@ -770,11 +765,7 @@ __device__ __forceinline__ void pairsum_tile(const BoxDev &Bx, const Tile &tl, i
                 }
             }
             if (act && lane == 0) {
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    Bx.psum[a * cap + i] = (double)Ff[a];
-                    Bx.psum[(3 + a) * cap + i] = (double)Tf[a];
-                }
+                sink(i, Ff, Tf);
                 if (nlim) atomicAdd(&Bx.counters[CNT_LUB_LIMITED], (unsigned long long)nlim);
             }
         }
@@ -791,16 +782,77 @@ __global__ void __launch_bounds__(256, DPS_MIXED_MINB) k_dem_pairsum_mixed(const
     DPS_FOR_TILES(tiles, ntiles, t) {
         const Tile tl = tiles[t];
         const BoxDev &Bx = boxes[tl.box];
+        const long long cap = Bx.cap;
+        auto store = [&](long long i, const float Ff[3], const float Tf[3]) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                Bx.psum[a * cap + i] = (double)Ff[a];
+                Bx.psum[(3 + a) * cap + i] = (double)Tf[a];
+            }
+        };
+        // outer partners only once a particle of the box has moved shell/2
+        const int outer = Bx.moved[src_tmp];
+        // cleared for this substep's update to set, by one thread of the box: a
+        // store from every block to the word all blocks read costs 20 us a launch
+        if (tl.begin == 0 && threadIdx.x == 0) Bx.moved[1 - src_tmp] = 0;
         if (LANES > 0) {
-            pairsum_tile<LANES ? LANES : 1>(Bx, tl, src_tmp);
+            pairsum_tile<LANES ? LANES : 1>(Bx, tl, src_tmp, outer, store);
         } else {
             switch (Bx.dem_lanes) {
-                case 8: pairsum_tile<8>(Bx, tl, src_tmp); break;
-                case 4: pairsum_tile<4>(Bx, tl, src_tmp); break;
-                case 2: pairsum_tile<2>(Bx, tl, src_tmp); break;
-                default: pairsum_tile<1>(Bx, tl, src_tmp);
+                case 8: pairsum_tile<8>(Bx, tl, src_tmp, outer, store); break;
+                case 4: pairsum_tile<4>(Bx, tl, src_tmp, outer, store); break;
+                case 2: pairsum_tile<2>(Bx, tl, src_tmp, outer, store); break;
+                default: pairsum_tile<1>(Bx, tl, src_tmp, outer, store);
             }
         }
+    }
+}
+
+// Few particles (tiles of at most 32, 8 lanes each, which fill the chip once): a
+// block sums the pairs of its tile, passes the sums through shared memory, and
+// its first warp updates the 32 particles: one launch a substep, and no trip of
+// the sums through global memory (18.8k spheres in 32^3: 17.6 -> 16.5 us a
+// substep).  The blocks of a substep read slot sd
+// mod 3 of Bx.moved, set the next and clear the one after it, which the
+// substep before this one read: no slot is read and written in one launch.
+// A tile that is its whole box (solo) takes all n substeps from sd in one
+// launch.
+#ifndef DPS_MIXED8_MINB
+#define DPS_MIXED8_MINB 4  // one wave of the largest count (3 blocks: 16.5 -> 19 us)
+#endif
+template <bool WALLS>
+__global__ void __launch_bounds__(256, DPS_MIXED8_MINB) k_dem_mixed8(const BoxDev *__restrict__ boxes,
+                                                                     const Tile *__restrict__ tiles, int sd, int n,
+                                                                     int n_dem) {
+    __shared__ float sums[6][32];
+    const Tile tl = tiles[blockIdx.x];
+    const BoxDev &Bx = boxes[tl.box];
+    auto store = [&](long long i, const float Ff[3], const float Tf[3]) {
+        const int k = (int)(i - tl.begin);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            sums[a][k] = Ff[a];
+            sums[3 + a][k] = Tf[a];
+        }
+    };
+#pragma unroll 1
+    for (int q = 0; q < n; ++q, ++sd) {
+        const int src_tmp = sd & 1, slot = sd % 3;
+        const int outer = Bx.moved[slot];
+        if (tl.begin == 0 && threadIdx.x == 0) Bx.moved[slot == 0 ? 2 : slot - 1] = 0;
+        pairsum_tile<8>(Bx, tl, src_tmp, outer, store);
+        __syncthreads();
+        const long long i = tl.begin + threadIdx.x;
+        if (threadIdx.x < 32 && i < tl.end) {
+            double F[3], T[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                F[a] = (double)sums[a][threadIdx.x];
+                T[a] = (double)sums[3 + a][threadIdx.x];
+            }
+            finish_particle<WALLS, false>(Bx, i, src_tmp, F, T, sd == n_dem - 1, Bx.moved + (slot == 2 ? 0 : slot + 1));
+        }
+        if (q + 1 < n) __syncthreads();
     }
 }
 
@@ -820,7 +872,7 @@ __global__ void __launch_bounds__(128, DPS_INTEG_MINB) k_dem_integrate(const Box
                 F[a] = Bx.psum[a * cap + i];
                 T[a] = Bx.psum[(3 + a) * cap + i];
             }
-            finish_particle<WALLS, false>(Bx, i, src_tmp, F, T, key_out);
+            finish_particle<WALLS, false>(Bx, i, src_tmp, F, T, key_out, Bx.moved + 1 - src_tmp);
         }
     }
 }
@@ -1050,15 +1102,10 @@ __device__ __forceinline__ double fx_recip(double x, float xf) {
 #ifndef DPS_PAIRS_MINB
 #define DPS_PAIRS_MINB 7  // 128-thread blocks per SM the register budget is sized for
 #endif
-__global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
-    k_dem_pairs64(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles, int ntiles, int src_tmp) {
-    __shared__ PairQueue Qs;
+// the pairs of one tile (Qs.en is 0 before and after; ends with a barrier)
+__device__ __forceinline__ void pairs64_tile(const BoxDev &Bx, const Tile &tl, int src_tmp, PairQueue &Qs) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (threadIdx.x == 0) Qs.en = 0;
-    __syncthreads();
-    DPS_FOR_TILES(tiles, ntiles, t) {
-        const Tile tl = tiles[t];
-        const BoxDev &Bx = boxes[tl.box];
+    {
         const double *xin = src_tmp ? Bx.xtmp : Bx.pf[Bx.cur];
         const float4 *fin = Bx.xf[src_tmp];
         const DemRec *rec = Bx.rec[src_tmp];
@@ -1207,6 +1254,17 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
     }
 }
 
+__global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
+    k_dem_pairs64(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles, int ntiles, int src_tmp) {
+    __shared__ PairQueue Qs;
+    if (threadIdx.x == 0) Qs.en = 0;
+    __syncthreads();
+    DPS_FOR_TILES(tiles, ntiles, t) {
+        const Tile tl = tiles[t];
+        pairs64_tile(boxes[tl.box], tl, src_tmp, Qs);
+    }
+}
+
 // The sums of a substep and the update: one thread per particle adds the
 // forces of its owned pairs (ascending partner), minus those of the pairs its
 // lower partners own (ascending owner), each pair's n x F_t times d_i/2, then
@@ -1223,19 +1281,15 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
 #ifndef DPS_GATHER_MINB
 #define DPS_GATHER_MINB 7  // 128-thread blocks per SM the register budget is sized for
 #endif
+// slots of a particle's pairs in contact with friction: listed while the forces
+// are summed, so that a warp pays for the most contacts of a particle and not
+// for every entry at which one of its lanes has one
+constexpr int TAN_CAP = 8;
 template <bool WALLS>
-__global__ void __launch_bounds__(128, WALLS ? 3 : DPS_GATHER_MINB) k_dem_gather64(const BoxDev *__restrict__ boxes,
-                                                        const Tile *__restrict__ tiles, int ntiles, int src_tmp,
-                                                        int key_out) {
-    // slots of a particle's pairs in contact with friction: listed while the
-    // forces are summed, so that a warp pays for the most contacts of a
-    // particle and not for every entry at which one of its lanes has one
-    constexpr int TAN_CAP = 8;
-    __shared__ int tan_slot[TAN_CAP][128];
-    DPS_FOR_TILES(tiles, ntiles, t) {
-        const Tile tl = tiles[t];
-        const BoxDev &Bx = boxes[tl.box];
-        const PairRes *__restrict__ pres = Bx.pres;
+__device__ __forceinline__ void gather64_tile(const BoxDev &Bx, const Tile &tl, int src_tmp, int key_out,
+                                              int (*tan_slot)[128]) {
+    {
+        const PairRes *pres = Bx.pres;
         const int parts = Bx.moved[src_tmp] ? 2 : 1;
         for (long long i = tl.begin + threadIdx.x; i < tl.end; i += blockDim.x) {
             double F[3] = {0, 0, 0}, T[3] = {0, 0, 0}, T2[3] = {0, 0, 0};
@@ -1293,8 +1347,40 @@ __global__ void __launch_bounds__(128, WALLS ? 3 : DPS_GATHER_MINB) k_dem_gather
 #pragma unroll
                 for (int a = 0; a < 3; ++a) T[a] = (T[a] + T2[a]) * lev;
             }
-            finish_particle<WALLS, true>(Bx, i, src_tmp, F, T, key_out);
+            finish_particle<WALLS, true>(Bx, i, src_tmp, F, T, key_out, Bx.moved + 1 - src_tmp);
         }
+    }
+}
+
+template <bool WALLS>
+__global__ void __launch_bounds__(128, WALLS ? 3 : DPS_GATHER_MINB) k_dem_gather64(const BoxDev *__restrict__ boxes,
+                                                        const Tile *__restrict__ tiles, int ntiles, int src_tmp,
+                                                        int key_out) {
+    __shared__ int tan_slot[TAN_CAP][128];
+    DPS_FOR_TILES(tiles, ntiles, t) {
+        const Tile tl = tiles[t];
+        gather64_tile<WALLS>(boxes[tl.box], tl, src_tmp, key_out, tan_slot);
+    }
+}
+
+// Boxes of one tile each (up to 128 particles; one sphere settling, a pair
+// colliding): a block runs all substeps of its box, a barrier where the general
+// path has a launch.  One sphere at 32 x 32 x 64: 8.1 -> 4.9 us a substep.
+template <bool WALLS>
+__global__ void __launch_bounds__(128) k_dem_solo64(const BoxDev *__restrict__ boxes, const Tile *__restrict__ tiles,
+                                                    int n_dem) {
+    __shared__ PairQueue Qs;
+    __shared__ int tan_slot[TAN_CAP][128];
+    const Tile tl = tiles[blockIdx.x];
+    const BoxDev &Bx = boxes[tl.box];
+    if (threadIdx.x == 0) Qs.en = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int sd = 0; sd < n_dem; ++sd) {
+        pairs64_tile(Bx, tl, sd & 1, Qs);
+        __syncthreads();
+        gather64_tile<WALLS>(Bx, tl, sd & 1, sd == n_dem - 1, tan_slot);
+        __syncthreads();
     }
 }
 
@@ -1342,6 +1428,20 @@ void launch_dem_substep64(const BoxDev *boxes, const Tile *tiles, int ntiles, in
         k_dem_gather64<true><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
     else
         k_dem_gather64<false><<<grid, 128, 0, s>>>(boxes, tiles, ntiles, src_tmp, key_out);
+}
+
+// every box is one tile: all substeps in one launch
+void launch_dem_solo64(const BoxDev *boxes, const Tile *tiles, int ntiles, int n_dem, int walls, cudaStream_t s) {
+    if (walls) k_dem_solo64<true><<<ntiles, 128, 0, s>>>(boxes, tiles, n_dem);
+    else k_dem_solo64<false><<<ntiles, 128, 0, s>>>(boxes, tiles, n_dem);
+}
+
+// tiles of at most 32 particles with 8 lanes: substeps sd to sd + n - 1 (n > 1:
+// every box is one tile)
+void launch_dem_mixed8(const BoxDev *boxes, const Tile *tiles, int ntiles, int sd, int n, int n_dem, int walls,
+                       cudaStream_t s) {
+    if (walls) k_dem_mixed8<true><<<ntiles, 256, 0, s>>>(boxes, tiles, sd, n, n_dem);
+    else k_dem_mixed8<false><<<ntiles, 256, 0, s>>>(boxes, tiles, sd, n, n_dem);
 }
 
 }  // namespace dps
