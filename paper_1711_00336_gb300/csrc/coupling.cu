@@ -357,7 +357,12 @@ template <typename Fn>
 __device__ __forceinline__ void for_brick_cells(const Geom &g, int ox, int oy, int oz, int ex, int ey, int ez, Fn &&fn) {
     const int nb = ex * ey * ez;
     for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-        const int lx = k % ex, ly = (k / ex) % ey, lz = k / (ex * ey);
+        int lx = k % BRICK, ly = k / BRICK % BRICK, lz = k / (BRICK * BRICK);
+        if (ex != BRICK || ey != BRICK) {  // a clipped brick: divisions at run time
+            lx = k % ex;
+            ly = k / ex % ey;
+            lz = k / (ex * ey);
+        }
         fn(cell_index(g, ox + lx, oy + ly, oz + lz), lx, ly, lz);
     }
 }
@@ -390,7 +395,8 @@ constexpr int SPARSE_CAP = 192, SPARSE_LIST = 12;
 template <typename FT, bool SPARSE> constexpr int brick_minb() {
     return SPARSE ? (sizeof(FT) == 8 ? 6 : 8) : (sizeof(FT) == 8 ? 3 : 4);
 }
-constexpr int BL_PER_THREAD = (HALO3 + BRICK_THREADS - 1) / BRICK_THREADS;
+constexpr int BL_PER_THREAD = HALO / 2;  // halo cells a thread stages
+static_assert(HALO3 / BL_PER_THREAD <= BRICK_THREADS, "half a halo row per thread");
 // staged entries: three (FP64) or four (FP32) blocks fit an SM's shared memory;
 // denser bricks take the walk over global memory
 template <typename FT, bool SPARSE> constexpr int stage_cap() {
@@ -418,26 +424,41 @@ __device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int
                                             const FT *__restrict__ w, BrickStage<FT, NV, SPARSE> &S, Val &&value) {
     constexpr int CAP = BrickStage<FT, NV, SPARSE>::CAP;
     const Geom &g = B.g;
+    // half a halo row (five cells along x) per thread, h = 5 t .. 5 t + 4: the
+    // row is decoded once and inside the box its cells' ranges share their ends
     int s0[BL_PER_THREAD], cnt[BL_PER_THREAD], tot = 0;
 #pragma unroll
-    for (int u = 0; u < BL_PER_THREAD; ++u) {
-        const int h = BL_PER_THREAD * threadIdx.x + u;
-        int a = 0, e = 0;
-        if (h < HALO3) {
-            const int hx = h % HALO, hy = (h / HALO) % HALO, hz = h / (HALO * HALO);
-            const int x = wrap_axis(ox + hx - 1, g.n[0], g.per[0]);
-            const int y = wrap_axis(oy + hy - 1, g.n[1], g.per[1]);
-            const int z = wrap_axis(oz + hz - 1, g.n[2], g.per[2]);
-            // (a clipped brick has a smaller halo)
-            if (hx <= ex + 1 && hy <= ey + 1 && hz <= ez + 1 && x >= 0 && y >= 0 && z >= 0) {
-                const long long n = cell_index(g, x, y, z);
-                a = B.cell_start[n];
-                e = B.cell_start[n + 1];
+    for (int u = 0; u < BL_PER_THREAD; ++u) s0[u] = cnt[u] = 0;
+    const int h0 = BL_PER_THREAD * threadIdx.x, hx0 = (threadIdx.x & 1) * BL_PER_THREAD;
+    if (h0 < HALO3) {
+        const int row = threadIdx.x >> 1, hz = row / HALO, hy = row - hz * HALO;
+        const int y = wrap_axis(oy + hy - 1, g.n[1], g.per[1]), z = wrap_axis(oz + hz - 1, g.n[2], g.per[2]);
+        const int x = ox + hx0 - 1;
+        // (a clipped brick has a smaller halo)
+        if (hy <= ey + 1 && hz <= ez + 1 && y >= 0 && z >= 0) {
+            const int *cs = B.cell_start + cell_index(g, 0, y, z);
+            if (x >= 0 && x + BL_PER_THREAD <= g.n[0] && hx0 + BL_PER_THREAD - 1 <= ex + 1) {
+                int e[BL_PER_THREAD + 1];
+#pragma unroll
+                for (int u = 0; u <= BL_PER_THREAD; ++u) e[u] = cs[x + u];
+#pragma unroll
+                for (int u = 0; u < BL_PER_THREAD; ++u) {
+                    s0[u] = e[u];
+                    cnt[u] = e[u + 1] - e[u];
+                }
+                tot = e[BL_PER_THREAD] - e[0];
+            } else {
+#pragma unroll
+                for (int u = 0; u < BL_PER_THREAD; ++u) {
+                    const int xu = wrap_axis(x + u, g.n[0], g.per[0]);
+                    if (hx0 + u <= ex + 1 && xu >= 0) {
+                        s0[u] = cs[xu];
+                        cnt[u] = cs[xu + 1] - s0[u];
+                        tot += cnt[u];
+                    }
+                }
             }
         }
-        s0[u] = a;
-        cnt[u] = e - a;
-        tot += e - a;
     }
     // block-wide exclusive prefix of the per-thread totals
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -457,18 +478,16 @@ __device__ __forceinline__ void stage_brick(const BoxDev &B, int ox, int oy, int
     }
     int run = base + incl - tot;
     const bool fits = total <= CAP;
+    if (fits && h0 < HALO3) {
 #pragma unroll
-    for (int u = 0; u < BL_PER_THREAD; ++u) {
-        const int h = BL_PER_THREAD * threadIdx.x + u;
-        if (h < HALO3 && fits) {
-            S.off[h] = (unsigned short)run;
-            if (cnt[u])
-                for (int m = 0; m < cnt[u]; ++m) {
-                    S.P[run + m] = s0[u] + m;
-                    S.hx[run + m] = (unsigned char)(h % HALO);
-                }
+        for (int u = 0; u < BL_PER_THREAD; ++u) {
+            S.off[h0 + u] = (unsigned short)run;
+            for (int m = 0; m < cnt[u]; ++m) {
+                S.P[run + m] = s0[u] + m;
+                S.hx[run + m] = (unsigned char)(hx0 + u);
+            }
+            run += cnt[u];
         }
-        run += cnt[u];
     }
     if (threadIdx.x == 0) {
         S.off[HALO3] = (unsigned short)total;
