@@ -11,8 +11,8 @@
 //    pass; it runs in 64-bit fixed point (lbm_fx.cuh), ~1500 integer
 //    instructions of which two to four issue per cycle.  128^3, walls at z:
 //    815 -> 228 us; 256^3, coupled step: 4.88 -> 1.93 ms (floor at the
-//    measured copy rate: 0.10 and 0.83 ms).  Boxes with a per-cell tau_e keep
-//    the FP64 relaxation, with rho and j from K2a.
+//    measured copy rate: 0.10 and 0.83 ms).  With a
+//    per-cell tau_e only tau_e is FP64: 75 x 61 x 90, 229 -> 107 us.
 // K2a moments: rho, j of f(x,t), u_D = (j + f_ext/2)/(rho eps_f) and
 //    1/(rho eps_f); one PDF read.
 // K2b fields: stencil over rho and u_D giving grad(eps_f p) and Du_f/Dt.
@@ -66,28 +66,15 @@ __device__ __forceinline__ CT tau_cell(const CT f[Q], CT s, CT rho, CT ux, CT uy
 // (Eq. LBM_Equation, relax_cell) and store each opposite pair as soon as it
 // is computed, which keeps few values live.  VISC: the box may
 // relax with a per-cell tau_e (vmode bit 0 Eilers, bit 1 Smagorinsky).
-template <typename ST, typename FT, typename CT, int PAR, bool VISC, bool MOMIN>
+template <typename ST, typename FT, typename CT, int PAR, bool VISC>
 __device__ __forceinline__ void relax_store_cell(ST *__restrict__ pdf, CT f[Q], const NbDelta &D, bool in,
                                                  const Geom &g, CT e, CT fpx, CT fpy, CT fpz, long long N, long long c,
                                                  CT fbx, CT fby, CT fbz, CT omega_box, CT kf_box, CT tau, int vmode,
-                                                 int *status, const CT *mom, const FxFluid *ff = nullptr);
+                                                 int *status, const FxFluid *ff = nullptr);
 
-// the moments of cell c from K2a (MOMIN: FP64 with a per-cell tau_e), else nothing
-template <typename FT, typename CT, bool MOMIN>
-__device__ __forceinline__ void load_moments(const FT *__restrict__ rho, const FT *__restrict__ j, long long N,
-                                             long long c, CT mom[4]) {
-    if (MOMIN) {
-        mom[0] = (CT)rho[c];
-        mom[1] = (CT)j[c];
-        mom[2] = (CT)j[N + c];
-        mom[3] = (CT)j[2 * N + c];
-    }
-}
-
-template <typename ST, typename FT, typename CT, int PAR, bool VISC, bool MOMIN>
+template <typename ST, typename FT, typename CT, int PAR, bool VISC>
 __device__ __forceinline__ void collide_stream_cell(ST *__restrict__ pdf, const FT *__restrict__ eps,
-                                                    const FT *__restrict__ fpf, const FT *__restrict__ rho_m,
-                                                    const FT *__restrict__ j_m, const Geom &g, long long c, CT fbx,
+                                                    const FT *__restrict__ fpf, const Geom &g, long long c, CT fbx,
                                                     CT fby, CT fbz, CT omega_box, CT kf_box, CT tau, int vmode,
                                                     int *status, const FxFluid *ff = nullptr) {
     const long long N = g.ncell;
@@ -106,19 +93,16 @@ __device__ __forceinline__ void collide_stream_cell(ST *__restrict__ pdf, const 
     } else {
         load_pdfs<ST, CT, PAR>(pdf, N, c, D, f);
     }
-    CT mom[4];
-    load_moments<FT, CT, MOMIN>(rho_m, j_m, N, c, mom);
-    relax_store_cell<ST, FT, CT, PAR, VISC, MOMIN>(pdf, f, D, in, g, (CT)eps[c], (CT)fpf[c], (CT)fpf[N + c],
+    relax_store_cell<ST, FT, CT, PAR, VISC>(pdf, f, D, in, g, (CT)eps[c], (CT)fpf[c], (CT)fpf[N + c],
                                                    (CT)fpf[2 * N + c], N, c, fbx, fby, fbz, omega_box, kf_box, tau,
-                                                   vmode, status, mom, ff);
+                                                   vmode, status, ff);
 }
 
 // two cells per thread (c and c + stride): the loads of both are issued before
 // either is relaxed, which doubles the bytes in flight per warp
-template <typename ST, typename FT, typename CT, int PAR, bool VISC, bool MOMIN>
+template <typename ST, typename FT, typename CT, int PAR, bool VISC>
 __device__ __forceinline__ void collide_stream_cell2(ST *__restrict__ pdf, const FT *__restrict__ eps,
-                                                     const FT *__restrict__ fpf, const FT *__restrict__ rho_m,
-                                                     const FT *__restrict__ j_m, const Geom &g, long long c,
+                                                     const FT *__restrict__ fpf, const Geom &g, long long c,
                                                      long long c2, bool two, CT fbx, CT fby, CT fbz, CT omega_box,
                                                      CT kf_box, CT tau, int vmode, int *status) {
     const long long N = g.ncell;
@@ -155,14 +139,11 @@ __device__ __forceinline__ void collide_stream_cell2(ST *__restrict__ pdf, const
         b1 = (CT)fpf[N + c2];
         b2 = (CT)fpf[2 * N + c2];
     }
-    CT mom[4], mom2[4];
-    load_moments<FT, CT, MOMIN>(rho_m, j_m, N, c, mom);
-    if (two) load_moments<FT, CT, MOMIN>(rho_m, j_m, N, c2, mom2);
-    relax_store_cell<ST, FT, CT, PAR, VISC, MOMIN>(pdf, f, D, in, g, e, a0, a1, a2, N, c, fbx, fby, fbz, omega_box,
-                                                   kf_box, tau, vmode, status, mom);
+    relax_store_cell<ST, FT, CT, PAR, VISC>(pdf, f, D, in, g, e, a0, a1, a2, N, c, fbx, fby, fbz, omega_box,
+                                                   kf_box, tau, vmode, status);
     if (two)
-        relax_store_cell<ST, FT, CT, PAR, VISC, MOMIN>(pdf, f2, D2, in2, g, e2, b0, b1, b2, N, c2, fbx, fby, fbz,
-                                                       omega_box, kf_box, tau, vmode, status, mom2);
+        relax_store_cell<ST, FT, CT, PAR, VISC>(pdf, f2, D2, in2, g, e2, b0, b1, b2, N, c2, fbx, fby, fbz,
+                                                       omega_box, kf_box, tau, vmode, status);
 }
 
 // two-element vectors of the stored type (low-precision forms): float2 or
@@ -198,10 +179,9 @@ template <> struct Vec2<__half> {
     }
 };
 
-template <typename ST, typename CT, bool VISC, bool MOMIN>
+template <typename ST, typename CT, bool VISC>
 __device__ __forceinline__ void relax_cell(CT f[Q], CT e, CT fpx, CT fpy, CT fpz, CT fbx, CT fby, CT fbz,
-                                           CT omega_box, CT kf_box, CT tau, int vmode, bool flag, int *status,
-                                           const CT *mom);
+                                           CT omega_box, CT kf_box, CT tau, int vmode, bool flag, int *status);
 
 // two consecutive cells c, c+1 (c and ncell even).  Even parity: own-cell
 // accesses only, any pair.  Odd parity: two cells of one x row (nx even: the
@@ -226,9 +206,9 @@ __device__ __forceinline__ void collide_stream_vec2(ST *__restrict__ pdf, const 
         D1 = neighbour_deltas(g, ix + 1, iy, iz);
     }
     if (PAR && (!no_wall_neighbour(D) || !no_wall_neighbour(D1))) {
-        collide_stream_cell<ST, FT, CT, PAR, VISC, false>(pdf, eps, fpf, nullptr, nullptr, g, c, fbx, fby, fbz,
+        collide_stream_cell<ST, FT, CT, PAR, VISC>(pdf, eps, fpf, g, c, fbx, fby, fbz,
                                                           omega_box, kf_box, tau, vmode, status);
-        collide_stream_cell<ST, FT, CT, PAR, VISC, false>(pdf, eps, fpf, nullptr, nullptr, g, c + 1, fbx, fby, fbz,
+        collide_stream_cell<ST, FT, CT, PAR, VISC>(pdf, eps, fpf, g, c + 1, fbx, fby, fbz,
                                                           omega_box, kf_box, tau, vmode, status);
         return;
     }
@@ -253,10 +233,10 @@ __device__ __forceinline__ void collide_stream_vec2(ST *__restrict__ pdf, const 
     Vec2<FT>::load(eps + cu, e0, e1);
 #pragma unroll
     for (int k = 0; k < 3; ++k) Vec2<FT>::load(fpf + ((unsigned)k * Nu + cu), a[k], b[k]);
-    relax_cell<ST, CT, VISC, false>(f, e0, a[0], a[1], a[2], fbx, fby, fbz, omega_box, kf_box, tau, vmode, true,
-                                    status, nullptr);
-    relax_cell<ST, CT, VISC, false>(f1, e1, b[0], b[1], b[2], fbx, fby, fbz, omega_box, kf_box, tau, vmode, true,
-                                    status, nullptr);
+    relax_cell<ST, CT, VISC>(f, e0, a[0], a[1], a[2], fbx, fby, fbz, omega_box, kf_box, tau, vmode, true,
+                                    status);
+    relax_cell<ST, CT, VISC>(f1, e1, b[0], b[1], b[2], fbx, fby, fbz, omega_box, kf_box, tau, vmode, true,
+                                    status);
     Vec2<ST>::store(pdf + cu, f[0], f1[0]);
 #pragma unroll
     for (int k = 1; k <= 9; ++k) {
@@ -299,32 +279,22 @@ __device__ __forceinline__ double r_sub(double a, double b) { return __dsub_rn(a
 // omega f^eq + F is E = K0 + cu (K1 cu + K2 cF), the odd part
 // O = K3 cu + K4 cF, with K0..K4 fixed per weight class.
 // `flag`: report a non-finite or non-positive density.
-// MOMIN: the moments s, j of these populations were computed by K2a in this
-// step (the FP64 form with a per-cell tau_e): they are passed in, not re-summed.
-template <typename ST, typename CT, bool VISC, bool MOMIN = false>
+template <typename ST, typename CT, bool VISC>
 __device__ __forceinline__ void relax_cell(CT f[Q], CT e, CT fpx, CT fpy, CT fpz, CT fbx, CT fby, CT fbz,
-                                           CT omega_box, CT kf_box, CT tau, int vmode, bool flag, int *status,
-                                           const CT *mom = nullptr) {
+                                           CT omega_box, CT kf_box, CT tau, int vmode, bool flag, int *status) {
     constexpr bool DEV = Store<ST>::shifted;
     // f_ext = f_pf + eps_f f_b (Eq. Forcing)
     const CT Fx = r_fma(e, fbx, fpx);
     const CT Fy = r_fma(e, fby, fpy);
     const CT Fz = r_fma(e, fbz, fpz);
     CT s = f[0], jx = 0, jy = 0, jz = 0;
-    if (MOMIN) {
-        s = mom[0];
-        jx = mom[1];
-        jy = mom[2];
-        jz = mom[3];
-    } else {
 #pragma unroll
-        for (int k = 1; k <= 9; ++k) {
-            s = r_add(s, r_add(f[k], f[k + 9]));
-            const CT d = r_sub(f[k], f[k + 9]);
-            if (CX(k) != 0) jx = CX(k) > 0 ? r_add(jx, d) : r_sub(jx, d);
-            if (CY(k) != 0) jy = CY(k) > 0 ? r_add(jy, d) : r_sub(jy, d);
-            if (CZ(k) != 0) jz = CZ(k) > 0 ? r_add(jz, d) : r_sub(jz, d);
-        }
+    for (int k = 1; k <= 9; ++k) {
+        s = r_add(s, r_add(f[k], f[k + 9]));
+        const CT d = r_sub(f[k], f[k + 9]);
+        if (CX(k) != 0) jx = CX(k) > 0 ? r_add(jx, d) : r_sub(jx, d);
+        if (CY(k) != 0) jy = CY(k) > 0 ? r_add(jy, d) : r_sub(jy, d);
+        if (CZ(k) != 0) jz = CZ(k) > 0 ? r_add(jz, d) : r_sub(jz, d);
     }
     const CT rho = DEV ? r_add(CT(1), s) : s;
     if (flag && (!(rho > CT(0)) || !(rho < CT(1e30)))) atomicOr(status, ST_NAN);
@@ -366,21 +336,20 @@ __device__ __forceinline__ void relax_cell(CT f[Q], CT e, CT fpx, CT fpy, CT fpz
 }
 
 // relaxation and parity-aware stores of one cell
-template <typename ST, typename FT, typename CT, int PAR, bool VISC, bool MOMIN>
+template <typename ST, typename FT, typename CT, int PAR, bool VISC>
 __device__ __forceinline__ void relax_store_cell(ST *__restrict__ pdf, CT f[Q], const NbDelta &D, bool in,
                                                  const Geom &g, CT e, CT fpx, CT fpy, CT fpz, long long N, long long c,
                                                  CT fbx, CT fby, CT fbz, CT omega_box, CT kf_box, CT tau, int vmode,
-                                                 int *status, const CT *mom, const FxFluid *ff) {
+                                                 int *status, const FxFluid *ff) {
     bool done = false;
-    if constexpr (sizeof(ST) == 8 && !VISC) {
+    if constexpr (sizeof(ST) == 8) {
         u64 b[Q];
 #pragma unroll
         for (int q = 0; q < Q; ++q) b[q] = fx_bits(f[q]);
-        done = fx_relax(b, e, fpx, fpy, fpz, *ff, f);
+        done = fx_relax<VISC>(b, e, fpx, fpy, fpz, *ff, tau, vmode, f);
     }
     if (!done)
-        relax_cell<ST, CT, VISC, MOMIN>(f, e, fpx, fpy, fpz, fbx, fby, fbz, omega_box, kf_box, tau, vmode, true, status,
-                                        mom);
+        relax_cell<ST, CT, VISC>(f, e, fpx, fpy, fpz, fbx, fby, fbz, omega_box, kf_box, tau, vmode, true, status);
     Store<ST>::store(pdf + (unsigned)c, f[0]);
 #pragma unroll
     for (int k = 1; k <= 9; ++k) {
@@ -398,9 +367,11 @@ template <> __device__ __forceinline__ float pick<float>(double, float f) { retu
 #ifndef DPS_K1_MINB
 #define DPS_K1_MINB 3  // FP64: 128-thread blocks per SM the register budget is sized for
 #endif
+#ifndef DPS_K1V_MINB
+#define DPS_K1V_MINB 3  // the same with a per-cell tau_e
+#endif
 // K1: every cell tile of every box, AA parity PAR (common to the batch).
-// MOMIN: rho and j come from K2a of the same step (FP64 coupled step, VISC)
-template <typename ST, typename FT, typename CT, int PAR, int MINB, bool VISC, int CPT, bool MOMIN = false>
+template <typename ST, typename FT, typename CT, int PAR, int MINB, bool VISC, int CPT>
 __global__ void __launch_bounds__(128, MINB) k_collide_stream(const BoxDev *__restrict__ boxes,
                                                            const Tile *__restrict__ tiles, int ntiles) {
     DPS_FOR_TILES(tiles, ntiles, t) {
@@ -409,14 +380,13 @@ __global__ void __launch_bounds__(128, MINB) k_collide_stream(const BoxDev *__re
         const Geom g = B.g;
         ST *pdf = (ST *)B.pdf;
         const FT *eps = (const FT *)B.eps, *fpf = (const FT *)B.fpf;
-        const FT *rho_m = (const FT *)B.rho, *j_m = (const FT *)B.j;
         const CT fbx = pick<CT>(B.ph.fb[0], B.ph.fb_f[0]), fby = pick<CT>(B.ph.fb[1], B.ph.fb_f[1]),
                  fbz = pick<CT>(B.ph.fb[2], B.ph.fb_f[2]);
         const CT omega = pick<CT>(B.ph.omega, B.ph.omega_f), kf = pick<CT>(B.ph.kf, B.ph.kf_f);
         const CT tau = (CT)B.ph.tau;
         const int vmode = VISC ? (B.ph.eilers ? 1 : 0) | (B.ph.smag ? 2 : 0) : 0;
         int *st = B.status;
-        if (CPT == 3 && sizeof(ST) < 8 && !MOMIN && !(g.ncell & 1) && !((tl.begin | tl.end) & 1) &&
+        if (CPT == 3 && sizeof(ST) < 8 && !(g.ncell & 1) && !((tl.begin | tl.end) & 1) &&
             (!PAR || !(g.n[0] & 1))) {
             // vector pairs; the odd parity at odd nx moves scalars, two cells a
             // thread in FP16 (161 x 150 x 139: 131 -> 107 us a step), one in
@@ -426,12 +396,12 @@ __global__ void __launch_bounds__(128, MINB) k_collide_stream(const BoxDev *__re
                                                            st);
         } else if (CPT == 1 || (CPT == 3 && sizeof(ST) == 4)) {
             for (long long c = tl.begin + threadIdx.x; c < tl.end; c += blockDim.x)
-                collide_stream_cell<ST, FT, CT, PAR, VISC, MOMIN>(pdf, eps, fpf, rho_m, j_m, g, c, fbx, fby, fbz,
+                collide_stream_cell<ST, FT, CT, PAR, VISC>(pdf, eps, fpf, g, c, fbx, fby, fbz,
                                                                   omega, kf, tau, vmode, st, &B.ph.ff);
         } else {
             for (long long c = tl.begin + threadIdx.x; c < tl.end; c += 2 * blockDim.x) {
                 const long long c2 = c + blockDim.x;
-                collide_stream_cell2<ST, FT, CT, PAR, VISC, MOMIN>(pdf, eps, fpf, rho_m, j_m, g, c, c2, c2 < tl.end,
+                collide_stream_cell2<ST, FT, CT, PAR, VISC>(pdf, eps, fpf, g, c, c2, c2 < tl.end,
                                                                    fbx, fby, fbz, omega, kf, tau, vmode, st);
             }
         }
@@ -929,28 +899,20 @@ static int grid_for(long long n, int block) {
 // autotuner.  visc: some box of the batch
 // relaxes with a per-cell tau_e (one register budget for that variant).
 template <typename ST, typename FT, typename CT>
-void launch_collide_stream(const BoxDev *boxes, const Tile *tiles, int ntiles, int parity, int variant, bool visc,
-                           bool mom_in, int grid, int block, cudaStream_t s) {
+void launch_collide_stream(const BoxDev *boxes, const Tile *tiles, int ntiles, int parity, int variant, bool visc, int grid, int block, cudaStream_t s) {
     block = 128;
     if (sizeof(CT) == 8) variant = 0;  // FP64: one register-heavy variant
-#define DPS_K1VM(MB, V, CPT, M)                                                                           \
+#define DPS_K1V(MB, V, CPT)                                                                           \
     do {                                                                                                  \
         if (parity)                                                                                       \
-            k_collide_stream<ST, FT, CT, 1, MB, V, CPT, M><<<grid, block, 0, s>>>(boxes, tiles, ntiles);  \
+            k_collide_stream<ST, FT, CT, 1, MB, V, CPT><<<grid, block, 0, s>>>(boxes, tiles, ntiles);  \
         else                                                                                              \
-            k_collide_stream<ST, FT, CT, 0, MB, V, CPT, M><<<grid, block, 0, s>>>(boxes, tiles, ntiles);  \
+            k_collide_stream<ST, FT, CT, 0, MB, V, CPT><<<grid, block, 0, s>>>(boxes, tiles, ntiles);  \
     } while (0)
-#define DPS_K1V(MB, V, CPT) DPS_K1VM(MB, V, CPT, false)
 #define DPS_K1(MB, CPT) DPS_K1V(MB, false, CPT)
     if constexpr (sizeof(CT) == 8) {
-        // per-cell tau_e: FP64 relaxation, rho and j of the coupled step
-        // from K2a.  Else the fixed-point relaxation, which sums them itself
-        if (visc) {
-            if (mom_in) DPS_K1VM(2, true, 1, true);
-            else DPS_K1V(2, true, 1);
-        } else {
-            DPS_K1(DPS_K1_MINB, 1);
-        }
+        if (visc) DPS_K1V(DPS_K1V_MINB, true, 1);
+        else DPS_K1(DPS_K1_MINB, 1);
     } else if (visc)
         DPS_K1V(3, true, 1);
     else if (variant == 1)
@@ -971,7 +933,6 @@ void launch_collide_stream(const BoxDev *boxes, const Tile *tiles, int ntiles, i
         DPS_K1(4, 1);
 #undef DPS_K1
 #undef DPS_K1V
-#undef DPS_K1VM
 }
 
 template <typename ST, typename FT, typename CT>
@@ -1015,7 +976,7 @@ void launch_pdf_import(void *pdf, long long N, const double *in, cudaStream_t s)
 
 // explicit instantiations for the three precision forms
 #define DPS_LBM_INST(ST, FT, CT)                                                                             \
-    template void launch_collide_stream<ST, FT, CT>(const BoxDev *, const Tile *, int, int, int, bool, bool, int, int, cudaStream_t); \
+    template void launch_collide_stream<ST, FT, CT>(const BoxDev *, const Tile *, int, int, int, bool, int, int, cudaStream_t); \
     template void launch_moments<ST, FT, CT>(const BoxDev *, const Tile *, int, int, int, int, cudaStream_t);
 DPS_LBM_INST(double, double, double)
 DPS_LBM_INST(float, float, float)

@@ -114,10 +114,58 @@ __host__ __device__ __forceinline__ u64 fx_recip(i64 rho, i64 e62, int &lz) {
     return ((u64)Y << 32) + (u64)(((c1 >> 32) * (i64)Y) * 2) + (((u64)(u32)c1 * Y) >> 31);
 }
 
+// omega = 1/tau_e of a cell (Eq. tau_e) from its populations f and rho (2^-62),
+// J = rho u (2^-62) and V = u/eps (2^-60).  The non-equilibrium flux Q_ab is
+// exact integer sums and three-half products; square roots and divisions are
+// FP64 (tau_* of the Eilers viscosity, tau_t of Smagorinsky, in the
+// cancellation-free form).
+__host__ __device__ __forceinline__ double fx_omega_cell(const i64 f[Q], i64 rho, const i64 J[3], const i64 V[3],
+                                                         i64 ir, double e, double tau, int eilers, int smag) {
+    double ts = tau;
+    if (eilers) {
+        double r = (1.0 - e) * (1.0 / 0.64);
+        r = r < 0.0 ? 0.0 : (r > 0.9 ? 0.9 : r);
+        const double a = 1.0 + (1.25 * 0.64) * r / (1.0 - r);
+        ts = 0.5 + (tau - 0.5) * (a * a);
+    }
+    if (!smag) return 1.0 / ts;
+    const i64 iso = fx_mulhi_s(rho, 6148914691236517205ll);  // rho/3
+    i64 P[6] = {-iso, -iso, -iso, 0, 0, 0};                  // xx yy zz xy xz yz
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int k = 1; k <= 9; ++k) {
+        const i64 p = f[k] + f[k + 9];
+        if (CX(k) != 0) P[0] += p;
+        if (CY(k) != 0) P[1] += p;
+        if (CZ(k) != 0) P[2] += p;
+        if (CX(k) * CY(k) != 0) P[3] += CX(k) * CY(k) > 0 ? p : -p;
+        if (CX(k) * CZ(k) != 0) P[4] += CX(k) * CZ(k) > 0 ? p : -p;
+        if (CY(k) * CZ(k) != 0) P[5] += CY(k) * CZ(k) > 0 ? p : -p;
+    }
+    const i64 J8[3] = {J[0] * 8, J[1] * 8, J[2] * 8};  // 2^-65, the products 2^-61
+    double q[6];
+    q[0] = fx_signed_to_double(P[0] - 2 * fx_mulhi_s(J8[0], V[0]), 62);
+    q[1] = fx_signed_to_double(P[1] - 2 * fx_mulhi_s(J8[1], V[1]), 62);
+    q[2] = fx_signed_to_double(P[2] - 2 * fx_mulhi_s(J8[2], V[2]), 62);
+    q[3] = fx_signed_to_double(P[3] - 2 * fx_mulhi_s(J8[0], V[1]), 62);
+    q[4] = fx_signed_to_double(P[4] - 2 * fx_mulhi_s(J8[0], V[2]), 62);
+    q[5] = fx_signed_to_double(P[5] - 2 * fx_mulhi_s(J8[1], V[2]), 62);
+    const double q2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + 2.0 * (q[3] * q[3] + q[4] * q[4] + q[5] * q[5]);
+    // 2 C_S^2 Qbar / (rho c_s^4)
+    const double x = (2 * 0.01 * 9) * sqrt(2.0 * q2) * fx_positive_to_double((u64)ir, 62);
+    const double y = 2.0 * (sqrt(ts * ts + x) + ts);
+    return y / (ts * y + x);  // 1/(tau_* + x/y)
+}
+
 // One cell: b the bits of the populations, e = eps_f, fp = f_pf; f receives the
-// post-collision populations.  False: outside the range, nothing is written.
+// post-collision populations.  VISC: omega from the cell's own tau_e (vmode bit
+// 0 Eilers, bit 1 Smagorinsky), else the box's.  False: outside the range,
+// nothing is written.
+template <bool VISC>
 __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, double fp0, double fp1, double fp2,
-                                                  const FxFluid &x, double out[Q]) {
+                                                  const FxFluid &xb, double tau, int vmode, double out[Q]) {
+    FxFluid x = xb;
     i64 f[Q], rho, j[3];
     const u64 eb = fx_bits(e), p0 = fx_bits(fp0), p1 = fx_bits(fp1), p2 = fx_bits(fp2);
     // 1/8 < eps <= 1, |f_pf| < 1/8
@@ -143,6 +191,20 @@ __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, doub
     const i64 ir = (i64)(fx_mulhi((u64)e62, R) << lz);  // 1/rho, 2^-62, < 2
     const u64 m = fx_mulhi((u64)rho << 1, R);
     const i64 ie = (i64)(lz >= 3 ? m << (lz - 3) : m >> (3 - lz));  // 1/eps, 2^-60, < 8
+    if (VISC && vmode) {
+        i64 W[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+        for (int a = 0; a < 3; ++a) W[a] = fx_mulhi_s(fx_mulhi_s(J[a] * 4, ir) * 4, ie);
+        const double om = fx_omega_cell(f, rho, J, W, ir, e, tau, vmode & 1, vmode & 2);
+        if (!(om > 0.0 && om < 2.0)) return false;
+        const u64 o = (u64)fx_from_pos(om, 60), k = (1ull << 60) - (o >> 1);  // omega, 1 - omega/2
+        x.om = o * 8;
+        x.om12 = o + fx_mulhi(o, 0x5555555555555555ull);
+        x.om36 = fx_mulhi(o, 0x71c71c71c71c71c7ull);
+        x.kf12 = k + fx_mulhi(k, 0x5555555555555555ull);
+    }
     const u64 c12 = fx_mulhi(x.om12, (u64)rho << 1) << 1;           // omega rho / 12, 2^-64
     i64 H[3], G[3], V[3];
 #ifdef __CUDA_ARCH__

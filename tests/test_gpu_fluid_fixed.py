@@ -73,6 +73,44 @@ def test_relaxation_across_the_fixed_point_ranges(name, tau):
     dom.close()
 
 
+@pytest.mark.parametrize("vk", [dict(eilers=1), dict(smagorinsky=1), dict(eilers=1, smagorinsky=1)],
+                         ids=["eilers", "smagorinsky", "both"])
+@pytest.mark.parametrize("name", list(RANGES))
+def test_cell_viscosity_across_the_fixed_point_ranges(name, vk):
+    """The same with a relaxation time per cell.  omega's own rounding (twenty
+    operations) multiplies f - f_eq, below the largest population: 5e-15."""
+    _need_gpu()
+    import oracle as O
+    from paper_1711_00336_gb300 import dps
+    scale, speed, noise, er, fa = RANGES[name]
+    n, per, tau = (13, 6, 9), (1, 0, 1), 0.55
+    nc = n[0] * n[1] * n[2]
+    c, w = dps.lattice()
+    co, _, _ = O.lattice()
+    perm = [next(k for k in range(19) if (co[k] == c[q]).all()) for q in range(19)]
+    rng = np.random.default_rng(len(name))
+    f = _populations(c, w, nc, scale, speed, noise, seed=len(name))
+    eps, fpf = rng.uniform(*er, nc), fa * rng.standard_normal((3, nc))
+    dom = dps.Domain(n, per, tau, "f64")
+    dom.set_closure(g=(0, 0, 0), fb_mode=0, fb=(0, 0, 0), n_int=1, n_dem=1, **vk)
+    dom.prepare()
+    dom.write_pdfs(f)
+    dom.write_fields(eps_f=eps, f_pf=fpf)
+    P = O.make_params(n, per, tau, n_int=1, n_dem=1, **vk)
+    ref = np.empty_like(f)
+    ref[perm] = f
+    for step in (1, 2):
+        try:
+            dom.collide_stream(1)
+        except dps.DPSError:
+            assert name in ("far_outside", "strong_force")
+            break
+        ref = O.collide_stream(P, ref, eps, fpf)
+        got = dom.read_pdfs()
+        assert np.abs(got - ref[perm]).max() <= step * 5e-15 * max(1.0, np.abs(ref).max() / eps.min()), step
+    dom.close()
+
+
 def test_non_finite_populations_are_reported():
     _need_gpu()
     from paper_1711_00336_gb300 import dps
