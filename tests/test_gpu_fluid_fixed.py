@@ -157,3 +157,44 @@ def test_step_gradients_against_plain_sums(n, per, speed):
     conv = np.array([(u * grad(u[b])).sum(0) for b in range(3)])
     assert np.abs(got["gradP"] - gp).max() <= 1e-15 * rho.max()
     assert np.abs(got["DuDt"] - conv).max() <= 2e-14 * np.abs(u).max()
+
+
+@pytest.mark.parametrize("form", ["f32", "f16s"])
+@pytest.mark.parametrize("steps", [0, 1])
+@pytest.mark.parametrize("n,per", [((8, 8, 8), (1, 1, 1)), ((17, 9, 4), (1, 1, 1)), ((6, 5, 7), (1, 0, 0)),
+                                   ((5, 3, 7), (0, 1, 1)), ((2, 9, 3), (0, 1, 1))])
+def test_fp32_moments_and_gradients(form, steps, n, per):
+    """The cell pairs of the moments pass (even and odd nx and cell counts, both
+    parities, walls) and the staged gradients.  rho carries 19 roundings of a sum
+    below 0.3 and that of 1 + s: 4e-7; grad P adds 18 terms, sum |w c| = 1/3: 6e-7."""
+    _need_gpu()
+    from paper_1711_00336_gb300 import dps
+    nc = n[0] * n[1] * n[2]
+    c, w = dps.lattice()
+    dom = dps.Domain(n, per, 0.7, form)
+    dom.set_closure(g=(0, 0, 0), fb_mode=0, fb=(0, 0, 0), n_int=1, n_dem=1)
+    dom.write_pdfs(_populations(c, w, nc, 1.0, 1e-2, 1e-2, seed=7))
+    if steps:
+        dom.step(steps)
+    f = dom.read_pdfs()
+    dom.step(1)
+    got = dom.read_fields(("gradP", "DuDt"))
+    dom.close()
+    rho = f.sum(0)
+    idx = np.arange(nc).reshape(n[2], n[1], n[0])
+
+    def nb(q):
+        i = idx
+        for a in range(3):
+            k = np.arange(n[a]) + c[q][a]
+            k = k % n[a] if per[a] else np.clip(k, 0, n[a] - 1)
+            i = np.take(i, k, axis=2 - a)
+        return i.ravel()
+
+    gp = sum(w[q] * np.outer(c[q], rho[nb(q)]) for q in range(1, 19))
+    assert np.abs(got["gradP"] - gp).max() <= 6e-7 * rho.max()
+    if not steps:  # no u_prev yet: the convective term alone; u good to 4e-7, its gradient to 1e-6
+        u = (c.T @ f) / rho
+        conv = np.array([(u * sum(3 * w[q] * np.outer(c[q], u[b][nb(q)]) for q in range(1, 19))).sum(0)
+                         for b in range(3)])
+        assert np.abs(got["DuDt"] - conv).max() <= 5e-6 * np.abs(u).max()
