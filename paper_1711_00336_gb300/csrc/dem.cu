@@ -1276,7 +1276,7 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
 // sector and one dependent load.  (A force plane and a flag array took three
 // sectors and two loads.)
 #ifndef DPS_GATHER_GC
-#define DPS_GATHER_GC 4  // entries whose loads are issued before any is added
+#define DPS_GATHER_GC 3  // entries whose loads are issued before any is added (4: 1% slower, 6: 4%)
 #endif
 #ifndef DPS_GATHER_MINB
 #define DPS_GATHER_MINB 7  // 128-thread blocks per SM the register budget is sized for
