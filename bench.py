@@ -71,23 +71,23 @@ def closure_of(wl):
 
 def algorithmic_bytes_collide(prec, mom_in=False):
     """K1 per cell: 19 PDF loads + 19 stores, eps_f and f_pf (3) loads; in the
-    FP64 coupled step (mom_in) also rho and j (4) from the moments pass."""
+    FP64 coupled step with a per-cell tau_e (mom_in) also rho and j (4) from the
+    moments pass."""
     s = {"f64": 8, "f32": 4, "f16s": 2}[prec]
     sf = 8 if prec == "f64" else 4
     return 2 * 19 * s + (8 if mom_in else 4) * sf
 
 
-# algorithmic FP64 flops (a division, square root or logarithm counted as one)
-# per cell of the collide-stream: velocity and invariants 36, 9 pairs x 16 +
-# 13 more (rho and j, 42 flops, come from the moments pass of the same step)
-K1_FLOPS_F64 = 207
+# algorithmic flops (a division, square root or logarithm counted as one).  They
+# count the method's work: the FP64 form does the relaxation (207 flops and 42
+# for rho and j per cell) and most of a lubrication pair in 64-bit fixed point
 DEM_FLOPS_PARTICLE = 32   # per particle and substep: semi-implicit Euler of u, w, x, skin check
 DEM_FLOPS_PAIR = 75       # per interacting pair (once: F_ji = -F_ij): separation 9, masses / normal 17,
                           # contact or Ball-Melrose force 49
 # DRAM bytes (read + write) per particle-substep of the FP64 DEM pair and
-# gather kernels, from the ncu capture of profiles/dem_pairs_fp64_settling_64.md
-# (a 64^3 box of the headline eps and d; traffic grows with the particle count)
-DEM_TRAFFIC_PER_PARTICLE = 748.0  # (4.54 + 17.64) MB / 29,669 spheres, cold-cache capture
+# gather kernels, from the ncu capture of profiles/dem_pairs_fp64_settling_128.md
+# (a 128^3 box of the headline eps and d)
+DEM_TRAFFIC_PER_PARTICLE = 969.0  # (48.3 + 181.7) MB / 237,349 spheres, cold-cache capture
 
 
 def interacting_pairs(x, d, n, periodic, h_c, sample=20000, seed=0):
@@ -357,16 +357,14 @@ def dem_roofline(phase, wl, st, steps, fp64_peak, hbm):
                          "bytes_per_particle": 184}}
 
 
-def collide_roofline(phase, ncell, steps, fp64_peak, hbm):
+def collide_roofline(phase, ncell, steps, hbm):
     cs = phase["collide_stream"]
     k1_ms = cs["ms"] / steps  # the phase: K1 and the end-of-step update
-    k1_flops = K1_FLOPS_F64 * ncell / (k1_ms * 1e-3) / 1e9
-    b = algorithmic_bytes_collide("f64", True)
-    return {"kernel": "k_collide_stream (K1, FP64)", "bound": "alu", "achieved": k1_flops, "peak": fp64_peak,
-            "unit": "GFLOP/s", "frac": k1_flops / fp64_peak, "traffic": None, "flops_per_cell": K1_FLOPS_F64,
-            "cells_per_launch": ncell, "per_launch_us": k1_ms * 1e3,
-            "hbm_view": {"achieved_GBps": b * ncell / (k1_ms * 1e-3) / 1e9, "peak_GBps": hbm, "bytes_per_cell": b},
-            "peak_source": "dps_probe_fp64_peak (of measured)"}
+    b = algorithmic_bytes_collide("f64")
+    ach = b * ncell / (k1_ms * 1e-3) / 1e9
+    return {"kernel": "k_collide_stream (K1, FP64 populations relaxed in 64-bit fixed point)", "bound": "hbm",
+            "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": None, "bytes_per_cell": b,
+            "cells_per_launch": ncell, "per_launch_us": k1_ms * 1e3, "peak_source": "MEASURED_PEAKS.json (of measured)"}
 
 
 def main():
@@ -423,7 +421,7 @@ def main():
     hbm = peaks.get("hbm_gbs", 6800.0)
     dom_phase = max((k for k in phase if k != "moments+fields"), key=lambda k: phase[k]["ms"])
     roof_dem = dem_roofline(phase, wl, st, args.steps, fp64_peak, hbm)
-    roof_k1 = collide_roofline(phase, ncell, args.steps, fp64_peak, hbm)
+    roof_k1 = collide_roofline(phase, ncell, args.steps, hbm)
     roof = dict(roof_dem if dom_phase != "collide_stream" else roof_k1, dominant_phase=dom_phase)
 
     forms = {}
