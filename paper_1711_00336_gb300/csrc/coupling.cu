@@ -377,7 +377,7 @@ __device__ __forceinline__ void for_brick_cells(const Geom &g, int ox, int oy, i
 // cell by cell of the support, for the busiest lane (~27 rounds of five
 // FP64 instructions); weights and values come from shared memory.  The three
 // gathers together, before / after: 17.9 / 7.6 ms a step (256^3, eps 0.2, two
-// subcycles, FP64), 3.1 / 1.9 ms (192^3, eps 0.38, FP32), 4.5 / 3.7 ms (256^3,
+// subcycles, FP64), 3.1 / 1.8 ms (192^3, eps 0.38, FP32), 4.5 / 3.7 ms (256^3,
 // eps 0.05, FP16 storage); FP64 is bound by its five FP64 instructions an entry.
 //
 // A dilute brick is a chain of waits instead (cell ranges, particles, cells),
@@ -386,8 +386,9 @@ __device__ __forceinline__ void for_brick_cells(const Geom &g, int ox, int oy, i
 // instances: a stage of SPARSE_CAP entries and lists of SPARSE_LIST, 8 (FP32)
 // or 6 (FP64) blocks per SM; a brick over that (particles that settled) is
 // staged in slabs of two layers (0.5 particles per cell), and walks global
-// memory past that.  Dilute cases: 3.7 -> 2.8 ms (FP16 storage), 7.6 -> 6.5 ms
-// (FP64 256^3); SPARSE_CAP 128 sends that FP64 box to the dense stage and 256
+// memory past that.  Dilute cases: 3.7 -> 2.4 ms (FP16 storage), 7.6 -> 6.4 ms
+// (FP64 256^3), with half a halo row per thread in the staging (2.8 and 6.5 with
+// four cells); SPARSE_CAP 128 sends that FP64 box to the dense stage and 256
 // costs the dilute one 5%.
 constexpr int BRICK_THREADS = 256;  // block size of every brick kernel
 constexpr int SPARSE_CAP = 192, SPARSE_LIST = 12;

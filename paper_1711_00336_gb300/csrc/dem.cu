@@ -1270,7 +1270,7 @@ __global__ void __launch_bounds__(32 * PAIR_WARPS, DPS_PAIRS_MINB)
 // lower partners own (ascending owner), each pair's n x F_t times d_i/2, then
 // the walls and Eq. particle_motion.  The order depends on the list alone.
 // WALLS: some box of the batch has a wall axis (else the wall code is left
-// out: 128 registers instead of 168, more warps for a kernel that waits on
+// out: 72 registers instead of 168, more warps for a kernel that waits on
 // the scattered loads of the pair results)
 // A pair's force and flag share one 32-byte record, so an entry costs one
 // sector and one dependent load.  (A force plane and a flag array took three

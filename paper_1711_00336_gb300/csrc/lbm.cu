@@ -10,7 +10,7 @@
 //    FP64: 207 FP64 warp instructions of ~19 cycles per 32 cells bound this
 //    pass; it runs in 64-bit fixed point (lbm_fx.cuh), ~1500 integer
 //    instructions of which two to four issue per cycle.  128^3, walls at z:
-//    815 -> 228 us; 256^3, coupled step: 4.88 -> 1.93 ms (floor at the
+//    815 -> 216 us; 256^3, coupled step: 4.88 -> 1.77 ms (floor at the
 //    measured copy rate: 0.10 and 0.83 ms).  With a
 //    per-cell tau_e only tau_e is FP64: 75 x 61 x 90, 229 -> 107 us.
 // K2a moments: rho, j of f(x,t), u_D = (j + f_ext/2)/(rho eps_f) and
