@@ -148,7 +148,7 @@ __device__ __forceinline__ long long particle_cell(const Geom &g, double x, doub
 struct FxFluid {
     u64 om;                // omega, 2^-63
     u64 om12, om36, kf12;  // omega/12, omega/36, (1 - omega/2)/12, 2^-64
-    i64 fb[3];             // body force, 2^-64
+    i64 fb[3];             // body force, 2^-66
     int ok;
 };
 

@@ -14,9 +14,15 @@
 //   f+-a+-b <- f - omega f + E' + D_a + D_b +- X_ab +- H_a +- H_b,
 // which needs no multiplication per direction beyond omega f.  Cells
 // outside the ranges below (populations about twice those at rest, or below
-// 2^-10) take the FP64 path, as do non-finite ones.  Products round down; the constants
-// added below balance the mean of that, so that neither mass nor momentum
-// drifts.
+// 2^-10) take the FP64 path, as do non-finite ones.
+//
+// A rounding of one sign would add up over cells and steps, so the sums that the
+// update conserves are kept: f_0 is what the other 18 leave of rho, exactly, and
+// f_ext and the odd part H, which carry the momentum, are rounded to nearest (zero
+// stays zero), and the halves of the final rounding cancel over the populations.
+// Mean error of a cell's mass and momentum per step against exact arithmetic, with
+// and without f_ext, tau 0.5045 to 3, 200,000 cells: below 8e-20 and 3e-20, the
+// noise of that mean (FP64: 7.5e-17 and 7e-20).  The even products round down.
 #pragma once
 #include "dps_internal.cuh"
 
@@ -29,23 +35,30 @@ __host__ __device__ __forceinline__ i64 fx_q62(u64 b) {
 __host__ __device__ __forceinline__ double fx_signed_to_double(i64 v, int frac) {
     return fx_with_sign(fx_to_double((u64)(v < 0 ? -v : v), frac), v);
 }
-// v >= 2^32, units of 2^-frac, rounded to double
+// v >= 2^32, units of 2^-frac, rounded to double (halves up; EVEN: halves to even)
+template <bool EVEN = false>
 __host__ __device__ __forceinline__ double fx_positive_to_double(u64 v, int frac) {
 #ifdef __CUDA_ARCH__
     const u32 hi = (u32)(v >> 32), lo = (u32)v;
     const int lz = __clz((int)hi);
     const u32 h = __funnelshift_l(lo, hi, lz), l = lo << lz;
-    const u64 r = (((u64)h << 32 | l) >> 11) + ((l >> 10) & 1);
-    return fx_double(r + ((u64)((u32)(1022 + 63 - frac - lz) << 20) << 32));
 #else
-    return fx_to_double(v, frac);
+    const int lz = fx_clz(v);
+    const u32 h = (u32)(v << lz >> 32), l = (u32)(v << lz);
 #endif
+    const u32 up = EVEN ? (l & 0x7ffu) + ((l >> 11) & 1) > 0x400u : (l >> 10) & 1;
+    return fx_double((((u64)h << 32 | l) >> 11) + up + ((u64)((u32)(1022 + 63 - frac - lz) << 20) << 32));
 }
 // a b 2^-64 for a, b >= 0, rounded down, the product of the low halves left
 // out: at most 3 units low, 1.25 in the mean
 __host__ __device__ __forceinline__ u64 fx_mulhi_short(u64 a, u64 b) {
     const u32 ah = (u32)(a >> 32), al = (u32)a, bh = (u32)(b >> 32), bl = (u32)b;
     return (u64)ah * bh + (((u64)ah * bl) >> 32) + (((u64)al * bh) >> 32);
+}
+// a b 2^-63 (below 2^63) rounded to nearest
+__host__ __device__ __forceinline__ i64 fx_mul_near63(i64 a, i64 b) {
+    const u64 lo = (u64)a * (u64)b;
+    return fx_mulhi_s(a, b) * 2 + (i64)(lo >> 63) + (i64)((lo >> 62) & 1);
 }
 __host__ __device__ __forceinline__ u32 fx_abs_hi(u64 b) { return (u32)(b >> 32) & 0x7fffffffu; }
 
@@ -92,11 +105,11 @@ __host__ __device__ inline FxFluid fx_fluid(double omega, double kf, const doubl
     if (!x.ok) return x;
     x.om = (u64)fx_from_pos(omega, 60) * 8;
     const u64 o = (u64)fx_from_pos(omega, 60), k = (u64)fx_from_pos(kf, 60);
-    // omega/12, omega/36, kf/12 in units of 2^-64: 16/12 = 4/3 and 16/36 = 4/9 of the 2^-60 value
-    x.om12 = o / 3 * 4 + (o % 3) * 4 / 3;
-    x.om36 = o / 9 * 4 + (o % 9) * 4 / 9;
-    x.kf12 = k / 3 * 4 + (k % 3) * 4 / 3;
-    for (int a = 0; a < 3; ++a) x.fb[a] = fx_from(fb[a], 63) * 2;  // 2^-64
+    // omega/12, omega/36, kf/12 in units of 2^-64 to nearest: 16/12 = 4/3 and 16/36 = 4/9 of the 2^-60 value
+    x.om12 = o / 3 * 4 + ((o % 3) * 4 + 1) / 3;
+    x.om36 = o / 9 * 4 + ((o % 9) * 4 + 4) / 9;
+    x.kf12 = k / 3 * 4 + ((k % 3) * 4 + 1) / 3;
+    for (int a = 0; a < 3; ++a) x.fb[a] = (i64)llrint(fb[a] * 0x1p66);
     return x;
 }
 
@@ -115,7 +128,7 @@ __host__ __device__ __forceinline__ u64 fx_recip(i64 rho, i64 e62, int &lz) {
 }
 
 // omega = 1/tau_e of a cell (Eq. tau_e) from its populations f and rho (2^-62),
-// J = rho u (2^-62) and V = u/eps (2^-60).  The non-equilibrium flux Q_ab is
+// J = rho u (2^-66) and V = u/eps (2^-60).  The non-equilibrium flux Q_ab is
 // exact integer sums and three-half products; square roots and divisions are
 // FP64 (tau_* of the Eilers viscosity, tau_t of Smagorinsky, in the
 // cancellation-free form).
@@ -143,14 +156,13 @@ __host__ __device__ __forceinline__ double fx_omega_cell(const i64 f[Q], i64 rho
         if (CX(k) * CZ(k) != 0) P[4] += CX(k) * CZ(k) > 0 ? p : -p;
         if (CY(k) * CZ(k) != 0) P[5] += CY(k) * CZ(k) > 0 ? p : -p;
     }
-    const i64 J8[3] = {J[0] * 8, J[1] * 8, J[2] * 8};  // 2^-65, the products 2^-61
     double q[6];
-    q[0] = fx_signed_to_double(P[0] - 2 * fx_mulhi_s(J8[0], V[0]), 62);
-    q[1] = fx_signed_to_double(P[1] - 2 * fx_mulhi_s(J8[1], V[1]), 62);
-    q[2] = fx_signed_to_double(P[2] - 2 * fx_mulhi_s(J8[2], V[2]), 62);
-    q[3] = fx_signed_to_double(P[3] - 2 * fx_mulhi_s(J8[0], V[1]), 62);
-    q[4] = fx_signed_to_double(P[4] - 2 * fx_mulhi_s(J8[0], V[2]), 62);
-    q[5] = fx_signed_to_double(P[5] - 2 * fx_mulhi_s(J8[1], V[2]), 62);
+    q[0] = fx_signed_to_double(P[0] - fx_mulhi_s(J[0], V[0]), 62);
+    q[1] = fx_signed_to_double(P[1] - fx_mulhi_s(J[1], V[1]), 62);
+    q[2] = fx_signed_to_double(P[2] - fx_mulhi_s(J[2], V[2]), 62);
+    q[3] = fx_signed_to_double(P[3] - fx_mulhi_s(J[0], V[1]), 62);
+    q[4] = fx_signed_to_double(P[4] - fx_mulhi_s(J[0], V[2]), 62);
+    q[5] = fx_signed_to_double(P[5] - fx_mulhi_s(J[1], V[2]), 62);
     const double q2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + 2.0 * (q[3] * q[3] + q[4] * q[4] + q[5] * q[5]);
     // 2 C_S^2 Qbar / (rho c_s^4)
     const double x = (2 * 0.01 * 9) * sqrt(2.0 * q2) * fx_positive_to_double((u64)ir, 62);
@@ -174,30 +186,30 @@ __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, doub
         return false;
     if (!fx_populations(b, f, rho, j)) return false;
     const i64 e62 = fx_from_pos(e, 62);
-    i64 F[3] = {fx_from(fp0, 62), fx_from(fp1, 62), fx_from(fp2, 62)}, J[3];
+    i64 F[3] = {fx_from(fp0, 65), fx_from(fp1, 65), fx_from(fp2, 65)}, J[3];
+    // f_ext = f_pf + eps_f f_b (|.| < 1/4), 2^-65; 1/2 < rho < 2, |j + F/2| < 1/8 per component
+    const i64 lim = 1ll << 59;
+    bool in = rho > (1ll << 61);
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
     for (int a = 0; a < 3; ++a) {
-        F[a] += fx_mulhi_s(e62, x.fb[a]);  // f_ext = f_pf + eps_f f_b (|.| < 1/4)
-        J[a] = j[a] + (F[a] >> 1);
+        F[a] += fx_mul_near63(e62, x.fb[a]);
+        const i64 t = j[a] + (F[a] >> 4);
+        in = in && t < lim && t > -lim;
+        J[a] = (i64)((u64)j[a] * 16 + (u64)F[a]);  // rho u = j + F/2, 2^-66
     }
-    // 1/2 < rho < 2, |j + F/2| < 1/8 per component
-    const i64 lim = 1ll << 59;
-    if (!(rho > (1ll << 61) && J[0] < lim && J[0] > -lim && J[1] < lim && J[1] > -lim && J[2] < lim && J[2] > -lim))
-        return false;
+    if (!in) return false;
     int lz;
     const u64 R = fx_recip(rho, e62, lz);
-    const i64 ir = (i64)(fx_mulhi((u64)e62, R) << lz);  // 1/rho, 2^-62, < 2
-    const u64 m = fx_mulhi((u64)rho << 1, R);
-    const i64 ie = (i64)(lz >= 3 ? m << (lz - 3) : m >> (3 - lz));  // 1/eps, 2^-60, < 8
-    if (VISC && vmode) {
-        i64 W[3];
+    i64 V[3];  // u/eps = (j + F/2)/(rho eps), 2^-60, |.| < 2
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
-        for (int a = 0; a < 3; ++a) W[a] = fx_mulhi_s(fx_mulhi_s(J[a] * 4, ir) * 4, ie);
-        const double om = fx_omega_cell(f, rho, J, W, ir, e, tau, vmode & 1, vmode & 2);
+    for (int a = 0; a < 3; ++a) V[a] = fx_mulhi_s(J[a], (i64)(R >> 1)) >> (5 - lz);
+    if (VISC && vmode) {
+        const i64 ir = (i64)(fx_mulhi((u64)e62, R) << lz);  // 1/rho, 2^-62, < 2
+        const double om = fx_omega_cell(f, rho, J, V, ir, e, tau, vmode & 1, vmode & 2);
         if (!(om > 0.0 && om < 2.0)) return false;
         const u64 o = (u64)fx_from_pos(om, 60), k = (1ull << 60) - (o >> 1);  // omega, 1 - omega/2
         x.om = o * 8;
@@ -205,52 +217,46 @@ __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, doub
         x.om36 = fx_mulhi(o, 0x71c71c71c71c71c7ull);
         x.kf12 = k + fx_mulhi(k, 0x5555555555555555ull);
     }
-    const u64 c12 = fx_mulhi(x.om12, (u64)rho << 1) << 1;           // omega rho / 12, 2^-64
-    i64 H[3], G[3], V[3];
+    i64 H[3], O[3], G[3];
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
     for (int a = 0; a < 3; ++a) {
-        const i64 u = fx_mulhi_s(J[a] * 4, ir);  // 2^-62, |u| < 1/4
-        G[a] = fx_mulhi_s(F[a] * 4, (i64)x.kf12);  // 2^-64
-        H[a] = fx_mulhi_s(u * 4, (i64)c12) + G[a] + 1;
-        V[a] = fx_mulhi_s(u * 4, ie);  // 2^-60
+        // omega rho u/12 + kf F/12 = h 2^-66, rounded once to 2^-63
+        const u64 jl = (u64)J[a] * x.om12, fl = (u64)F[a] * x.kf12;
+        const i64 g = fx_mulhi_s(F[a], (i64)x.kf12);  // 2^-65
+        const i64 h = fx_mulhi_s(J[a], (i64)x.om12) + 2 * g + (i64)(fl >> 63) + (i64)(jl + 2 * fl < jl);
+        O[a] = (h + 4) >> 3;
+        H[a] = h * 2;  // 2^-67
+        G[a] = g * 4;
     }
+    // the even parts in units of 2^-63
     i64 D[3], S = 0;
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
     for (int a = 0; a < 3; ++a) {
-        const i64 p = fx_mulhi_s(H[a] + G[a], V[a]);  // 2^-60
+        const i64 p = fx_mulhi_s(H[a] + G[a], V[a]);
         D[a] = p + (p >> 1);
         S += D[a];
     }
-    // E' in units of 2^-63
-    const i64 E = (i64)fx_mulhi(x.om36, (u64)rho << 1) - fx_mulhi_s(S * 4, 6148914691236517205ll) * 2;
-    const i64 xy = fx_mulhi_s(H[0], V[1]) + fx_mulhi_s(G[1], V[0]);
-    const i64 xz = fx_mulhi_s(H[0], V[2]) + fx_mulhi_s(G[2], V[0]);
-    const i64 yz = fx_mulhi_s(H[1], V[2]) + fx_mulhi_s(G[2], V[1]);
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-    for (int a = 0; a < 3; ++a) {
-        D[a] *= 8;  // 2^-63
-        H[a] = (H[a] + 1) >> 1;
-    }
-    const i64 Xxy = xy * 24, Xxz = xz * 24, Xyz = yz * 24;
-    // f - omega f + ...; the constant in f_0 balances the mean of the
-    // rounded-down products over the 19 populations
+    const i64 E = (i64)fx_mulhi(x.om36, (u64)rho << 1) - fx_mulhi_s(S, 6148914691236517205ll);
+    const i64 Xxy = 3 * (fx_mulhi_s(H[0], V[1]) + fx_mulhi_s(G[1], V[0]));
+    const i64 Xxz = 3 * (fx_mulhi_s(H[0], V[2]) + fx_mulhi_s(G[2], V[0]));
+    const i64 Xyz = 3 * (fx_mulhi_s(H[1], V[2]) + fx_mulhi_s(G[2], V[1]));
+    // f - omega f + ...; f_0 takes what the others leave of rho (the even parts
+    // of the nine pairs add to 12 E + 6 S a side)
     i64 v[Q];
-    v[0] = (f[0] - (i64)fx_mulhi(x.om, (u64)f[0] << 1) + 6 * E) * 2 - 42;
-    int low = (int)(v[0] >> 32);
+    u64 rest = (u64)f[0] * 2 - (u64)E * 24 - (u64)S * 12 - 1;
+    int low = 0x7fffffff;
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
     for (int k = 1; k <= 9; ++k) {
         i64 ev = E, od = 0;
-        if (CX(k) != 0) { ev += D[0]; od += CX(k) > 0 ? H[0] : -H[0]; }
-        if (CY(k) != 0) { ev += D[1]; od += CY(k) > 0 ? H[1] : -H[1]; }
-        if (CZ(k) != 0) { ev += D[2]; od += CZ(k) > 0 ? H[2] : -H[2]; }
+        if (CX(k) != 0) { ev += D[0]; od += CX(k) > 0 ? O[0] : -O[0]; }
+        if (CY(k) != 0) { ev += D[1]; od += CY(k) > 0 ? O[1] : -O[1]; }
+        if (CZ(k) != 0) { ev += D[2]; od += CZ(k) > 0 ? O[2] : -O[2]; }
         if (CX(k) * CY(k) != 0) ev += CX(k) * CY(k) > 0 ? Xxy : -Xxy;
         if (CX(k) * CZ(k) != 0) ev += CX(k) * CZ(k) > 0 ? Xxz : -Xxz;
         if (CY(k) * CZ(k) != 0) ev += CY(k) * CZ(k) > 0 ? Xyz : -Xyz;
@@ -258,17 +264,25 @@ __host__ __device__ __forceinline__ bool fx_relax(const u64 b[Q], double e, doub
             ev *= 2;
             od *= 2;
         }
-        v[k] = f[k] * 2 - (i64)fx_mulhi_short(x.om, (u64)f[k] << 2) + ev + od;
-        v[k + 9] = f[k + 9] * 2 - (i64)fx_mulhi_short(x.om, (u64)f[k + 9] << 2) + ev - od;
+        const i64 p = (i64)fx_mulhi_short(x.om, (u64)f[k] << 2), r = (i64)fx_mulhi_short(x.om, (u64)f[k + 9] << 2);
+        rest += (u64)(p + r);
+        // the halves of a pair round up below, or down with one unit less: five
+        // pairs up and four down, and f_0 with its halves to even one unit less
+        if (!(k & 1)) ev -= 1;
+        v[k] = f[k] * 2 - p + ev + od;
+        v[k + 9] = f[k + 9] * 2 - r + ev - od;
         const int a = (int)(v[k] >> 32), c = (int)(v[k + 9] >> 32);
         low = low < a ? low : a;
         low = low < c ? low : c;
     }
+    v[0] = (i64)rest;
+    low = low < (int)(v[0] >> 32) ? low : (int)(v[0] >> 32);
     if (low > 0) {
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
-        for (int q = 0; q < Q; ++q) out[q] = fx_positive_to_double((u64)v[q], 63);
+        for (int q = 1; q < Q; ++q) out[q] = fx_positive_to_double((u64)v[q], 63);
+        out[0] = fx_positive_to_double<true>((u64)v[0], 63);
     } else {  // a population at or below zero
 #ifdef __CUDA_ARCH__
 #pragma unroll
