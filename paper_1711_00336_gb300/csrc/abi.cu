@@ -547,6 +547,11 @@ static int force_lanes(const BoxHost *h) {
     return lanes;
 }
 
+// particles per tile.  The pair lists of the FP64 form outlive a layout: a slot keeps its owner as the
+// index within 32 particles, and the slots of such a chunk are consecutive.  So
+// every particle tile starts at a multiple of 32, whatever size was asked for.
+static int part_tile(const Tuning &u) { return (u.part_tile + 31) / 32 * 32; }
+
 // rebuild the device table and the tile lists from the host boxes (the
 // device step state must have been pulled first)
 static int push_layout(Batch *B) {
@@ -586,6 +591,7 @@ static int push_layout(Batch *B) {
         while (ct > 128 && nc < 8LL * 152 * ct) ct /= 2;
         B->tune.cell_tile = ct;
     }
+    const int PT = part_tile(B->tune);
     std::vector<Tile> partc[4];  // particle tiles by DEM lanes class
     B->any_lift = false;
     B->any_walls = false;
@@ -606,13 +612,12 @@ static int push_layout(Batch *B) {
         h->d.ufield = B->prec == DPS_F64 && 27 * h->d.np >= 2 * h->d.g.ncell;
         tab[k] = h->d;
         const long long N = h->d.g.ncell, np = h->d.np;
-        B->solo &= np <= std::min(128, B->tune.part_tile);
+        B->solo &= np <= std::min(128, PT);
         B->sparse &= 1000 * np <= sparse_stage_mean() * N;
         for (long long c = 0; c < N; c += B->tune.cell_tile)
             ct.push_back(Tile{k, 0, c, std::min(N, c + B->tune.cell_tile)});
         B->cpl_lanes = std::max(B->cpl_lanes, fl);
-        for (long long p = 0; p < np; p += B->tune.part_tile)
-            partc[lc].push_back(Tile{k, fl, p, std::min(np, p + B->tune.part_tile)});
+        for (long long p = 0; p < np; p += PT) partc[lc].push_back(Tile{k, fl, p, std::min(np, p + PT)});
         int idx = 0;
         for (long long c = 0; c < N; c += ST) scan.push_back(Tile{k, idx++, c, std::min(N, c + ST)});
         B->most_scan = std::max(B->most_scan, idx);
@@ -660,7 +665,7 @@ static int grid_of(int ntiles) { return std::max(1, std::min(ntiles, 152 * 8)); 
 // block: these kernels hold 100-200 registers a thread, and 256-thread blocks
 // would leave one block per SM.
 static int part_threads(const Tuning &u, int lanes) {
-    const long long want = (long long)u.part_tile * lanes;
+    const long long want = (long long)part_tile(u) * lanes;
     const long long b = lanes > 1 && want > u.part_block && want <= 256 ? want : u.part_block;
     return (int)((b + 31) / 32 * 32);
 }
@@ -798,7 +803,7 @@ static void enqueue_step(Batch *B) {
             for (int sd = 0; sd < B->n_dem; ++sd) {
                 const int key_out = sd == B->n_dem - 1;
                 if (B->prec == DPS_F64) {
-                    launch_dem_substep64(T, B->d_part, B->n_part, sd & 1, key_out, B->any_walls, u.part_tile, s);
+                    launch_dem_substep64(T, B->d_part, B->n_part, sd & 1, key_out, B->any_walls, part_tile(u), s);
                     ndl += 2;  // pair kernel + gather kernel
                     continue;
                 }
@@ -811,7 +816,7 @@ static void enqueue_step(Batch *B) {
                         ++classes;
                     }
                 if (classes > 1) lanes = 0;
-                if (lanes == 8 && u.part_tile <= 32) {
+                if (lanes == 8 && part_tile(u) <= 32) {
                     const int n = B->solo ? B->n_dem : 1;
                     launch_dem_mixed8(T, B->d_part, B->n_part, sd, n, B->n_dem, B->any_walls, s);
                     sd += n - 1;
@@ -821,7 +826,7 @@ static void enqueue_step(Batch *B) {
                 // a block holds all lane groups of a particle tile, at most
                 // 256 threads (four such blocks fit an SM)
                 const int blk = (int)std::min<long long>(
-                    256, (std::max<long long>(u.part_block, (long long)u.part_tile * (lanes ? lanes : 8)) + 31) / 32 * 32);
+                    256, (std::max<long long>(u.part_block, (long long)part_tile(u) * (lanes ? lanes : 8)) + 31) / 32 * 32);
                 launch_dem_substep(T, B->d_part, B->n_part, sd & 1, key_out, lanes, B->any_walls, grid_of(B->n_part),
                                    blk, s);
                 ndl += 2;  // pair kernel + integration kernel
