@@ -60,8 +60,10 @@ extern "C" {
 typedef struct dps_domain *dps_handle;
 
 /* Device allocator hooks.  alloc returns a device pointer (NULL on failure,
- * which the library reports as DPS_ERR_OOM); free releases it.  Both NULL:
- * the library uses cudaMalloc / cudaFree. */
+ * which the library reports as DPS_ERR_OOM); free releases it.  Memory of any
+ * alignment is taken: a pointer off a multiple of 32 bytes is given back and
+ * asked for again with 32 bytes more.  Both NULL: the library uses cudaMalloc /
+ * cudaFree. */
 typedef void *(*dps_alloc_fn)(size_t bytes, void *ctx);
 typedef void (*dps_free_fn)(void *ptr, void *ctx);
 

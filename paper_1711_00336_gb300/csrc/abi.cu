@@ -12,6 +12,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 #include <system_error>
 #include <sys/mman.h>
@@ -142,6 +143,7 @@ struct Batch {
     dps_alloc_fn alloc = nullptr;
     dps_free_fn free = nullptr;
     void *ctx = nullptr;
+    std::map<void *, void *> shifted;  // memory moved up to DEV_ALIGN: as allocated
     std::string err;
     std::vector<BoxHost *> boxes;
     std::vector<BoxHost *> dev_order;  // box of each device-table entry (null: removed since)
@@ -194,23 +196,42 @@ static thread_local std::string g_create_err;
         if (_e != cudaSuccess) FAILB(b, DPS_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(_e)); \
     } while (0)
 
-static void *dalloc_raw(Batch *B, size_t bytes) {
-    if (bytes == 0) bytes = 16;
-    void *p = nullptr;
-    if (B->alloc) {
-        p = B->alloc(bytes, B->ctx);
-    } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        p = nullptr;
-    }
-    return p;
-}
-static void dfree_raw(Batch *B, void *p) {
-    if (!p) return;
+static void release_raw(Batch *B, void *p) {
     if (B->free)
         B->free(p, B->ctx);
     else
         cudaFree(p);
+}
+// the records of a pair (PairRes) are read as 32-byte words, the scans and the
+// float copies as 16-byte ones; a caller's allocator promises no alignment, so
+// memory off a multiple of 32 is given back and asked for with 32 bytes more
+constexpr size_t DEV_ALIGN = 32;
+static void *dalloc_raw(Batch *B, size_t bytes) {
+    if (bytes == 0) bytes = 16;
+    void *p = nullptr;
+    if (!B->alloc) {
+        if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
+    }
+    p = B->alloc(bytes, B->ctx);
+    if ((size_t)p % DEV_ALIGN == 0) return p;
+    release_raw(B, p);
+    void *const q = B->alloc(bytes + DEV_ALIGN, B->ctx);
+    if (!q) return nullptr;
+    p = (void *)(((size_t)q + DEV_ALIGN - 1) / DEV_ALIGN * DEV_ALIGN);
+    if (p != q) B->shifted[p] = q;
+    return p;
+}
+static void dfree_raw(Batch *B, void *p) {
+    if (!p) return;
+    const auto q = B->shifted.find(p);
+    if (q == B->shifted.end()) {
+        release_raw(B, p);
+    } else {
+        release_raw(B, q->second);
+        B->shifted.erase(q);
+    }
 }
 static void *box_alloc(Batch *B, BoxHost *h, size_t bytes) {
     void *p = dalloc_raw(B, bytes);
