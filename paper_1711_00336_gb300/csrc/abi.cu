@@ -85,6 +85,7 @@ void launch_fluid_sums(const void *, const void *, const void *, const Geom &, c
 void launch_particle_sums(const double *, const double *, long long, long long, double *, double *, cudaStream_t);
 void launch_particles_import(double *, int, long long, long long, const int *, const double *, cudaStream_t);
 void launch_rec_velocity(DemRec *, const double *, long long, long long, cudaStream_t);
+void launch_float_velocity(float4 *, float4 *, const double *, long long, long long, cudaStream_t);
 void launch_particles_export4(const BoxDev *, int, const double *, const int *, long long, long long, double *,
                               cudaStream_t);
 long long reduce_partials_doubles();
@@ -1414,8 +1415,11 @@ static int box_write_particles(Batch *B, BoxHost *h, long long n, const double *
         launch_particles_import(pf, 3 * k, h->d.cap, n, ids, buf, B->stream);
     }
     // without new positions the box is not sorted again, which would renew
-    // the records of the FP64 pair kernel
-    if (u3 && !x3 && h->d.rec[0]) launch_rec_velocity(h->d.rec[0], pf, h->d.cap, n, B->stream);
+    // the records of the FP64 pair kernel and the float copies of the mixed forms
+    if (!x3 && (u3 || w3)) {
+        if (h->d.lowp) launch_float_velocity(h->d.vf[0], h->d.of[0], pf, h->d.cap, n, B->stream);
+        else launch_rec_velocity(h->d.rec[0], pf, h->d.cap, n, B->stream);
+    }
     CKB(B, cudaFreeAsync(buf, B->stream));
     CKB(B, cudaStreamSynchronize(B->stream));
     if (x3) h->prepared = false;

@@ -323,6 +323,16 @@ __global__ void k_rec_velocity(DemRec *rec, const double *pf, long long cap, lon
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < np; i += (long long)gridDim.x * blockDim.x)
         for (int a = 0; a < 3; ++a) rec[i].u[a] = pf[(PU + a) * cap + i];
 }
+// the float copies of the mixed forms' velocities (v; .w keeps the mass) and spins (o), likewise
+__global__ void k_float_velocity(float4 *v, float4 *o, const double *pf, long long cap, long long np) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < np; i += (long long)gridDim.x * blockDim.x) {
+        v[i] = make_float4(to_float(pf[PU * cap + i]), to_float(pf[PV * cap + i]), to_float(pf[PW * cap + i]), v[i].w);
+        o[i] = make_float4(to_float(pf[POX * cap + i]), to_float(pf[POY * cap + i]), to_float(pf[POZ * cap + i]), 0.f);
+    }
+}
+void launch_float_velocity(float4 *v, float4 *o, const double *pf, long long cap, long long np, cudaStream_t s) {
+    if (np > 0) k_float_velocity<<<grid_for(np, 256), 256, 0, s>>>(v, o, pf, cap, np);
+}
 void launch_rec_velocity(DemRec *rec, const double *pf, long long cap, long long np, cudaStream_t s) {
     if (np > 0) k_rec_velocity<<<grid_for(np, 256), 256, 0, s>>>(rec, pf, cap, np);
 }
