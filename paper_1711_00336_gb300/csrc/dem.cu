@@ -568,7 +568,7 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
     const float4 xs = Bx.xs[i];  // position at the last sort, and d
     // walls: the faces of every non-periodic axis (m_ij = m_i, <d> = 2 d_i),
     // screened in FP32 (xs carries d) with the margin of the pair screen.  The
-    // FP64 form takes the lubrication from the integer path of the pairs and
+    // FP64 form takes the lubrication from the integer path (fx_wall) and
     // leaves contact to the FP64 body out of line: inlined, six faces' worth of
     // FP64 cost 211 registers a thread (closures with walls, 75 x 61 x 90: DEM
     // substep 67 -> 55 us with three blocks per SM, 64 with one)
@@ -585,16 +585,12 @@ __device__ __forceinline__ void finish_particle(const BoxDev &Bx, long long i, i
             if (per || (!(away < reach) && ph.far_ok)) continue;
             const double xa = a == 0 ? xi[0] : (a == 1 ? xi[1] : xi[2]);
             int kind = FX_EXACT;
-            if (F64 && ph.fx.ok && ph.lubrication && away > 0.f && away < 16.f) {
-                // lubrication as for a pair, with the wall a partner of no
-                // radius: 1/<d> = 1/(2 d_i)
+            if (F64 && ph.fx.ok && ph.lubrication) {
                 const DemPart q = Bx.part[Bx.cur][i];
-                const i64 x = fx_from(xa, ph.fx.frac);
-                const i64 dx[3] = {0, 0, side ? ((i64)n_a << ph.fx.frac) - x : x};
-                FxPair o;
-                kind = dx[2] > 0 ? fx_pair(dx, q.rad, (u64)q.inv_d, ph.fx, o) : FX_EXACT;
+                double al, be;
+                kind = fx_wall(fma(-0.5, pf[PD * cap + i], side ? n_a - xa : xa), (u64)q.inv_d, ph.h_c, ph.h_min,
+                               ph.fx, al, be);
                 if (kind == FX_LUB) {
-                    double al = o.alpha, be = o.beta;
                     const float capf = (float)ph.capfac * 0.999f;
                     if (ph.lub_limiter && !(fx_approx(be) * q.imf < capf && fx_approx(al) * q.imf < capf)) {
                         const double lim = pf[PM * cap + i] * ph.capfac;

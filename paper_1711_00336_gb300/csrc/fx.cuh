@@ -7,10 +7,12 @@
 // and an addition a tenth.  The separation, the unit normal, the gap, the
 // logarithm and the reciprocal of a lubrication pair therefore run on 64-bit
 // integers with 58 to 63 fraction bits, each value scaled so that its leading
-// bits are used: every intermediate result is at least as precise as the
-// FP64 one it replaces (53 bits).  The reciprocal and the reciprocal square
-// root are Newton's iteration from a single-precision seed, the logarithm a
-// table of 128 reciprocals and the Taylor series of ln(1 + u).
+// bits are used.  Against exact arithmetic the coefficients of a pair of spheres
+// are 2 to 40 times as close as FP64's (as close next to the origin of a box of
+// 512 cells or more); those of a wall, whose gap is taken in FP64, 2 to 3 times
+// (largest error of 20,000: 2.0e-16 and 5.8e-16).  The reciprocal and the
+// reciprocal square root are Newton's iteration from a single-precision seed, the
+// logarithm a table of 128 reciprocals and the Taylor series of ln(1 + u).
 //
 // Every function is host and device code with the same results up to the
 // single-precision seeds, whose last bits do not survive the iterations'
@@ -180,51 +182,11 @@ struct FxPair {
     double alpha, beta;  // shear and squeeze coefficients a_sh (2/(h+<d>))^2 and a_sq, before the limiter
 };
 
-// One pair (Sec. 3.1.3).  dx: x_j - x_i (minimum image) in units of 2^-frac, S
-// = rad_i + rad_j (fx_radius), I = fx_inv_d of i plus that of j.  FX_EXACT:
-// the pair overlaps or leaves the range of this path, the FP64 body decides;
-// FX_NONE: no force; FX_LUB: o holds the coefficients.
-__host__ __device__ __forceinline__ int fx_pair(const i64 dx[3], i64 S, u64 I, const FxBox &bx, FxPair &o) {
-    u64 a[3];
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-    for (int k = 0; k < 3; ++k) a[k] = (u64)(dx[k] < 0 ? -dx[k] : dx[k]);
-    // leading bit of the largest component at bit 62: a = x' 2^63, |x'| < 1
-    const u64 any = a[0] | a[1] | a[2];
-    const int s = fx_clz(any) - 1;
-    const int gf = s + bx.frac - 3, sl = gf - 56;
-    if (sl < 0 || sl > 24) return FX_EXACT;  // |dx| >= 16, or far below any radius of the path
-    u64 X[3], N2 = 0;
-#ifdef __CUDA_ARCH__
-#pragma unroll
-#endif
-    for (int k = 0; k < 3; ++k) {
-        X[k] = a[k] << s;
-        N2 += fx_mulhi(X[k], X[k]);  // |x'|^2 in units of 2^-62, in [1/4, 3)
-    }
-    // r = 1/|x'|: y (1 + e/2 + 3/8 e^2) with e = 1 - |x'|^2 y^2
-    const float yf = fx_rsqrt_seed((float)(u32)(N2 >> 32) * 0x1p-30f);
-    const u32 Y = (u32)(yf * 0x1p30f);
-    const i64 e = (i64)(1ull << 58) - (i64)fx_mulhi(N2, (u64)Y * Y);  // 2^-58
-    const i64 eh = (i64)(int)(e >> 8);
-    const i64 c = (e >> 1) + ((3 * ((eh * eh) >> 42)) >> 3);
-    const u64 R = ((u64)Y << 32) + (u64)(((c >> 32) * (i64)Y) * 64) + (((u64)(u32)c * Y) >> 26);  // 2^-62
-    // gap in units of 2^-gf: |dx| - S
-    const i64 D = (i64)fx_mulhi(N2, R);
-    if ((S >> (62 - sl)) != 0) return FX_EXACT;  // S past the scale of |dx|: deep overlap
-    const i64 G = D - (S << sl);
-    if (G < 0) return FX_EXACT;
-    if ((G >> sl) >= bx.hc) return FX_NONE;
-    // the floored gap hh = Hm 2^He
-    u64 Hm = bx.hmin_m;
-    int He = bx.hmin_e;
-    if ((G >> sl) >= bx.hmin) {
-        const int lz = fx_clz((u64)G);
-        Hm = (u64)G << lz;
-        He = -gf - lz;
-    }
-    // 1/<d> = I 2^-59; ir = hh/<d>, P = hh/<d>^2
+// The lubrication coefficients (Sec. 3.1.3) at the floored gap hh = Hm 2^He (leading
+// bit of Hm set) and 1/<d> = I 2^-59: alpha and beta as in FxPair.  FX_LUB, FX_NONE (both
+// are zero) or FX_EXACT (out of range).
+__host__ __device__ __forceinline__ int fx_lub(u64 Hm, int He, u64 I, const FxBox &bx, double &alpha, double &beta) {
+    // ir = hh/<d>, P = hh/<d>^2
     const int li = fx_clz(I);
     const u64 Im = I << li;
     u64 ir = fx_mulhi(Hm, Im);
@@ -269,12 +231,61 @@ __host__ __device__ __forceinline__ int fx_pair(const i64 dx[3], i64 S, u64 I, c
     const u64 La = (u64)(L < 0 ? -L : L);
     const int lL = fx_clz(La | 1);
     const u64 LI = fx_mulhi(La << lL, ir);  // |L| ir = LI 2^-(58+lL+q)
-    o.alpha = L > 0 ? fx_to_double(fx_mulhi(LI, CP), 56 + lL + q + Pe - bx.c_e) : 0.0;
+    alpha = L > 0 ? fx_to_double(fx_mulhi(LI, CP), 56 + lL + q + Pe - bx.c_e) : 0.0;
     const int st = lL + q - 2;  // >= 3: |L| ir < 1
     const i64 ta = (i64)(LI >> (st > 63 ? 63 : st));  // 2^-60
     const i64 W = 6225776124876973670ll + (i64)fx_mulhi(ir >> q, 1482327648780231826ull);  // 27/20 + 9/28 ir, 2^-62
     const i64 B3 = (3ll << 56) + fx_mulhi_s(L < 0 ? -ta : ta, W);  // 2^-58
-    o.beta = B3 > 0 ? fx_to_double(fx_mulhi((u64)B3 << 4, CP), 60 + Pe - bx.c_e) : 0.0;
+    beta = B3 > 0 ? fx_to_double(fx_mulhi((u64)B3 << 4, CP), 60 + Pe - bx.c_e) : 0.0;
+    return FX_LUB;
+}
+
+// One pair (Sec. 3.1.3).  dx: x_j - x_i (minimum image) in units of 2^-frac, S
+// = rad_i + rad_j (fx_radius), I = fx_inv_d of i plus that of j.  FX_EXACT:
+// the pair overlaps or leaves the range of this path, the FP64 body decides;
+// FX_NONE: no force; FX_LUB: o holds the coefficients.
+__host__ __device__ __forceinline__ int fx_pair(const i64 dx[3], i64 S, u64 I, const FxBox &bx, FxPair &o) {
+    u64 a[3];
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k) a[k] = (u64)(dx[k] < 0 ? -dx[k] : dx[k]);
+    // leading bit of the largest component at bit 62: a = x' 2^63, |x'| < 1
+    const u64 any = a[0] | a[1] | a[2];
+    const int s = fx_clz(any) - 1;
+    const int gf = s + bx.frac - 3, sl = gf - 56;
+    if (sl < 0 || sl > 24) return FX_EXACT;  // |dx| >= 16, or far below any radius of the path
+    u64 X[3], N2 = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int k = 0; k < 3; ++k) {
+        X[k] = a[k] << s;
+        N2 += fx_mulhi(X[k], X[k]);  // |x'|^2 in units of 2^-62, in [1/4, 3)
+    }
+    // r = 1/|x'|: y (1 + e/2 + 3/8 e^2) with e = 1 - |x'|^2 y^2
+    const float yf = fx_rsqrt_seed((float)(u32)(N2 >> 32) * 0x1p-30f);
+    const u32 Y = (u32)(yf * 0x1p30f);
+    const i64 e = (i64)(1ull << 58) - (i64)fx_mulhi(N2, (u64)Y * Y);  // 2^-58
+    const i64 eh = (i64)(int)(e >> 8);
+    const i64 c = (e >> 1) + ((3 * ((eh * eh) >> 42)) >> 3);
+    const u64 R = ((u64)Y << 32) + (u64)(((c >> 32) * (i64)Y) * 64) + (((u64)(u32)c * Y) >> 26);  // 2^-62
+    // gap in units of 2^-gf: |dx| - S
+    const i64 D = (i64)fx_mulhi(N2, R);
+    if ((S >> (62 - sl)) != 0) return FX_EXACT;  // S past the scale of |dx|: deep overlap
+    const i64 G = D - (S << sl);
+    if (G < 0) return FX_EXACT;
+    if ((G >> sl) >= bx.hc) return FX_NONE;
+    // the floored gap hh = Hm 2^He
+    u64 Hm = bx.hmin_m;
+    int He = bx.hmin_e;
+    if ((G >> sl) >= bx.hmin) {
+        const int lz = fx_clz((u64)G);
+        Hm = (u64)G << lz;
+        He = -gf - lz;
+    }
+    const int kind = fx_lub(Hm, He, I, bx, o.alpha, o.beta);
+    if (kind != FX_LUB) return kind;
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
@@ -282,6 +293,19 @@ __host__ __device__ __forceinline__ int fx_pair(const i64 dx[3], i64 S, u64 I, c
         o.n[k] = fx_with_sign(fx_to_double(fx_mulhi(X[k], R), 61), dx[k]);
     }
     return FX_LUB;
+}
+
+// A wall of gap h >= 0 (FP64: one subtraction, exact for small gaps; through the
+// positions' fixed-point copies the gap 1e-5 of a sphere at x < 1/4 would lose five
+// digits) and I = fx_inv_d of the sphere, 1/<d> = 1/(2 d).
+__host__ __device__ __forceinline__ int fx_wall(double h, u64 I, double h_c, double h_min, const FxBox &bx,
+                                                double &alpha, double &beta) {
+    if ((i64)fx_bits(h) < 0) return FX_EXACT;  // overlap
+    if (fx_bits(h) >= fx_bits(h_c)) return FX_NONE;
+    u64 Hm = bx.hmin_m;
+    int He = bx.hmin_e;
+    if (fx_bits(h) >= fx_bits(h_min)) fx_split(h, Hm, He);
+    return fx_lub(Hm, He, I, bx, alpha, beta);
 }
 
 }  // namespace dps
