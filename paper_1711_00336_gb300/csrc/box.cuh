@@ -98,14 +98,18 @@ struct Tile {
 // iterate the tiles of a launch: one block per tile, blocks stride over tiles
 #define DPS_FOR_TILES(tiles, ntiles, t) for (int t = blockIdx.x; t < (ntiles); t += gridDim.x)
 
-// a brick tile packs its origin (Tile::begin) and extent (Tile::end), 21 bits an axis
-__host__ __device__ inline long long brick_pack(int x, int y, int z) {
-    return (long long)x | ((long long)y << 21) | ((long long)z << 42);
+// a brick tile: its origin (any cell of a box of 2^27) and extent (up to 8 an axis)
+__host__ __device__ inline Tile brick_tile(int box, int x, int y, int z, int ex, int ey, int ez) {
+    return Tile{box, 0, (long long)x | ((long long)y << 32),
+                (long long)z | ((long long)ex << 32) | ((long long)ey << 40) | ((long long)ez << 48)};
 }
-__device__ __forceinline__ void brick_unpack(long long v, int &x, int &y, int &z) {
-    x = (int)(v & 0x1FFFFF);
-    y = (int)((v >> 21) & 0x1FFFFF);
-    z = (int)((v >> 42) & 0x1FFFFF);
+__host__ __device__ __forceinline__ void brick_of(const Tile &t, int &x, int &y, int &z, int &ex, int &ey, int &ez) {
+    x = (int)t.begin;
+    y = (int)(t.begin >> 32);
+    z = (int)t.end;
+    ex = (int)(t.end >> 32) & 0xff;
+    ey = (int)(t.end >> 40) & 0xff;
+    ez = (int)(t.end >> 48) & 0xff;
 }
 
 }  // namespace dps

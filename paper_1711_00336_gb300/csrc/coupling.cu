@@ -343,7 +343,7 @@ template <> __device__ __forceinline__ const float *weights_of<float>(const BoxD
 
 // ---- brick-tiled gathers ---------------------------------------------------------
 // A brick is a block of up to 8x8x8 cells of one box (Tile::begin and
-// Tile::end pack its origin and extent, 21 bits per axis).  The block first
+// Tile::end pack its origin and extent).  The block first
 // stages the particles of the brick's cells and their one-cell halo in
 // shared memory, then every thread gathers over the 27 neighbours of its cells
 // in a fixed order: o_z, o_y, o_x ascending, then the sorted order inside a
@@ -586,8 +586,7 @@ __device__ __forceinline__ void brick_gather(const BoxDev &B, unsigned char *sme
                                              const FT *__restrict__ w, Val &&value, Fin &&fin) {
     BrickStage<FT, NV, SPARSE> &S = *(BrickStage<FT, NV, SPARSE> *)smem;
     int ox, oy, oz, ex, ey, ez;
-    brick_unpack(tl.begin, ox, oy, oz);
-    brick_unpack(tl.end, ex, ey, ez);
+    brick_of(tl, ox, oy, oz, ex, ey, ez);
     int z = 0, dz = ez;
 #pragma unroll 1
     while (z < ez) {
@@ -1028,7 +1027,7 @@ void brick_tiles(int box, const int n[3], std::vector<Tile> &out) {
                 const int ex = n[0] - x < BRICK ? n[0] - x : BRICK;
                 const int ey = n[1] - y < BRICK ? n[1] - y : BRICK;
                 const int ez = n[2] - z < BRICK ? n[2] - z : BRICK;
-                out.push_back(Tile{box, 0, brick_pack(x, y, z), brick_pack(ex, ey, ez)});
+                out.push_back(brick_tile(box, x, y, z, ex, ey, ez));
             }
 }
 

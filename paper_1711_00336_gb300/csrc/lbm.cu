@@ -569,8 +569,7 @@ __global__ void __launch_bounds__(256, DPS_FIELDS32_MINB) k_fields32(const BoxDe
         const Geom g = B.g;
         const long long N = g.ncell;
         int ox, oy, oz, ex, ey, ez;
-        brick_unpack(tl.begin, ox, oy, oz);
-        brick_unpack(tl.end, ex, ey, ez);
+        brick_of(tl, ox, oy, oz, ex, ey, ez);
         const float *rho = (const float *)B.rho, *uD = (const float *)B.uD;
         float *uprev = (float *)B.uprev, *gradP = (float *)B.gradP, *DuDt = (float *)B.DuDt;
         const int have_prev = B.have_uprev;
@@ -680,8 +679,7 @@ __global__ void __launch_bounds__(256) k_fields64(const BoxDev *__restrict__ box
         const Geom g = B.g;
         const long long N = g.ncell;
         int ox, oy, oz, ex, ey, ez;
-        brick_unpack(tl.begin, ox, oy, oz);
-        brick_unpack(tl.end, ex, ey, ez);
+        brick_of(tl, ox, oy, oz, ex, ey, ez);
         const double *rho = (const double *)B.rho, *uD = (const double *)B.uD;
         if (threadIdx.x < 2) top[threadIdx.x] = 0;
         __syncthreads();  // (also: the previous brick is done with S)
@@ -828,8 +826,7 @@ __global__ void __launch_bounds__(256) k_curl64(const BoxDev *__restrict__ boxes
         const Geom g = B.g;
         const long long N = g.ncell;
         int ox, oy, oz, ex, ey, ez;
-        brick_unpack(tl.begin, ox, oy, oz);
-        brick_unpack(tl.end, ex, ey, ez);
+        brick_of(tl, ox, oy, oz, ex, ey, ez);
         const double *rho = (const double *)B.rho, *j = (const double *)B.j, *eps = (const double *)B.eps;
         const double hb[3] = {0.5 * B.ph.fb[0], 0.5 * B.ph.fb[1], 0.5 * B.ph.fb[2]};
         double *uf = (double *)B.fam, *curl = (double *)B.curl;
