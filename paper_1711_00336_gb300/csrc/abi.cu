@@ -290,10 +290,14 @@ struct ReadSeg {
 };
 constexpr size_t RING_CHUNK = 1u << 20;
 constexpr int RING_N = 8;
-constexpr size_t DIRECT_MAX = 24u << 20;
 
-// every page of [p, p + n) is in memory
+// [p, p + n) is memory of CUDA's own (pinned, managed), or every page of it is in memory
 static bool pages_exist(void *p, size_t n) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess)
+        cudaGetLastError();
+    else if (at.type != cudaMemoryTypeUnregistered)
+        return true;
     const size_t pg = (size_t)sysconf(_SC_PAGESIZE), a = (size_t)p / pg * pg;
     std::vector<unsigned char> in(((size_t)p + n - a + pg - 1) / pg);
     if (mincore((void *)a, (size_t)p + n - a, in.data()) != 0) return false;
@@ -309,10 +313,10 @@ static int read_back(Batch *B, const std::vector<ReadSeg> &segs) {
         total += segs[k].bytes;
         joined &= k == 0 || (const char *)segs[k - 1].src + segs[k - 1].bytes == segs[k].src;
     }
-    // one array up to this size whose pages exist: the driver's pageable copy, 15
-    // GB/s (6.3 MB 0.40 ms, through the ring 0.52; 50 MB 2.9 and 1.8).  Into
-    // pages not touched yet it makes 1 GB/s (16.8 MB 15 ms, the ring 1.2).
-    if (segs.size() == 1 && total <= DIRECT_MAX && pages_exist(segs[0].dst, total)) {
+    // one array whose pages exist, pinned or not: the driver's copy (50 MB 0.49 ms,
+    // through the ring 1.14; 170 MB 1.45 and 3.0).  Into pages not touched yet it
+    // makes 1 GB/s (16.8 MB 15 ms, the ring 1.2).
+    if (segs.size() == 1 && total > 0 && pages_exist(segs[0].dst, total)) {
         CKB(B, cudaMemcpyAsync(segs[0].dst, segs[0].src, total, cudaMemcpyDeviceToHost, B->stream));
         CKB(B, cudaStreamSynchronize(B->stream));
         return DPS_OK;
