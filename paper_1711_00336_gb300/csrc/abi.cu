@@ -281,8 +281,9 @@ static void tend(Batch *B, int phase, int nl, cudaStream_t on = nullptr) {
 // buffer into fresh pages moves ~5 GB/s (page faults), which made the read of
 // 1.6 million particles 29 ms of a 76 ms pass; so the data goes through a ring
 // of eight pinned 1 MB chunks (kept with the batch) that up to
-// eight threads empty while the copies of the next chunks run: that read 29 ->
-// 15 ms, the particles of 256^3 (182 MB) 24 -> 6 ms.
+// eight threads (seven helpers over all calls of the process) empty while the
+// copies of the next chunks run: that read 29 -> 15 ms, the particles of 256^3
+// (182 MB) 24 -> 6 ms.
 struct ReadSeg {
     void *dst;
     const void *src;
@@ -305,6 +306,17 @@ static bool pages_exist(void *p, size_t n) {
         if (!(v & 1)) return false;
     return true;
 }
+
+// threads that help with a read-back, over all calls of the process
+constexpr int HELPERS_MAX = 7;
+static std::atomic<int> g_helpers{0};
+struct Helpers {
+    int n;
+    explicit Helpers(int want) : n(std::max(0, std::min(want, HELPERS_MAX - g_helpers.fetch_add(want)))) {
+        g_helpers -= want - n;
+    }
+    ~Helpers() { g_helpers -= n; }
+};
 
 static int read_back(Batch *B, const std::vector<ReadSeg> &segs) {
     size_t total = 0;
@@ -398,9 +410,10 @@ static int read_back(Batch *B, const std::vector<ReadSeg> &segs) {
             }
         }
     };
+    const Helpers helpers(std::min(n, want) - 1);
     std::vector<std::thread> team;
     try {
-        for (int k = 1; k < std::min(n, want); ++k) team.emplace_back(work, false);
+        for (int k = 0; k < helpers.n; ++k) team.emplace_back(work, false);
     } catch (const std::system_error &) {  // no more threads: those that run do the work
     }
     work(true);
