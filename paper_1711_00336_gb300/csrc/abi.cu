@@ -13,8 +13,8 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <new>
 #include <string>
-#include <system_error>
 #include <sys/mman.h>
 #include <thread>
 #include <unistd.h>
@@ -318,17 +318,17 @@ struct Helpers {
     ~Helpers() { g_helpers -= n; }
 };
 
-static int read_back(Batch *B, const std::vector<ReadSeg> &segs) {
+static int read_back_segs(Batch *B, const ReadSeg *segs, size_t ns) {
     size_t total = 0;
     bool joined = true;  // the sources follow one another
-    for (size_t k = 0; k < segs.size(); ++k) {
+    for (size_t k = 0; k < ns; ++k) {
         total += segs[k].bytes;
         joined &= k == 0 || (const char *)segs[k - 1].src + segs[k - 1].bytes == segs[k].src;
     }
     // one array whose pages exist, pinned or not: the driver's copy (50 MB 0.49 ms,
     // through the ring 1.14; 170 MB 1.45 and 3.0).  Into pages not touched yet it
     // makes 1 GB/s (16.8 MB 15 ms, the ring 1.2).
-    if (segs.size() == 1 && total > 0 && pages_exist(segs[0].dst, total)) {
+    if (ns == 1 && total > 0 && pages_exist(segs[0].dst, total)) {
         CKB(B, cudaMemcpyAsync(segs[0].dst, segs[0].src, total, cudaMemcpyDeviceToHost, B->stream));
         CKB(B, cudaStreamSynchronize(B->stream));
         return DPS_OK;
@@ -341,9 +341,9 @@ static int read_back(Batch *B, const std::vector<ReadSeg> &segs) {
                                                  1 + total / (2u << 20));
     const size_t len = std::min(RING_CHUNK, std::max<size_t>(256u << 10, (total / (2 * want) + 4095) / 4096 * 4096));
     std::vector<ReadSeg> ch;
-    for (const ReadSeg &g : segs)
-        for (size_t o = 0; o < g.bytes; o += len)
-            ch.push_back({(char *)g.dst + o, (const char *)g.src + o, std::min(len, g.bytes - o)});
+    for (size_t k = 0; k < ns; ++k)
+        for (size_t o = 0; o < segs[k].bytes; o += len)
+            ch.push_back({(char *)segs[k].dst + o, (const char *)segs[k].src + o, std::min(len, segs[k].bytes - o)});
     const int n = (int)ch.size();
     if (n == 0) {
         CKB(B, cudaStreamSynchronize(B->stream));
@@ -412,14 +412,21 @@ static int read_back(Batch *B, const std::vector<ReadSeg> &segs) {
     };
     const Helpers helpers(std::min(n, want) - 1);
     std::vector<std::thread> team;
+    team.reserve((size_t)helpers.n);  // (nothing throws between the first thread and the joins)
     try {
         for (int k = 0; k < helpers.n; ++k) team.emplace_back(work, false);
-    } catch (const std::system_error &) {  // no more threads: those that run do the work
+    } catch (const std::exception &) {  // no more threads or memory for one: those that run do the work
     }
     work(true);
     for (std::thread &t : team) t.join();
     if (err != (int)cudaSuccess) FAILB(B, DPS_ERR_CUDA, "read-back: %s", cudaGetErrorString((cudaError_t)(int)err));
     return DPS_OK;
+}
+// no exception leaves a C entry
+static int read_back(Batch *B, const ReadSeg *segs, size_t ns) try {
+    return read_back_segs(B, segs, ns);
+} catch (const std::bad_alloc &) {
+    FAILB(B, DPS_ERR_OOM, "read-back: out of host memory");
 }
 
 // ---- physics constants of a box ---------------------------------------------
@@ -1367,7 +1374,8 @@ static int box_read_fields(Batch *B, BoxHost *h, uint32_t mask, double *out, lon
             else
                 launch_to_double<float>(src, planes[b] * N, buf, B->stream);
         }
-        if ((rc = read_back(B, {{out + off, buf, (size_t)(8 * planes[b] * N)}}))) {
+        const ReadSeg seg = {out + off, buf, (size_t)(8 * planes[b] * N)};
+        if ((rc = read_back(B, &seg, 1))) {
             cudaFreeAsync(buf, B->stream);
             return rc;
         }
@@ -1407,10 +1415,11 @@ static int box_read_particles(Batch *B, BoxHost *h, double *x3, double *u3, doub
     launch_particles_export4(k >= 0 ? B->d_table : nullptr, k, h->d.pf[h->d.cur], h->d.pi[h->d.cur] + IID * h->d.cap,
                              h->d.cap, np, B->d_pstage, B->stream);
     double *dst[4] = {x3, u3, w3, F3};
-    std::vector<ReadSeg> segs;
+    ReadSeg segs[4];
+    size_t ns = 0;
     for (int q = 0; q < 4; ++q)
-        if (dst[q]) segs.push_back({dst[q], B->d_pstage + (size_t)q * 3 * np, 8 * 3 * (size_t)np});
-    return read_back(B, segs);
+        if (dst[q]) segs[ns++] = {dst[q], B->d_pstage + (size_t)q * 3 * np, 8 * 3 * (size_t)np};
+    return read_back(B, segs, ns);
 }
 
 static int box_write_particles(Batch *B, BoxHost *h, long long n, const double *x3, const double *u3, const double *w3) {
@@ -1860,7 +1869,8 @@ int dps_read_pdfs(dps_handle h, double *out, int64_t cap) {
     PREC_CALL(B, launch_pdf_export<double>(d.pdf, d.g, B->parity, buf, B->stream),
               launch_pdf_export<float>(d.pdf, d.g, B->parity, buf, B->stream),
               launch_pdf_export<__half>(d.pdf, d.g, B->parity, buf, B->stream));
-    rc = read_back(B, {{out, buf, (size_t)(8 * Q * N)}});
+    const ReadSeg seg = {out, buf, (size_t)(8 * Q * N)};
+    rc = read_back(B, &seg, 1);
     CKB(B, cudaFreeAsync(buf, B->stream));
     CKB(B, cudaStreamSynchronize(B->stream));
     return rc;
