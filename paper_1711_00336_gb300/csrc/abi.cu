@@ -49,6 +49,7 @@ void launch_bsort_flip(BoxDev *, int, int, cudaStream_t);
 void launch_end_step(BoxDev *, int, cudaStream_t);
 int launch_bscan(const BoxDev *, int, const Tile *, int, int, cudaStream_t);
 int scan_tile_cells();
+int bscan_launches(int);
 void brick_tiles(int, const int *, std::vector<Tile> &);
 template <typename FT>
 void launch_eps(const BoxDev *, const Tile *, int, int, cudaStream_t);
@@ -598,6 +599,29 @@ static int force_lanes(const BoxHost *h) {
 // every particle tile starts at a multiple of 32, whatever size was asked for.
 static int part_tile(const Tuning &u) { return (u.part_tile + 31) / 32 * 32; }
 
+// the launch shapes of the batch: those that were set, or the defaults for its size
+static Tuning launch_shapes(const Batch *B) {
+    Tuning u = B->tune;
+    if (B->shape_fixed) return u;
+    // particle tiles: small enough that every SM gets a block when
+    // the batch holds few particles (a particle thread is latency- or
+    // FP64-bound, so spreading them over all SMs is what counts)
+    long long npt = 0, nc = 0;
+    for (const BoxHost *h : B->boxes) {
+        npt += h->d.np;
+        nc += h->d.g.ncell;
+    }
+    u.part_tile = 256;
+    while (u.part_tile > 32 && npt < 2LL * 152 * u.part_tile) u.part_tile /= 2;
+    u.part_block = std::min(128, u.part_tile);
+    // the same for the cell tiles: 32 x 32 x 64 cells in tiles of 1024
+    // would keep 64 of the 152 SMs busy (step of that box, FP64: 264 us;
+    // with tiles of 128: 201 us; 64^3: 548 and 526 us)
+    u.cell_tile = 1024;
+    while (u.cell_tile > 128 && nc < 8LL * 152 * u.cell_tile) u.cell_tile /= 2;
+    return u;
+}
+
 // rebuild the device table and the tile lists from the host boxes (the
 // device step state must have been pulled first)
 static int push_layout(Batch *B) {
@@ -618,25 +642,7 @@ static int push_layout(Batch *B) {
     std::vector<Tile> cell, part, scan, brick;
     const long long ST = scan_tile_cells();
     std::vector<Tile> cellv;  // cell tiles of the boxes with a per-cell tau_e
-    if (!B->shape_fixed) {
-        // default particle tiles: small enough that every SM gets a block when
-        // the batch holds few particles (a particle thread is latency- or
-        // FP64-bound, so spreading them over all SMs is what counts)
-        long long npt = 0;
-        for (BoxHost *h : B->boxes) npt += h->d.np;
-        int pt = 256;
-        while (pt > 32 && npt < 2LL * 152 * pt) pt /= 2;
-        B->tune.part_tile = pt;
-        B->tune.part_block = std::min(128, pt);
-        // the same for the cell tiles: 32 x 32 x 64 cells in tiles of 1024
-        // would keep 64 of the 152 SMs busy (step of that box, FP64: 264 us;
-        // with tiles of 128: 201 us; 64^3: 548 and 526 us)
-        long long nc = 0;
-        for (BoxHost *h : B->boxes) nc += h->d.g.ncell;
-        int ct = 1024;
-        while (ct > 128 && nc < 8LL * 152 * ct) ct /= 2;
-        B->tune.cell_tile = ct;
-    }
+    B->tune = launch_shapes(B);
     const int PT = part_tile(B->tune);
     std::vector<Tile> partc[4];  // particle tiles by DEM lanes class
     B->any_lift = false;
@@ -717,6 +723,7 @@ static int part_threads(const Tuning &u, int lanes) {
 }
 
 // ---- the coupled step --------------------------------------------------------------
+constexpr int SOLO_TILES = 4 * 152;  // boxes that one launch for all FP64 substeps takes
 #define PREC_CALL(B, F64CALL, F32CALL, F16CALL) \
     do {                                        \
         if ((B)->prec == DPS_F64) {             \
@@ -842,7 +849,7 @@ static void enqueue_step(Batch *B) {
         if (fork) cudaEventRecord(B->ev_join, B->side);
         tbegin(B);
         int ndl = 0;
-        if (pl && f64 && B->solo && B->n_part <= 4 * 152) {
+        if (pl && f64 && B->solo && B->n_part <= SOLO_TILES) {
             launch_dem_solo64(T, B->d_part, B->n_part, B->n_dem, B->any_walls, s);
             ndl = 1;
         } else if (pl)
@@ -2006,15 +2013,32 @@ static void b_get_timing(Batch *B, double *ms, int64_t *nl, int reset) {
         }
     }
 }
+// launches of the next step: counted as it was recorded, or, before the first step
+// and after a change of the boxes or closures, as enqueue_step will launch
 static long long b_launches_per_step(Batch *B) {
-    if (B->launches_step > 0) return B->launches_step;  // counted as the step was recorded
-    long long np = 0;
-    for (BoxHost *h : B->boxes) np += h->d.np;
-    const int pl = np > 0;
-    const int n_int = B->boxes.empty() ? 1 : B->boxes[0]->cl.n_int;
-    const int n_dem = B->boxes.empty() ? 1 : B->boxes[0]->cl.n_dem;
-    const int f64 = B->prec == DPS_F64;
-    return 2 + 2 + (long long)n_int * (2 * pl + 2 + pl * n_dem * 2 + 2 + (5 + 2 * f64) * pl + 1 + 1);
+    if (B->launches_step > 0 && !B->layout_dirty) return B->launches_step;
+    const int PT = part_tile(launch_shapes(B)), ST = scan_tile_cells();
+    long long tiles = 0;
+    int classes = 0, most_scan = 0, kinds = 0;  // bits of the lane classes and of the K1 variants
+    bool lift = false, solo = true;
+    for (const BoxHost *h : B->boxes) {
+        const bool c = h->have_closure;
+        lift |= c && h->cl.lift && h->d.np > 0;
+        kinds |= c && (h->cl.eilers || h->cl.smagorinsky) ? 2 : 1;
+        solo &= h->d.np <= std::min(128, PT);
+        tiles += (h->d.np + PT - 1) / PT;
+        if (h->d.np > 0) classes |= 1 << dem_lanes_class(h);
+        most_scan = std::max(most_scan, (int)((h->d.g.ncell + ST - 1) / ST));
+    }
+    const int pl = tiles > 0;
+    const long long n_int = B->boxes.empty() ? 1 : B->boxes[0]->cl.n_int;
+    const long long n_dem = B->boxes.empty() ? 1 : B->boxes[0]->cl.n_dem;
+    long long dem = 2 * n_dem;
+    if (B->prec == DPS_F64 && solo && tiles <= SOLO_TILES) dem = 1;
+    if (B->prec != DPS_F64 && classes == 8 && PT <= 32) dem = solo ? 1 : n_dem;
+    const int rows = B->prec == DPS_F64 ? 2 : (B->prec == DPS_F16S ? 1 : 0);  // of the pair lists
+    const long long sort = bscan_launches(most_scan) + 1 + pl * (4 + rows);
+    return 2 + n_int * (pl * (2 + lift + dem) + 2 + sort + 1) + (kinds == 3 ? 2 : 1) + 1;
 }
 
 int dps_set_timing(dps_handle h, int enable) { return h ? b_set_timing(&h->B, enable) : DPS_ERR_ARG; }

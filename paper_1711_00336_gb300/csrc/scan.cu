@@ -232,13 +232,15 @@ __global__ void __launch_bounds__(BSCAN_THREADS) k_bscan_tiles(const BoxDev *__r
     if (base <= n - 1 && n - 1 < base + BSCAN_ITEMS) B.cell_start[n] = off;
 }
 
+int bscan_launches(int most_tiles) { return most_tiles <= BSCAN_DIRECT ? 2 : 3; }
+
 // most_tiles: scan tiles of the largest box; returns the launches
 int launch_bscan(const BoxDev *boxes, int nboxes, const Tile *scan_tiles, int ntiles, int most_tiles, cudaStream_t s) {
-    const int direct = most_tiles <= BSCAN_DIRECT;
+    const int direct = bscan_launches(most_tiles) == 2;
     k_bscan_sums<<<ntiles, BSCAN_THREADS, 0, s>>>(boxes, scan_tiles);
     if (!direct) k_bscan_parts<<<nboxes, BSCAN_THREADS, 0, s>>>(boxes, nboxes);
     k_bscan_tiles<<<ntiles, BSCAN_THREADS, 0, s>>>(boxes, scan_tiles, direct);
-    return direct ? 2 : 3;
+    return bscan_launches(most_tiles);
 }
 int scan_tile_cells() { return BSCAN_TILE; }
 
