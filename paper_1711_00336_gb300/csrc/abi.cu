@@ -293,19 +293,17 @@ struct ReadSeg {
 constexpr size_t RING_CHUNK = 1u << 20;
 constexpr int RING_N = 8;
 
-// [p, p + n) is memory of CUDA's own (pinned, managed), or every page of it is in memory
+// every page of [p, p + n) is in memory, or it is memory of CUDA's own (pinned, managed)
 static bool pages_exist(void *p, size_t n) {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess)
-        cudaGetLastError();
-    else if (at.type != cudaMemoryTypeUnregistered)
-        return true;
     const size_t pg = (size_t)sysconf(_SC_PAGESIZE), a = (size_t)p / pg * pg;
     std::vector<unsigned char> in(((size_t)p + n - a + pg - 1) / pg);
-    if (mincore((void *)a, (size_t)p + n - a, in.data()) != 0) return false;
-    for (unsigned char v : in)
-        if (!(v & 1)) return false;
-    return true;
+    if (mincore((void *)a, (size_t)p + n - a, in.data()) == 0 &&
+        std::all_of(in.begin(), in.end(), [](unsigned char v) { return v & 1; }))
+        return true;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type != cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+    return false;
 }
 
 // threads that help with a read-back, over all calls of the process
