@@ -70,9 +70,9 @@ def closure_of(wl):
 
 
 def algorithmic_bytes_collide(prec, mom_in=False):
-    """K1 per cell: 19 PDF loads + 19 stores, eps_f and f_pf (3) loads; in the
-    FP64 coupled step with a per-cell tau_e (mom_in) also rho and j (4) from the
-    moments pass."""
+    """K1 per cell: 19 PDF loads + 19 stores, eps_f and f_pf (3) loads.  mom_in: for
+    a collide-stream that reads rho and j (4) from the moments pass too, which
+    none of the present kernels does."""
     s = {"f64": 8, "f32": 4, "f16s": 2}[prec]
     sf = 8 if prec == "f64" else 4
     return 2 * 19 * s + (8 if mom_in else 4) * sf

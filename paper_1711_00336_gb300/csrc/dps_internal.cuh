@@ -10,8 +10,11 @@
 //   fields    planes of ncell values of the field type FT (double for DPS_F64,
 //             float otherwise): eps_f, rho, j(3), u_D(3), u_prev(3), DuDt(3),
 //             gradP(3), f_pf applied (3), f_pf of the subcycle (3), f_pf sum (3);
-//             with the lift force the u_D planes hold, during the subcycles,
-//             the curl of the subcycle-start fluid velocity
+//             during the subcycles the u_D planes hold, with the lift force, the
+//             curl of the subcycle-start fluid velocity until the added-mass
+//             forces are taken, then (FP64, BoxDev::ufield) u_f for the drag;
+//             the planes of the subcycle's f_pf hold u_f for the lift (FP64)
+//             until the added-mass reaction is gathered
 //   particles SoA of doubles [field][cap] in cell-sorted order, two sets
 //             (main / alternate) for the sort gather and the DEM ping-pong.
 #pragma once

@@ -10,9 +10,9 @@
 //    FP64: 207 FP64 warp instructions of ~19 cycles per 32 cells bound this
 //    pass; it runs in 64-bit fixed point (lbm_fx.cuh), ~1500 integer
 //    instructions of which two to four issue per cycle.  128^3, walls at z:
-//    815 -> 216 us; 256^3, coupled step: 4.88 -> 1.77 ms (floor at the
+//    815 -> 215 us; 256^3, coupled step: 4.88 -> 1.67 ms (floor at the
 //    measured copy rate: 0.10 and 0.83 ms).  With a
-//    per-cell tau_e only tau_e is FP64: 75 x 61 x 90, 229 -> 107 us.
+//    per-cell tau_e only tau_e is FP64: 75 x 61 x 90, 229 -> 105 us.
 // K2a moments: rho, j of f(x,t), u_D = (j + f_ext/2)/(rho eps_f) and
 //    1/(rho eps_f); one PDF read.
 // K2b fields: stencil over rho and u_D giving grad(eps_f p) and Du_f/Dt.
